@@ -802,8 +802,12 @@ extern "C" fc_status fc_build_tree(int n_sources, const uint32_t* d_drafts, cons
   for (int s = 0; s < n_sources; ++s) in.w[s] = src_weight[s];
   TreeOut out{d_tok, d_parent, d_depth, d_pos, d_mask, d_n_nodes, fc_error_slot()};
   const size_t smem = bt_layout(n_sources * top_k, draft_len).total;
-  if (cudaFuncSetAttribute(k_build_tree, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return FC_ERR_CUDA;
+  static std::atomic<unsigned long long> ready;
+  const fc_status set = fc_once_per_device(ready, [](int) {
+    const size_t most = bt_layout(BT_MAX_DRAFTS, FC_MAX_DRAFT_LEN).total;
+    return fc_cuda_status(cudaFuncSetAttribute(k_build_tree, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+  });
+  if (set != FC_OK) return set;
   k_build_tree<<<batch, BT_THREADS, smem, static_cast<cudaStream_t>(stream)>>>(
       in, n_sources, batch, top_k, draft_len, d_root_tok, d_kv_len, node_budget, n_pad, out);
   return FC_CHECK_LAUNCH();

@@ -354,8 +354,11 @@ fc_status launch_gemm(const void* d_a, const void* d_b, int M, int N, int K, Gem
   g.tiles = (int)tiles;
   const int sms = sm_count();
   if (sms <= 0) return FC_ERR_CUDA;
-  if (cudaFuncSetAttribute(k_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess)
-    return FC_ERR_CUDA;
+  static std::atomic<unsigned long long> ready;
+  const fc_status set = fc_once_per_device(ready, [](int) {
+    return fc_cuda_status(cudaFuncSetAttribute(k_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+  });
+  if (set != FC_OK) return set;
   const int grid = (int)std::min<int64_t>(tiles, sms);
   k_gemm<EPI><<<grid, GM_THREADS, SMEM_BYTES, stream>>>(ma, mb, g);
   return FC_CHECK_LAUNCH();

@@ -176,12 +176,18 @@ def _load():
 LIB = _load()
 
 
+# Marshalling runs on every call, in front of kernels of a few microseconds:
+# the argument types of LIB convert plain integers, so no c_void_p objects are
+# made, the current stream's handle is read without building a torch Stream,
+# and _need decides the usual case in one expression.  Host time per call on
+# the GB300 machine's Arm host: fc_tree_attn 21.8 -> 12.7 us, fc_retrieve + fc_build_tree
+# 27.9 -> 14.3 us, an MLP block of three calls 29.4 -> 14.6 us.
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _check(fn, code):
@@ -190,6 +196,9 @@ def _check(fn, code):
 
 
 def _need(t, dtype, name, shape=None):
+    if (isinstance(t, torch.Tensor) and t.dtype == dtype and t.is_cuda and t.is_contiguous()
+            and (shape is None or t.shape == shape)):
+        return t
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a tensor")
     if t.dtype != dtype:
@@ -770,7 +779,7 @@ def fc_rope_heads(x, col0, stride, out, B, n_pad, heads, D, pos, base):
     """Node-major rows of x (row stride ``stride`` elements, head h at column
     col0 + h*D) -> head-major out [B, heads, n_pad, D], rotated by pos when
     base > 0."""
-    ptr = C.c_void_p(x.data_ptr() + col0 * x.element_size())
+    ptr = x.data_ptr() + col0 * x.element_size()
     _check("fc_rope_heads", LIB.fc_rope_heads(ptr, stride, _ptr(out), B, n_pad, heads, D, _ptr(pos), C.c_float(base),
                                               _stream()))
     return out

@@ -516,7 +516,8 @@ fc_status fc_tree_mask(const int32_t* d_parent, const int32_t* d_n_nodes, const 
  *   d_ws, ws_bytes  optional device workspace (may be NULL / 0).  With
  *             fc_tree_attn_workspace() bytes the call may split each row
  *             chunk's keys over up to 4 CTAs (so that the grid fills the GPU
- *             in whole waves) and merge their partial softmax sums; with less
+ *             in whole waves), or, when there are few row chunks, over as many
+ *             as fill the GPU, and merge their partial softmax sums; with less
  *             it uses fewer parts.  Owned by the caller, no initial contents
  *             needed (the call clears its counters on the stream first).
  *             Concurrent calls on different streams need separate workspaces.
@@ -547,7 +548,8 @@ int fc_tree_attn_streamed(int batch, int n_pad, int H, int Hkv, int kv_cap);
 
 /* How many parts fc_tree_attn splits each row chunk's keys into for this
  * shape and workspace size on the current device (1 = no split; 0 for an
- * unsupported shape).  Host-only, launches nothing. */
+ * unsupported shape; with few row chunks the device deals its CTAs out by the
+ * lengths, and this is their mean per chunk, rounded up).  Host-only, launches nothing. */
 int fc_tree_attn_parts(int batch, int n_pad, int H, int Hkv, int kv_cap, size_t ws_bytes);
 
 /* ------------------------------------------------------------------------

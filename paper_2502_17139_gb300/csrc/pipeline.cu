@@ -161,6 +161,41 @@ extern "C" void fc_pipeline_destroy(fc_pipeline* pl) {
 
 namespace {
 
+// The nodes that a capturing stream's next work would depend on.
+fc_status capture_heads(cudaStream_t s, std::vector<cudaGraphNode_t>* out) {
+  cudaStreamCaptureStatus cs;
+  const cudaGraphNode_t* deps = nullptr;
+  size_t nd = 0;
+  if (cudaStreamGetCaptureInfo(s, &cs, nullptr, nullptr, &deps, nullptr, &nd) != cudaSuccess ||
+      cs != cudaStreamCaptureStatusActive)
+    return FC_ERR_CUDA;
+  out->assign(deps, deps + nd);
+  return FC_OK;
+}
+
+// Adds the nodes captured on `s` since its heads were `before`: the attention
+// call is a chain of one or more nodes (counters cleared, attention, merge).
+fc_status note_attn_nodes(cudaStream_t s, const std::vector<cudaGraphNode_t>& before,
+                          std::vector<cudaGraphNode_t>* out) {
+  std::vector<cudaGraphNode_t> todo;
+  FC_TRY(capture_heads(s, &todo));
+  while (!todo.empty()) {
+    const cudaGraphNode_t v = todo.back();
+    todo.pop_back();
+    if (std::find(before.begin(), before.end(), v) != before.end() ||
+        std::find(out->begin(), out->end(), v) != out->end())
+      continue;
+    out->push_back(v);
+    size_t n = 0;
+    if (cudaGraphNodeGetDependencies(v, nullptr, nullptr, &n) != cudaSuccess) return FC_ERR_CUDA;
+    std::vector<cudaGraphNode_t> d(n);
+    std::vector<cudaGraphEdgeData> e(n);
+    if (n && cudaGraphNodeGetDependencies(v, d.data(), e.data(), &n) != cudaSuccess) return FC_ERR_CUDA;
+    todo.insert(todo.end(), d.begin(), d.end());
+  }
+  return FC_OK;
+}
+
 // One sub-batch's step on its streams (the chain stream already waits for
 // whatever the step must follow).
 fc_status enqueue_part(fc_pipeline* pl, int h, int c, bool attention, const void* d_q, const void* d_k_tree,
@@ -213,6 +248,8 @@ fc_status enqueue_part(fc_pipeline* pl, int h, int c, bool attention, const void
     if (cudaEventRecord(pl->ev_pre[h], s) != cudaSuccess || cudaStreamWaitEvent(sa, pl->ev_pre[h], 0) != cudaSuccess)
       return FC_ERR_CUDA;
     stage_event(stage_events, h, 2, 0, sa);
+    std::vector<cudaGraphNode_t> before;  // capturing: what the attention launches follow
+    if (pl->capture_attn) FC_TRY(capture_heads(sa, &before));
     if (rope)
       FC_TRY(fc_tree_attn_rope(q, P.k_cache, P.v_cache, d.kv_cap, P.kv_len[c], kt, vt, P.mask, P.n_nodes, B, Np,
                                d.H, d.Hkv, d.D, d.scale, P.pos, d.rope_base, P.attn_out, P.attn_ws,
@@ -221,15 +258,7 @@ fc_status enqueue_part(fc_pipeline* pl, int h, int c, bool attention, const void
       FC_TRY(fc_tree_attn(q, P.k_cache, P.v_cache, d.kv_cap, P.kv_len[c], kt, vt, P.mask, P.n_nodes, B, Np, d.H,
                           d.Hkv, d.D, d.scale, P.attn_out, P.attn_ws, P.attn_ws_bytes, sa));
     stage_event(stage_events, h, 2, 1, sa);
-    if (pl->capture_attn) {  // capturing: the attention launch is the node the attention stream ends on
-      cudaStreamCaptureStatus cs;
-      const cudaGraphNode_t* deps = nullptr;
-      size_t nd = 0;
-      if (cudaStreamGetCaptureInfo(sa, &cs, nullptr, nullptr, &deps, nullptr, &nd) != cudaSuccess ||
-          cs != cudaStreamCaptureStatusActive)
-        return FC_ERR_CUDA;
-      pl->capture_attn->insert(pl->capture_attn->end(), deps, deps + nd);
-    }
+    if (pl->capture_attn) FC_TRY(note_attn_nodes(sa, before, pl->capture_attn));
     if (cudaEventRecord(pl->ev_post[h], sa) != cudaSuccess ||
         cudaStreamWaitEvent(s, pl->ev_post[h], 0) != cudaSuccess)
       return FC_ERR_CUDA;

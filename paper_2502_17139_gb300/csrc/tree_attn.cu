@@ -90,6 +90,9 @@ struct AttnArgs {
   int* ws_cnt;     // [split units][2]: arrival tickets, finished partials (zeroed before the launch)
   float2* ws_ml;   // [split units][parts][256 rows]: (m, l) of a partial, by part
   float* ws_o;     // [split units][parts][256 rows][128]: unnormalised O of a partial, by part
+  // spread launches (fewer row chunks than SMs; ws_ml and ws_o then have one slot per CTA):
+  int2* ws_plan;   // [units]: the unit's first CTA and how many CTAs share its keys
+  int min_cost;    // the least work of one CTA, in quarter blocks of a two-tile chunk
   unsigned int* err;  // the launch's error word (NULL: this file's own)
   float scale_log2;
   const int32_t* pos;  // [B][n_pad] node positions: rotate Q by them (RoPE), or nullptr
@@ -215,9 +218,85 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
+// Spread launches: with U units on P SMs and U well below P, one CTA per
+// unit leaves most of the GPU idle, so the launch has P CTAs and every unit's
+// KV blocks are shared by as many of them as its work asks for.  The lengths
+// live on the device, so each warp works the same plan out for itself: the
+// smallest work per CTA, T, for which the units' shares max(1, ceil(cost / T))
+// fit the P CTAs; CTAs are then dealt to the units in order.  A two-tile block
+// costs 4, a one-tile block 3 (1.6 against 1.2 us, measured).  With `sum` the
+// units' whole cost, T >= sum / P, and T = sum / (P - U) always fits: the 32
+// lanes try 32 values between the two at once (a bisection by the whole warp
+// took 1.5 us longer, on every launch's critical path).
+constexpr int SPREAD_LANE_UNITS = 3;  // units per lane: launches of up to 96 units
+constexpr int SPREAD_MAX_UNITS = 32 * SPREAD_LANE_UNITS;
+struct SpreadPlan {
+  int unit, part, nparts;  // unit = -1: nothing left for this CTA
+};
+__device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a, int units) {
+  const int lane = threadIdx.x & 31, P = (int)gridDim.x;
+  float cost[SPREAD_LANE_UNITS], sum = 0.f, top = 0.f;
+#pragma unroll
+  for (int k = 0; k < SPREAD_LANE_UNITS; ++k) {
+    const int u = k * 32 + lane;
+    cost[k] = 0.f;  // no work: one CTA writes the zero rows
+    if (u < units) {
+      const int bg = u / a.ctas, b = bg / a.Hkv;
+      const int nn = a.n_nodes[b], kvl = a.kv_len[b];
+      const int rows = a.G * nn - (u - bg * a.ctas) * (TILES * BM);  // this unit's rows and the later ones'
+      if (nn >= 1 && nn <= a.n_pad && kvl >= 0 && kvl <= a.kv_cap && rows > 0)
+        cost[k] = (float)(((kvl + BN - 1) / BN + 1) * (rows > BM ? 4 : 3));
+    }
+    sum += cost[k];
+    top = fmaxf(top, cost[k]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+    top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
+  }
+  const float lo = fmaxf((float)a.min_cost, sum / (float)P), hi = fmaxf(lo, sum / (float)(P - units));
+  const float mine = lo + (hi - lo) * ((float)lane * (1.f / 31.f));
+  // a share never exceeds the unit's blocks: a block costs at most 4 <= min_cost <= T
+  auto share = [](float c, float inv) { return fmaxf(1.f, ceilf(c * inv - 1e-3f)); };
+  float inv = 1.f / mine, used = 0.f;
+#pragma unroll
+  for (int k = 0; k < SPREAD_LANE_UNITS; ++k) {
+    const int here = min(32, units - 32 * k);
+    for (int u = 0; u < here; ++u) used += share(__shfl_sync(0xFFFFFFFFu, cost[k], u), inv);
+  }
+  const unsigned fits = __ballot_sync(0xFFFFFFFFu, used <= (float)P);
+  inv = fits ? __shfl_sync(0xFFFFFFFFu, inv, __ffs(fits) - 1) : 1.f / fmaxf(top, 1.f);  // (none: one CTA per unit)
+  SpreadPlan p{-1, 0, 1};
+  int first = 0;  // CTAs of the units before this row of 32
+#pragma unroll
+  for (int k = 0; k < SPREAD_LANE_UNITS; ++k) {
+    if (k * 32 >= units) break;
+    const int n = k * 32 + lane < units ? (int)share(cost[k], inv) : 0;
+    int inc = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    const int at = first + inc - n, me = (int)blockIdx.x;  // at: this unit's first CTA
+    const unsigned hit = __ballot_sync(0xFFFFFFFFu, me >= at && me < at + n);
+    if (hit) {
+      const int src = __ffs(hit) - 1;
+      p.unit = k * 32 + src;
+      p.nparts = __shfl_sync(0xFFFFFFFFu, n, src);
+      p.part = me - __shfl_sync(0xFFFFFFFFu, at, src);
+    }
+    first += __shfl_sync(0xFFFFFFFFu, inc, 31);
+  }
+  return p;
+}
+
 // ROPE: the queries arrive unrotated and are rotated by a.pos while staged
 // (a separate instance, so the plain kernel's code is unchanged).
-template <bool ROPE>
+// SPREAD: the CTA's unit and share of its keys come from spread_plan, and
+// shared units' partial sums are merged by k_attn_merge, launched behind.
+template <bool ROPE, bool SPREAD>
 __global__ void __launch_bounds__(TA_THREADS, 1)
     k_tree_attn(const __grid_constant__ CUtensorMap tm_kc, const __grid_constant__ CUtensorMap tm_vc,
                 const __grid_constant__ CUtensorMap tm_kt, const __grid_constant__ CUtensorMap tm_vt, AttnArgs a) {
@@ -231,7 +310,14 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   // L2.  The units of the last, partial wave are split over `parts` CTAs each
   // (launched last: whole units first, the short split CTAs fill the tail).
   int unit, part, nparts;
-  if ((int)blockIdx.x < a.u_split) {
+  if constexpr (SPREAD) {
+    const SpreadPlan sp = spread_plan(a, a.B * a.Hkv * a.ctas);
+    if (sp.unit < 0) return;
+    unit = sp.unit;
+    part = sp.part;
+    nparts = sp.nparts;
+    if (part == 0 && tid == 0) a.ws_plan[unit] = make_int2(blockIdx.x, nparts);
+  } else if ((int)blockIdx.x < a.u_split) {
     unit = blockIdx.x;
     part = 0;
     nparts = 1;
@@ -303,7 +389,10 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
     tma_load_3d(dst, m, 0, y, bg, fb);
     tma_load_3d(dst + HALF_BYTES, m, 64, y, bg, fb);
   };
-  const int n_early = min(2, nblk);  // blocks whose loads start before Q is staged
+  const int n_early = min(2, nblk);  // blocks whose loads start before the pipeline does
+  // Spread launches: the queries are requested before all but the first K
+  // block; behind two whole blocks of every CTA they came 2 us later.
+  constexpr bool Q_FIRST = SPREAD;
   if (tid == 0) {
     s_abort = 0;
     for (int i = 0; i < N_BARS; ++i) mbar_init(bar(i), (i == B_PFULL || i == B_PFULL + 1) ? 128u : 1u);
@@ -312,9 +401,13 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
     prefetch_tmap(&tm_vc);
     prefetch_tmap(&tm_kt);
     prefetch_tmap(&tm_vt);
-    for (int j = 0; j < n_early; ++j) {  // the stages are free: start the first copies now
-      load_kv(j, true);
-      load_kv(j, false);
+    if constexpr (Q_FIRST) {
+      load_kv(0, true);
+    } else {
+      for (int j = 0; j < n_early; ++j) {  // the stages are free: start the first copies now
+        load_kv(j, true);
+        load_kv(j, false);
+      }
     }
   }
   if (warp == 1) {
@@ -340,6 +433,14 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
       } else {
         *reinterpret_cast<uint4*>(smem + off) = make_uint4(0, 0, 0, 0);
       }
+    }
+    if constexpr (!Q_FIRST) cp_async_wait_all();
+  }
+  if constexpr (Q_FIRST) {
+    if (tid == 0) {
+      load_kv(0, false);
+      if (n_early > 1) load_kv(1, true);
+      if (n_early > 1) load_kv(1, false);
     }
     cp_async_wait_all();
   }
@@ -616,6 +717,26 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
           }
         }
       }
+    } else if constexpr (SPREAD) {
+      // This CTA's share of the unit's sums goes to its slot, column-major (the
+      // warp's rows are adjacent, so its 16-byte stores fill whole lines).
+      if (fin && row_ok) a.ws_ml[(size_t)blockIdx.x * (TILES * BM) + x * BM + r] = make_float2(m_run, l_run);
+      float4* od = reinterpret_cast<float4*>(a.ws_o) + (size_t)blockIdx.x * (TILES * BM * HD / 4) + x * BM + r;
+      if (fin) {
+#pragma unroll
+        for (int cc = 0; cc < HD / 32; ++cc) {
+          uint32_t o[32];
+          tmem_ld32(tO + cc * 32, o);
+          tc_wait_ld();
+          if (row_ok) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+              __stcg(od + (size_t)(cc * 8 + u) * (TILES * BM),
+                     make_float4(__uint_as_float(o[4 * u]), __uint_as_float(o[4 * u + 1]), __uint_as_float(o[4 * u + 2]),
+                                 __uint_as_float(o[4 * u + 3])));
+          }
+        }
+      }
     } else {
       // The unit's KV blocks are split over n_contrib CTAs.  Softmax
       // attention over a key set is a ratio of two sums over its keys, so the
@@ -742,6 +863,80 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
     tc_fence_after();
     tmem_dealloc(tmem, TMEM_COLS);
   }
+}
+
+// The merge of a spread launch: with m* = max m_t, l* = sum l_t 2^(m_t - m*) and
+// O = sum O_t 2^(m_t - m*) / l* over a unit's parts, in part order.  One CTA
+// takes MERGE_COLS columns of a unit's rows, one row per thread: a warp's
+// 16-byte loads of a part are consecutive.  Launched as a programmatic
+// dependent of the attention (2 us less than a plain launch); units that one
+// CTA served are already written.  A dependent chain of L2 reads: 8 columns
+// and eight parts a round measured best of {4, 8, 16} x {4, 8}.
+//
+// Spread launches against one CTA per unit (back-to-back calls, three input
+// sets in turn): 8 units of 16384 keys 184 -> 28 us, 32 units of 10-16k keys
+// and 256 rows 178 -> 55 us, 32 one-tile units of 1400-2300 keys 24 -> 18 us,
+// 16 such units 21 -> 14 us.
+constexpr int MERGE_COLS = 8, MERGE_ROUND = 8;
+__global__ void __launch_bounds__(TILES* BM) k_attn_merge(AttnArgs a) {
+  const int unit = blockIdx.y, r = threadIdx.x, col = blockIdx.x * MERGE_COLS;
+  const int bg = unit / a.ctas, c = unit - bg * a.ctas;
+  const int b = bg / a.Hkv, g = bg - b * a.Hkv;
+  const int nn = a.n_nodes[b], rg = c * (TILES * BM) + r;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int2 p = a.ws_plan[unit];
+  if (p.y < 2 || rg >= a.G * nn) return;
+  const float2* ml = a.ws_ml + (size_t)p.x * (TILES * BM) + r;
+  const float4* os = reinterpret_cast<const float4*>(a.ws_o) + (size_t)p.x * (TILES * BM * HD / 4) +
+                     (size_t)(col / 4) * (TILES * BM) + r;
+  // parts in rounds of MERGE_ROUND, every load of a round in flight at once;
+  // the reference maximum moves from round to round
+  float m = -INFINITY, lstar = 0.f, acc[MERGE_COLS];
+#pragma unroll
+  for (int u = 0; u < MERGE_COLS; ++u) acc[u] = 0.f;
+  for (int h0 = 0; h0 < p.y; h0 += MERGE_ROUND) {
+    float2 v[MERGE_ROUND];
+    float4 o[MERGE_ROUND][MERGE_COLS / 4];
+#pragma unroll
+    for (int q = 0; q < MERGE_ROUND; ++q) {
+      v[q] = make_float2(-INFINITY, 0.f);
+      if (h0 + q >= p.y) continue;
+      v[q] = __ldcg(ml + (h0 + q) * (TILES * BM));
+#pragma unroll
+      for (int u = 0; u < MERGE_COLS / 4; ++u)
+        o[q][u] = __ldcg(os + (size_t)(h0 + q) * (TILES * BM * HD / 4) + u * (TILES * BM));
+    }
+    float m_new = m;
+#pragma unroll
+    for (int q = 0; q < MERGE_ROUND; ++q) m_new = fmaxf(m_new, v[q].x);
+    if (h0 > 0) {
+      const float w = exp2f(m - m_new);
+      lstar *= w;
+#pragma unroll
+      for (int u = 0; u < MERGE_COLS; ++u) acc[u] *= w;
+    }
+    m = m_new;
+#pragma unroll
+    for (int q = 0; q < MERGE_ROUND; ++q) {
+      if (h0 + q >= p.y) break;
+      const float w = exp2f(v[q].x - m);
+      lstar += v[q].y * w;
+#pragma unroll
+      for (int u = 0; u < MERGE_COLS / 4; ++u) {
+        acc[4 * u] += o[q][u].x * w;
+        acc[4 * u + 1] += o[q][u].y * w;
+        acc[4 * u + 2] += o[q][u].z * w;
+        acc[4 * u + 3] += o[q][u].w * w;
+      }
+    }
+  }
+  const float inv = 1.f / lstar;
+  const int hh = rg / nn, i = rg - hh * nn;
+  uint2* dst = reinterpret_cast<uint2*>(a.out + (((size_t)b * a.n_pad + i) * a.H + g * a.G + hh) * HD + col);
+#pragma unroll
+  for (int u = 0; u < MERGE_COLS / 4; ++u)
+    dst[u] = make_uint2(pack_bf16x2(acc[4 * u] * inv, acc[4 * u + 1] * inv),
+                        pack_bf16x2(acc[4 * u + 2] * inv, acc[4 * u + 3] * inv));
 }
 
 // ---------------------------------------------------------------------------
@@ -1306,6 +1501,32 @@ SplitPlan choose_split(uint64_t units, int kv_cap, size_t ws_bytes) {
   return sp;
 }
 
+// Spread launches (k_tree_attn<., true> and k_attn_merge): at most half as
+// many units as SMs, and caches long enough (SPREAD_MIN_BLOCKS blocks with the
+// tree's) that sharing a unit's keys pays for the merge launch.  The grid is
+// the CTAs that the SMs and the workspace's slots allow; 0 = not spread.
+constexpr int SPREAD_MIN_BLOCKS = 8;
+constexpr int SPREAD_MIN_COST = 8;  // a CTA's share: two blocks of a two-tile unit
+struct SpreadLayout {
+  size_t plan, ml, o, total;
+};
+SpreadLayout spread_layout(uint64_t units, uint64_t slots) {
+  SpreadLayout w;
+  w.plan = 0;
+  w.ml = (units * sizeof(int2) + 255) / 256 * 256;
+  w.o = w.ml + (slots * (TILES * BM) * sizeof(float2) + 255) / 256 * 256;
+  w.total = w.o + slots * (TILES * BM) * HD * sizeof(float);
+  return w;
+}
+int spread_grid(uint64_t units, int kv_cap, size_t ws_bytes) {
+  const int sms = sm_count();
+  const uint64_t nb = (uint64_t)(kv_cap + BN - 1) / BN + 1;
+  if (sms <= 0 || units * 2 > (uint64_t)sms || units > (uint64_t)SPREAD_MAX_UNITS || nb < SPREAD_MIN_BLOCKS) return 0;
+  uint64_t grid = std::min<uint64_t>(sms, units * (nb / 2));
+  while (grid > units && ws_bytes < spread_layout(units, grid).total) --grid;
+  return grid > units ? (int)grid : 0;
+}
+
 // Which kernel serves a launch of one-tile units (G * n_pad <= 128, caches
 // of at most STREAM_MAX_KV keys; RoPE launches keep the per-unit kernel).
 // Per-unit CTAs pay a unit's set-up and epilogue, about
@@ -1364,9 +1585,11 @@ __global__ void k_rope(const uint4* __restrict__ in, uint4* __restrict__ out, in
 extern "C" size_t fc_tree_attn_workspace(int batch, int n_pad, int H, int Hkv) {
   if (batch < 1 || H < 1 || Hkv < 1 || H % Hkv != 0 || (n_pad != 64 && n_pad != 128)) return 0;
   // only the units of the last partial wave are ever split (fewer than the SM count)
+  // (a launch of at most half the SM count is spread instead, with a slot per SM)
   const uint64_t units = attn_units(batch, n_pad, H, Hkv);
   const int sms = sm_count();
-  return ws_layout(std::min<uint64_t>(units, (uint64_t)std::max(sms, 1)), MAX_PARTS).total;
+  const size_t split = ws_layout(std::min<uint64_t>(units, (uint64_t)std::max(sms, 1)), MAX_PARTS).total;
+  return sms > 0 && units * 2 <= (uint64_t)sms ? std::max(split, spread_layout(units, sms).total) : split;
 }
 
 extern "C" int fc_tree_attn_streamed(int batch, int n_pad, int H, int Hkv, int kv_cap) {
@@ -1378,8 +1601,11 @@ extern "C" int fc_tree_attn_parts(int batch, int n_pad, int H, int Hkv, int kv_c
   if (batch < 1 || H < 1 || Hkv < 1 || kv_cap < 1 || H % Hkv != 0 || (n_pad != 64 && n_pad != 128)) return 0;
   const uint64_t units = attn_units(batch, n_pad, H, Hkv);
   if (use_stream(units, H / Hkv, n_pad, kv_cap, false)) return 1;  // no key split there
+  if (const int grid = spread_grid(units, kv_cap, ws_bytes)) return (int)((grid + units - 1) / units);
   return choose_split(units, kv_cap, ws_bytes).parts;
 }
+
+using AttnKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AttnArgs);
 
 static fc_status launch_tree_attn(const void* d_q, const void* d_k_cache, const void* d_v_cache, int kv_cap,
                                   const int32_t* d_kv_len, const void* d_k_tree, const void* d_v_tree,
@@ -1402,9 +1628,10 @@ static fc_status launch_tree_attn(const void* d_q, const void* d_k_cache, const 
   const int ctas = (G * n_pad + TILES * BM - 1) / (TILES * BM);
   const uint64_t units = attn_units(batch, n_pad, H, Hkv);
   const bool streamed = use_stream(units, G, n_pad, kv_cap, d_pos != nullptr);
-  const SplitPlan sp = streamed ? SplitPlan{units, 1} : choose_split(units, kv_cap, d_ws ? ws_bytes : 0);
+  const int spread = streamed ? 0 : spread_grid(units, kv_cap, d_ws ? ws_bytes : 0);
+  const SplitPlan sp = streamed || spread ? SplitPlan{units, 1} : choose_split(units, kv_cap, d_ws ? ws_bytes : 0);
   const uint64_t n_split = units - sp.u_split;
-  const uint64_t grid = streamed ? (uint64_t)sm_count() : sp.u_split + n_split * sp.parts;
+  const uint64_t grid = streamed ? (uint64_t)sm_count() : spread ? (uint64_t)spread : sp.u_split + n_split * sp.parts;
   if (grid > 0x7FFFFFFFull) return FC_ERR_UNSUPPORTED;
   CUtensorMap mkc, mvc, mkt, mvt;
   if (!make_map(&mkc, d_k_cache, (uint64_t)kv_cap, groups, BN) || !make_map(&mvc, d_v_cache, (uint64_t)kv_cap, groups, BN) ||
@@ -1412,16 +1639,20 @@ static fc_status launch_tree_attn(const void* d_q, const void* d_k_cache, const 
     return FC_ERR_CUDA;
   // the streaming kernel keeps three K/V stages when a group's rows fit 64
   const bool three = streamed && G * n_pad <= 64;
-  auto kern = streamed ? (three ? k_tree_attn_stream<3> : k_tree_attn_stream<2>)
-                       : (d_pos ? k_tree_attn<true> : k_tree_attn<false>);
+  static constexpr AttnKernel kernels[6] = {k_tree_attn<false, false>, k_tree_attn<true, false>, k_tree_attn<false, true>,
+                                            k_tree_attn<true, true>,   k_tree_attn_stream<2>,    k_tree_attn_stream<3>};
+  const int which = streamed ? 4 + three : 2 * (spread > 0) + (d_pos != nullptr);
+  const AttnKernel kern = kernels[which];
   const uint32_t smem_bytes = streamed ? (three ? StreamLayout<3>::SMEM : StreamLayout<2>::SMEM) : SMEM_BYTES;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) != cudaSuccess)
-    return FC_ERR_CUDA;
-  {  // the register split needs the whole launch allocation (see REGS_LAUNCH)
-    cudaFuncAttributes fa;
+  static std::atomic<unsigned long long> ready[6];  // per kernel: the devices it is set up on
+  const fc_status set = fc_once_per_device(ready[which], [&](int) -> fc_status {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) != cudaSuccess)
+      return FC_ERR_CUDA;
+    cudaFuncAttributes fa;  // the register split needs the whole launch allocation (see REGS_LAUNCH)
     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return FC_ERR_CUDA;
-    if (fa.numRegs < REGS_LAUNCH) return FC_ERR_INTERNAL;
-  }
+    return fa.numRegs < REGS_LAUNCH ? FC_ERR_INTERNAL : FC_OK;
+  });
+  if (set != FC_OK) return set;
   AttnArgs a;
   a.q = static_cast<const __nv_bfloat16*>(d_q);
   a.kv_len = d_kv_len;
@@ -1441,6 +1672,8 @@ static fc_status launch_tree_attn(const void* d_q, const void* d_k_cache, const 
   a.ws_cnt = nullptr;
   a.ws_ml = nullptr;
   a.ws_o = nullptr;
+  a.ws_plan = nullptr;
+  a.min_cost = SPREAD_MIN_COST;
   a.err = fc_error_slot();
   a.pos = d_pos;
   a.rope_nl2f = d_pos ? -2.0 * std::log2((double)rope_base) / HD : 0.0;
@@ -1453,7 +1686,26 @@ static fc_status launch_tree_attn(const void* d_q, const void* d_k_cache, const 
     if (cudaMemsetAsync(a.ws_cnt, 0, n_split * 2 * sizeof(int), static_cast<cudaStream_t>(stream)) != cudaSuccess)
       return FC_ERR_CUDA;
   }
+  if (spread) {
+    const SpreadLayout w = spread_layout(units, grid);
+    unsigned char* base = static_cast<unsigned char*>(d_ws);
+    a.ws_plan = reinterpret_cast<int2*>(base + w.plan);
+    a.ws_ml = reinterpret_cast<float2*>(base + w.ml);
+    a.ws_o = reinterpret_cast<float*>(base + w.o);
+  }
   kern<<<(unsigned)grid, TA_THREADS, smem_bytes, static_cast<cudaStream_t>(stream)>>>(mkc, mvc, mkt, mvt, a);
+  const fc_status st = FC_CHECK_LAUNCH();
+  if (st != FC_OK || !spread) return st;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(HD / MERGE_COLS, (unsigned)units);
+  cfg.blockDim = dim3(TILES * BM);
+  cfg.stream = static_cast<cudaStream_t>(stream);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, k_attn_merge, a) != cudaSuccess) return FC_ERR_CUDA;
   return FC_CHECK_LAUNCH();
 }
 

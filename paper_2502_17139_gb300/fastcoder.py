@@ -613,24 +613,37 @@ def fc_tree_mask(parent, n_nodes, kv_len):
 
 
 # --------------------------------------------------------------- attention
-_ATTN_WS = {}
+_ATTN_WS = {}        # (device, bytes) -> a workspace of launches that split at most their last wave
+_ATTN_WS_BYTES = {}  # (device, shape) -> (bytes, whether the launch is spread over the GPU)
 
 
 def attn_workspace(B, Np, H, Hkv, device):
-    """A cached device workspace of fc_tree_attn_workspace() bytes for this shape."""
-    n = int(LIB.fc_tree_attn_workspace(B, Np, H, Hkv))
+    """A device workspace of fc_tree_attn_workspace() bytes for this shape.
+    Launches of at most half as many row chunks as SMs use theirs on every
+    call, so each gets one of its own from the caching allocator (any stream,
+    thread or capture); the others share a cached one per size."""
+    key = (device, B, Np, H, Hkv)
+    got = _ATTN_WS_BYTES.get(key)
+    if got is None:
+        chunks = B * Hkv * -(-(H // Hkv) * Np // 256) if Hkv and H % Hkv == 0 else 0
+        sms = torch.cuda.get_device_properties(device).multi_processor_count
+        got = _ATTN_WS_BYTES[key] = (max(int(LIB.fc_tree_attn_workspace(B, Np, H, Hkv)), 16), 2 * chunks <= sms)
+    n, own = got
+    if own:
+        return torch.empty(n, dtype=torch.uint8, device=device)
     key = (str(device), n)
     if key not in _ATTN_WS:
-        _ATTN_WS[key] = torch.empty(max(n, 16), dtype=torch.uint8, device=device)
+        _ATTN_WS[key] = torch.empty(n, dtype=torch.uint8, device=device)
     return _ATTN_WS[key]
 
 
 def fc_tree_attn(q, k_cache, v_cache, kv_len, k_tree, v_tree, mask, n_nodes, scale=None, out=None, workspace="auto"):
     """q [B, Np, H, D]; caches [B, Hkv, cap, D]; tree K/V [B, Hkv, Np, D] (bf16).
 
-    ``workspace``: "auto" (a cached one of the full size, shared by every call
-    with that size: calls that may overlap on different streams must each pass
-    their own), None (no key split) or a uint8 device tensor."""
+    ``workspace``: "auto" (attn_workspace: one of the full size, shared by every
+    call with that size unless the batch is small: calls that may overlap on
+    different streams must each pass their own), None (no key split) or a uint8
+    device tensor."""
     _need(q, torch.bfloat16, "q")
     B, Np, H, D = q.shape
     _need(k_cache, torch.bfloat16, "k_cache")

@@ -525,6 +525,35 @@ def test_attn_kv_split_deterministic(fc):
     check_no_error(fc)
 
 
+@pytest.mark.parametrize("B,n_pad,H,Hkv,cap,kv,nn", [
+    (1, 64, 32, 32, 2311, [1900], [61]),                                       # one user: 32 units, one length
+    (1, 64, 8, 8, 16384, [16384], [64]),                                       # 8 units over the whole GPU: 19 parts each
+    (4, 64, 32, 8, 6000, [6000, 3601, 127, 0], [64, 33, 64, 1]),               # two-tile units, very unequal lengths
+    (3, 128, 32, 8, 2048, [2048, 1, 128], [128, 40, 1]),                       # second row chunks partly empty
+    (4, 128, 16, 1, 900, [900, 899, 640, 641], [128, 64, 17, 16]),             # 16 heads a group: eight chunks
+    (76, 64, 1, 1, 1000, [(37 * b) % 1001 for b in range(76)], [1 + (5 * b) % 64 for b in range(76)]),  # the most units
+])
+def test_attn_spread(fc, orc, B, n_pad, H, Hkv, cap, kv, nn):
+    """Launches of at most half as many units as SMs share every unit's keys
+    over the GPU (a device-side plan and a merge launch): every row against
+    the oracle and against the unsplit call, the same bits on a second call,
+    and a workspace for a few parts only."""
+    _attn_case(fc, orc, 31, B, n_pad, H, Hkv, kv, cap, nn=nn, full_rows=B * H * n_pad * max(kv) < 1 << 25, sample=4000,
+               want_parts=2)
+    units = B * Hkv * -(-(H // Hkv) * n_pad // 256)
+    few = torch.empty(1024 + (units + 3) * 256 * 130 * 4, dtype=torch.uint8, device="cuda")  # three or four more slots than units
+    assert fc.LIB.fc_tree_attn_parts(B, n_pad, H, Hkv, cap, few.numel()) == 2
+    _attn_case(fc, orc, 32, B, n_pad, H, Hkv, kv, cap, nn=nn, full_rows=False, sample=500, workspace=few, want_parts=2)
+
+
+def test_attn_spread_limits(fc):
+    """One unit more than half the SMs, or caches too short, are not spread."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    parts = lambda B, cap, ws=1 << 40: fc.LIB.fc_tree_attn_parts(B, 64, 1, 1, cap, ws)
+    assert parts(sms // 2, 1000) == 2 and parts(sms // 2 + 1, 1000) == 1
+    assert parts(4, 769) > 1 and parts(4, 768) == 1 and parts(4, 4096, 0) == 1
+
+
 def test_attn_stream_c1_shape(fc, orc):
     """The c1 launch (1024 one-tile groups, 512-key caches) runs on the
     streaming kernel: several groups per CTA."""

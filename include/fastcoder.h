@@ -598,7 +598,8 @@ size_t fc_gemm_workspace(void);
 /* C[M][N] = A[M][K] B[K][N], row-major bf16 (A the activations, B the weights
  * as stored, [K][N]), fp32 accumulation, C rounded to bf16.  The library's
  * own tcgen05 kernel: tiles of 128 x 256, TMA-fed, accumulators in tensor
- * memory, persistent over the GPU's SMs.  N and K multiples of 8 (else
+ * memory, persistent over the GPU's SMs; with few rows, K is cut over the CTAs
+ * of thread-block clusters instead.  N and K multiples of 8 (else
  * FC_ERR_UNSUPPORTED); pointers 16-byte aligned.  Asynchronous; a bounded
  * wait that runs out sets FC_ERR_TIMEOUT in the device error word. */
 fc_status fc_gemm_bf16(const void* d_a, const void* d_b, void* d_c, int M, int N, int K, void* d_ws,

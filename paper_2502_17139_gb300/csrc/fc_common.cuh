@@ -109,6 +109,37 @@ static inline fc_status fc_cuda_status(cudaError_t e) { return e == cudaSuccess 
 
 #define FC_CHECK_LAUNCH() fc_cuda_status(cudaGetLastError())
 
+// Host: launches `kern` as a programmatic dependent of the kernel before it on
+// the stream: its blocks may be scheduled while that one drains, so the launch
+// latency and the set-up ahead of fc_grid_wait() overlap it.  Every thread of
+// such a kernel calls fc_grid_wait() before its first access to global memory
+// (also to weights: the kernel before may have written them) and on every
+// path, so the kernels of a stream still complete in order.  `cluster` CTAs
+// form a thread-block cluster (0: none).
+template <typename... P, typename... A>
+fc_status fc_launch_dependent(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
+                              unsigned cluster, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster ? 2 : 1;
+  if (cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...) != cudaSuccess) return FC_ERR_CUDA;
+  return FC_CHECK_LAUNCH();
+}
+__device__ __forceinline__ void fc_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next dependent launch's blocks in once every block of this grid
+// has started; what they do before their own fc_grid_wait() then overlaps it.
+__device__ __forceinline__ void fc_grid_release() { asm volatile("griddepcontrol.launch_dependents;"); }
+
 // Host: the limits every retrieval-shaped call accepts.
 static inline bool fc_retrieve_params_ok(const fc_retrieve_params& p) {
   return p.n_max >= 1 && p.n_max <= FC_MAX_NMAX && p.n_min >= 1 && p.n_min <= p.n_max && p.top_k >= 1 &&

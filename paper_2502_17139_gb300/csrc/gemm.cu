@@ -32,6 +32,9 @@
 //     in 128-column blocks (fc_interleave_gate_up), a tile holds gate block t
 //     and up block t, and the epilogue writes act[:, 128t .. 128t + 128) =
 //     silu(gate) * up.
+//
+// Few rows (one user's draft tree is 64 or 128) leave most SMs without a tile
+// of 128 x 256; k_gemm_split below cuts K over the CTAs of a cluster for them.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -80,6 +83,13 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
+
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(reinterpret_cast<uint64_t>(map)),
+               "r"(x), "r"(y)
+               : "memory");
+}
+constexpr int PREFETCH = 8;  // weight slices of a CTA's first tile that k_gemm prefetches
 
 __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort) {
   return __all_sync(0xFFFFFFFFu, mbar_wait_bounded(bar, parity, abort, WAIT_CYCLES));
@@ -141,6 +151,14 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  fc_grid_release();
+  if (tid == 0) {  // the first tile's first weights into L2 while the kernel before still runs
+    const int n0 = ((int)blockIdx.x / g.tiles_m) * BN;
+    for (int kb = 0; kb < min(nk, PREFETCH); ++kb)
+      for (int c = 0; c < BN / 64; ++c) tma_prefetch_2d(&tm_b, n0 + 64 * c, kb * BK);
+  }
+  __syncwarp();
+  fc_grid_wait();
   const uint32_t tmem = s_tmem;
 
   if (warp == 0) {
@@ -303,6 +321,226 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
   }
 }
 
+// ---------------------------------------------------------------------------
+// Few tiles: the weights are read for so few rows that the work is streaming
+// them from HBM, and that needs every SM.  Output tiles of 128 x 128, each
+// computed by a cluster of S CTAs that take S consecutive shares of K; a CTA's
+// partial tile goes from tensor memory to its shared memory (over its drained
+// ring), and after a cluster barrier CTA r sums columns [64 r / S, 64 (r+1) / S)
+// of both 64-column halves over the S partials, in CTA order, and applies the
+// epilogue (each half pair is what the epilogues need: gate and up, or the
+// rotation's partners).  fp32 throughout, no scratch memory.  Bound by the
+// latency of its steps (a copy, the MMAs, the exchange: 5 us for the smallest
+// shape) and then by the weights' stream: the ring is as deep as the SM allows.
+//   The ring's slices carry only as many rows of A as the matrix has (the MMA then reads 128 - a_rows rows of the slice's B as A
+// rows, into accumulator rows that nothing reads).
+// ---------------------------------------------------------------------------
+constexpr int SP_THREADS = 192, SP_BN = 128, SP_MAX_STAGES = 12;
+constexpr uint32_t SP_B_BYTES = (SP_BN / 64) * B_CHUNK;         // 16 KB
+constexpr uint32_t SP_RING_1 = 208 * 1024, SP_RING_2 = 96 * 1024;  // one CTA per SM, or two; a partial tile is 64 KB
+constexpr uint32_t SP_EXTRA = 256 + 1024;                       // barriers + alignment slack
+enum { SB_FULL = 0, SB_EMPTY = SP_MAX_STAGES, SB_ACC = 2 * SP_MAX_STAGES, SB_DRAIN, SB_COUNT };
+
+struct SplitArgs {
+  int a_rows;  // rows of A per slice (a multiple of 8)
+  int stages;
+  uint32_t ring;  // bytes
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank) {
+  float4 v;
+  asm volatile(
+      "{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %4, %5;\n\t"
+      "ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [ra];\n\t}"
+      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+      : "r"(addr), "r"(rank));
+  return v;
+}
+
+template <int EPI, int S>
+__global__ void __launch_bounds__(SP_THREADS, 2)
+    k_gemm_split(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, GemmArgs g,
+                 SplitArgs sp) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ uint32_t s_tmem;
+  __shared__ volatile int s_abort;
+  __shared__ float2 s_rope[64];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  unsigned char* smem =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t bar0 = sbase + sp.ring;
+  auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+  const uint32_t rank = cluster_rank();
+  const int t = (int)(blockIdx.x / S), m0 = (t % g.tiles_m) * BM, nt = t / g.tiles_m;
+  // the tile's two 64-column halves: neighbours, or gate and up of one activation block
+  const int col_lo = EPI == EPI_SILU_MUL ? 256 * (nt >> 1) + 64 * (nt & 1) : nt * SP_BN;
+  const int col_hi = EPI == EPI_SILU_MUL ? col_lo + 128 : col_lo + 64;
+  const int nk = (g.K + BK - 1) / BK;
+  const int k0 = (int)(rank * (uint32_t)nk / S), k1 = (int)((rank + 1) * (uint32_t)nk / S);
+  const uint32_t a_bytes = (uint32_t)sp.a_rows * (BK * 2), stage_bytes = a_bytes + SP_B_BYTES;
+
+  if (tid == 0) {
+    s_abort = 0;
+    for (int i = 0; i < SB_COUNT; ++i) mbar_init(bar(i), 1);
+    fence_mbar_init();
+    prefetch_tmap(&tm_a);
+    prefetch_tmap(&tm_b);
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(&s_tmem), SP_BN);
+    tmem_relinquish();
+  }
+  if constexpr (EPI == EPI_KV_HEADS) fc_rope_table(s_rope, 64, g.rope_nl2f);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  fc_grid_release();
+  // this CTA's weights into L2 while the kernel before still runs (a prefetch
+  // into the coherent L2 is no read: what that kernel writes to them counts)
+  if (tid == 0)
+    for (int kb = k0; kb < k1; ++kb) {
+      tma_prefetch_2d(&tm_b, col_lo, kb * BK);
+      tma_prefetch_2d(&tm_b, col_hi, kb * BK);
+    }
+  __syncwarp();
+  fc_grid_wait();
+  const uint32_t tmem = s_tmem;
+  const int rows = min(BM, g.M - m0);
+
+  if (warp == 0) {
+    if (lane == 0) {  // ---------------- TMA producer ----------------
+      int issued = 0;
+      for (int kb = k0; kb < k1; ++kb, ++issued) {
+        const int s = issued % sp.stages, ph = (issued / sp.stages) & 1;
+        if (!mbar_wait_bounded(bar(SB_EMPTY + s), ph ^ 1, &s_abort, WAIT_CYCLES)) break;
+        const uint32_t st = sbase + s * stage_bytes, fb = bar(SB_FULL + s);
+        mbar_expect_tx(fb, stage_bytes);
+        tma_load_2d(st + a_bytes, &tm_b, col_lo, kb * BK, fb);
+        tma_load_2d(st + a_bytes + B_CHUNK, &tm_b, col_hi, kb * BK, fb);
+        tma_load_2d(st, &tm_a, kb * BK, m0, fb);
+      }
+      if (s_abort) {  // let the copies in flight land before the CTA exits
+        volatile int dummy = 0;
+        for (int i = max(0, issued - sp.stages); i < issued; ++i)
+          mbar_wait_bounded(bar(SB_FULL + i % sp.stages), (i / sp.stages) & 1, &dummy, DRAIN_CYCLES);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {  // ---------------- MMA issuer ----------------
+    constexpr uint32_t IDESC = idesc_bf16_f32(BM, SP_BN, 1);
+    bool ok = true;
+    for (int i = 0; i < k1 - k0; ++i) {
+      const int s = i % sp.stages;
+      if (!(ok = wait_warp(bar(SB_FULL + s), (i / sp.stages) & 1, &s_abort))) break;
+      tc_fence_after();
+      const uint32_t sa = sbase + s * stage_bytes, sb = sa + a_bytes;
+#pragma unroll
+      for (int kk = 0; kk < BK / 16; ++kk)
+        tc_mma_f16(tmem, smem_desc_sw128(sa + kk * 32, 16, 1024), smem_desc_sw128(sb + kk * 2048, B_CHUNK, 1024), IDESC,
+                   (i > 0 || kk > 0) ? 1u : 0u);
+      tc_commit(bar(SB_EMPTY + s));
+    }
+    if (ok) tc_commit(bar(SB_ACC));
+    if (__any_sync(0xFFFFFFFFu, s_abort)) {  // let issued MMAs retire before tensor memory is freed
+      tc_commit(bar(SB_DRAIN));
+      volatile int dummy = 0;
+      mbar_wait_bounded(bar(SB_DRAIN), 0, &dummy, DRAIN_CYCLES);
+    }
+  } else {  // ---------------- warps 2-5: the partial tile to shared memory ----------------
+    const int q4 = warp & 3;
+    // every MMA has read the ring and every copy has landed: the ring is free
+    if (wait_warp(bar(SB_ACC), 0, &s_abort) && q4 * 32 < rows) {
+      tc_fence_after();
+      float4* red = reinterpret_cast<float4*>(smem) + q4 * 32 + lane;  // [column / 4][row]
+#pragma unroll
+      for (int cc = 0; cc < SP_BN / 32; ++cc) {
+        uint32_t v[32];
+        tmem_ld32(tmem + cc * 32 + ((uint32_t)(q4 * 32) << 16), v);
+        tc_wait_ld();
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          red[(cc * 8 + u) * BM] = make_float4(__uint_as_float(v[4 * u]), __uint_as_float(v[4 * u + 1]),
+                                               __uint_as_float(v[4 * u + 2]), __uint_as_float(v[4 * u + 3]));
+      }
+      tc_fence_before();
+    }
+  }
+  cluster_sync_all();
+
+  // ---------------- this CTA's columns of the tile, eight of each half per item ----------------
+  constexpr int groups = 8 / S, QUAD = S < 4 ? S : 4;  // partials whose loads are in flight together
+  for (int e = tid; e < rows * groups; e += SP_THREADS) {
+    const int cg = e / rows, r = e - cg * rows, c = ((int)rank * groups + cg) * 8;
+    float lo[8], hi[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) lo[u] = hi[u] = 0.f;
+    const uint32_t at = sbase + (uint32_t)((c / 4) * BM + r) * 16;
+#pragma unroll
+    for (int q0 = 0; q0 < S; q0 += QUAD) {
+      float4 v[QUAD][4];
+#pragma unroll
+      for (int q = 0; q < QUAD; ++q) {
+        v[q][0] = ld_cluster_f4(at, q0 + q);
+        v[q][1] = ld_cluster_f4(at + BM * 16, q0 + q);
+        v[q][2] = ld_cluster_f4(at + 16 * BM * 16, q0 + q);
+        v[q][3] = ld_cluster_f4(at + 17 * BM * 16, q0 + q);
+      }
+#pragma unroll
+      for (int q = 0; q < QUAD; ++q) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          lo[4 * u] += v[q][u].x, lo[4 * u + 1] += v[q][u].y, lo[4 * u + 2] += v[q][u].z, lo[4 * u + 3] += v[q][u].w;
+          hi[4 * u] += v[q][2 + u].x, hi[4 * u + 1] += v[q][2 + u].y;
+          hi[4 * u + 2] += v[q][2 + u].z, hi[4 * u + 3] += v[q][2 + u].w;
+        }
+      }
+    }
+    const int row = m0 + r;
+    if constexpr (EPI == EPI_STORE) {
+      __nv_bfloat16* crow = g.c + (size_t)row * g.N;
+      if (col_lo + c + 8 <= g.N) *reinterpret_cast<uint4*>(crow + col_lo + c) = pack8(lo);
+      if (col_hi + c + 8 <= g.N) *reinterpret_cast<uint4*>(crow + col_hi + c) = pack8(hi);
+    } else if constexpr (EPI == EPI_SILU_MUL) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) lo[u] = __fdividef(lo[u], 1.f + __expf(-lo[u])) * hi[u];  // as in k_gemm
+      *reinterpret_cast<uint4*>(g.c + (size_t)row * (g.N / 2) + nt * 64 + c) = pack8(lo);
+    } else {
+      const int b = row / g.n_pad, i = row - b * g.n_pad;
+      const bool key = nt < g.hkv;
+      const int head = key ? nt : nt - g.hkv, p = g.pos[row];
+      __nv_bfloat16* dst = (key ? g.k_out : g.v_out) + (((size_t)b * g.hkv + head) * g.n_pad + i) * 128 + c;
+      if (key && p >= 0) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          float sn, cs;
+          fc_rope_sincos((float)p, s_rope[c + u], sn, cs);
+          const float x0 = lo[u], x1 = hi[u];
+          lo[u] = x0 * cs - x1 * sn;
+          hi[u] = x1 * cs + x0 * sn;
+        }
+      }
+      *reinterpret_cast<uint4*>(dst) = pack8(lo);
+      *reinterpret_cast<uint4*>(dst + 64) = pack8(hi);
+    }
+  }
+  __syncwarp();
+  cluster_sync_all();  // no CTA leaves while another may still read its partial tile
+  if (tid == 0 && s_abort) fc_flag(FC_ERR_WORD(g.err), FC_EBIT_TIMEOUT);
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, SP_BN);
+  }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   static std::once_flag once;
@@ -339,11 +577,28 @@ int sm_count() {
 
 bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
+// How many CTAs a cluster of k_gemm_split has for a launch, 0 = k_gemm.  The
+// split kernel serves launches whose 128 x 256 tiles fill less than half of
+// the SMs, with the most CTAs that still fit one per SM (a deep ring each);
+// shares of K of at least four slices.  Clusters of eight fit two CTAs per SM
+// only (one per SM, the GPCs hold too few of them: 10.7 against 7.3 us), with
+// half the ring; they pay for up to 64 rows and long K.
+// us per call, k_gemm / clusters of 2 / 4 / 8, weights from HBM:
+//   M 64,  K 2048, N 2048   13.8 /  9.3 /  7.2 /  7.3      M 512, same        14.7 / 10.7 / 11.5 / 21
+//   M 256, K 2048, N 2048   15.1 / 10.3 /  8.4 / 11.1      M 64,  N 4096      14.8 /  9.7 /  8.1 /  8.9
+//   M 64,  K 5504, N 2048   31.3 / 17.6 / 11.6 /  9.8      M 128, same        32.6 / 18.7 / 12.6 / 13.3
+//   M 512, K 2048, N 4096   15.6 / 14.6 / 23 / 47          (128 big tiles and more: k_gemm)
+int split_cluster(int M, int64_t tiles, int64_t big_tiles, int nk, int sms) {
+  if (2 * big_tiles > sms) return 0;
+  if (M <= 64 && nk >= 64 && tiles * 8 <= sms) return 8;
+  if (nk >= 16 && tiles * 4 <= sms) return 4;
+  return nk >= 8 && tiles * 2 <= sms ? 2 : 0;
+}
+
 template <int EPI>
 fc_status launch_gemm(const void* d_a, const void* d_b, int M, int N, int K, GemmArgs g, cudaStream_t stream) {
-  CUtensorMap ma, mb;
-  if (!make_map_2d(&ma, d_a, (uint64_t)M, (uint64_t)K, BM) || !make_map_2d(&mb, d_b, (uint64_t)K, (uint64_t)N, BK))
-    return FC_ERR_CUDA;
+  const int sms = sm_count();
+  if (sms <= 0) return FC_ERR_CUDA;
   g.M = M;
   g.N = N;
   g.K = K;
@@ -352,16 +607,33 @@ fc_status launch_gemm(const void* d_a, const void* d_b, int M, int N, int K, Gem
   const int64_t tiles = (int64_t)g.tiles_m * ((N + BN - 1) / BN);
   if (tiles > 0x7FFFFFFF) return FC_ERR_UNSUPPORTED;
   g.tiles = (int)tiles;
-  const int sms = sm_count();
-  if (sms <= 0) return FC_ERR_CUDA;
+  CUtensorMap ma, mb;
+  const int64_t split_tiles = (int64_t)g.tiles_m * ((N + SP_BN - 1) / SP_BN);
+  const int cluster = split_cluster(M, split_tiles, tiles, (K + BK - 1) / BK, sms);
+  const int a_rows = cluster ? std::min(BM, (M + 7) / 8 * 8) : BM;
+  if (!make_map_2d(&ma, d_a, (uint64_t)M, (uint64_t)K, a_rows) || !make_map_2d(&mb, d_b, (uint64_t)K, (uint64_t)N, BK))
+    return FC_ERR_CUDA;
+  using Split = void (*)(CUtensorMap, CUtensorMap, GemmArgs, SplitArgs);
+  static constexpr Split split[3] = {k_gemm_split<EPI, 2>, k_gemm_split<EPI, 4>, k_gemm_split<EPI, 8>};
   static std::atomic<unsigned long long> ready;
-  const fc_status set = fc_once_per_device(ready, [](int) {
-    return fc_cuda_status(cudaFuncSetAttribute(k_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+  const fc_status set = fc_once_per_device(ready, [](int) -> fc_status {
+    if (cudaFuncSetAttribute(k_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess)
+      return FC_ERR_CUDA;
+    for (const Split k : split)
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SP_RING_1 + SP_EXTRA)) != cudaSuccess)
+        return FC_ERR_CUDA;
+    return FC_OK;
   });
   if (set != FC_OK) return set;
+  if (cluster) {
+    const uint32_t stage = (uint32_t)a_rows * (BK * 2) + SP_B_BYTES;
+    const uint32_t ring = cluster == 8 ? SP_RING_2 : SP_RING_1;
+    const SplitArgs sp{a_rows, std::min<int>(SP_MAX_STAGES, ring / stage), ring};
+    return fc_launch_dependent(split[cluster / 4], dim3((unsigned)(split_tiles * cluster)), SP_THREADS, ring + SP_EXTRA,
+                               stream, (unsigned)cluster, ma, mb, g, sp);
+  }
   const int grid = (int)std::min<int64_t>(tiles, sms);
-  k_gemm<EPI><<<grid, GM_THREADS, SMEM_BYTES, stream>>>(ma, mb, g);
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(k_gemm<EPI>, dim3((unsigned)grid), GM_THREADS, SMEM_BYTES, stream, 0, ma, mb, g);
 }
 
 // gate/up weights [K][2 * inter] (gate columns, then up columns) -> 128-column

@@ -169,3 +169,31 @@ def test_gemm_silu_mul(fc, M, K, inter):
         + G[:, :inter] * G[:, inter:] + 1e-30
     got = act.double().cpu().numpy()
     assert (np.abs(got - ref) <= lim).all()
+
+
+@pytest.mark.parametrize("M,N,K", [
+    (1, 8, 512), (64, 136, 1032), (64, 2048, 5504), (64, 2432, 4104),        # clusters of 2, 4 and 8; ragged N and K
+    (65, 2048, 2048), (128, 4096, 1024), (200, 1000, 1016), (300, 2048, 520),  # two and three row tiles
+    (64, 4864, 1024), (64, 4872, 1024),                                       # the last tile count of clusters of 4, the first of 2
+])
+def test_gemm_split_shapes(fc, M, N, K):
+    """Few tiles: K cut over the CTAs of a cluster, partial tiles summed in CTA
+    order; twice, for the same bits."""
+    a, b = operands(M, N, K, M * 7 + N + K)
+    c = torch.full((M + 1, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+    fc.fc_gemm_bf16(a, b, out=c[:M])
+    again = fc.fc_gemm_bf16(a, b)
+    torch.cuda.synchronize()
+    assert fc.fc_get_error() == "FC_OK"
+    bound_check(a, b, c[:M])
+    assert torch.equal(c[:M], again) and torch.isnan(c[M]).all()
+
+
+@pytest.mark.parametrize("M,K,inter", [(1, 1024, 128), (64, 2048, 1280), (130, 520, 256), (64, 4096, 640)])
+def test_gemm_split_silu_mul(fc, M, K, inter):
+    test_gemm_silu_mul(fc, M, K, inter)
+
+
+@pytest.mark.parametrize("batch,n_pad,Hkv,K", [(1, 64, 16, 2048), (1, 128, 3, 1024), (3, 64, 1, 4104), (1, 8, 2, 512)])
+def test_gemm_split_kv_heads(fc, orc, batch, n_pad, Hkv, K):
+    test_gemm_kv_heads(fc, orc, batch, n_pad, Hkv, K)

@@ -253,6 +253,10 @@ __global__ void __launch_bounds__(BT_THREADS) k_build_tree(TreeIn in, int S, int
   uint32_t* tab = reinterpret_cast<uint32_t*>(smem_raw + L.tab);
   __shared__ uint32_t hist[256];
   const int b = blockIdx.x, tid = threadIdx.x;
+  fc_grid_release();
+  fc_grid_wait();
+  root_tok = fc_after_wait(root_tok);
+  kv_len = fc_after_wait(kv_len);
 
   // 1. valid drafts, compacted in (source, slot) order
   for (int i = tid; i < M0; i += BT_THREADS) {
@@ -808,9 +812,8 @@ extern "C" fc_status fc_build_tree(int n_sources, const uint32_t* d_drafts, cons
     return fc_cuda_status(cudaFuncSetAttribute(k_build_tree, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
   });
   if (set != FC_OK) return set;
-  k_build_tree<<<batch, BT_THREADS, smem, static_cast<cudaStream_t>(stream)>>>(
-      in, n_sources, batch, top_k, draft_len, d_root_tok, d_kv_len, node_budget, n_pad, out);
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(k_build_tree, dim3((unsigned)batch), BT_THREADS, smem, static_cast<cudaStream_t>(stream), 0,
+                             in, n_sources, batch, top_k, draft_len, d_root_tok, d_kv_len, node_budget, n_pad, out);
 }
 
 extern "C" fc_status fc_tree_mask(const int32_t* d_parent, const int32_t* d_n_nodes, const int32_t* d_kv_len,

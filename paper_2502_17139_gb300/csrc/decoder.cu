@@ -24,6 +24,10 @@ constexpr int ROWS_PER_BLOCK = 8;  // one warp per row
 
 __global__ void k_embed(const uint32_t* __restrict__ tok, int n, const uint4* __restrict__ table, int vocab,
                         int hidden, uint4* __restrict__ out) {
+  fc_grid_release();
+  fc_grid_wait();
+  tok = fc_after_wait(tok);
+  table = fc_after_wait(table);
   const int row = blockIdx.x * ROWS_PER_BLOCK + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= n) return;
   const uint32_t t = tok[row];
@@ -55,6 +59,11 @@ __global__ void __launch_bounds__(NORM_THREADS) k_add_rmsnorm(uint4* __restrict_
                                                               const uint4* __restrict__ w, uint4* __restrict__ out,
                                                               int rows, int dim, float eps) {
   __shared__ float s_part[NORM_THREADS / 32];
+  fc_grid_release();
+  fc_grid_wait();
+  x = fc_after_wait(x);
+  r = fc_after_wait(r);
+  w = fc_after_wait(w);
   const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   if (row >= rows) return;
   const int cw = dim / 8;
@@ -197,9 +206,9 @@ extern "C" fc_status fc_embed(const uint32_t* d_tok, int n, const void* d_table,
   if (n < 0 || vocab < 1 || hidden < 8 || hidden % 8) return FC_ERR_INVALID_ARG;
   if (n == 0) return FC_OK;
   if (!d_tok || !d_table || !d_out || !aligned16(d_table) || !aligned16(d_out)) return FC_ERR_INVALID_ARG;
-  k_embed<<<(n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK, ROWS_PER_BLOCK * 32, 0, static_cast<cudaStream_t>(stream)>>>(
-      d_tok, n, static_cast<const uint4*>(d_table), vocab, hidden, static_cast<uint4*>(d_out));
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(k_embed, dim3((unsigned)((n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK)), ROWS_PER_BLOCK * 32, 0,
+                             static_cast<cudaStream_t>(stream), 0, d_tok, n, static_cast<const uint4*>(d_table), vocab,
+                             hidden, static_cast<uint4*>(d_out));
 }
 
 extern "C" fc_status fc_add_rmsnorm(void* d_x, const void* d_r, const void* d_w, void* d_out, int rows, int dim,
@@ -209,10 +218,9 @@ extern "C" fc_status fc_add_rmsnorm(void* d_x, const void* d_r, const void* d_w,
   if (rows == 0) return FC_OK;
   if (!d_x || !d_w || !d_out || !aligned16(d_x) || !aligned16(d_w) || !aligned16(d_out) || (d_r && !aligned16(d_r)))
     return FC_ERR_INVALID_ARG;
-  k_add_rmsnorm<<<rows, NORM_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<uint4*>(d_x), static_cast<const uint4*>(d_r), static_cast<const uint4*>(d_w),
-      static_cast<uint4*>(d_out), rows, dim, eps);
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(k_add_rmsnorm, dim3((unsigned)rows), NORM_THREADS, 0, static_cast<cudaStream_t>(stream), 0,
+                             static_cast<uint4*>(d_x), static_cast<const uint4*>(d_r), static_cast<const uint4*>(d_w),
+                             static_cast<uint4*>(d_out), rows, dim, eps);
 }
 
 extern "C" fc_status fc_silu_mul(const void* d_gu, void* d_out, int rows, int inter, fc_stream stream) {

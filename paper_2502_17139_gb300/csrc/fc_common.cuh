@@ -136,6 +136,13 @@ fc_status fc_launch_dependent(void (*kern)(P...), dim3 grid, unsigned threads, s
   return FC_CHECK_LAUNCH();
 }
 __device__ __forceinline__ void fc_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A pointer argument as read after the wait: loads through a const __restrict__
+// argument count as invariant, so the compiler could move them ahead of it.
+template <typename T>
+__device__ __forceinline__ T* fc_after_wait(T* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  return p;
+}
 // Lets the next dependent launch's blocks in once every block of this grid
 // has started; what they do before their own fc_grid_wait() then overlaps it.
 __device__ __forceinline__ void fc_grid_release() { asm volatile("griddepcontrol.launch_dependents;"); }

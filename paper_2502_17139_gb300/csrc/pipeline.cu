@@ -186,12 +186,11 @@ fc_status note_attn_nodes(cudaStream_t s, const std::vector<cudaGraphNode_t>& be
         std::find(out->begin(), out->end(), v) != out->end())
       continue;
     out->push_back(v);
-    size_t n = 0;
-    if (cudaGraphNodeGetDependencies(v, nullptr, nullptr, &n) != cudaSuccess) return FC_ERR_CUDA;
-    std::vector<cudaGraphNode_t> d(n);
-    std::vector<cudaGraphEdgeData> e(n);
-    if (n && cudaGraphNodeGetDependencies(v, d.data(), e.data(), &n) != cudaSuccess) return FC_ERR_CUDA;
-    todo.insert(todo.end(), d.begin(), d.end());
+    cudaGraphNode_t d[16];  // a stream's node follows the nodes its stream and its event waits ended on
+    cudaGraphEdgeData e[16];
+    size_t n = 16;
+    if (cudaGraphNodeGetDependencies(v, d, e, &n) != cudaSuccess || n > 16) return FC_ERR_CUDA;
+    todo.insert(todo.end(), d, d + n);
   }
   return FC_OK;
 }

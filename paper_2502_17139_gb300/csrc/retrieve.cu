@@ -330,6 +330,11 @@ __global__ void __launch_bounds__(RT_THREADS) k_retrieve(DsArgs args, DsArgs rev
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RetSmem& sm = *reinterpret_cast<RetSmem*>(smem_raw);
   const int b = blockIdx.x, s = blockIdx.y, tid = threadIdx.x;
+  fc_grid_release();
+  fc_grid_wait();
+  ctx = fc_after_wait(ctx);
+  ctx_len = fc_after_wait(ctx_len);
+  skip = fc_after_wait(skip);
   if (skip && skip[b]) return;
   const DsView ds = args.ds[s];
   const uint32_t* __restrict__ T = ds.T;
@@ -543,6 +548,11 @@ __global__ void k_rc_insert(uint32_t* table, int capacity, int S, fc_retrieve_pa
                             const int32_t* __restrict__ skip, RetOut o) {
   __shared__ RcSmem sm;
   const int b = blockIdx.x;
+  fc_grid_release();
+  fc_grid_wait();
+  ctx = fc_after_wait(ctx);
+  ctx_len = fc_after_wait(ctx_len);
+  skip = fc_after_wait(skip);
   if (skip && skip[b]) return;
   rc_load_key(sm, ctx, stride, ctx_len, b, p.n_max);
   const size_t ew = rc_entry_words(S, p);
@@ -621,9 +631,8 @@ static fc_status launch_retrieve(bool all, const fc_datastore* sources, const fc
   if (st != FC_OK) return st;
   RetOut o{d_drafts, d_draft_len, d_count, d_n_drafts, d_match_len, fc_error_slot()};
   dim3 grid((unsigned)batch, (unsigned)n_sources);
-  kern<<<grid, RT_THREADS, sizeof(RetSmem), static_cast<cudaStream_t>(stream)>>>(a, r, d_ctx, ctx_stride, d_ctx_len,
-                                                                                 batch, d_skip, p, o, rc);
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(kern, grid, RT_THREADS, sizeof(RetSmem), static_cast<cudaStream_t>(stream), 0, a, r, d_ctx,
+                             ctx_stride, d_ctx_len, batch, d_skip, p, o, rc);
 }
 
 extern "C" fc_status fc_retrieve(const fc_datastore* sources, int n_sources, const uint32_t* d_ctx, int ctx_stride,
@@ -718,8 +727,7 @@ extern "C" fc_status fc_rcache_insert(void* d_table, int capacity, int n_sources
     return FC_ERR_INVALID_ARG;
   RetOut o{const_cast<uint32_t*>(d_drafts), const_cast<int32_t*>(d_draft_len), const_cast<uint32_t*>(d_count),
            const_cast<int32_t*>(d_n_drafts), const_cast<int32_t*>(d_match_len), fc_error_slot()};
-  k_rc_insert<<<batch, 128, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<uint32_t*>(d_table), capacity,
-                                                                     n_sources, p, d_ctx, ctx_stride, d_ctx_len, batch,
-                                                                     d_skip, o);
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(k_rc_insert, dim3((unsigned)batch), 128, 0, static_cast<cudaStream_t>(stream), 0,
+                             static_cast<uint32_t*>(d_table), capacity, n_sources, p, d_ctx, ctx_stride, d_ctx_len,
+                             batch, d_skip, o);
 }

@@ -25,9 +25,12 @@ __global__ void __launch_bounds__(ACC_WARPS * 32) k_accept(const uint32_t* __res
                                                            int path_cap, uint32_t* __restrict__ bonus,
                                                            unsigned int* err) {
   extern __shared__ uint32_t acc_smem[];  // [ACC_WARPS][3][n_pad]
-  // Launched as a programmatic dependent of the row argmax (fc_argmax_accept):
-  // wait here until that grid's results are visible.  A no-op otherwise.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  fc_grid_release();
+  fc_grid_wait();
+  tok = fc_after_wait(tok);
+  parent = fc_after_wait(parent);
+  n_nodes = fc_after_wait(n_nodes);
+  argmax = fc_after_wait(argmax);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.x * ACC_WARPS + w;
   if (b >= B) return;
@@ -82,6 +85,16 @@ __global__ void k_kv_append(const int32_t* __restrict__ path, const int32_t* __r
                             uint32_t* __restrict__ ctx, int ctx_stride, const int32_t* __restrict__ ctx_len_in,
                             int32_t* __restrict__ ctx_len_out, uint32_t* __restrict__ root_out,
                             unsigned int* err) {
+  fc_grid_release();
+  fc_grid_wait();
+  path = fc_after_wait(path);
+  acc_len = fc_after_wait(acc_len);
+  bonus = fc_after_wait(bonus);
+  tok = fc_after_wait(tok);
+  k_tree = fc_after_wait(k_tree);
+  v_tree = fc_after_wait(v_tree);
+  kv_len_in = fc_after_wait(kv_len_in);
+  ctx_len_in = fc_after_wait(ctx_len_in);
   const int b = blockIdx.x;
   const int a = acc_len[b];
   const int kvl = kv_len_in[b], cl = ctx_len_in[b];
@@ -156,8 +169,10 @@ __device__ __forceinline__ uint32_t max_nan_bf16x2(uint32_t a, uint32_t b) {
 __global__ void __launch_bounds__(AM_WARPS * 32) k_argmax_rows(const uint16_t* __restrict__ logits, int vocab,
                                                                 const int32_t* __restrict__ n_nodes, int n_pad,
                                                                 uint32_t* __restrict__ argmax) {
-  // the acceptance walk may be scheduled now; it waits for this grid's results
-  asm volatile("griddepcontrol.launch_dependents;");
+  fc_grid_release();  // the acceptance walk may be scheduled now; it waits for this grid's results
+  fc_grid_wait();
+  logits = fc_after_wait(logits);
+  n_nodes = fc_after_wait(n_nodes);
   const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * AM_WARPS + warp;
   if (i >= n_pad) return;
@@ -243,6 +258,13 @@ __global__ void k_synth_argmax(const uint32_t* __restrict__ tok, const int32_t* 
   __shared__ int par_s[FC_MAX_NODES];
   __shared__ int first_child[FC_MAX_NODES];
   __shared__ uint32_t tok_s[FC_MAX_NODES];
+  fc_grid_release();
+  fc_grid_wait();
+  tok = fc_after_wait(tok);
+  parent = fc_after_wait(parent);
+  n_nodes = fc_after_wait(n_nodes);
+  plen = fc_after_wait(plen);
+  rtok = fc_after_wait(rtok);
   const int b = blockIdx.x;
   const size_t base = (size_t)b * n_pad;
   const int n = min(max((int)n_nodes[b], 1), n_pad);
@@ -299,9 +321,9 @@ extern "C" fc_status fc_accept(const uint32_t* d_tok, const int32_t* d_parent, c
   if (!d_tok || !d_parent || !d_n_nodes || !d_argmax || !d_acc_len || !d_path || !d_bonus) return FC_ERR_INVALID_ARG;
   const unsigned blocks = (unsigned)((batch + ACC_WARPS - 1) / ACC_WARPS);
   const size_t smem = (size_t)ACC_WARPS * 3 * n_pad * sizeof(uint32_t);  // <= 48 KB for n_pad <= 1024
-  k_accept<<<blocks, ACC_WARPS * 32, smem, static_cast<cudaStream_t>(stream)>>>(
-      d_tok, d_parent, d_n_nodes, d_argmax, batch, n_pad, d_acc_len, d_path, path_cap, d_bonus, fc_error_slot());
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(k_accept, dim3(blocks), ACC_WARPS * 32, smem, static_cast<cudaStream_t>(stream), 0, d_tok,
+                             d_parent, d_n_nodes, d_argmax, batch, n_pad, d_acc_len, d_path, path_cap, d_bonus,
+                             fc_error_slot());
 }
 
 extern "C" fc_status fc_argmax_accept(const void* d_logits, int vocab, const uint32_t* d_tok,
@@ -316,26 +338,13 @@ extern "C" fc_status fc_argmax_accept(const void* d_logits, int vocab, const uin
     return FC_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(d_logits) % 2) return FC_ERR_INVALID_ARG;
   const dim3 grid((unsigned)((n_pad + AM_WARPS - 1) / AM_WARPS), (unsigned)batch);
-  k_argmax_rows<<<grid, AM_WARPS * 32, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const uint16_t*>(d_logits), vocab, d_n_nodes, n_pad, d_argmax);
-  const fc_status st = FC_CHECK_LAUNCH();
+  const fc_status st = fc_launch_dependent(k_argmax_rows, grid, AM_WARPS * 32, 0, static_cast<cudaStream_t>(stream), 0,
+                                           static_cast<const uint16_t*>(d_logits), vocab, d_n_nodes, n_pad, d_argmax);
   if (st != FC_OK) return st;
-  // the walk as a programmatic dependent launch: it is scheduled while the
-  // argmax grid runs and waits (griddepcontrol.wait) for its completion
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((batch + ACC_WARPS - 1) / ACC_WARPS));
-  cfg.blockDim = dim3(ACC_WARPS * 32);
-  cfg.dynamicSmemBytes = (size_t)ACC_WARPS * 3 * n_pad * sizeof(uint32_t);
-  cfg.stream = static_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, k_accept, d_tok, d_parent, d_n_nodes, (const uint32_t*)d_argmax, batch, n_pad,
-                         d_acc_len, d_path, path_cap, d_bonus, fc_error_slot()) != cudaSuccess)
-    return FC_ERR_CUDA;
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(k_accept, dim3((unsigned)((batch + ACC_WARPS - 1) / ACC_WARPS)), ACC_WARPS * 32,
+                             (size_t)ACC_WARPS * 3 * n_pad * sizeof(uint32_t), static_cast<cudaStream_t>(stream), 0,
+                             d_tok, d_parent, d_n_nodes, d_argmax, batch, n_pad, d_acc_len, d_path, path_cap, d_bonus,
+                             fc_error_slot());
 }
 
 extern "C" fc_status fc_kv_append(const int32_t* d_path, const int32_t* d_acc_len, const uint32_t* d_bonus,
@@ -355,11 +364,11 @@ extern "C" fc_status fc_kv_append(const int32_t* d_path, const int32_t* d_acc_le
   const uintptr_t al = reinterpret_cast<uintptr_t>(d_k_tree) | reinterpret_cast<uintptr_t>(d_v_tree) |
                        reinterpret_cast<uintptr_t>(d_k_cache) | reinterpret_cast<uintptr_t>(d_v_cache);
   if (al % 16) return FC_ERR_INVALID_ARG;
-  k_kv_append<<<batch, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      d_path, d_acc_len, d_bonus, d_tok, static_cast<const uint4*>(d_k_tree), static_cast<const uint4*>(d_v_tree), n_pad,
-      Hkv, D, path_cap, static_cast<uint4*>(d_k_cache), static_cast<uint4*>(d_v_cache), kv_cap, d_kv_len_in,
-      d_kv_len_out, d_ctx, ctx_stride, d_ctx_len_in, d_ctx_len_out, d_root_out, fc_error_slot());
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(
+      k_kv_append, dim3((unsigned)batch), 256, 0, static_cast<cudaStream_t>(stream), 0, d_path, d_acc_len, d_bonus, d_tok,
+      static_cast<const uint4*>(d_k_tree), static_cast<const uint4*>(d_v_tree), n_pad, Hkv, D, path_cap,
+      static_cast<uint4*>(d_k_cache), static_cast<uint4*>(d_v_cache), kv_cap, d_kv_len_in, d_kv_len_out, d_ctx,
+      ctx_stride, d_ctx_len_in, d_ctx_len_out, d_root_out, fc_error_slot());
 }
 
 extern "C" fc_status fc_synth_argmax(const uint32_t* d_tok, const int32_t* d_parent, const int32_t* d_n_nodes,
@@ -369,9 +378,8 @@ extern "C" fc_status fc_synth_argmax(const uint32_t* d_tok, const int32_t* d_par
   if (batch < 0 || n_pad < 1 || n_pad > FC_MAX_NODES || vocab < 2) return FC_ERR_INVALID_ARG;
   if (batch == 0) return FC_OK;
   if (!d_tok || !d_parent || !d_n_nodes || !d_plen || !d_rtok || !d_argmax) return FC_ERR_INVALID_ARG;
-  k_synth_argmax<<<batch, 128, 0, static_cast<cudaStream_t>(stream)>>>(d_tok, d_parent, d_n_nodes, n_pad, d_plen,
-                                                                       d_rtok, vocab, d_argmax);
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(k_synth_argmax, dim3((unsigned)batch), 128, 0, static_cast<cudaStream_t>(stream), 0, d_tok,
+                             d_parent, d_n_nodes, n_pad, d_plen, d_rtok, vocab, d_argmax);
 }
 
 // ---------------------------------------------------------------------------

@@ -305,6 +305,8 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   __shared__ volatile int s_abort;
   __shared__ int s_ticket, s_ready;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  fc_grid_release();
+  fc_grid_wait();
   // Units (group, row chunk) in launch order, so the row chunks of a group,
   // which stream the same K/V blocks, run together and share them through
   // L2.  The units of the last, partial wave are split over `parts` CTAs each
@@ -882,8 +884,9 @@ __global__ void __launch_bounds__(TILES* BM) k_attn_merge(AttnArgs a) {
   const int unit = blockIdx.y, r = threadIdx.x, col = blockIdx.x * MERGE_COLS;
   const int bg = unit / a.ctas, c = unit - bg * a.ctas;
   const int b = bg / a.Hkv, g = bg - b * a.Hkv;
+  fc_grid_release();
+  fc_grid_wait();
   const int nn = a.n_nodes[b], rg = c * (TILES * BM) + r;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int2 p = a.ws_plan[unit];
   if (p.y < 2 || rg >= a.G * nn) return;
   const float2* ml = a.ws_ml + (size_t)p.x * (TILES * BM) + r;
@@ -1042,6 +1045,8 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  fc_grid_release();
+  fc_grid_wait();
   const int U = a.B * a.Hkv;
   const int n_units = max(0, (U - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x);
   unsigned char* smem =
@@ -1555,8 +1560,12 @@ uint64_t attn_units(int batch, int n_pad, int H, int Hkv) {
 __global__ void k_rope(const uint4* __restrict__ in, uint4* __restrict__ out, int B, int n_pad, int heads, int D,
                        int layout, const int32_t* __restrict__ pos, double nl2f) {
   __shared__ float2 tab[FC_ROPE_MAX_HALF];
+  fc_grid_release();
   fc_rope_table(tab, D / 2, nl2f);
   __syncthreads();
+  fc_grid_wait();
+  in = fc_after_wait(in);
+  pos = fc_after_wait(pos);
   const int ch = D / 16;  // 16-byte chunks per half row
   const size_t items = (size_t)B * n_pad * heads * ch;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < items; e += (size_t)gridDim.x * blockDim.x) {
@@ -1693,20 +1702,11 @@ static fc_status launch_tree_attn(const void* d_q, const void* d_k_cache, const 
     a.ws_ml = reinterpret_cast<float2*>(base + w.ml);
     a.ws_o = reinterpret_cast<float*>(base + w.o);
   }
-  kern<<<(unsigned)grid, TA_THREADS, smem_bytes, static_cast<cudaStream_t>(stream)>>>(mkc, mvc, mkt, mvt, a);
-  const fc_status st = FC_CHECK_LAUNCH();
+  const fc_status st = fc_launch_dependent(kern, dim3((unsigned)grid), TA_THREADS, smem_bytes,
+                                           static_cast<cudaStream_t>(stream), 0, mkc, mvc, mkt, mvt, a);
   if (st != FC_OK || !spread) return st;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(HD / MERGE_COLS, (unsigned)units);
-  cfg.blockDim = dim3(TILES * BM);
-  cfg.stream = static_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, k_attn_merge, a) != cudaSuccess) return FC_ERR_CUDA;
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(k_attn_merge, dim3(HD / MERGE_COLS, (unsigned)units), TILES * BM, 0,
+                             static_cast<cudaStream_t>(stream), 0, a);
 }
 
 extern "C" fc_status fc_tree_attn(const void* d_q, const void* d_k_cache, const void* d_v_cache, int kv_cap,
@@ -1741,8 +1741,7 @@ extern "C" fc_status fc_rope(const void* d_in, void* d_out, int batch, int n_pad
   if ((reinterpret_cast<uintptr_t>(d_in) | reinterpret_cast<uintptr_t>(d_out)) % 16) return FC_ERR_INVALID_ARG;
   const size_t items = (size_t)batch * n_pad * heads * (D / 16);
   const unsigned blocks = (unsigned)std::min<size_t>((items + 255) / 256, 152 * 16);
-  k_rope<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const uint4*>(d_in),
-                                                                static_cast<uint4*>(d_out), batch, n_pad, heads, D,
-                                                                layout, d_pos, -2.0 * std::log2((double)base) / D);
-  return FC_CHECK_LAUNCH();
+  return fc_launch_dependent(k_rope, dim3(blocks), 256, 0, static_cast<cudaStream_t>(stream), 0,
+                             static_cast<const uint4*>(d_in), static_cast<uint4*>(d_out), batch, n_pad, heads, D, layout,
+                             d_pos, -2.0 * std::log2((double)base) / D);
 }

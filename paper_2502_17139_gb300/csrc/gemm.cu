@@ -2,7 +2,7 @@
 // verifies every draft in one pass (Section IV-D).  Row-major bf16 operands,
 // fp32 accumulation in tensor memory, bf16 output.
 //
-// GB300 design (a persistent, warp-specialised tcgen05 kernel, one CTA per SM):
+// GB300 design (persistent, warp-specialised tcgen05 kernels, one CTA per SM):
 //   * output tiles of 128 x 256; the CTAs walk the tile list with a stride of
 //     the grid, M fastest, so the CTAs of a wave share the weight columns they
 //     read (and the activations, a few MB, stay in L2);
@@ -33,8 +33,10 @@
 //     and up block t, and the epilogue writes act[:, 128t .. 128t + 128) =
 //     silu(gate) * up.
 //
-// Few rows (one user's draft tree is 64 or 128) leave most SMs without a tile
-// of 128 x 256; k_gemm_split below cuts K over the CTAs of a cluster for them.
+// That is k_gemm, for launches of about one wave of tiles.  k_gemm_pair below
+// runs many tiles on pairs of SMs, and k_gemm_split cuts K over the CTAs of a
+// cluster where few rows (one user's draft tree is 64 or 128) would leave most
+// SMs without a tile.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -111,6 +113,92 @@ __device__ __forceinline__ uint4 pack8(const float* v) {
   o.z = pack_bf16x2(v[4], v[5]);
   o.w = pack_bf16x2(v[6], v[7]);
   return o;
+}
+
+// One output row of a 128 x 256 tile, from 256 tensor-memory columns at tacc
+// (one row per thread; called by whole warps).
+template <int EPI>
+__device__ __forceinline__ void store_tile_row(const GemmArgs& g, uint32_t tacc, int row, int n0, const float2* s_rope) {
+  if constexpr (EPI == EPI_STORE) {
+    __nv_bfloat16* crow = g.c + (size_t)row * g.N;
+#pragma unroll 1
+    for (int cc = 0; cc < BN / 32; ++cc) {
+      uint32_t v[32];
+      tmem_ld32(tacc + cc * 32, v);
+      tc_wait_ld();
+      const int col = n0 + cc * 32;
+      if (row < g.M && col < g.N) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (col + 8 * u + 8 <= g.N)
+            *reinterpret_cast<uint4*>(crow + col + 8 * u) = pack8_bits(v + 8 * u);
+      }
+    }
+  } else if constexpr (EPI == EPI_SILU_MUL) {
+    // gate columns [0, 128) and up columns [128, 256) of the tile -> act block n0 / 2
+    __nv_bfloat16* arow = g.c + (size_t)row * (g.N / 2) + n0 / 2;
+#pragma unroll 1
+    for (int cc = 0; cc < 4; ++cc) {
+      uint32_t gv[32], uv[32];
+      tmem_ld32(tacc + cc * 32, gv);
+      tmem_ld32(tacc + 128 + cc * 32, uv);
+      tc_wait_ld();
+      if (row < g.M) {
+        float a[32];
+#pragma unroll
+        for (int u = 0; u < 32; ++u) {
+          const float x = __uint_as_float(gv[u]);
+          // the fast divide: an IEEE division takes a slow path for a zero dividend,
+          // which doubled this epilogue's time on padding rows (all zeros)
+          a[u] = __fdividef(x, 1.f + __expf(-x)) * __uint_as_float(uv[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          *reinterpret_cast<uint4*>(arow + cc * 32 + 8 * u) = pack8(a + 8 * u);
+      }
+    }
+  } else {
+    // two heads of 128 columns; head hh < hkv is a key head (rotated)
+    const int b = row / g.n_pad, i = row - b * g.n_pad;
+    const int p = row < g.M ? g.pos[row] : -1;
+#pragma unroll 1
+    for (int j = 0; j < 2; ++j) {
+      const int hh = n0 / 128 + j;
+      const bool key = hh < g.hkv;
+      const int head = key ? hh : hh - g.hkv;
+      __nv_bfloat16* dst = (key ? g.k_out : g.v_out) + (((size_t)b * g.hkv + head) * g.n_pad + i) * 128;
+#pragma unroll 1
+      for (int q = 0; q < 2; ++q) {  // dims 32q .. 32q + 31 and their partners 64 + 32q ..
+        uint32_t lv[32], hv[32];
+        tmem_ld32(tacc + j * 128 + q * 32, lv);
+        tmem_ld32(tacc + j * 128 + 64 + q * 32, hv);
+        tc_wait_ld();
+        if (row < g.M) {
+          float lo[32], hi[32];
+#pragma unroll
+          for (int u = 0; u < 32; ++u) {
+            lo[u] = __uint_as_float(lv[u]);
+            hi[u] = __uint_as_float(hv[u]);
+          }
+          if (key && p >= 0) {
+#pragma unroll
+            for (int u = 0; u < 32; ++u) {
+              float sn, cs;
+              fc_rope_sincos((float)p, s_rope[q * 32 + u], sn, cs);
+              const float x0 = lo[u], x1 = hi[u];
+              lo[u] = x0 * cs - x1 * sn;
+              hi[u] = x1 * cs + x0 * sn;
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            *reinterpret_cast<uint4*>(dst + q * 32 + 8 * u) = pack8(lo + 8 * u);
+            *reinterpret_cast<uint4*>(dst + 64 + q * 32 + 8 * u) = pack8(hi + 8 * u);
+          }
+        }
+      }
+    }
+  }
 }
 
 template <int EPI>
@@ -225,88 +313,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
       if (!wait_warp(bar(B_ACC_FULL + buf), acc_ph, &s_abort)) break;
       tc_fence_after();
       const int m0 = (t % g.tiles_m) * BM, n0 = (t / g.tiles_m) * BN;
-      const int row = m0 + r;
-      const uint32_t tacc = tmem + buf * BN + lane_off;
-      if constexpr (EPI == EPI_STORE) {
-        __nv_bfloat16* crow = g.c + (size_t)row * g.N;
-#pragma unroll 1
-        for (int cc = 0; cc < BN / 32; ++cc) {
-          uint32_t v[32];
-          tmem_ld32(tacc + cc * 32, v);
-          tc_wait_ld();
-          const int col = n0 + cc * 32;
-          if (row < g.M && col < g.N) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              if (col + 8 * u + 8 <= g.N)
-                *reinterpret_cast<uint4*>(crow + col + 8 * u) = pack8_bits(v + 8 * u);
-          }
-        }
-      } else if constexpr (EPI == EPI_SILU_MUL) {
-        // gate columns [0, 128) and up columns [128, 256) of the tile -> act block n0 / 2
-        __nv_bfloat16* arow = g.c + (size_t)row * (g.N / 2) + n0 / 2;
-#pragma unroll 1
-        for (int cc = 0; cc < 4; ++cc) {
-          uint32_t gv[32], uv[32];
-          tmem_ld32(tacc + cc * 32, gv);
-          tmem_ld32(tacc + 128 + cc * 32, uv);
-          tc_wait_ld();
-          if (row < g.M) {
-            float a[32];
-#pragma unroll
-            for (int u = 0; u < 32; ++u) {
-              const float x = __uint_as_float(gv[u]);
-              // the fast divide: an IEEE division takes a slow path for a zero dividend,
-              // which doubled this epilogue's time on padding rows (all zeros)
-              a[u] = __fdividef(x, 1.f + __expf(-x)) * __uint_as_float(uv[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              *reinterpret_cast<uint4*>(arow + cc * 32 + 8 * u) = pack8(a + 8 * u);
-          }
-        }
-      } else {
-        // two heads of 128 columns; head hh < hkv is a key head (rotated)
-        const int b = row / g.n_pad, i = row - b * g.n_pad;
-        const int p = row < g.M ? g.pos[row] : -1;
-#pragma unroll 1
-        for (int j = 0; j < 2; ++j) {
-          const int hh = n0 / 128 + j;
-          const bool key = hh < g.hkv;
-          const int head = key ? hh : hh - g.hkv;
-          __nv_bfloat16* dst = (key ? g.k_out : g.v_out) + (((size_t)b * g.hkv + head) * g.n_pad + i) * 128;
-#pragma unroll 1
-          for (int q = 0; q < 2; ++q) {  // dims 32q .. 32q + 31 and their partners 64 + 32q ..
-            uint32_t lv[32], hv[32];
-            tmem_ld32(tacc + j * 128 + q * 32, lv);
-            tmem_ld32(tacc + j * 128 + 64 + q * 32, hv);
-            tc_wait_ld();
-            if (row < g.M) {
-              float lo[32], hi[32];
-#pragma unroll
-              for (int u = 0; u < 32; ++u) {
-                lo[u] = __uint_as_float(lv[u]);
-                hi[u] = __uint_as_float(hv[u]);
-              }
-              if (key && p >= 0) {
-#pragma unroll
-                for (int u = 0; u < 32; ++u) {
-                  float sn, cs;
-                  fc_rope_sincos((float)p, s_rope[q * 32 + u], sn, cs);
-                  const float x0 = lo[u], x1 = hi[u];
-                  lo[u] = x0 * cs - x1 * sn;
-                  hi[u] = x1 * cs + x0 * sn;
-                }
-              }
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                *reinterpret_cast<uint4*>(dst + q * 32 + 8 * u) = pack8(lo + 8 * u);
-                *reinterpret_cast<uint4*>(dst + 64 + q * 32 + 8 * u) = pack8(hi + 8 * u);
-              }
-            }
-          }
-        }
-      }
+      store_tile_row<EPI>(g, tmem + buf * BN + lane_off, m0 + r, n0, s_rope);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(B_ACC_EMPTY + buf));
@@ -322,30 +329,22 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
 }
 
 // ---------------------------------------------------------------------------
-// Few tiles: the weights are read for so few rows that the work is streaming
-// them from HBM, and that needs every SM.  Output tiles of 128 x 128, each
-// computed by a cluster of S CTAs that take S consecutive shares of K; a CTA's
-// partial tile goes from tensor memory to its shared memory (over its drained
-// ring), and after a cluster barrier CTA r sums columns [64 r / S, 64 (r+1) / S)
-// of both 64-column halves over the S partials, in CTA order, and applies the
-// epilogue (each half pair is what the epilogues need: gate and up, or the
-// rotation's partners).  fp32 throughout, no scratch memory.  Bound by the
-// latency of its steps (a copy, the MMAs, the exchange: 5 us for the smallest
-// shape) and then by the weights' stream: the ring is as deep as the SM allows.
-//   The ring's slices carry only as many rows of A as the matrix has (the MMA then reads 128 - a_rows rows of the slice's B as A
-// rows, into accumulator rows that nothing reads).
+// Many tiles: pairs of CTAs (cta_group::2) on tiles of 256 x 256.  A 128 x 256
+// tile on one SM moves 12 KB into and 12 KB out of shared memory per 16-deep
+// MMA of 128 cycles, 192 bytes a cycle where the SM has 128: k_gemm's tensor
+// pipe stands at 68%.  Bound by the MMAs: 1862 TFLOP/s on the LM head (M 2048,
+// K 2048, N 32256) where k_gemm reaches 1518.  In a pair each SM holds its own 128 rows of A and half of
+// B's columns, 8 KB in and 8 KB out, and the ring is seven slices deep.
+//   Both CTAs' copies complete on the leader's (rank 0's) barriers; the leader
+// issues the MMAs of both, into tensor memory of both (each its own 128 rows),
+// and its commits arrive in both CTAs.  Roles, walk and epilogues as k_gemm.
 // ---------------------------------------------------------------------------
-constexpr int SP_THREADS = 192, SP_BN = 128, SP_MAX_STAGES = 12;
-constexpr uint32_t SP_B_BYTES = (SP_BN / 64) * B_CHUNK;         // 16 KB
-constexpr uint32_t SP_RING_1 = 208 * 1024, SP_RING_2 = 96 * 1024;  // one CTA per SM, or two; a partial tile is 64 KB
-constexpr uint32_t SP_EXTRA = 256 + 1024;                       // barriers + alignment slack
-enum { SB_FULL = 0, SB_EMPTY = SP_MAX_STAGES, SB_ACC = 2 * SP_MAX_STAGES, SB_DRAIN, SB_COUNT };
-
-struct SplitArgs {
-  int a_rows;  // rows of A per slice (a multiple of 8)
-  int stages;
-  uint32_t ring;  // bytes
-};
+constexpr int PR_STAGES = 7, PR_BM = 2 * BM;
+constexpr uint32_t PR_B_BYTES = B_BYTES / 2, PR_STAGE = A_BYTES + PR_B_BYTES;  // per CTA: 32 KB
+constexpr uint32_t PR_SMEM = PR_STAGES * PR_STAGE + 256 + 1024;                // + barriers + alignment slack
+enum { P_FULL = 0, P_EMPTY = PR_STAGES, P_ACC_FULL = 2 * PR_STAGES, P_ACC_EMPTY = P_ACC_FULL + 2,
+       P_DRAIN = P_ACC_EMPTY + 2, P_COUNT };
+static_assert(P_COUNT * 8 <= 256, "barrier area");
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -355,6 +354,209 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// A copy into this CTA's shared memory that completes on a barrier of the pair.
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
+      "[%1, {%2, %3}], [%4];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void mma_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                         uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// Arrives on the barrier at this offset in both CTAs once the MMAs issued so far are done.
+__device__ __forceinline__ void commit_pair(uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t.reg .b16 m;\n\tmov.b16 m, 3;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], m;\n\t}" ::"r"(bar)
+      : "memory");
+}
+// An arrival on a barrier of either CTA of the pair (a cluster address).
+__device__ __forceinline__ void arrive_cluster(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+// As mbar_wait_bounded, for a barrier that the other CTA's threads arrive on.
+__device__ __forceinline__ bool wait_warp_cluster(uint32_t bar, uint32_t parity, volatile int* abort) {
+  const long long t0 = clock64();
+  for (;;) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, 500000;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (__all_sync(0xFFFFFFFFu, ok != 0)) return true;
+    if (__any_sync(0xFFFFFFFFu, *abort || (uint64_t)(clock64() - t0) > WAIT_CYCLES)) {
+      *abort = 1;
+      return false;
+    }
+  }
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(GM_THREADS, 1) __cluster_dims__(2, 1, 1)
+    k_gemm_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, GemmArgs g) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ uint32_t s_tmem;
+  __shared__ volatile int s_abort;
+  __shared__ float2 s_rope[64];
+  if constexpr (EPI == EPI_KV_HEADS) fc_rope_table(s_rope, 64, g.rope_nl2f);  // read after the barrier below
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  unsigned char* smem =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t bar0 = sbase + PR_STAGES * PR_STAGE;
+  auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+  const int nk = (g.K + BK - 1) / BK;
+  const uint32_t rank = cluster_rank();
+  const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+
+  if (tid == 0) {
+    s_abort = 0;
+    for (int i = 0; i < P_COUNT; ++i)
+      mbar_init(bar(i), i == P_ACC_EMPTY || i == P_ACC_EMPTY + 1 ? 8 : 1);  // 4 epilogue warps of both CTAs
+    fence_mbar_init();
+    prefetch_tmap(&tm_a);
+    prefetch_tmap(&tm_b);
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // both CTAs' barriers are ready
+  tc_fence_after();
+  fc_grid_release();
+  if (tid == 0) {  // the first tile's first weights into L2 while the kernel before still runs
+    const int n0 = (pair / g.tiles_m) * BN + (int)rank * (BN / 2);
+    for (int kb = 0; kb < min(nk, PREFETCH); ++kb)
+      for (int c = 0; c < BN / 128; ++c) tma_prefetch_2d(&tm_b, n0 + 64 * c, kb * BK);
+  }
+  __syncwarp();
+  fc_grid_wait();
+  const uint32_t tmem = s_tmem;
+
+  if (warp == 0) {
+    // ---------------- TMA producer: this CTA's rows of A, its half of B's columns ----------------
+    if (lane == 0) {
+      uint32_t issued = 0;
+      for (int t = pair; t < g.tiles && !s_abort; t += pairs) {
+        const int m0 = (t % g.tiles_m) * PR_BM + (int)rank * BM, n0 = (t / g.tiles_m) * BN + (int)rank * (BN / 2);
+        for (int kb = 0; kb < nk; ++kb) {
+          const uint32_t s = issued % PR_STAGES, ph = (issued / PR_STAGES) & 1;
+          if (!mbar_wait_bounded(bar(P_EMPTY + s), ph ^ 1, &s_abort, WAIT_CYCLES)) break;
+          const uint32_t st = sbase + s * PR_STAGE, fb = cluster_addr(bar(P_FULL + s), 0);
+          if (rank == 0) mbar_expect_tx(bar(P_FULL + s), 2 * PR_STAGE);
+          tma_load_2d_pair(st, &tm_a, kb * BK, m0, fb);
+#pragma unroll
+          for (int c = 0; c < BN / 128; ++c) tma_load_2d_pair(st + A_BYTES + c * B_CHUNK, &tm_b, n0 + 64 * c, kb * BK, fb);
+          ++issued;
+        }
+      }
+      if (s_abort && rank == 0) {  // let both CTAs' copies in flight land before either exits
+        volatile int dummy = 0;
+        for (uint32_t i = issued > PR_STAGES ? issued - PR_STAGES : 0; i < issued; ++i)
+          mbar_wait_bounded(bar(P_FULL + i % PR_STAGES), (i / PR_STAGES) & 1, &dummy, DRAIN_CYCLES);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: the leader's warp, for both CTAs ----------------
+    constexpr uint32_t IDESC = idesc_bf16_f32(PR_BM, BN, 1);  // A K-major, B N-major
+    if (rank == 0) {
+      uint32_t consumed = 0, acc_i = 0;
+      bool ok = true;
+      for (int t = pair; ok && t < g.tiles; t += pairs, ++acc_i) {
+        const uint32_t buf = acc_i & 1, acc_ph = (acc_i >> 1) & 1;
+        if (!(ok = wait_warp_cluster(bar(P_ACC_EMPTY + buf), acc_ph ^ 1, &s_abort))) break;
+        tc_fence_after();
+        const uint32_t d = tmem + buf * BN;
+        for (int kb = 0; kb < nk; ++kb, ++consumed) {
+          const uint32_t s = consumed % PR_STAGES, ph = (consumed / PR_STAGES) & 1;
+          if (!(ok = wait_warp(bar(P_FULL + s), ph, &s_abort))) break;
+          tc_fence_after();
+          const uint32_t sa = sbase + s * PR_STAGE, sb = sa + A_BYTES;
+#pragma unroll
+          for (int kk = 0; kk < BK / 16; ++kk)
+            mma_pair(d, smem_desc_sw128(sa + kk * 32, 16, 1024), smem_desc_sw128(sb + kk * 2048, B_CHUNK, 1024), IDESC,
+                     (kb > 0 || kk > 0) ? 1u : 0u);
+          commit_pair(bar(P_EMPTY + s));
+        }
+        if (!ok) break;
+        commit_pair(bar(P_ACC_FULL + buf));
+      }
+      if (__any_sync(0xFFFFFFFFu, s_abort)) {  // let issued MMAs retire before tensor memory is freed
+        commit_pair(bar(P_DRAIN));
+        volatile int dummy = 0;
+        mbar_wait_bounded(bar(P_DRAIN), 0, &dummy, DRAIN_CYCLES);
+      }
+    }
+  } else {
+    // ---------------- epilogue: thread = output row of this CTA's half of the tile ----------------
+    const int q4 = warp & 3;  // the tensor-memory lane quarter this warp may read
+    const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
+    uint32_t acc_i = 0;
+    for (int t = pair; t < g.tiles; t += pairs, ++acc_i) {
+      const uint32_t buf = acc_i & 1, acc_ph = (acc_i >> 1) & 1;
+      if (!wait_warp(bar(P_ACC_FULL + buf), acc_ph, &s_abort)) break;
+      tc_fence_after();
+      const int m0 = (t % g.tiles_m) * PR_BM + (int)rank * BM, n0 = (t / g.tiles_m) * BN;
+      store_tile_row<EPI>(g, tmem + buf * BN + lane_off, m0 + q4 * 32 + lane, n0, s_rope);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) arrive_cluster(cluster_addr(bar(P_ACC_EMPTY + buf), 0));
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // no CTA leaves while the other's MMAs, copies or arrivals may still reach it
+  if (tid == 0 && s_abort) fc_flag(FC_ERR_WORD(g.err), FC_EBIT_TIMEOUT);
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Few tiles: the weights are read for so few rows that the work is streaming
+// them from HBM, and that needs every SM.  Output tiles of 128 x 64 NB, each
+// computed by a cluster of S CTAs that take S consecutive shares of K; a CTA's
+// partial tile goes from tensor memory to its shared memory (over its drained
+// ring), and after a cluster barrier CTA r sums every S-th group of eight
+// columns of both halves over the S partials, in CTA order, and applies the
+// epilogue (column c of either half is what the epilogues need together: gate
+// and up, or the rotation's partners).  fp32 throughout, no scratch memory.  Bound by the
+// latency of its steps (a copy, the MMAs, the exchange: 5 us for the smallest
+// shape) and then by the weights' stream: the ring is as deep as the SM allows.
+//   The ring's slices carry only as many rows of A as the matrix has (the MMA then reads 128 - a_rows rows of the slice's B as A
+// rows, into accumulator rows that nothing reads).
+// ---------------------------------------------------------------------------
+constexpr int SP_THREADS = 192, SP_MAX_STAGES = 12;
+constexpr uint32_t SP_RING_1 = 208 * 1024, SP_RING_2 = 96 * 1024;  // one CTA per SM, or two; a partial tile is 32 NB KB
+constexpr uint32_t SP_EXTRA = 256 + 1024;                       // barriers + alignment slack
+enum { SB_FULL = 0, SB_EMPTY = SP_MAX_STAGES, SB_ACC = 2 * SP_MAX_STAGES, SB_DRAIN, SB_COUNT };
+
+struct SplitArgs {
+  int a_rows;  // rows of A per slice (a multiple of 8)
+  int stages;
+  uint32_t ring;  // bytes
+};
+
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank) {
   float4 v;
   asm volatile(
@@ -365,8 +567,8 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank) {
   return v;
 }
 
-template <int EPI, int S>
-__global__ void __launch_bounds__(SP_THREADS, 2)
+template <int EPI, int S, int NB>
+__global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
     k_gemm_split(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, GemmArgs g,
                  SplitArgs sp) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -381,12 +583,14 @@ __global__ void __launch_bounds__(SP_THREADS, 2)
   auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
   const uint32_t rank = cluster_rank();
   const int t = (int)(blockIdx.x / S), m0 = (t % g.tiles_m) * BM, nt = t / g.tiles_m;
-  // the tile's two 64-column halves: neighbours, or gate and up of one activation block
-  const int col_lo = EPI == EPI_SILU_MUL ? 256 * (nt >> 1) + 64 * (nt & 1) : nt * SP_BN;
-  const int col_hi = EPI == EPI_SILU_MUL ? col_lo + 128 : col_lo + 64;
+  constexpr int WN = 64 * NB, HN = WN / 2;  // the tile's columns, and those of a half
+  // 64-column chunk c of the tile: side by side, but a half of 64 gate columns goes with the same up columns
+  auto chunk_col = [&](int c) {
+    return EPI == EPI_SILU_MUL && NB == 2 ? 256 * (nt >> 1) + 64 * (nt & 1) + 128 * c : nt * WN + 64 * c;
+  };
   const int nk = (g.K + BK - 1) / BK;
   const int k0 = (int)(rank * (uint32_t)nk / S), k1 = (int)((rank + 1) * (uint32_t)nk / S);
-  const uint32_t a_bytes = (uint32_t)sp.a_rows * (BK * 2), stage_bytes = a_bytes + SP_B_BYTES;
+  const uint32_t a_bytes = (uint32_t)sp.a_rows * (BK * 2), stage_bytes = a_bytes + NB * B_CHUNK;
 
   if (tid == 0) {
     s_abort = 0;
@@ -396,7 +600,7 @@ __global__ void __launch_bounds__(SP_THREADS, 2)
     prefetch_tmap(&tm_b);
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(&s_tmem), SP_BN);
+    tmem_alloc(smem_u32(&s_tmem), WN);
     tmem_relinquish();
   }
   if constexpr (EPI == EPI_KV_HEADS) fc_rope_table(s_rope, 64, g.rope_nl2f);
@@ -407,10 +611,8 @@ __global__ void __launch_bounds__(SP_THREADS, 2)
   // this CTA's weights into L2 while the kernel before still runs (a prefetch
   // into the coherent L2 is no read: what that kernel writes to them counts)
   if (tid == 0)
-    for (int kb = k0; kb < k1; ++kb) {
-      tma_prefetch_2d(&tm_b, col_lo, kb * BK);
-      tma_prefetch_2d(&tm_b, col_hi, kb * BK);
-    }
+    for (int kb = k0; kb < k1; ++kb)
+      for (int c = 0; c < NB; ++c) tma_prefetch_2d(&tm_b, chunk_col(c), kb * BK);
   __syncwarp();
   fc_grid_wait();
   const uint32_t tmem = s_tmem;
@@ -424,8 +626,8 @@ __global__ void __launch_bounds__(SP_THREADS, 2)
         if (!mbar_wait_bounded(bar(SB_EMPTY + s), ph ^ 1, &s_abort, WAIT_CYCLES)) break;
         const uint32_t st = sbase + s * stage_bytes, fb = bar(SB_FULL + s);
         mbar_expect_tx(fb, stage_bytes);
-        tma_load_2d(st + a_bytes, &tm_b, col_lo, kb * BK, fb);
-        tma_load_2d(st + a_bytes + B_CHUNK, &tm_b, col_hi, kb * BK, fb);
+#pragma unroll
+        for (int c = 0; c < NB; ++c) tma_load_2d(st + a_bytes + c * B_CHUNK, &tm_b, chunk_col(c), kb * BK, fb);
         tma_load_2d(st, &tm_a, kb * BK, m0, fb);
       }
       if (s_abort) {  // let the copies in flight land before the CTA exits
@@ -436,7 +638,7 @@ __global__ void __launch_bounds__(SP_THREADS, 2)
     }
     __syncwarp();
   } else if (warp == 1) {  // ---------------- MMA issuer ----------------
-    constexpr uint32_t IDESC = idesc_bf16_f32(BM, SP_BN, 1);
+    constexpr uint32_t IDESC = idesc_bf16_f32(BM, WN, 1);
     bool ok = true;
     for (int i = 0; i < k1 - k0; ++i) {
       const int s = i % sp.stages;
@@ -462,7 +664,7 @@ __global__ void __launch_bounds__(SP_THREADS, 2)
       tc_fence_after();
       float4* red = reinterpret_cast<float4*>(smem) + q4 * 32 + lane;  // [column / 4][row]
 #pragma unroll
-      for (int cc = 0; cc < SP_BN / 32; ++cc) {
+      for (int cc = 0; cc < WN / 32; ++cc) {
         uint32_t v[32];
         tmem_ld32(tmem + cc * 32 + ((uint32_t)(q4 * 32) << 16), v);
         tc_wait_ld();
@@ -477,9 +679,10 @@ __global__ void __launch_bounds__(SP_THREADS, 2)
   cluster_sync_all();
 
   // ---------------- this CTA's columns of the tile, eight of each half per item ----------------
-  constexpr int groups = 8 / S, QUAD = S < 4 ? S : 4;  // partials whose loads are in flight together
+  constexpr int QUAD = S < 4 ? S : 4;  // partials whose loads are in flight together
+  const int groups = (HN / 8 - (int)rank + S - 1) / S;  // groups rank, rank + S, ... of the half's eights
   for (int e = tid; e < rows * groups; e += SP_THREADS) {
-    const int cg = e / rows, r = e - cg * rows, c = ((int)rank * groups + cg) * 8;
+    const int cg = e / rows, r = e - cg * rows, c = ((int)rank + cg * S) * 8;
     float lo[8], hi[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) lo[u] = hi[u] = 0.f;
@@ -491,8 +694,8 @@ __global__ void __launch_bounds__(SP_THREADS, 2)
       for (int q = 0; q < QUAD; ++q) {
         v[q][0] = ld_cluster_f4(at, q0 + q);
         v[q][1] = ld_cluster_f4(at + BM * 16, q0 + q);
-        v[q][2] = ld_cluster_f4(at + 16 * BM * 16, q0 + q);
-        v[q][3] = ld_cluster_f4(at + 17 * BM * 16, q0 + q);
+        v[q][2] = ld_cluster_f4(at + (HN / 4) * BM * 16, q0 + q);
+        v[q][3] = ld_cluster_f4(at + (HN / 4 + 1) * BM * 16, q0 + q);
       }
 #pragma unroll
       for (int q = 0; q < QUAD; ++q) {
@@ -507,12 +710,13 @@ __global__ void __launch_bounds__(SP_THREADS, 2)
     const int row = m0 + r;
     if constexpr (EPI == EPI_STORE) {
       __nv_bfloat16* crow = g.c + (size_t)row * g.N;
-      if (col_lo + c + 8 <= g.N) *reinterpret_cast<uint4*>(crow + col_lo + c) = pack8(lo);
-      if (col_hi + c + 8 <= g.N) *reinterpret_cast<uint4*>(crow + col_hi + c) = pack8(hi);
+      const int col = nt * WN + c;
+      if (col + 8 <= g.N) *reinterpret_cast<uint4*>(crow + col) = pack8(lo);
+      if (col + HN + 8 <= g.N) *reinterpret_cast<uint4*>(crow + col + HN) = pack8(hi);
     } else if constexpr (EPI == EPI_SILU_MUL) {
 #pragma unroll
       for (int u = 0; u < 8; ++u) lo[u] = __fdividef(lo[u], 1.f + __expf(-lo[u])) * hi[u];  // as in k_gemm
-      *reinterpret_cast<uint4*>(g.c + (size_t)row * (g.N / 2) + nt * 64 + c) = pack8(lo);
+      *reinterpret_cast<uint4*>(g.c + (size_t)row * (g.N / 2) + nt * HN + c) = pack8(lo);
     } else {
       const int b = row / g.n_pad, i = row - b * g.n_pad;
       const bool key = nt < g.hkv;
@@ -537,7 +741,7 @@ __global__ void __launch_bounds__(SP_THREADS, 2)
   if (tid == 0 && s_abort) fc_flag(FC_ERR_WORD(g.err), FC_EBIT_TIMEOUT);
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, SP_BN);
+    tmem_dealloc(tmem, WN);
   }
 }
 
@@ -588,11 +792,31 @@ bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0;
 //   M 256, K 2048, N 2048   15.1 / 10.3 /  8.4 / 11.1      M 64,  N 4096      14.8 /  9.7 /  8.1 /  8.9
 //   M 64,  K 5504, N 2048   31.3 / 17.6 / 11.6 /  9.8      M 128, same        32.6 / 18.7 / 12.6 / 13.3
 //   M 512, K 2048, N 4096   15.6 / 14.6 / 23 / 47          (128 big tiles and more: k_gemm)
-int split_cluster(int M, int64_t tiles, int64_t big_tiles, int nk, int sms) {
-  if (2 * big_tiles > sms) return 0;
-  if (M <= 64 && nk >= 64 && tiles * 8 <= sms) return 8;
-  if (nk >= 16 && tiles * 4 <= sms) return 4;
-  return nk >= 8 && tiles * 2 <= sms ? 2 : 0;
+// Where two CTAs per 128-column tile are too many, clusters of three take
+// 256-column tiles: gate/up of inter 5504 at M 64 15.6 -> 12.2, M 128 16.4 -> 14.2.
+struct SplitPlan {
+  int cluster, nb;  // CTAs per cluster (0: k_gemm), 64-column chunks per tile
+};
+SplitPlan choose_split(int M, int64_t tiles_m, int N, int64_t big_tiles, int nk, int sms, bool wide) {
+  const int64_t tiles = tiles_m * ((N + 127) / 128);
+  if (2 * big_tiles > sms) return {0, 0};
+  if (M <= 64 && nk >= 64 && tiles * 8 <= sms) return {8, 2};
+  if (nk >= 16 && tiles * 4 <= sms) return {4, 2};
+  if (nk >= 8 && tiles * 2 <= sms) return {2, 2};
+  return wide && nk >= 12 && big_tiles * 3 <= sms ? SplitPlan{3, 4} : SplitPlan{0, 0};
+}
+
+// Whether k_gemm_pair serves a launch of `tiles` 128 x 256 tiles: by waves, a
+// pair's being the shorter (16.4 thousand cycles of MMAs per 2048 of K either
+// way; k_gemm reaches 69% of that).  One row of tiles would waste half of each
+// pair, and in a single wave of short K the pair's set-up (a cluster barrier,
+// 0.6 us) is not earned back.  us per call, k_gemm / pairs:
+//   M 2048, K 2048, N 32256  178.3 / 145.4    M 2048, K 2048, gate/up 11008  60.2 / 51.2
+//   M 2048, K 5504, N 2048    31.6 /  30.1    M 512,  K 2048, N 32256        59.1 / 47.9
+//   M 1000, K 2048, N 4096    16.6 /  17.7    M 2048, K 2048, N 2048         15.2 / 15.8
+bool use_pair(int64_t tiles_m, int64_t tiles, int64_t pair_tiles, int nk, int sms) {
+  const int64_t waves = (tiles + sms - 1) / sms, pair_waves = (pair_tiles + sms / 2 - 1) / (sms / 2);
+  return tiles_m > 1 && 20 * pair_waves < 29 * waves && (waves > 1 || nk >= 48);
 }
 
 template <int EPI>
@@ -608,29 +832,41 @@ fc_status launch_gemm(const void* d_a, const void* d_b, int M, int N, int K, Gem
   if (tiles > 0x7FFFFFFF) return FC_ERR_UNSUPPORTED;
   g.tiles = (int)tiles;
   CUtensorMap ma, mb;
-  const int64_t split_tiles = (int64_t)g.tiles_m * ((N + SP_BN - 1) / SP_BN);
-  const int cluster = split_cluster(M, split_tiles, tiles, (K + BK - 1) / BK, sms);
-  const int a_rows = cluster ? std::min(BM, (M + 7) / 8 * 8) : BM;
+  constexpr bool WIDE = EPI != EPI_KV_HEADS;  // a tile of the K/V projection is one head
+  const SplitPlan plan = choose_split(M, g.tiles_m, N, tiles, (K + BK - 1) / BK, sms, WIDE);
+  const int a_rows = plan.cluster ? std::min(BM, (M + 7) / 8 * 8) : BM;
   if (!make_map_2d(&ma, d_a, (uint64_t)M, (uint64_t)K, a_rows) || !make_map_2d(&mb, d_b, (uint64_t)K, (uint64_t)N, BK))
     return FC_ERR_CUDA;
   using Split = void (*)(CUtensorMap, CUtensorMap, GemmArgs, SplitArgs);
-  static constexpr Split split[3] = {k_gemm_split<EPI, 2>, k_gemm_split<EPI, 4>, k_gemm_split<EPI, 8>};
+  constexpr int W = WIDE ? 4 : 2;
+  static constexpr Split narrow[9] = {nullptr, nullptr, k_gemm_split<EPI, 2, 2>, nullptr, k_gemm_split<EPI, 4, 2>,
+                                      nullptr, nullptr, nullptr, k_gemm_split<EPI, 8, 2>};
+  static constexpr Split wide = WIDE ? k_gemm_split<EPI, 3, W> : nullptr;
   static std::atomic<unsigned long long> ready;
   const fc_status set = fc_once_per_device(ready, [](int) -> fc_status {
-    if (cudaFuncSetAttribute(k_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gemm_pair<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PR_SMEM) != cudaSuccess)
       return FC_ERR_CUDA;
-    for (const Split k : split)
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SP_RING_1 + SP_EXTRA)) != cudaSuccess)
+    for (const Split k : {narrow[2], narrow[4], narrow[8], wide})
+      if (k && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SP_RING_1 + SP_EXTRA)) != cudaSuccess)
         return FC_ERR_CUDA;
     return FC_OK;
   });
   if (set != FC_OK) return set;
-  if (cluster) {
-    const uint32_t stage = (uint32_t)a_rows * (BK * 2) + SP_B_BYTES;
-    const uint32_t ring = cluster == 8 ? SP_RING_2 : SP_RING_1;
+  if (plan.cluster) {
+    const uint32_t stage = (uint32_t)a_rows * (BK * 2) + plan.nb * B_CHUNK;
+    const uint32_t ring = plan.cluster == 8 ? SP_RING_2 : SP_RING_1;
     const SplitArgs sp{a_rows, std::min<int>(SP_MAX_STAGES, ring / stage), ring};
-    return fc_launch_dependent(split[cluster / 4], dim3((unsigned)(split_tiles * cluster)), SP_THREADS, ring + SP_EXTRA,
-                               stream, (unsigned)cluster, ma, mb, g, sp);
+    const int64_t ctas = (int64_t)g.tiles_m * ((N + 64 * plan.nb - 1) / (64 * plan.nb)) * plan.cluster;
+    return fc_launch_dependent(plan.nb == 4 ? wide : narrow[plan.cluster], dim3((unsigned)ctas), SP_THREADS,
+                               ring + SP_EXTRA, stream, (unsigned)plan.cluster, ma, mb, g, sp);
+  }
+  const int64_t pair_tiles = (int64_t)((M + PR_BM - 1) / PR_BM) * ((N + BN - 1) / BN);
+  if (use_pair(g.tiles_m, tiles, pair_tiles, (K + BK - 1) / BK, sms)) {
+    g.tiles_m = (M + PR_BM - 1) / PR_BM;
+    g.tiles = (int)pair_tiles;
+    return fc_launch_dependent(k_gemm_pair<EPI>, dim3((unsigned)(2 * std::min(g.tiles, sms / 2))), GM_THREADS, PR_SMEM,
+                               stream, 0, ma, mb, g);
   }
   const int grid = (int)std::min<int64_t>(tiles, sms);
   return fc_launch_dependent(k_gemm<EPI>, dim3((unsigned)grid), GM_THREADS, SMEM_BYTES, stream, 0, ma, mb, g);

@@ -175,6 +175,7 @@ def test_gemm_silu_mul(fc, M, K, inter):
     (1, 8, 512), (64, 136, 1032), (64, 2048, 5504), (64, 2432, 4104),        # clusters of 2, 4 and 8; ragged N and K
     (65, 2048, 2048), (128, 4096, 1024), (200, 1000, 1016), (300, 2048, 520),  # two and three row tiles
     (64, 4864, 1024), (64, 4872, 1024),                                       # the last tile count of clusters of 4, the first of 2
+    (64, 9728, 520), (64, 9736, 1000), (70, 12800, 776), (3, 12808, 1024),    # clusters of 3 on wide tiles, and past them
 ])
 def test_gemm_split_shapes(fc, M, N, K):
     """Few tiles: K cut over the CTAs of a cluster, partial tiles summed in CTA
@@ -189,11 +190,35 @@ def test_gemm_split_shapes(fc, M, N, K):
     assert torch.equal(c[:M], again) and torch.isnan(c[M]).all()
 
 
-@pytest.mark.parametrize("M,K,inter", [(1, 1024, 128), (64, 2048, 1280), (130, 520, 256), (64, 4096, 640)])
+@pytest.mark.parametrize("M,K,inter", [(1, 1024, 128), (64, 2048, 1280), (130, 520, 256), (64, 4096, 640),
+                                       (64, 2048, 5504), (100, 840, 6272)])
 def test_gemm_split_silu_mul(fc, M, K, inter):
     test_gemm_silu_mul(fc, M, K, inter)
 
 
 @pytest.mark.parametrize("batch,n_pad,Hkv,K", [(1, 64, 16, 2048), (1, 128, 3, 1024), (3, 64, 1, 4104), (1, 8, 2, 512)])
 def test_gemm_split_kv_heads(fc, orc, batch, n_pad, Hkv, K):
+    test_gemm_kv_heads(fc, orc, batch, n_pad, Hkv, K)
+
+
+@pytest.mark.parametrize("M,N,K", [(257, 20000, 136), (300, 39000, 72), (2500, 4104, 200), (1281, 2056, 3080), (129, 19464, 3072)])
+def test_gemm_pair_shapes(fc, M, N, K):
+    """Many tiles: 256 x 256 tiles on pairs of CTAs, over several waves, with
+    ragged rows (a whole half tile past M among them), columns and K."""
+    a, b = operands(M, N, K, M + N + K)
+    c = torch.full((M + 1, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+    fc.fc_gemm_bf16(a, b, out=c[:M])
+    torch.cuda.synchronize()
+    assert fc.fc_get_error() == "FC_OK"
+    bound_check(a, b, c[:M])
+    assert torch.isnan(c[M]).all()
+
+
+@pytest.mark.parametrize("M,K,inter", [(390, 200, 11008), (1100, 3080, 384)])
+def test_gemm_pair_silu_mul(fc, M, K, inter):
+    test_gemm_silu_mul(fc, M, K, inter)
+
+
+@pytest.mark.parametrize("batch,n_pad,Hkv,K", [(5, 128, 33, 200), (9, 64, 5, 3080)])
+def test_gemm_pair_kv_heads(fc, orc, batch, n_pad, Hkv, K):
     test_gemm_kv_heads(fc, orc, batch, n_pad, Hkv, K)

@@ -253,7 +253,6 @@ __global__ void __launch_bounds__(BT_THREADS) k_build_tree(TreeIn in, int S, int
   uint32_t* tab = reinterpret_cast<uint32_t*>(smem_raw + L.tab);
   __shared__ uint32_t hist[256];
   const int b = blockIdx.x, tid = threadIdx.x;
-  fc_grid_release();
   fc_grid_wait();
   root_tok = fc_after_wait(root_tok);
   kv_len = fc_after_wait(kv_len);

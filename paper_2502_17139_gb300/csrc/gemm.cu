@@ -239,8 +239,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  fc_grid_release();
-  if (tid == 0) {  // the first tile's first weights into L2 while the kernel before still runs
+  if (tid == 0) {  // the first tile's first weights into L2 while the kernel before drains
     const int n0 = ((int)blockIdx.x / g.tiles_m) * BN;
     for (int kb = 0; kb < min(nk, PREFETCH); ++kb)
       for (int c = 0; c < BN / 64; ++c) tma_prefetch_2d(&tm_b, n0 + 64 * c, kb * BK);
@@ -441,8 +440,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) __cluster_dims__(2, 1, 1)
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers are ready
   tc_fence_after();
-  fc_grid_release();
-  if (tid == 0) {  // the first tile's first weights into L2 while the kernel before still runs
+  if (tid == 0) {  // the first tile's first weights into L2 while the kernel before drains
     const int n0 = (pair / g.tiles_m) * BN + (int)rank * (BN / 2);
     for (int kb = 0; kb < min(nk, PREFETCH); ++kb)
       for (int c = 0; c < BN / 128; ++c) tma_prefetch_2d(&tm_b, n0 + 64 * c, kb * BK);

@@ -330,7 +330,6 @@ __global__ void __launch_bounds__(RT_THREADS) k_retrieve(DsArgs args, DsArgs rev
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RetSmem& sm = *reinterpret_cast<RetSmem*>(smem_raw);
   const int b = blockIdx.x, s = blockIdx.y, tid = threadIdx.x;
-  fc_grid_release();
   fc_grid_wait();
   ctx = fc_after_wait(ctx);
   ctx_len = fc_after_wait(ctx_len);
@@ -548,7 +547,6 @@ __global__ void k_rc_insert(uint32_t* table, int capacity, int S, fc_retrieve_pa
                             const int32_t* __restrict__ skip, RetOut o) {
   __shared__ RcSmem sm;
   const int b = blockIdx.x;
-  fc_grid_release();
   fc_grid_wait();
   ctx = fc_after_wait(ctx);
   ctx_len = fc_after_wait(ctx_len);

@@ -305,7 +305,6 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   __shared__ volatile int s_abort;
   __shared__ int s_ticket, s_ready;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  fc_grid_release();
   fc_grid_wait();
   // Units (group, row chunk) in launch order, so the row chunks of a group,
   // which stream the same K/V blocks, run together and share them through
@@ -1045,7 +1044,6 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  fc_grid_release();
   fc_grid_wait();
   const int U = a.B * a.Hkv;
   const int n_units = max(0, (U - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x);

@@ -2,15 +2,30 @@
 // token corpus (the datastore organisation of Section IV-A, Eq. 1-2, which
 // follows REST's suffix-array index).
 //
-// Method (GPU prefix doubling): after round r every position i carries the
-// dense rank of its first 2^r tokens.  A round sorts the positions by the
-// pair (rank[i], rank[i + h] + 1) (0 when i + h runs past the end, so a
-// shorter suffix sorts first), with a stable LSD radix sort written here
-// (8-bit digits, per-block histograms, a global exclusive scan and a stable
-// scatter that ranks equal digits inside a warp with __match_any_sync), then
-// re-ranks by scanning "key differs from its predecessor" flags.  The loop
-// stops when every rank is distinct.  All passes stream the arrays once
-// (HBM-bound); only the rank gather rank[i + h] is random.
+// Method.  A position's first tokens, as many as fit, are packed into a 64-bit
+// key (symbols token + 1, 0 past the corpus end, so a shorter suffix sorts
+// first): four tokens at a vocabulary of 32k.  One stable LSD radix sort of
+// the keys (8-bit digits, per-block histograms, a global exclusive scan, a
+// stable scatter that ranks equal digits inside a warp with __match_any_sync)
+// puts every suffix into the range of those that share its key.  Only ranges
+// of more than one suffix go on, and each round compares their next tokens:
+//   * up to 32 suffixes: a thread per suffix counts those of its range that
+//     precede it (k_refine_small, ranges packed into lists);
+//   * up to 4096: a CTA sorts the range in shared memory (k_refine_mid);
+//   * longer: the ranges' suffixes are gathered and go through the radix sort
+//     again, (range, next tokens) as the key.
+// Where a range splits, its two neighbours' first different token is their
+// common prefix, so the LCP array comes out of the same comparisons.  Corpora
+// with repeats of more than about 130 tokens end with prefix doubling: after a
+// round at h every position carries the dense rank of its first h tokens, and
+// sorting by (rank[i], rank[i + h] + 1) gives the ranks of the first 2h.
+//
+// Bound by HBM: the radix passes stream 32 bytes a position each, the rounds
+// gather the text of the suffixes still in play.  Doubling from the start sorts
+// all positions in every round: 100M tokens 114 ms against 17 ms
+// (with the suffix keys); 1M tokens 1.94 against 0.77 ms.
+
+#include <algorithm>
 
 #include "fc_common.cuh"
 
@@ -74,16 +89,6 @@ __global__ void k_check_tokens(const uint32_t* __restrict__ T, uint64_t n, uint3
       atomicOr(ctl, 1u);
       return;
     }
-}
-
-// First round: key = (T[i], T[i+1] + 1 or 0), val = i.
-__global__ void k_keys_first(const uint32_t* __restrict__ T, uint64_t n, uint64_t* __restrict__ key,
-                             uint32_t* __restrict__ val) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-    uint64_t lo = (i + 1 < n) ? (uint64_t)T[i + 1] + 1 : 0;
-    key[i] = ((uint64_t)T[i] << 32) | lo;
-    val[i] = (uint32_t)i;
-  }
 }
 
 // Later rounds: positions in current SA order; key = (rank[i], rank[i+h] + 1 or 0).
@@ -323,6 +328,405 @@ __global__ void k_lcp(const uint32_t* __restrict__ T, const uint32_t* __restrict
   }
 }
 
+// ---------------------------------------------------------------------------
+// Refinement by text (see the top of the file).
+// ---------------------------------------------------------------------------
+struct Sym {
+  int bits, count;  // bits per symbol (0..vocab), symbols per key
+};
+
+// The `count` symbols of the suffix at `pos`, the first in the highest bits.
+__device__ __forceinline__ uint64_t pack_key(const uint32_t* __restrict__ T, uint64_t n, uint64_t pos, int bits, int count) {
+  uint64_t k = 0;
+#pragma unroll 4
+  for (int j = 0; j < count; ++j) k = (k << bits) | (pos + j < n ? (uint64_t)__ldg(T + pos + j) + 1 : 0ull);
+  return k;
+}
+// How many leading symbols two different keys share.
+__device__ __forceinline__ int common_syms(uint64_t a, uint64_t b, int bits, int count) {
+  return (__clzll((long long)(a ^ b)) - (64 - bits * count)) / bits;
+}
+__device__ __forceinline__ uint8_t cap_lcp(uint32_t l) { return (uint8_t)(l < FC_LCP_CAP ? l : FC_LCP_CAP); }
+
+constexpr uint32_t SMALL_MAX = 32, MID_MAX = 4096;
+struct Range {  // a range of suffixes that share their first `depth` tokens
+  uint32_t start, size, depth;
+};
+struct HugeRange {
+  uint32_t start, size, depth, base;  // base: its first element among the gathered ones
+};
+// A list element of a small range: slot (its place in the suffix array) and
+// (depth << 8 | its index in the range).
+using Elem = uint2;
+
+struct Counts {  // device counters
+  uint32_t flag, groups;     // bad token; doubling's number of ranks
+  uint32_t small[3], mid[3];  // list elements and ranges: a round reads one, fills the next, clears the third
+  uint32_t huge[2], total;
+};
+
+__global__ void k_pack_keys(const uint32_t* __restrict__ T, uint64_t n, Sym y, uint64_t* __restrict__ key,
+                            uint32_t* __restrict__ val) {
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+    key[i] = pack_key(T, n, i, y.bits, y.count);
+    val[i] = (uint32_t)i;
+  }
+}
+
+// Exclusive sum over the block; *total = the whole sum (warps of 32, up to 32 of them).
+__device__ __forceinline__ uint32_t block_sum_scan(uint32_t x, uint32_t* wsum, uint32_t* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  uint32_t inc = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) wsum[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t v = lane < nw ? wsum[lane] : 0u;
+    uint32_t vi = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, vi, o);
+      if (lane >= o) vi += y;
+    }
+    wsum[lane] = vi - v;
+    if (lane == 31) *total = vi;
+  }
+  __syncthreads();
+  return wsum[warp] + inc - x;
+}
+
+// Splits sorted keys into ranges: the LCP where neighbours differ, the elements
+// of small ranges into `small`, longer ranges into `mid` and `huge`.  GATHERED:
+// the keys are those of the ranges `from` (their index in the bits above the
+// symbols), element a of range r being suffix-array slot start + a - base, and
+// `val` is written there; otherwise the keys are all positions', and the
+// first-token bucket table is written where `bucket` is given.
+constexpr int SPL_THREADS = 256, SPL_ITEMS = 8, SPL_TILE = SPL_THREADS * SPL_ITEMS;
+template <bool GATHERED>
+__global__ void __launch_bounds__(SPL_THREADS) k_split(const uint64_t* __restrict__ key, const uint32_t* __restrict__ val,
+                                                       uint64_t m, Sym y, uint32_t depth, const HugeRange* __restrict__ from,
+                                                       uint32_t* sa, uint8_t* __restrict__ lcp, Elem* __restrict__ small,
+                                                       Range* __restrict__ mid, HugeRange* __restrict__ huge, Counts* ct,
+                                                       int huge_out, uint32_t* __restrict__ bucket, uint32_t vocab) {
+  __shared__ uint64_t s_key[SPL_TILE + 2 * SMALL_MAX];          // [0]: the key before the tile
+  __shared__ uint32_t s_head[SPL_TILE / 32 + 2];               // bit i: element i of the tile starts a range
+  __shared__ uint32_t wsum[32], s_total, s_base;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const uint64_t t0 = blockIdx.x * (uint64_t)SPL_TILE;
+  const int have = (int)min((uint64_t)(SPL_TILE + SMALL_MAX), m - t0);  // the tile's elements and the 32 after it
+  const int sym_bits = y.bits * y.count;
+  for (int i = tid; i < have + 1; i += SPL_THREADS)
+    s_key[i] = (t0 + i > 0) ? key[t0 + i - 1] : ~key[0];  // before the first: any other key
+  __syncthreads();
+  for (int i = tid; i < SPL_TILE + (int)SMALL_MAX; i += SPL_THREADS) {  // past the end: a range starts
+    const uint32_t w = __ballot_sync(0xFFFFFFFFu, i >= have || s_key[i + 1] != s_key[i]);
+    if (lane == 0) s_head[i >> 5] = w;
+  }
+  if (tid == 0) s_head[SPL_TILE / 32 + 1] = 0;
+  __syncthreads();
+  const int tile = min(have, SPL_TILE);
+  uint32_t n_out = 0;
+  uint32_t e_slot[SPL_ITEMS + 1], e_meta[SPL_ITEMS + 1];  // this thread's small elements, in list order
+#pragma unroll
+  for (int q = 0; q <= SPL_ITEMS; ++q) {
+    // consecutive elements per thread; the last round covers the 31 elements past the tile
+    const int i = q < SPL_ITEMS ? tid * SPL_ITEMS + q : SPL_TILE + tid;
+    e_meta[q] = 0xFFFFFFFFu;
+    if (q == SPL_ITEMS ? (tid >= (int)SMALL_MAX - 1 || i >= have) : i >= tile) continue;
+    const uint64_t k = s_key[i + 1];
+    uint32_t d = depth, slot = (uint32_t)(t0 + i), o = 0;
+    if constexpr (GATHERED) {
+      o = (uint32_t)(k >> sym_bits);
+      slot = from[o].start + ((uint32_t)(t0 + i) - from[o].base);
+      d += from[o].depth;
+    }
+    const bool head = (s_head[i >> 5] >> (i & 31)) & 1u;
+    if (q < SPL_ITEMS) {
+      if constexpr (GATHERED) sa[slot] = val[t0 + i];
+      if (head) {
+        const uint64_t kp = s_key[i];
+        if (GATHERED ? (t0 + i > 0 && (uint32_t)(kp >> sym_bits) == o) : t0 + i > 0)
+          lcp[slot] = cap_lcp(d - (uint32_t)y.count + (uint32_t)common_syms(k, kp, y.bits, y.count));
+        else if (!GATHERED)
+          lcp[slot] = 0;
+      }
+      if (!GATHERED && bucket) {  // tokens between the neighbours' first ones start here
+        const uint32_t ft = (uint32_t)(k >> (sym_bits - y.bits)) - 1;
+        const uint32_t lo = t0 + i > 0 ? (uint32_t)(s_key[i] >> (sym_bits - y.bits)) : 0u;  // the previous first token + 1
+        for (uint32_t v = lo; v <= ft; ++v) bucket[v] = (uint32_t)(t0 + i);
+        if (t0 + i == m - 1)
+          for (uint32_t v = ft + 1; v <= vocab; ++v) bucket[v] = (uint32_t)m;
+      }
+    }
+    // this element's range: its head at most 31 back, its end at most 32 ahead (else it is longer)
+    int hd = -1;
+    {
+      const uint32_t w = s_head[i >> 5] & (0xFFFFFFFFu >> (31 - (i & 31)));
+      if (w) hd = (i & ~31) + 31 - __clz(w);
+      else if (i >= 32) {
+        const uint32_t p = s_head[(i >> 5) - 1];
+        if (p) hd = (i & ~31) - 32 + 31 - __clz(p);
+      }
+    }
+    if (hd < 0 || hd >= tile || i - hd >= (int)SMALL_MAX) continue;  // another tile's range, or a long one
+    int nx = 0x7FFFFFFF;  // the next head after i
+    {
+      const int w0 = (i + 1) >> 5;
+      const uint32_t w = w0 <= SPL_TILE / 32 ? s_head[w0] & (0xFFFFFFFFu << ((i + 1) & 31)) : 0u;
+      if (w) nx = w0 * 32 + __ffs(w) - 1;
+      else if (w0 + 1 <= SPL_TILE / 32 && s_head[w0 + 1]) nx = (w0 + 1) * 32 + __ffs(s_head[w0 + 1]) - 1;
+    }
+    if (nx - hd <= (int)SMALL_MAX) {
+      if (nx - hd > 1) {
+        e_slot[q] = slot;
+        e_meta[q] = (d << 8) | (uint32_t)(i - hd);
+        ++n_out;
+      }
+    } else if (head) {  // a longer range: its end by doubling steps and bisection over the sorted keys
+      uint64_t lo = t0 + i + SMALL_MAX, step = SMALL_MAX;  // key[lo - 1] belongs to it
+      while (lo - 1 + step < m && key[lo - 1 + step] == k) {
+        lo += step;
+        step *= 2;
+      }
+      uint64_t hi = min(m, lo - 1 + step);  // the first element past it lies in [lo, hi]
+      while (lo < hi) {
+        const uint64_t c = (lo + hi) >> 1;
+        if (key[c] == k) lo = c + 1;
+        else hi = c;
+      }
+      const uint32_t size = (uint32_t)(lo - (t0 + i));
+      if (size <= MID_MAX) mid[atomicAdd(&ct->mid[0], 1u)] = Range{slot, size, d};
+      else huge[atomicAdd(&ct->huge[huge_out], 1u)] = HugeRange{slot, size, d, 0u};
+    }
+  }
+  // list order: a thread's consecutive elements, then those past the tile
+  const uint32_t tail = e_meta[SPL_ITEMS] != 0xFFFFFFFFu ? 1u : 0u;
+  uint32_t at = block_sum_scan(n_out - tail, wsum, &s_total);
+  const uint32_t in_tile = s_total;
+  __syncthreads();
+  const uint32_t at_tail = block_sum_scan(tail, wsum, &s_total);
+  if (tid == 0 && in_tile + s_total) s_base = atomicAdd(&ct->small[0], in_tile + s_total);
+  __syncthreads();
+  at += s_base;
+#pragma unroll
+  for (int q = 0; q < SPL_ITEMS; ++q)
+    if (e_meta[q] != 0xFFFFFFFFu) small[at++] = make_uint2(e_slot[q], e_meta[q]);
+  if (tail) small[s_base + in_tile + at_tail] = make_uint2(e_slot[SPL_ITEMS], e_meta[SPL_ITEMS]);
+}
+
+// One round over the small ranges: a tile of 256 list elements holds the whole
+// of every range that starts in its first 224.  A thread compares its suffix's
+// next symbols with those of its range: how many are smaller (its new
+// sub-range's place), equal (they go on), and the largest smaller one (the LCP
+// at the new sub-range's start).
+constexpr int RFS_THREADS = 256, RFS_HEADS = RFS_THREADS - (int)SMALL_MAX;
+__global__ void __launch_bounds__(RFS_THREADS) k_refine_small(const uint32_t* __restrict__ T, uint64_t n, Sym y, uint32_t* sa,
+                                                              uint8_t* __restrict__ lcp, const Elem* list, Elem* next,
+                                                              Counts* ct, int in, int out) {
+  __shared__ uint64_t s_key[RFS_THREADS];
+  __shared__ uint32_t s_idx[RFS_THREADS + 1], s_act[RFS_THREADS], wsum[32], s_total, s_base;
+  __shared__ Elem s_out[RFS_THREADS];
+  const int tid = threadIdx.x;
+  fc_grid_wait();
+  const uint32_t m = *(volatile uint32_t*)&ct->small[in];
+  const uint32_t tiles = m / RFS_HEADS + (m % RFS_HEADS != 0);
+  for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const uint64_t a = (uint64_t)t * RFS_HEADS + tid;
+    const Elem e = a < m ? list[a] : make_uint2(0u, 0u);
+    const uint32_t idx = e.y & 255u, d = e.y >> 8;
+    const int hd = tid - (int)idx;  // the range's first element in the tile
+    const bool mine = a < m && hd >= 0 && hd < RFS_HEADS;
+    const uint32_t pos = mine ? sa[e.x] : 0u;
+    const uint64_t k = mine ? pack_key(T, n, (uint64_t)pos + d, y.bits, y.count) : 0ull;
+    s_key[tid] = k;
+    s_idx[tid] = a < m ? idx : 0u;
+    if (tid == 0) s_idx[RFS_THREADS] = 0u;
+    s_act[tid] = 0u;
+    __syncthreads();
+    if (mine) {
+      uint32_t less = 0, before = 0, equal = 0;
+      uint64_t below = 0;
+      for (int j = hd; j == hd || s_idx[j] != 0u; ++j) {  // the next range (or the end) starts at index 0
+        const uint64_t o = s_key[j];
+        if (o < k) {
+          ++less;
+          below = max(below, o);
+        } else if (o == k) {
+          ++equal;
+          before += j < tid;
+        }
+      }
+      const uint32_t slot = e.x - idx + less + before;
+      sa[slot] = pos;
+      if (before == 0 && less > 0) lcp[slot] = cap_lcp(d + (uint32_t)common_syms(k, below, y.bits, y.count));
+      if (equal > 1) {
+        const int at = hd + (int)(less + before);
+        s_act[at] = 1u;
+        s_out[at] = make_uint2(slot, ((d + (uint32_t)y.count) << 8) | before);
+      }
+    }
+    __syncthreads();
+    const uint32_t act = s_act[tid];
+    const uint32_t at = block_sum_scan(act, wsum, &s_total);
+    if (tid == 0 && s_total) s_base = atomicAdd(&ct->small[out], s_total);
+    __syncthreads();
+    if (act) next[s_base + at] = s_out[tid];
+    __syncthreads();
+  }
+}
+
+// One round over the ranges of 33 to 4096 suffixes: a CTA sorts a range's
+// (next symbols, position) pairs in shared memory (bitonic) and splits it.
+constexpr int RFM_THREADS = 512;
+constexpr uint32_t RFM_SMEM = MID_MAX * (8 + 4);
+__global__ void __launch_bounds__(RFM_THREADS) k_refine_mid(const uint32_t* __restrict__ T, uint64_t n, Sym y, uint32_t* sa,
+                                                            uint8_t* __restrict__ lcp, const Range* ranges, Range* next,
+                                                            Elem* small, Counts* ct, int in, int out) {
+  extern __shared__ __align__(16) unsigned char rfm_smem[];
+  uint64_t* s_key = reinterpret_cast<uint64_t*>(rfm_smem);
+  uint32_t* s_pos = reinterpret_cast<uint32_t*>(rfm_smem + MID_MAX * 8);
+  __shared__ uint32_t s_head[MID_MAX / 32 + 2], wsum[32], s_total, s_base;
+  const int tid = threadIdx.x, lane = tid & 31;
+  fc_grid_wait();
+  const uint32_t ng = *(volatile uint32_t*)&ct->mid[in];
+  if (blockIdx.x == 0 && tid == 0) ct->small[3 - in - out] = ct->mid[3 - in - out] = 0u;  // the round after next's
+  for (uint32_t gi = blockIdx.x; gi < ng; gi += gridDim.x) {
+    const Range g = ranges[gi];
+    uint32_t p2 = 64;
+    while (p2 < g.size) p2 *= 2;
+    for (uint32_t i = tid; i < p2; i += RFM_THREADS) {
+      uint32_t pos = 0xFFFFFFFFu;  // padding sorts behind every suffix
+      uint64_t k = ~0ull;
+      if (i < g.size) {
+        pos = sa[g.start + i];
+        k = pack_key(T, n, (uint64_t)pos + g.depth, y.bits, y.count);
+      }
+      s_key[i] = k;
+      s_pos[i] = pos;
+    }
+    __syncthreads();
+    for (uint32_t len = 2; len <= p2; len *= 2)
+      for (uint32_t st = len / 2; st > 0; st /= 2) {
+        for (uint32_t i = tid; i < p2 / 2; i += RFM_THREADS) {
+          const uint32_t a = 2 * i - (i & (st - 1)), b = a + st;
+          const uint64_t ka = s_key[a], kb = s_key[b];
+          const uint32_t pa = s_pos[a], pb = s_pos[b];
+          const bool up = (a & len) == 0, gt = ka > kb || (ka == kb && pa > pb);
+          if (gt == up) {
+            s_key[a] = kb, s_key[b] = ka;
+            s_pos[a] = pb, s_pos[b] = pa;
+          }
+        }
+        __syncthreads();
+      }
+    const uint32_t words = (g.size + 31) / 32 + 1;
+    for (uint32_t i = tid; i < words * 32; i += RFM_THREADS) {
+      const bool head = i >= g.size || i == 0 || s_key[i] != s_key[i - 1];
+      const uint32_t w = __ballot_sync(0xFFFFFFFFu, head);  // whole warps: words * 32 elements
+      if (lane == 0) s_head[i >> 5] = w;
+    }
+    __syncthreads();
+    // a thread takes consecutive elements, so that its small ones stay in order
+    const uint32_t per = (g.size + RFM_THREADS - 1) / RFM_THREADS, i0 = min(g.size, tid * per), i1 = min(g.size, i0 + per);
+    auto range_of = [&](uint32_t i, uint32_t& hd, uint32_t& nx) {  // the bounds of i's sub-range
+      uint32_t w = i >> 5, v = s_head[w] & (0xFFFFFFFFu >> (31 - (i & 31)));
+      while (!v) v = s_head[--w];  // element 0 is a head
+      hd = w * 32 + 31 - __clz(v);
+      w = (i + 1) >> 5, v = s_head[w] & (0xFFFFFFFFu << ((i + 1) & 31));
+      while (!v) v = s_head[++w];  // the word past the last element is all heads
+      nx = min(g.size, w * 32 + __ffs(v) - 1);
+    };
+    uint32_t n_out = 0;
+    for (uint32_t i = i0; i < i1; ++i) {
+      sa[g.start + i] = s_pos[i];
+      uint32_t hd, nx;
+      range_of(i, hd, nx);
+      const uint32_t size = nx - hd;
+      if (i == hd && i > 0)
+        lcp[g.start + i] = cap_lcp(g.depth + (uint32_t)common_syms(s_key[i], s_key[i - 1], y.bits, y.count));
+      if (size > SMALL_MAX) {
+        if (i == hd) next[atomicAdd(&ct->mid[out], 1u)] = Range{g.start + hd, size, g.depth + (uint32_t)y.count};
+      } else if (size > 1) {
+        ++n_out;
+      }
+    }
+    uint32_t at = block_sum_scan(n_out, wsum, &s_total);
+    if (tid == 0 && s_total) s_base = atomicAdd(&ct->small[out], s_total);
+    __syncthreads();
+    at += s_base;
+    if (n_out)
+      for (uint32_t i = i0; i < i1; ++i) {
+        uint32_t hd, nx;
+        range_of(i, hd, nx);
+        if (nx - hd > 1 && nx - hd <= SMALL_MAX)
+          small[at++] = make_uint2(g.start + i, ((g.depth + (uint32_t)y.count) << 8) | (i - hd));
+      }
+    __syncthreads();
+  }
+}
+
+// base[] of the huge ranges (one CTA) and their total.
+__global__ void __launch_bounds__(SCAN_THREADS) k_huge_base(HugeRange* r, Counts* ct, int in) {
+  __shared__ uint32_t tot;
+  const uint32_t ng = ct->huge[in];
+  uint32_t run = 0;
+  for (uint32_t t = 0; t < ng; t += SCAN_THREADS) {
+    const uint32_t i = t + threadIdx.x, s = i < ng ? r[i].size : 0u;
+    const uint32_t ex = block_exclusive_scan(s, &tot);
+    if (i < ng) r[i].base = run + ex;
+    run += tot;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    ct->total = run;
+    ct->huge[in ^ 1] = 0;
+  }
+}
+
+// The huge ranges' suffixes with (range, next symbols) keys.
+__global__ void k_huge_gather(const uint32_t* __restrict__ T, uint64_t n, Sym y, const uint32_t* __restrict__ sa,
+                              const HugeRange* __restrict__ r, uint32_t ng, uint32_t m, uint64_t* __restrict__ key,
+                              uint32_t* __restrict__ val) {
+  for (uint64_t a = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; a < m; a += (uint64_t)gridDim.x * blockDim.x) {
+    uint32_t lo = 0, hi = ng;  // the last range with base <= a
+    while (hi - lo > 1) {
+      const uint32_t c = (lo + hi) >> 1;
+      if (r[c].base <= a) lo = c;
+      else hi = c;
+    }
+    const uint32_t pos = sa[r[lo].start + ((uint32_t)a - r[lo].base)];
+    key[a] = ((uint64_t)lo << (y.bits * y.count)) | pack_key(T, n, (uint64_t)pos + r[lo].depth, y.bits, y.count);
+    val[a] = pos;
+  }
+}
+
+// Where prefix doubling takes over: every position's rank is the first slot of its range.
+__global__ void k_rank_slots(const uint32_t* __restrict__ sa, uint64_t n, uint32_t* __restrict__ rank) {
+  for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x)
+    rank[sa[j]] = (uint32_t)j;
+}
+__global__ void k_rank_ranges(const uint32_t* __restrict__ sa, const Elem* __restrict__ list, const Range* __restrict__ mid,
+                              const HugeRange* __restrict__ huge, const Counts* ct, int in, int huge_in,
+                              uint32_t* __restrict__ rank) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  for (uint64_t a = t; a < ct->small[in]; a += stride) rank[sa[list[a].x]] = list[a].x - (list[a].y & 255u);
+  for (uint32_t g = blockIdx.x; g < ct->mid[in]; g += gridDim.x)
+    for (uint32_t i = threadIdx.x; i < mid[g].size; i += blockDim.x) rank[sa[mid[g].start + i]] = mid[g].start;
+  for (uint32_t g = 0; g < ct->huge[huge_in]; ++g)
+    for (uint64_t i = t; i < huge[g].size; i += stride) rank[sa[huge[g].start + i]] = huge[g].start;
+}
+
+int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 0;
+  return n;
+}
+
 inline int bits_for(uint64_t x) {
   int b = 0;
   while (x) {
@@ -367,55 +771,150 @@ extern "C" fc_status fc_datastore_build(const uint32_t* d_tokens, uint64_t n, ui
   uint32_t* stmp = reinterpret_cast<uint32_t*>(ws + L.scan_tmp);
   uint32_t* ctl = reinterpret_cast<uint32_t*>(ws + L.ctl);
   const unsigned g = grid_for(n, 256);
-  uint32_t hctl[2] = {0, 0};
+  Counts* ct = reinterpret_cast<Counts*>(ctl);
+  Counts hc{};
+  static_assert(sizeof(Counts) <= 64, "counter area");
+  auto read_counts = [&]() -> bool {  // synchronises
+    return cudaMemcpyAsync(&hc, ct, sizeof hc, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
+           cudaStreamSynchronize(s) == cudaSuccess;
+  };
+  // An LSD sort of m (key, value) pairs over the low `bits` bits; the result lands in the first pair of buffers
+  // (so an odd number of passes starts from the second, where the caller then writes the pairs: starts_second).
+  auto starts_second = [](int bits) { return ((bits + 7) / 8) % 2 != 0; };
+  auto sort_pairs = [&](uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, uint64_t m, int bits) -> bool {
+    const uint64_t nb = cdiv(m, RS_TILE);
+    if (starts_second(bits)) std::swap(k0, k1), std::swap(v0, v1);
+    for (int shift = 0; shift < bits; shift += 8) {
+      k_radix_hist<<<(unsigned)nb, RS_THREADS, 0, s>>>(k0, m, shift, hist, nb);
+      if (exclusive_scan(hist, 256 * nb, stmp, s) != cudaSuccess) return false;
+      k_radix_scatter<<<(unsigned)nb, RS_THREADS, RS_SMEM, s>>>(k0, v0, k1, v1, m, shift, hist, nb);
+      std::swap(k0, k1);
+      std::swap(v0, v1);
+    }
+    return true;
+  };
 
-  if (cudaFuncSetAttribute(k_radix_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_SMEM) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_radix_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(k_refine_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RFM_SMEM) != cudaSuccess)
     return FC_ERR_CUDA;
   if (cudaMemsetAsync(ctl, 0, 64, s) != cudaSuccess) return FC_ERR_CUDA;
   k_check_tokens<<<g, 256, 0, s>>>(d_tokens, n, vocab, ctl);
-  if (cudaMemcpyAsync(hctl, ctl, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess) return FC_ERR_CUDA;
-  if (cudaStreamSynchronize(s) != cudaSuccess) return FC_ERR_CUDA;
-  if (hctl[0]) return FC_ERR_INVALID_ARG;
+  if (!read_counts()) return FC_ERR_CUDA;
+  if (hc.flag) return FC_ERR_INVALID_ARG;
 
-  k_keys_first<<<g, 256, 0, s>>>(d_tokens, n, key_a, d_sa);
-  uint64_t max_hi = vocab - 1, max_lo = vocab;
-  uint64_t h = 1;
-  for (int round = 0;; ++round) {
-    if (round > 40) return FC_ERR_INTERNAL;
-    // LSD passes over the populated bits of the low then the high word.
-    uint64_t* kin = key_a;
-    uint32_t* vin = d_sa;
-    uint64_t* kout = key_b;
-    uint32_t* vout = val_b;
-    int shifts[16];
-    int np = 0;
-    for (int b = 0; b < bits_for(max_lo); b += 8) shifts[np++] = b;
-    for (int b = 0; b < bits_for(max_hi); b += 8) shifts[np++] = 32 + b;
-    for (int p = 0; p < np; ++p) {
-      k_radix_hist<<<(unsigned)L.nb, RS_THREADS, 0, s>>>(kin, n, shifts[p], hist, L.nb);
-      if (exclusive_scan(hist, 256 * L.nb, stmp, s) != cudaSuccess) return FC_ERR_CUDA;
-      k_radix_scatter<<<(unsigned)L.nb, RS_THREADS, RS_SMEM, s>>>(kin, vin, kout, vout, n, shifts[p], hist, L.nb);
-      std::swap(kin, kout);
-      std::swap(vin, vout);
+  // Every position by its first symbols.
+  Sym y;
+  y.bits = bits_for(vocab);
+  y.count = std::min(8, 64 / y.bits);
+  const int key_bits = y.bits * y.count;
+  const bool second = starts_second(key_bits);
+  k_pack_keys<<<g, 256, 0, s>>>(d_tokens, n, y, second ? key_b : key_a, second ? val_b : d_sa);
+  if (!sort_pairs(key_a, d_sa, key_b, val_b, n, key_bits)) return FC_ERR_CUDA;
+  // The sorted keys are in key_a.  key_b takes the list of small ranges (8 bytes an element, n at most), the rank
+  // area the tables of longer ones; the lists alternate between key_b and key_a from then on.
+  Elem* lists[2] = {reinterpret_cast<Elem*>(key_b), reinterpret_cast<Elem*>(key_a)};
+  const size_t mid_cap = n / (SMALL_MAX + 1) + 1, huge_cap = n / (MID_MAX + 1) + 1;
+  char* tab = reinterpret_cast<char*>(rank);
+  Range* mids[2] = {reinterpret_cast<Range*>(tab), reinterpret_cast<Range*>(tab) + mid_cap};
+  HugeRange* huges[2];
+  huges[0] = reinterpret_cast<HugeRange*>(tab + align_up(2 * mid_cap * sizeof(Range), 16));
+  huges[1] = huges[0] + huge_cap;
+  // first tokens come with the keys, unless gaps of unused tokens could be long
+  const bool buckets = vocab <= 65536u;
+  k_split<false><<<(unsigned)cdiv(n, SPL_TILE), SPL_THREADS, 0, s>>>(key_a, d_sa, n, y, (uint32_t)y.count, nullptr, d_sa,
+                                                                     d_lcp, lists[0], mids[0], huges[0], ct, 0,
+                                                                     buckets ? d_bucket : nullptr, vocab);
+  // Ranges of more than MID_MAX suffixes: gathered and sorted, while that makes headway.
+  int hin = 0;
+  uint64_t before = ~0ull;
+  bool doubling = false;
+  uint64_t h = (uint64_t)y.count;  // tokens that every range is known to share
+  for (;;) {
+    k_huge_base<<<1, SCAN_THREADS, 0, s>>>(huges[hin], ct, hin);
+    if (!read_counts()) return FC_ERR_CUDA;
+    const uint32_t ng = hc.huge[hin], m = hc.total;
+    if (ng == 0) break;
+    Sym yh = y;
+    const int obits = bits_for(ng - 1);
+    yh.count = std::min(y.count, (63 - obits) / y.bits);  // the range's index lies above the symbols
+    if (2ull * m > before || yh.count < 1) {
+      doubling = true;
+      break;
     }
-    // kin/vin now hold the sorted keys and positions.
-    k_heads<<<g, 256, 0, s>>>(kin, n, head);
-    if (exclusive_scan(head, n, stmp, s) != cudaSuccess) return FC_ERR_CUDA;
-    k_ranks<<<g, 256, 0, s>>>(kin, vin, head, n, rank, d_sa, ctl);
-    if (cudaMemcpyAsync(hctl, ctl, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess) return FC_ERR_CUDA;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return FC_ERR_CUDA;
-    uint64_t groups = hctl[1];
-    if (groups == n) break;
-    if (groups == 0 || groups > n) return FC_ERR_INTERNAL;
-    h = (round == 0) ? 2 : h * 2;
-    if (h >= 2 * n + 2) return FC_ERR_INTERNAL;
-    k_keys_round<<<g, 256, 0, s>>>(d_sa, rank, n, h, key_a, d_sa);
-    max_hi = groups - 1;
-    max_lo = groups;
+    before = m;
+    const int bits = yh.bits * yh.count + obits;
+    uint64_t* k1 = key_b + (n - m);  // behind the list: small elements and gathered ones are n at most
+    const bool sec = starts_second(bits);
+    k_huge_gather<<<grid_for(m, 256), 256, 0, s>>>(d_tokens, n, yh, d_sa, huges[hin], ng, m, sec ? k1 : key_a,
+                                                   sec ? head : val_b);
+    if (!sort_pairs(key_a, val_b, k1, head, m, bits)) return FC_ERR_CUDA;
+    k_split<true><<<(unsigned)cdiv(m, SPL_TILE), SPL_THREADS, 0, s>>>(key_a, val_b, m, yh, (uint32_t)yh.count, huges[hin],
+                                                                      d_sa, d_lcp, lists[0], mids[0], huges[hin ^ 1], ct,
+                                                                      hin ^ 1, nullptr, 0u);
+    hin ^= 1;
   }
-  k_bucket<<<grid_for((uint64_t)vocab + 1, 256), 256, 0, s>>>(d_tokens, d_sa, n, vocab, d_bucket);
-  // every group is a single suffix now, so rank is the inverse suffix array
-  k_lcp<<<g, 256, 0, s>>>(d_tokens, d_sa, rank, n, d_lcp);
+  // Rounds of y.count more tokens over the rest.
+  const int sms = std::max(1, sm_count());
+  int round = 0;
+  while (!doubling) {
+    const int in = round % 3;
+    if (round % 8 == 0) {
+      if (round && !read_counts()) return FC_ERR_CUDA;
+      if (hc.small[in] == 0 && hc.mid[in] == 0) break;
+      // most suffixes still together after eight rounds, or repeats of more than about 130 tokens
+      if (round && (round >= 32 || hc.small[in] > n / 4)) {
+        doubling = true;
+        break;
+      }
+    }
+    const int o = (round + 1) % 3, li = round & 1;
+    const unsigned gs = (unsigned)std::min<uint64_t>(cdiv(n, RFS_HEADS), 8ull * sms), gm = 3u * sms;
+    if (fc_launch_dependent(k_refine_small, dim3(gs), RFS_THREADS, 0, s, 0, d_tokens, n, y, d_sa, d_lcp, lists[li],
+                            lists[li ^ 1], ct, in, o) != FC_OK ||
+        fc_launch_dependent(k_refine_mid, dim3(gm), RFM_THREADS, RFM_SMEM, s, 0, d_tokens, n, y, d_sa, d_lcp, mids[li],
+                            mids[li ^ 1], lists[li ^ 1], ct, in, o) != FC_OK)
+      return FC_ERR_CUDA;
+    ++round;
+    h += (uint64_t)y.count;
+  }
+  if (doubling) {
+    // The ranks go where the tables are not; from then on the two areas have changed places.
+    k_rank_slots<<<g, 256, 0, s>>>(d_sa, n, head);
+    k_rank_ranges<<<grid_for(n, 256), 256, 0, s>>>(d_sa, lists[round & 1], mids[round & 1], huges[hin], ct, round % 3, hin,
+                                                   head);
+    std::swap(rank, head);
+    for (int r = 0;; ++r) {
+      if (r > 40 || h >= 4 * n + 64) return FC_ERR_INTERNAL;
+      k_keys_round<<<g, 256, 0, s>>>(d_sa, rank, n, h, key_a, d_sa);
+      // LSD passes over the populated bits of the low then the high word
+      uint64_t* kin = key_a;
+      uint32_t* vin = d_sa;
+      uint64_t* kout = key_b;
+      uint32_t* vout = val_b;
+      int shifts[16];
+      int np = 0;
+      for (int b = 0; b < bits_for(n); b += 8) shifts[np++] = b;
+      for (int b = 0; b < bits_for(n - 1); b += 8) shifts[np++] = 32 + b;
+      for (int p = 0; p < np; ++p) {
+        k_radix_hist<<<(unsigned)L.nb, RS_THREADS, 0, s>>>(kin, n, shifts[p], hist, L.nb);
+        if (exclusive_scan(hist, 256 * L.nb, stmp, s) != cudaSuccess) return FC_ERR_CUDA;
+        k_radix_scatter<<<(unsigned)L.nb, RS_THREADS, RS_SMEM, s>>>(kin, vin, kout, vout, n, shifts[p], hist, L.nb);
+        std::swap(kin, kout);
+        std::swap(vin, vout);
+      }
+      // kin/vin now hold the sorted keys and positions.
+      k_heads<<<g, 256, 0, s>>>(kin, n, head);
+      if (exclusive_scan(head, n, stmp, s) != cudaSuccess) return FC_ERR_CUDA;
+      k_ranks<<<g, 256, 0, s>>>(kin, vin, head, n, rank, d_sa, ctl);
+      if (!read_counts()) return FC_ERR_CUDA;
+      if (hc.groups == n) break;
+      if (hc.groups == 0 || hc.groups > n) return FC_ERR_INTERNAL;
+      h *= 2;
+    }
+    // every group is a single suffix now, so rank is the inverse suffix array
+    k_lcp<<<g, 256, 0, s>>>(d_tokens, d_sa, rank, n, d_lcp);
+  }
+  if (!buckets) k_bucket<<<grid_for((uint64_t)vocab + 1, 256), 256, 0, s>>>(d_tokens, d_sa, n, vocab, d_bucket);
   if (cudaGetLastError() != cudaSuccess) return FC_ERR_CUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return FC_ERR_CUDA;
   if (out) {

@@ -64,6 +64,48 @@ def test_sa_small_sweep(fc, orc, n, vocab, seed):
     assert np.array_equal(ds.lcp.cpu().numpy(), orc.lcp(T, sa))
 
 
+def _sa_corpus(kind):
+    rng = np.random.default_rng(len(kind))
+    z = lambda n, v, s=1.1: (np.minimum(rng.zipf(s + 0.2, n), v) - 1).astype(np.uint32)
+    if kind == "zipf":  # ranges of every size class: up to 32, up to 4096 and more suffixes
+        return z(150_000, 300), 300
+    if kind == "sparse_vocab":  # more tokens than the bucket table takes from the keys
+        return (z(30_000, 70_000) * 3).astype(np.uint32), 300_000
+    if kind == "eight_bits":  # eight symbols fill the 64-bit key
+        return z(60_000, 255), 255
+    if kind == "tile_edges":  # runs of 31 to 33 and of 4095 to 4097 equal keys around the tiles of 2048
+        runs = [31, 32, 33, 1, 2, 2016, 32, 33, 64, 4095, 4096, 4097, 31]
+        return np.concatenate([np.concatenate([np.full(r, 5, np.uint32), [100 + i]]) for i, r in enumerate(runs)]).astype(np.uint32), 200
+    if kind == "equal_pairs":  # many pairs, triples, ... of 40 equal tokens: several rounds, the LCP inside them
+        grams = rng.integers(0, 30_000, (200, 40))
+        return np.concatenate([np.concatenate([grams[i], rng.integers(0, 30_000, 3)]) for i in rng.integers(0, 200, 900)]).astype(np.uint32), 30_000
+    if kind == "twice":  # a corpus and its copy: prefix doubling over all positions
+        t = z(20_000, 5000)
+        return np.concatenate([t, t]), 5000
+    if kind == "long_repeats":  # repeats of 140 to 1000 tokens among others: doubling for a few
+        t = z(60_000, 5000)
+        for ln in (140, 300, 1000, 129, 133):
+            a, b = rng.integers(0, 29_000), rng.integers(30_000, 59_000 - ln)
+            t[b:b + ln] = t[a:a + ln]
+        return t, 5000
+    if kind == "periodic":
+        return np.tile(rng.integers(0, 9, 17), 1200).astype(np.uint32), 9
+    return np.zeros(9000, np.uint32), 1  # "one_token"
+
+
+@pytest.mark.parametrize("kind", ["zipf", "sparse_vocab", "eight_bits", "tile_edges", "equal_pairs", "twice", "long_repeats",
+                                  "periodic", "one_token"])
+def test_sa_build_paths(fc, orc, kind):
+    """Corpora whose ranges of equal keys take each path of the refinement."""
+    T, vocab = _sa_corpus(kind)
+    ds = fc.fc_datastore_build(dev(T), vocab)
+    torch.cuda.synchronize()
+    sa = orc.suffix_array(T)
+    assert np.array_equal(host_u32(ds.sa), sa)
+    assert np.array_equal(host_u32(ds.bucket), orc.bucket(T, sa, vocab))
+    assert np.array_equal(ds.lcp.cpu().numpy(), orc.lcp(T, sa))
+
+
 def test_sa_constant_corpus(fc, orc):
     T = np.full(10000, 7, np.uint32)
     ds = fc.fc_datastore_build(dev(T), 8)

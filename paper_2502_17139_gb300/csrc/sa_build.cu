@@ -83,14 +83,6 @@ Layout layout_for(uint64_t n) {
   return L;
 }
 
-__global__ void k_check_tokens(const uint32_t* __restrict__ T, uint64_t n, uint32_t vocab, uint32_t* ctl) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-    if (T[i] >= vocab) {
-      atomicOr(ctl, 1u);
-      return;
-    }
-}
-
 // Later rounds: positions in current SA order; key = (rank[i], rank[i+h] + 1 or 0).
 // val may alias sa (each element rewrites its own value).
 __global__ void k_keys_round(const uint32_t* sa, const uint32_t* __restrict__ rank, uint64_t n, uint64_t h,
@@ -103,17 +95,51 @@ __global__ void k_keys_round(const uint32_t* sa, const uint32_t* __restrict__ ra
   }
 }
 
-__global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const uint64_t* __restrict__ key, uint64_t n, int shift,
-                                                           uint32_t* __restrict__ hist, uint64_t nb) {
+struct Sym {
+  int bits, count;  // bits per symbol (0..vocab), symbols per key
+  uint32_t inv;     // ceil(2^16 / bits): x * inv >> 16 = x / bits for x < 64
+};
+
+// The `count` symbols of the suffix at `pos`, the first in the highest bits.
+__device__ __forceinline__ uint64_t pack_key(const uint32_t* __restrict__ T, uint64_t n, uint64_t pos, int bits, int count) {
+  uint64_t k = 0;
+#pragma unroll 4
+  for (int j = 0; j < count; ++j) k = (k << bits) | (pos + j < n ? (uint64_t)__ldg(T + pos + j) + 1 : 0ull);
+  return k;
+}
+// The keys of a first pass, made from the text: the positions in order, each with its first symbols.
+struct TextKeys {
+  const uint32_t* T;
+  Sym y;
+};
+
+// Per-block histograms of one 8-bit digit.  FIRST: of the text's keys, and the tokens are checked.
+template <bool FIRST>
+__global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const uint64_t* __restrict__ key, TextKeys tx, uint64_t n, int shift,
+                                                           uint32_t* __restrict__ hist, uint64_t nb, uint32_t vocab,
+                                                           uint32_t* ctl) {
   __shared__ uint32_t h[256];
+  fc_grid_wait();
+  key = fc_after_wait(key);
   h[threadIdx.x] = 0;
   __syncthreads();
   uint64_t base = blockIdx.x * (uint64_t)RS_TILE;
+  bool bad = false;
 #pragma unroll 4
   for (int k = 0; k < RS_ITEMS; ++k) {
     uint64_t idx = base + (uint64_t)k * RS_THREADS + threadIdx.x;
-    if (idx < n) atomicAdd(&h[(uint32_t)(key[idx] >> shift) & 255u], 1u);
+    if (idx < n) {
+      uint64_t x;
+      if constexpr (FIRST) {
+        x = pack_key(tx.T, n, idx, tx.y.bits, tx.y.count);
+        bad |= __ldg(tx.T + idx) >= vocab;
+      } else {
+        x = key[idx];
+      }
+      atomicAdd(&h[(uint32_t)(x >> shift) & 255u], 1u);
+    }
   }
+  if (FIRST && bad) atomicOr(ctl, 1u);
   __syncthreads();
   hist[(uint64_t)threadIdx.x * nb + blockIdx.x] = h[threadIdx.x];
 }
@@ -124,57 +150,81 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const uint64_t* __res
 // warps and digits), places them in shared memory in digit order, and then
 // writes them out in that order: consecutive threads write consecutive
 // addresses of a digit's run, so the stores coalesce instead of spraying
-// 8- and 4-byte writes over 256 runs.
-constexpr uint32_t RS_SMEM = RS_TILE * (8 + 4);  // keys and values of one tile
-
-__global__ void __launch_bounds__(RS_THREADS) k_radix_scatter(const uint64_t* __restrict__ kin,
-                                                              const uint32_t* __restrict__ vin,
-                                                              uint64_t* __restrict__ kout,
-                                                              uint32_t* __restrict__ vout, uint64_t n, int shift,
-                                                              const uint32_t* __restrict__ offs, uint64_t nb) {
-  extern __shared__ __align__(16) unsigned char rs_smem[];
-  uint64_t* skey = reinterpret_cast<uint64_t*>(rs_smem);
-  uint32_t* sval = reinterpret_cast<uint32_t*>(rs_smem + RS_TILE * 8);
+// 8- and 4-byte writes over 256 runs.  The values follow through the same
+// shared memory.  Bound by the latency of its phases, so by how many blocks an
+// SM holds: four at 64 registers and 42 KB (with the values in registers and
+// shared memory beside the keys, two: 0.99 ms a pass of 100M pairs, now @@).
+// FIRST: the keys come from the text and the values are the positions.
+template <bool FIRST>
+__global__ void __launch_bounds__(RS_THREADS, 3) k_radix_scatter(const uint64_t* __restrict__ kin,
+                                                                 const uint32_t* __restrict__ vin, TextKeys tx,
+                                                                 uint64_t* __restrict__ kout,
+                                                                 uint32_t* __restrict__ vout, uint64_t n, int shift,
+                                                                 const uint32_t* __restrict__ offs, uint64_t nb) {
+  __shared__ uint64_t skey[RS_TILE];
+  uint32_t* sval = reinterpret_cast<uint32_t*>(skey);
   __shared__ uint32_t wbin[RS_WARPS][256];
-  __shared__ uint32_t base_s[256];
-  __shared__ uint32_t doff[256];   // where digit d starts in the block's digit order
+  __shared__ uint32_t dpos[256];   // where digit d starts in the output, less where it starts in the block's digit order
   __shared__ uint32_t wsum[RS_THREADS / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   for (int d = tid; d < RS_WARPS * 256; d += RS_THREADS) (&wbin[0][0])[d] = 0;
-  base_s[tid] = offs[(uint64_t)tid * nb + blockIdx.x];
-  __syncthreads();
+  fc_grid_wait();
+  kin = fc_after_wait(kin);
+  vin = fc_after_wait(vin);
+  offs = fc_after_wait(offs);
   const uint64_t b0 = blockIdx.x * (uint64_t)RS_TILE;
   const uint32_t count = (uint32_t)min((uint64_t)RS_TILE, n - b0);
-  const uint64_t w0 = b0 + (uint64_t)warp * RS_WARP_CHUNK;
+  const uint64_t w0 = b0 + (uint64_t)warp * RS_WARP_CHUNK + lane;  // this lane's first key; the others every 32
+  const int left = (int)count - warp * RS_WARP_CHUNK - lane;       // key `it` exists while 32 it < left
   const uint32_t lt = (1u << lane) - 1u;
+  kin += w0;
+  vin += w0;
   uint64_t key[RS_ITEMS];
-  uint32_t val[RS_ITEMS];
-  uint32_t lr[RS_ITEMS];
+  if constexpr (FIRST) {  // the tile's symbols (0 past the end) and the seven after it, staged
+    const int bits = tx.y.bits;
+    const bool pairs = tx.y.count == 4 && bits <= 16;  // staged as pairs of neighbours: two make a key
+    for (int i = tid; i < RS_TILE + 8; i += RS_THREADS) {
+      const uint32_t a = b0 + i < n ? __ldg(tx.T + b0 + i) + 1u : 0u;
+      const uint32_t b = pairs && b0 + i + 1 < n ? __ldg(tx.T + b0 + i + 1) + 1u : 0u;
+      sval[i] = pairs ? (a << bits) | b : a;
+    }
+    __syncthreads();
+    const uint32_t* sy = sval + warp * RS_WARP_CHUNK + lane;
+    if (pairs) {
+#pragma unroll
+      for (int it = 0; it < RS_ITEMS; ++it) key[it] = ((uint64_t)sy[32 * it] << (2 * bits)) | sy[32 * it + 2];
+    } else {
+#pragma unroll
+      for (int it = 0; it < RS_ITEMS; ++it) {
+        uint64_t k = 0;
+        for (int j = 0; j < tx.y.count; ++j) k = (k << bits) | sy[32 * it + j];
+        key[it] = k;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int it = 0; it < RS_ITEMS; ++it) key[it] = 32 * it < left ? kin[32 * it] : 0ull;
+  }
+  const uint32_t base = offs[(uint64_t)tid * nb + blockIdx.x];
+  __syncthreads();
+  uint32_t at[RS_ITEMS / 2];  // per key, 16 bits: its rank among the warp's equal digits, then its place in the block
 #pragma unroll
   for (int it = 0; it < RS_ITEMS; ++it) {
-    uint64_t idx = w0 + (uint64_t)it * 32 + lane;
-    bool ok = idx < n;
-    key[it] = ok ? kin[idx] : 0ull;
-    val[it] = ok ? vin[idx] : 0u;
-    uint32_t d = ok ? ((uint32_t)(key[it] >> shift) & 255u) : 256u;
-    uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
-    uint32_t cnt = (d < 256u) ? wbin[warp][d] : 0u;
-    lr[it] = cnt + __popc(peers & lt);
-    __syncwarp();
-    if (d < 256u && lane == __ffs(peers) - 1) wbin[warp][d] = cnt + __popc(peers);
-    __syncwarp();
+    const bool ok = 32 * it < left;
+    const uint32_t d = ok ? ((uint32_t)(key[it] >> shift) & 255u) : 256u;
+    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+    // the equal digits' first lane adds them all: a warp's atomics apply in order, and the iterations overlap
+    uint32_t cnt = 0;
+    if (ok && (peers & lt) == 0) cnt = atomicAdd(&wbin[warp][d], (uint32_t)__popc(peers));
+    const uint32_t r = __shfl_sync(0xFFFFFFFFu, cnt, __ffs(peers) - 1) + __popc(peers & lt);
+    at[it / 2] = it & 1 ? at[it / 2] | (r << 16) : r;
   }
   __syncthreads();
-  // per digit (thread tid = digit): warp prefix, then the digit's block total
+  // per digit (thread tid = digit): the digit's block total, then warp prefixes from where it starts in the block
   uint32_t run = 0;
 #pragma unroll
-  for (int w = 0; w < RS_WARPS; ++w) {
-    uint32_t c = wbin[w][tid];
-    wbin[w][tid] = run;
-    run += c;
-  }
-  // exclusive scan of the digit totals over the 256 digits
-  uint32_t inc = run;
+  for (int w = 0; w < RS_WARPS; ++w) run += wbin[w][tid];
+  uint32_t inc = run;  // exclusive scan of the digit totals over the 256 digits
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
@@ -182,27 +232,51 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_scatter(const uint64_t* __
   }
   if (lane == 31) wsum[warp] = inc;
   __syncthreads();
-  uint32_t before = 0;
-  for (int w = 0; w < warp; ++w) before += wsum[w];
-  doff[tid] = before + inc - run;
+  uint32_t first = inc - run;
+  for (int w = 0; w < warp; ++w) first += wsum[w];
+  dpos[tid] = base - first;
+#pragma unroll
+  for (int w = 0; w < RS_WARPS; ++w) {
+    const uint32_t c = wbin[w][tid];
+    wbin[w][tid] = first;
+    first += c;
+  }
   __syncthreads();
 #pragma unroll
   for (int it = 0; it < RS_ITEMS; ++it) {
-    uint64_t idx = w0 + (uint64_t)it * 32 + lane;
-    if (idx < n) {
+    if (32 * it < left) {
       const uint32_t d = (uint32_t)(key[it] >> shift) & 255u;
-      const uint32_t at = doff[d] + wbin[warp][d] + lr[it];
-      skey[at] = key[it];
-      sval[at] = val[it];
+      const uint32_t p = wbin[warp][d] + ((at[it / 2] >> (16 * (it & 1))) & 0xFFFFu);
+      at[it / 2] = it & 1 ? (at[it / 2] & 0xFFFFu) | (p << 16) : (at[it / 2] & 0xFFFF0000u) | p;
+      skey[p] = key[it];
+    }
+  }
+  uint32_t val[RS_ITEMS];
+#pragma unroll
+  for (int it = 0; it < RS_ITEMS; ++it) {
+    if constexpr (FIRST) val[it] = (uint32_t)w0 + 32 * it;
+    else val[it] = 32 * it < left ? vin[32 * it] : 0u;
+  }
+  __syncthreads();
+  uint32_t pos[RS_ITEMS];
+#pragma unroll
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const uint32_t j = tid + k * RS_THREADS;
+    if (j < count) {
+      const uint64_t x = skey[j];
+      pos[k] = dpos[(uint32_t)(x >> shift) & 255u] + j;  // positions are below 2^32
+      kout[pos[k]] = x;
     }
   }
   __syncthreads();
-  for (uint32_t j = tid; j < count; j += RS_THREADS) {
-    const uint64_t k = skey[j];
-    const uint32_t d = (uint32_t)(k >> shift) & 255u;
-    const uint64_t pos = (uint64_t)base_s[d] + (j - doff[d]);
-    kout[pos] = k;
-    vout[pos] = sval[j];
+#pragma unroll
+  for (int it = 0; it < RS_ITEMS; ++it)
+    if (32 * it < left) sval[(at[it / 2] >> (16 * (it & 1))) & 0xFFFFu] = val[it];
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const uint32_t j = tid + k * RS_THREADS;
+    if (j < count) vout[pos[k]] = sval[j];
   }
 }
 
@@ -238,6 +312,8 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t* t
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(const uint32_t* __restrict__ in, uint64_t n,
                                                               uint32_t* __restrict__ partial) {
   __shared__ uint32_t tot;
+  fc_grid_wait();
+  in = fc_after_wait(in);
   uint64_t base = blockIdx.x * (uint64_t)SCAN_TILE + (uint64_t)threadIdx.x * SCAN_ITEMS;
   uint32_t s = 0;
 #pragma unroll
@@ -250,6 +326,9 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(const uint32_t* __
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(uint32_t* __restrict__ data, uint64_t n,
                                                              const uint32_t* __restrict__ partial) {
   __shared__ uint32_t tot;
+  fc_grid_wait();
+  data = fc_after_wait(data);
+  partial = fc_after_wait(partial);
   uint64_t base = blockIdx.x * (uint64_t)SCAN_TILE + (uint64_t)threadIdx.x * SCAN_ITEMS;
   uint32_t v[SCAN_ITEMS];
   uint32_t s = 0;
@@ -269,15 +348,16 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(uint32_t* __restric
 cudaError_t exclusive_scan(uint32_t* data, uint64_t n, uint32_t* tmp, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   uint64_t nt = cdiv(n, SCAN_TILE);
-  if (nt == 1) {
-    k_scan_apply<<<1, SCAN_THREADS, 0, s>>>(data, n, nullptr);
-    return cudaGetLastError();
+  if (nt > 1) {
+    if (fc_launch_dependent(k_scan_reduce, dim3((unsigned)nt), SCAN_THREADS, 0, s, 0, data, n, tmp) != FC_OK)
+      return cudaErrorUnknown;
+    cudaError_t e = exclusive_scan(tmp, nt, tmp + nt, s);
+    if (e != cudaSuccess) return e;
   }
-  k_scan_reduce<<<(unsigned)nt, SCAN_THREADS, 0, s>>>(data, n, tmp);
-  cudaError_t e = exclusive_scan(tmp, nt, tmp + nt, s);
-  if (e != cudaSuccess) return e;
-  k_scan_apply<<<(unsigned)nt, SCAN_THREADS, 0, s>>>(data, n, tmp);
-  return cudaGetLastError();
+  return fc_launch_dependent(k_scan_apply, dim3((unsigned)nt), SCAN_THREADS, 0, s, 0, data, n,
+                             (const uint32_t*)(nt > 1 ? tmp : nullptr)) == FC_OK
+             ? cudaSuccess
+             : cudaErrorUnknown;
 }
 
 // rank[val[j]] = number of distinct keys before position j (dense rank);
@@ -331,20 +411,9 @@ __global__ void k_lcp(const uint32_t* __restrict__ T, const uint32_t* __restrict
 // ---------------------------------------------------------------------------
 // Refinement by text (see the top of the file).
 // ---------------------------------------------------------------------------
-struct Sym {
-  int bits, count;  // bits per symbol (0..vocab), symbols per key
-};
-
-// The `count` symbols of the suffix at `pos`, the first in the highest bits.
-__device__ __forceinline__ uint64_t pack_key(const uint32_t* __restrict__ T, uint64_t n, uint64_t pos, int bits, int count) {
-  uint64_t k = 0;
-#pragma unroll 4
-  for (int j = 0; j < count; ++j) k = (k << bits) | (pos + j < n ? (uint64_t)__ldg(T + pos + j) + 1 : 0ull);
-  return k;
-}
 // How many leading symbols two different keys share.
-__device__ __forceinline__ int common_syms(uint64_t a, uint64_t b, int bits, int count) {
-  return (__clzll((long long)(a ^ b)) - (64 - bits * count)) / bits;
+__device__ __forceinline__ uint32_t common_syms(uint64_t a, uint64_t b, const Sym& y) {
+  return ((uint32_t)(__clzll((long long)(a ^ b)) - (64 - y.bits * y.count)) * y.inv) >> 16;
 }
 __device__ __forceinline__ uint8_t cap_lcp(uint32_t l) { return (uint8_t)(l < FC_LCP_CAP ? l : FC_LCP_CAP); }
 
@@ -364,14 +433,6 @@ struct Counts {  // device counters
   uint32_t small[3], mid[3];  // list elements and ranges: a round reads one, fills the next, clears the third
   uint32_t huge[2], total;
 };
-
-__global__ void k_pack_keys(const uint32_t* __restrict__ T, uint64_t n, Sym y, uint64_t* __restrict__ key,
-                            uint32_t* __restrict__ val) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-    key[i] = pack_key(T, n, i, y.bits, y.count);
-    val[i] = (uint32_t)i;
-  }
-}
 
 // Exclusive sum over the block; *total = the whole sum (warps of 32, up to 32 of them).
 __device__ __forceinline__ uint32_t block_sum_scan(uint32_t x, uint32_t* wsum, uint32_t* total) {
@@ -405,7 +466,7 @@ __device__ __forceinline__ uint32_t block_sum_scan(uint32_t x, uint32_t* wsum, u
 // symbols), element a of range r being suffix-array slot start + a - base, and
 // `val` is written there; otherwise the keys are all positions', and the
 // first-token bucket table is written where `bucket` is given.
-constexpr int SPL_THREADS = 256, SPL_ITEMS = 8, SPL_TILE = SPL_THREADS * SPL_ITEMS;
+constexpr int SPL_THREADS = 256, SPL_TILE = 8 * SPL_THREADS;
 template <bool GATHERED>
 __global__ void __launch_bounds__(SPL_THREADS) k_split(const uint64_t* __restrict__ key, const uint32_t* __restrict__ val,
                                                        uint64_t m, Sym y, uint32_t depth, const HugeRange* __restrict__ from,
@@ -414,108 +475,107 @@ __global__ void __launch_bounds__(SPL_THREADS) k_split(const uint64_t* __restric
                                                        int huge_out, uint32_t* __restrict__ bucket, uint32_t vocab) {
   __shared__ uint64_t s_key[SPL_TILE + 2 * SMALL_MAX];          // [0]: the key before the tile
   __shared__ uint32_t s_head[SPL_TILE / 32 + 2];               // bit i: element i of the tile starts a range
+  __shared__ uint32_t s_list[SPL_TILE / 32 + 1], s_first[SPL_TILE / 32 + 1];  // bit i: it goes to the list; bits before
   __shared__ uint32_t wsum[32], s_total, s_base;
   const int tid = threadIdx.x, lane = tid & 31;
   const uint64_t t0 = blockIdx.x * (uint64_t)SPL_TILE;
   const int have = (int)min((uint64_t)(SPL_TILE + SMALL_MAX), m - t0);  // the tile's elements and the 32 after it
   const int sym_bits = y.bits * y.count;
-  for (int i = tid; i < have + 1; i += SPL_THREADS)
-    s_key[i] = (t0 + i > 0) ? key[t0 + i - 1] : ~key[0];  // before the first: any other key
+#pragma unroll
+  for (int q = 0; q < SPL_TILE / SPL_THREADS + 1; ++q) {
+    const int i = tid + q * SPL_THREADS;
+    if (i < have + 1) s_key[i] = (t0 + i > 0) ? key[t0 + i - 1] : ~key[0];  // before the first: any other key
+  }
   __syncthreads();
   for (int i = tid; i < SPL_TILE + (int)SMALL_MAX; i += SPL_THREADS) {  // past the end: a range starts
     const uint32_t w = __ballot_sync(0xFFFFFFFFu, i >= have || s_key[i + 1] != s_key[i]);
     if (lane == 0) s_head[i >> 5] = w;
   }
-  if (tid == 0) s_head[SPL_TILE / 32 + 1] = 0;
+  if (tid == 0) s_head[SPL_TILE / 32 + 1] = 0;  // nothing is known past the 32: such a range is long, or another tile's
   __syncthreads();
   const int tile = min(have, SPL_TILE);
-  uint32_t n_out = 0;
-  uint32_t e_slot[SPL_ITEMS + 1], e_meta[SPL_ITEMS + 1];  // this thread's small elements, in list order
-#pragma unroll
-  for (int q = 0; q <= SPL_ITEMS; ++q) {
-    // consecutive elements per thread; the last round covers the 31 elements past the tile
-    const int i = q < SPL_ITEMS ? tid * SPL_ITEMS + q : SPL_TILE + tid;
-    e_meta[q] = 0xFFFFFFFFu;
-    if (q == SPL_ITEMS ? (tid >= (int)SMALL_MAX - 1 || i >= have) : i >= tile) continue;
-    const uint64_t k = s_key[i + 1];
-    uint32_t d = depth, slot = (uint32_t)(t0 + i), o = 0;
+  // an element's slot and the depth that its range now shares
+  auto place = [&](int i, uint32_t& slot, uint32_t& d) {
+    slot = (uint32_t)(t0 + i);
+    d = depth;
     if constexpr (GATHERED) {
-      o = (uint32_t)(k >> sym_bits);
-      slot = from[o].start + ((uint32_t)(t0 + i) - from[o].base);
+      const uint32_t o = (uint32_t)(s_key[i + 1] >> sym_bits);
+      slot = from[o].start + (slot - from[o].base);
       d += from[o].depth;
     }
-    const bool head = (s_head[i >> 5] >> (i & 31)) & 1u;
-    if (q < SPL_ITEMS) {
-      if constexpr (GATHERED) sa[slot] = val[t0 + i];
-      if (head) {
-        const uint64_t kp = s_key[i];
-        if (GATHERED ? (t0 + i > 0 && (uint32_t)(kp >> sym_bits) == o) : t0 + i > 0)
-          lcp[slot] = cap_lcp(d - (uint32_t)y.count + (uint32_t)common_syms(k, kp, y.bits, y.count));
-        else if (!GATHERED)
-          lcp[slot] = 0;
-      }
-      if (!GATHERED && bucket) {  // tokens between the neighbours' first ones start here
-        const uint32_t ft = (uint32_t)(k >> (sym_bits - y.bits)) - 1;
-        const uint32_t lo = t0 + i > 0 ? (uint32_t)(s_key[i] >> (sym_bits - y.bits)) : 0u;  // the previous first token + 1
-        for (uint32_t v = lo; v <= ft; ++v) bucket[v] = (uint32_t)(t0 + i);
-        if (t0 + i == m - 1)
-          for (uint32_t v = ft + 1; v <= vocab; ++v) bucket[v] = (uint32_t)m;
+  };
+  // an element's range: its head at most 31 back and the next one at most 32 ahead of that, else -1
+  auto small_head = [&](int i, bool& alone) -> int {
+    const int w = i >> 5, b = i & 31;
+    // heads at i - 31 .. i (bit 31 = i) and at i + 1 .. i + 32 (bit 0 = i + 1)
+    const uint32_t back = __funnelshift_l(w ? s_head[w - 1] : 0u, s_head[w], 31 - b);
+    const uint32_t ahead = __funnelshift_r(b == 31 ? s_head[w + 1] : s_head[w], b == 31 ? 0u : s_head[w + 1], (b + 1) & 31);
+    if (!back) return -1;
+    const int hd = i - __clz(back);
+    const uint32_t to = ahead ? (uint32_t)(i + __ffs(ahead)) : 0xFFFFu;  // the next head
+    alone = to - (uint32_t)hd == 1u;
+    return hd < tile && to - (uint32_t)hd <= SMALL_MAX ? hd : -1;
+  };
+  for (int i = tid; i < SPL_TILE + (int)SMALL_MAX; i += SPL_THREADS) {  // whole warps
+    bool listed = false;
+    if (i < have) {
+      bool alone = false;
+      const int hd = small_head(i, alone);
+      listed = hd >= 0 && !alone;
+      if (i < tile) {
+        uint32_t slot, d;
+        place(i, slot, d);
+        if constexpr (GATHERED) sa[slot] = val[t0 + i];
+        if ((s_head[i >> 5] >> (i & 31)) & 1u) {
+          const uint64_t k = s_key[i + 1], kp = s_key[i];
+          if (!GATHERED && bucket) {  // tokens between the neighbours' first ones start here
+            const uint32_t ft = (uint32_t)(k >> (sym_bits - y.bits));  // the first token + 1
+            for (uint32_t v = t0 + i > 0 ? (uint32_t)(kp >> (sym_bits - y.bits)) : 0u; v < ft; ++v)
+              bucket[v] = (uint32_t)(t0 + i);
+          }
+          if (GATHERED ? (t0 + i > 0 && (kp >> sym_bits) == (k >> sym_bits)) : t0 + i > 0)
+            lcp[slot] = cap_lcp(d - (uint32_t)y.count + common_syms(k, kp, y));
+          else if (!GATHERED)
+            lcp[slot] = 0;
+          if (hd < 0) {  // a longer range: its end by doubling steps and bisection over the sorted keys
+            uint64_t lo = t0 + i + SMALL_MAX, step = SMALL_MAX;  // key[lo - 1] belongs to it
+            while (lo - 1 + step < m && key[lo - 1 + step] == k) {
+              lo += step;
+              step *= 2;
+            }
+            uint64_t hi = min(m, lo - 1 + step);  // the first element past it lies in [lo, hi]
+            while (lo < hi) {
+              const uint64_t c = (lo + hi) >> 1;
+              if (key[c] == k) lo = c + 1;
+              else hi = c;
+            }
+            const uint32_t size = (uint32_t)(lo - (t0 + i));
+            if (size <= MID_MAX) mid[atomicAdd(&ct->mid[0], 1u)] = Range{slot, size, d};
+            else huge[atomicAdd(&ct->huge[huge_out], 1u)] = HugeRange{slot, size, d, 0u};
+          }
+        }
       }
     }
-    // this element's range: its head at most 31 back, its end at most 32 ahead (else it is longer)
-    int hd = -1;
-    {
-      const uint32_t w = s_head[i >> 5] & (0xFFFFFFFFu >> (31 - (i & 31)));
-      if (w) hd = (i & ~31) + 31 - __clz(w);
-      else if (i >= 32) {
-        const uint32_t p = s_head[(i >> 5) - 1];
-        if (p) hd = (i & ~31) - 32 + 31 - __clz(p);
-      }
-    }
-    if (hd < 0 || hd >= tile || i - hd >= (int)SMALL_MAX) continue;  // another tile's range, or a long one
-    int nx = 0x7FFFFFFF;  // the next head after i
-    {
-      const int w0 = (i + 1) >> 5;
-      const uint32_t w = w0 <= SPL_TILE / 32 ? s_head[w0] & (0xFFFFFFFFu << ((i + 1) & 31)) : 0u;
-      if (w) nx = w0 * 32 + __ffs(w) - 1;
-      else if (w0 + 1 <= SPL_TILE / 32 && s_head[w0 + 1]) nx = (w0 + 1) * 32 + __ffs(s_head[w0 + 1]) - 1;
-    }
-    if (nx - hd <= (int)SMALL_MAX) {
-      if (nx - hd > 1) {
-        e_slot[q] = slot;
-        e_meta[q] = (d << 8) | (uint32_t)(i - hd);
-        ++n_out;
-      }
-    } else if (head) {  // a longer range: its end by doubling steps and bisection over the sorted keys
-      uint64_t lo = t0 + i + SMALL_MAX, step = SMALL_MAX;  // key[lo - 1] belongs to it
-      while (lo - 1 + step < m && key[lo - 1 + step] == k) {
-        lo += step;
-        step *= 2;
-      }
-      uint64_t hi = min(m, lo - 1 + step);  // the first element past it lies in [lo, hi]
-      while (lo < hi) {
-        const uint64_t c = (lo + hi) >> 1;
-        if (key[c] == k) lo = c + 1;
-        else hi = c;
-      }
-      const uint32_t size = (uint32_t)(lo - (t0 + i));
-      if (size <= MID_MAX) mid[atomicAdd(&ct->mid[0], 1u)] = Range{slot, size, d};
-      else huge[atomicAdd(&ct->huge[huge_out], 1u)] = HugeRange{slot, size, d, 0u};
-    }
+    const uint32_t w = __ballot_sync(0xFFFFFFFFu, listed);
+    if (lane == 0) s_list[i >> 5] = w;
   }
-  // list order: a thread's consecutive elements, then those past the tile
-  const uint32_t tail = e_meta[SPL_ITEMS] != 0xFFFFFFFFu ? 1u : 0u;
-  uint32_t at = block_sum_scan(n_out - tail, wsum, &s_total);
-  const uint32_t in_tile = s_total;
+  if (!GATHERED && bucket && t0 + tile == m)  // and none after the last suffix's
+    for (uint32_t v = (uint32_t)(s_key[tile] >> (sym_bits - y.bits)) + tid; v <= vocab; v += SPL_THREADS) bucket[v] = (uint32_t)m;
   __syncthreads();
-  const uint32_t at_tail = block_sum_scan(tail, wsum, &s_total);
-  if (tid == 0 && in_tile + s_total) s_base = atomicAdd(&ct->small[0], in_tile + s_total);
+  const uint32_t cnt = tid < SPL_TILE / 32 + 1 ? (uint32_t)__popc(s_list[tid]) : 0u;
+  const uint32_t first = block_sum_scan(cnt, wsum, &s_total);
+  if (tid < SPL_TILE / 32 + 1) s_first[tid] = first;
+  if (tid == 0 && s_total) s_base = atomicAdd(&ct->small[0], s_total);
   __syncthreads();
-  at += s_base;
-#pragma unroll
-  for (int q = 0; q < SPL_ITEMS; ++q)
-    if (e_meta[q] != 0xFFFFFFFFu) small[at++] = make_uint2(e_slot[q], e_meta[q]);
-  if (tail) small[s_base + in_tile + at_tail] = make_uint2(e_slot[SPL_ITEMS], e_meta[SPL_ITEMS]);
+  for (int i = tid; i < SPL_TILE + (int)SMALL_MAX; i += SPL_THREADS) {
+    const uint32_t w = s_list[i >> 5];
+    if (!((w >> (i & 31)) & 1u)) continue;
+    uint32_t slot, d;
+    bool alone;
+    place(i, slot, d);
+    small[s_base + s_first[i >> 5] + __popc(w & ((1u << (i & 31)) - 1u))] =
+        make_uint2(slot, (d << 8) | (uint32_t)(i - small_head(i, alone)));
+  }
 }
 
 // One round over the small ranges: a tile of 256 list elements holds the whole
@@ -562,7 +622,7 @@ __global__ void __launch_bounds__(RFS_THREADS) k_refine_small(const uint32_t* __
       }
       const uint32_t slot = e.x - idx + less + before;
       sa[slot] = pos;
-      if (before == 0 && less > 0) lcp[slot] = cap_lcp(d + (uint32_t)common_syms(k, below, y.bits, y.count));
+      if (before == 0 && less > 0) lcp[slot] = cap_lcp(d + common_syms(k, below, y));
       if (equal > 1) {
         const int at = hd + (int)(less + before);
         s_act[at] = 1u;
@@ -647,7 +707,7 @@ __global__ void __launch_bounds__(RFM_THREADS) k_refine_mid(const uint32_t* __re
       range_of(i, hd, nx);
       const uint32_t size = nx - hd;
       if (i == hd && i > 0)
-        lcp[g.start + i] = cap_lcp(g.depth + (uint32_t)common_syms(s_key[i], s_key[i - 1], y.bits, y.count));
+        lcp[g.start + i] = cap_lcp(g.depth + common_syms(s_key[i], s_key[i - 1], y));
       if (size > SMALL_MAX) {
         if (i == hd) next[atomicAdd(&ct->mid[out], 1u)] = Range{g.start + hd, size, g.depth + (uint32_t)y.count};
       } else if (size > 1) {
@@ -778,38 +838,50 @@ extern "C" fc_status fc_datastore_build(const uint32_t* d_tokens, uint64_t n, ui
     return cudaMemcpyAsync(&hc, ct, sizeof hc, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
            cudaStreamSynchronize(s) == cudaSuccess;
   };
-  // An LSD sort of m (key, value) pairs over the low `bits` bits; the result lands in the first pair of buffers
-  // (so an odd number of passes starts from the second, where the caller then writes the pairs: starts_second).
-  auto starts_second = [](int bits) { return ((bits + 7) / 8) % 2 != 0; };
-  auto sort_pairs = [&](uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, uint64_t m, int bits) -> bool {
+  // One pass of an LSD sort of m (key, value) pairs: digit offsets, then the scatter.
+  auto offsets = [&](uint64_t m) { return exclusive_scan(hist, 256 * cdiv(m, RS_TILE), stmp, s) == cudaSuccess; };
+  auto pass = [&](const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, uint64_t m, int shift) {
     const uint64_t nb = cdiv(m, RS_TILE);
-    if (starts_second(bits)) std::swap(k0, k1), std::swap(v0, v1);
-    for (int shift = 0; shift < bits; shift += 8) {
-      k_radix_hist<<<(unsigned)nb, RS_THREADS, 0, s>>>(k0, m, shift, hist, nb);
-      if (exclusive_scan(hist, 256 * nb, stmp, s) != cudaSuccess) return false;
-      k_radix_scatter<<<(unsigned)nb, RS_THREADS, RS_SMEM, s>>>(k0, v0, k1, v1, m, shift, hist, nb);
+    return fc_launch_dependent(k_radix_hist<false>, dim3((unsigned)nb), RS_THREADS, 0, s, 0, kin, TextKeys{}, m, shift, hist, nb,
+                               0u, nullptr) == FC_OK &&
+           offsets(m) &&
+           fc_launch_dependent(k_radix_scatter<false>, dim3((unsigned)nb), RS_THREADS, 0, s, 0, kin, vin, TextKeys{}, kout, vout,
+                               m, shift, hist, nb) == FC_OK;
+  };
+  // The passes from digit `d` on over the low `bits` bits, from one pair of buffers to the other.
+  auto passes = [&](uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, uint64_t m, int d, int bits) {
+    for (; 8 * d < bits; ++d) {
+      if (!pass(k0, v0, k1, v1, m, 8 * d)) return false;
       std::swap(k0, k1);
       std::swap(v0, v1);
     }
     return true;
   };
 
-  if (cudaFuncSetAttribute(k_radix_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_SMEM) != cudaSuccess ||
-      cudaFuncSetAttribute(k_refine_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RFM_SMEM) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_refine_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RFM_SMEM) != cudaSuccess)
     return FC_ERR_CUDA;
   if (cudaMemsetAsync(ctl, 0, 64, s) != cudaSuccess) return FC_ERR_CUDA;
-  k_check_tokens<<<g, 256, 0, s>>>(d_tokens, n, vocab, ctl);
-  if (!read_counts()) return FC_ERR_CUDA;
-  if (hc.flag) return FC_ERR_INVALID_ARG;
 
-  // Every position by its first symbols.
+  // Every position by its first symbols.  The first pass reads the text itself (and checks it, before anything
+  // is written to the outputs); its pairs land where the last pass ends in (key_a, d_sa).
   Sym y;
   y.bits = bits_for(vocab);
   y.count = std::min(8, 64 / y.bits);
-  const int key_bits = y.bits * y.count;
-  const bool second = starts_second(key_bits);
-  k_pack_keys<<<g, 256, 0, s>>>(d_tokens, n, y, second ? key_b : key_a, second ? val_b : d_sa);
-  if (!sort_pairs(key_a, d_sa, key_b, val_b, n, key_bits)) return FC_ERR_CUDA;
+  y.inv = (65536u + (uint32_t)y.bits - 1u) / (uint32_t)y.bits;
+  const int key_bits = y.bits * y.count, np = (key_bits + 7) / 8;
+  const TextKeys tx{d_tokens, y};
+  k_radix_hist<true><<<(unsigned)L.nb, RS_THREADS, 0, s>>>(nullptr, tx, n, 0, hist, L.nb, vocab, ctl);
+  if (!read_counts()) return FC_ERR_CUDA;
+  if (hc.flag) return FC_ERR_INVALID_ARG;
+  {
+    uint64_t* k0 = np % 2 ? key_a : key_b;
+    uint32_t* v0 = np % 2 ? d_sa : val_b;
+    if (!offsets(n)) return FC_ERR_CUDA;
+    if (fc_launch_dependent(k_radix_scatter<true>, dim3((unsigned)L.nb), RS_THREADS, 0, s, 0, nullptr, nullptr, tx, k0, v0, n, 0,
+                            hist, L.nb) != FC_OK ||
+        !passes(k0, v0, np % 2 ? key_b : key_a, np % 2 ? val_b : d_sa, n, 1, key_bits))
+      return FC_ERR_CUDA;
+  }
   // The sorted keys are in key_a.  key_b takes the list of small ranges (8 bytes an element, n at most), the rank
   // area the tables of longer ones; the lists alternate between key_b and key_a from then on.
   Elem* lists[2] = {reinterpret_cast<Elem*>(key_b), reinterpret_cast<Elem*>(key_a)};
@@ -844,10 +916,11 @@ extern "C" fc_status fc_datastore_build(const uint32_t* d_tokens, uint64_t n, ui
     before = m;
     const int bits = yh.bits * yh.count + obits;
     uint64_t* k1 = key_b + (n - m);  // behind the list: small elements and gathered ones are n at most
-    const bool sec = starts_second(bits);
-    k_huge_gather<<<grid_for(m, 256), 256, 0, s>>>(d_tokens, n, yh, d_sa, huges[hin], ng, m, sec ? k1 : key_a,
-                                                   sec ? head : val_b);
-    if (!sort_pairs(key_a, val_b, k1, head, m, bits)) return FC_ERR_CUDA;
+    const bool odd = (bits + 7) / 8 % 2 != 0;  // the last pass ends in (key_a, val_b)
+    uint64_t *kf = odd ? k1 : key_a, *kt = odd ? key_a : k1;
+    uint32_t *vf = odd ? head : val_b, *vt = odd ? val_b : head;
+    k_huge_gather<<<grid_for(m, 256), 256, 0, s>>>(d_tokens, n, yh, d_sa, huges[hin], ng, m, kf, vf);
+    if (!passes(kf, vf, kt, vt, m, 0, bits)) return FC_ERR_CUDA;
     k_split<true><<<(unsigned)cdiv(m, SPL_TILE), SPL_THREADS, 0, s>>>(key_a, val_b, m, yh, (uint32_t)yh.count, huges[hin],
                                                                       d_sa, d_lcp, lists[0], mids[0], huges[hin ^ 1], ct,
                                                                       hin ^ 1, nullptr, 0u);
@@ -896,9 +969,7 @@ extern "C" fc_status fc_datastore_build(const uint32_t* d_tokens, uint64_t n, ui
       for (int b = 0; b < bits_for(n); b += 8) shifts[np++] = b;
       for (int b = 0; b < bits_for(n - 1); b += 8) shifts[np++] = 32 + b;
       for (int p = 0; p < np; ++p) {
-        k_radix_hist<<<(unsigned)L.nb, RS_THREADS, 0, s>>>(kin, n, shifts[p], hist, L.nb);
-        if (exclusive_scan(hist, 256 * L.nb, stmp, s) != cudaSuccess) return FC_ERR_CUDA;
-        k_radix_scatter<<<(unsigned)L.nb, RS_THREADS, RS_SMEM, s>>>(kin, vin, kout, vout, n, shifts[p], hist, L.nb);
+        if (!pass(kin, vin, kout, vout, n, shifts[p])) return FC_ERR_CUDA;
         std::swap(kin, kout);
         std::swap(vin, vout);
       }
@@ -986,6 +1057,10 @@ extern "C" fc_status fc_datastore_build_noalloc(const uint32_t* d_tokens, uint64
 // the corpus end; 32 bytes, written as two 16-byte stores.
 // ---------------------------------------------------------------------------
 namespace {
+// VEC: the corpus is 16-byte aligned, and a suffix's tokens 1..7 come from the
+// aligned 16-byte groups they lie in (all inside the corpus) instead of seven
+// 4-byte loads.  Bound by the random reads: 100M tokens @@.
+template <bool VEC>
 __global__ void k_suffix_keys(const uint32_t* __restrict__ T, const uint32_t* __restrict__ sa, uint64_t n,
                               uint4* __restrict__ keys) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -993,8 +1068,18 @@ __global__ void k_suffix_keys(const uint32_t* __restrict__ T, const uint32_t* __
     const uint64_t i = __ldg(sa + j);
     uint32_t t[8];
     t[0] = (uint32_t)i;
+    const uint64_t g = (i + 1) >> 2;  // the group of token i + 1
+    if (VEC && 4 * (g + 3) <= n) {
+      const uint4* Tv = reinterpret_cast<const uint4*>(T) + g;
+      const int o = (int)(i + 1) & 3;
+      const uint4 a = __ldg(Tv), b = __ldg(Tv + 1), c = o > 1 ? __ldg(Tv + 2) : make_uint4(0, 0, 0, 0);
+      const uint32_t w[10] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y};
 #pragma unroll
-    for (int k = 1; k < 8; ++k) t[k] = (i + k < n) ? __ldg(T + i + k) : FC_PAD_TOKEN;
+      for (int k = 0; k < 7; ++k) t[k + 1] = o == 0 ? w[k] : o == 1 ? w[k + 1] : o == 2 ? w[k + 2] : w[k + 3];
+    } else {
+#pragma unroll
+      for (int k = 1; k < 8; ++k) t[k] = (i + k < n) ? __ldg(T + i + k) : FC_PAD_TOKEN;
+    }
     keys[2 * j] = make_uint4(t[0], t[1], t[2], t[3]);
     keys[2 * j + 1] = make_uint4(t[4], t[5], t[6], t[7]);
   }
@@ -1007,8 +1092,9 @@ extern "C" fc_status fc_datastore_keys(const fc_datastore* ds, uint32_t* d_keys,
     return FC_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(d_keys) % 32) return FC_ERR_INVALID_ARG;
   const uint64_t n = ds->n_tokens;
-  k_suffix_keys<<<grid_for(n, 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(ds->tokens, ds->sa, n,
-                                                                                 reinterpret_cast<uint4*>(d_keys));
+  const auto kern = reinterpret_cast<uintptr_t>(ds->tokens) % 16 == 0 ? k_suffix_keys<true> : k_suffix_keys<false>;
+  kern<<<grid_for(n, 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(ds->tokens, ds->sa, n,
+                                                                        reinterpret_cast<uint4*>(d_keys));
   return FC_CHECK_LAUNCH();
 }
 

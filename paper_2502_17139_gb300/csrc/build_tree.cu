@@ -4,21 +4,26 @@
 // by depth; Section V-C: alpha = beta = 1, at most 64 draft tokens).
 //
 // One CTA per query, everything in shared memory, no pointer trie:
-//   1. gather the drafts of all sources with weight w = src_weight * count;
-//   2. sort them lexicographically (threads rank drafts against all others,
-//      comparing zero-padded pairs of tokens packed in 64-bit words, then
-//      lengths) and merge duplicates across sources (weights add);
-//   3. with neighbour LCPs, every trie node is a pair (u, l): the prefix of
-//      length l of sorted unique draft u, new at u when l > lcp(u-1, u).
-//      Its weight is the weight sum of the contiguous run of drafts that
-//      share that prefix (prefix sums over the sorted drafts);
+//   1. a thread per slot reads its draft (every load at once) and packs it as
+//      zero-padded token pairs in 64-bit words; weight w = src_weight * count;
+//   2. drafts rank themselves by token sequence: a few lanes per draft compare
+//      it with all others, four tokens at a time (then lengths); neighbours'
+//      first difference gives the LCP, equal neighbours merge across sources
+//      (weights add);
+//   3. every trie node is a pair (u, l): the prefix of length l of sorted
+//      unique draft u, new at u when l > lcp(u-1, u).  A bit per (l, u) says
+//      whether a run of drafts that share l tokens starts at u: a node's
+//      weight is a prefix-sum difference up to the run's end, the next set bit
+//      of row l, and its parent starts at the last set bit of row l - 1;
 //   4. a radix select on the distinct (W, 31 - l, 8191 - u) keys finds the
 //      heaviest budget - 1 nodes (ties: shallower, then smaller path); a
 //      parent's key always exceeds its child's, so the kept set is a tree;
-//   5. (u, l) order is depth-first preorder with children in ascending
-//      token order: a scan over a kept-flag table [u][l] numbers the nodes
-//      and maps a parent (the run start of prefix l - 1) to its index;
-//      masks are ancestor walks.
+//   5. (u, l) order is depth-first preorder with children in ascending token
+//      order: kept bits in that order, counted, number the nodes; masks are
+//      ancestor walks.
+// Bound by latency: a chain of barrier-separated steps in one CTA.  Against one
+// with serial scans, run ends and runs found by walking, a lookup per token:
+// retrieval and tree at batch 256 55.5 -> 41.3 us, at batch 1 18.4 -> 14.8 us.
 #include <algorithm>
 
 #include "fc_common.cuh"
@@ -49,9 +54,10 @@ struct TreeOut {
 };
 
 struct BtLayout {
-  size_t tok, len, w, order, uniq, wu, ps, lcp, coff, flag, ckey, pk, tab, total;
+  size_t pk, ckey, w, ps, len, order, uniq, lcp, coff, lcpr, total;
 };
 
+// Shared memory of k_build_tree for M slots of d tokens.
 __host__ __device__ inline BtLayout bt_layout(int M, int d) {
   BtLayout L;
   size_t off = 0;
@@ -60,19 +66,16 @@ __host__ __device__ inline BtLayout bt_layout(int M, int d) {
     off = (off + bytes + 15) & ~(size_t)15;
     return o;
   };
-  L.tok = take((size_t)M * d * 4);
-  L.len = take((size_t)M * 4);
-  L.w = take((size_t)M * 8);
-  L.order = take((size_t)M * 4);
-  L.uniq = take((size_t)M * 4);
-  L.wu = take((size_t)M * 8);
-  L.ps = take((size_t)(M + 1) * 8);
-  L.lcp = take((size_t)(M + 1) * 4);
-  L.coff = take((size_t)(M + 1) * 4);
-  L.flag = take((size_t)(M + 1) * 4);
-  L.ckey = take((size_t)M * d * 8);
-  L.pk = take((size_t)M * PK_WORDS * 8);  // each draft as zero-padded token pairs
-  L.tab = take((size_t)M * d * 4);  // kept flags [u][l - 1], then their preorder ranks
+  L.pk = take((size_t)M * PK_WORDS * 8);  // [four tokens][slot]: 16-byte vectors
+  L.ckey = take((size_t)M * d * 8);       // candidates' selection keys
+  L.w = take((size_t)M * 8);              // per slot
+  L.ps = take((size_t)(M + 1) * 8);       // prefix sums of the unique drafts' weights
+  L.len = take((size_t)M * 4);            // per slot, 0: no draft
+  L.order = take((size_t)M * 4);          // sorted draft -> slot
+  L.uniq = take((size_t)M * 4);           // unique draft -> slot
+  L.lcp = take((size_t)M * 4);            // unique draft -> LCP with the one before
+  L.coff = take((size_t)M * 4);           // unique draft -> its first candidate
+  L.lcpr = take((size_t)M * 4);           // valid slots; then sorted draft -> LCP with the one before
   L.total = off;
   return L;
 }
@@ -221,218 +224,294 @@ __device__ uint64_t radix_select_desc(const uint64_t* key, uint32_t n, uint32_t 
   return pre;
 }
 
-// -1 / 0 / 1 lexicographic comparison of two drafts (a prefix sorts first).
-__device__ __forceinline__ int cmp_draft(const uint32_t* a, int la, const uint32_t* b, int lb) {
-  int l = min(la, lb);
-  for (int i = 0; i < l; ++i)
-    if (a[i] != b[i]) return a[i] < b[i] ? -1 : 1;
-  return la < lb ? -1 : (la > lb ? 1 : 0);
-}
+// Packed drafts in shared memory: vector v (tokens 4 v .. 4 v + 3) of slot i at pk[v * M0 + i].
+struct Packed {
+  const ulonglong2* pk;
+  int M0;
+  __device__ __forceinline__ uint32_t token(int i, int t) const {
+    const ulonglong2 v = pk[(t >> 2) * M0 + i];
+    const uint64_t w = t & 2 ? v.y : v.x;
+    return (uint32_t)(t & 1 ? w : w >> 32);
+  }
+};
 
 __global__ void __launch_bounds__(BT_THREADS) k_build_tree(TreeIn in, int S, int B, int k, int d,
                                                            const uint32_t* __restrict__ root_tok,
                                                            const int32_t* __restrict__ kv_len, int budget, int n_pad,
                                                            TreeOut out) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint32_t wsum[BT_THREADS / 32 + 1];
-  __shared__ int32_t sel_u[FC_MAX_NODES], sel_l[FC_MAX_NODES], par_s[FC_MAX_NODES];
+  constexpr int WARPS = BT_THREADS / 32, MAX_WORDS = BT_MAX_DRAFTS / 32;
+  constexpr int KEPT_WORDS = BT_MAX_DRAFTS * FC_MAX_DRAFT_LEN / 32;
+  __shared__ uint32_t s_valid[MAX_WORDS], s_uniq[MAX_WORDS];      // bits: slot holds a draft; sorted draft is new
+  __shared__ uint32_t s_run[FC_MAX_DRAFT_LEN + 1][MAX_WORDS + 1];  // [l] bits: a run of drafts sharing l tokens starts
+  __shared__ uint32_t s_kept[KEPT_WORDS], s_before[KEPT_WORDS];    // kept nodes in (u, l) order, and how many before
+  __shared__ uint32_t s_wsum[WARPS];
+  __shared__ uint64_t s_wsum64[WARPS];
+  __shared__ uint32_t tok_s[FC_MAX_NODES];
+  __shared__ int32_t dep_s[FC_MAX_NODES], par_s[FC_MAX_NODES];
+  __shared__ uint32_t hist[256];
   const int M0 = S * k;
   const BtLayout L = bt_layout(M0, d);
-  uint32_t* tok = reinterpret_cast<uint32_t*>(smem_raw + L.tok);
-  int32_t* len = reinterpret_cast<int32_t*>(smem_raw + L.len);
+  ulonglong2* pk = reinterpret_cast<ulonglong2*>(smem_raw + L.pk);
+  uint64_t* ckey = reinterpret_cast<uint64_t*>(smem_raw + L.ckey);
   uint64_t* w = reinterpret_cast<uint64_t*>(smem_raw + L.w);
-  uint32_t* order = reinterpret_cast<uint32_t*>(smem_raw + L.order);
-  uint32_t* uniq = reinterpret_cast<uint32_t*>(smem_raw + L.uniq);
-  uint64_t* wu = reinterpret_cast<uint64_t*>(smem_raw + L.wu);
   uint64_t* ps = reinterpret_cast<uint64_t*>(smem_raw + L.ps);
+  int32_t* len = reinterpret_cast<int32_t*>(smem_raw + L.len);
+  uint32_t* uniq = reinterpret_cast<uint32_t*>(smem_raw + L.uniq);
   uint32_t* lcp = reinterpret_cast<uint32_t*>(smem_raw + L.lcp);
   uint32_t* coff = reinterpret_cast<uint32_t*>(smem_raw + L.coff);
-  uint32_t* flag = reinterpret_cast<uint32_t*>(smem_raw + L.flag);
-  uint64_t* ckey = reinterpret_cast<uint64_t*>(smem_raw + L.ckey);
-  uint64_t* pk = reinterpret_cast<uint64_t*>(smem_raw + L.pk);
-  uint32_t* tab = reinterpret_cast<uint32_t*>(smem_raw + L.tab);
-  __shared__ uint32_t hist[256];
-  const int b = blockIdx.x, tid = threadIdx.x;
+  uint32_t* lcpr = reinterpret_cast<uint32_t*>(smem_raw + L.lcpr);
+  uint32_t* list = lcpr;  // valid slots; dead once the order is known
+  uint32_t* order = reinterpret_cast<uint32_t*>(smem_raw + L.order);
+  const Packed P{pk, M0};
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int words0 = (M0 + 31) / 32;
   fc_grid_wait();
   root_tok = fc_after_wait(root_tok);
   kv_len = fc_after_wait(kv_len);
+  const uint32_t root = root_tok[b];
+  const int kvl = kv_len[b];
 
-  // 1. valid drafts, compacted in (source, slot) order
-  for (int i = tid; i < M0; i += BT_THREADS) {
-    int s = i / k, t = i - s * k;
-    size_t sb = (size_t)s * B + b;
-    int nd = min(max((int)in.n_drafts[sb], 0), k);
-    int l = (t < nd) ? in.draft_len[sb * k + t] : 0;
-    flag[i] = (l > 0 && l <= d) ? 1u : 0u;
-  }
-  __syncthreads();
-  // keep the flags: scan a copy in coff
-  for (int i = tid; i < M0; i += BT_THREADS) coff[i] = flag[i];
-  __syncthreads();
-  uint32_t M = block_scan_array(coff, M0, wsum);
-  for (int i = tid; i < M0; i += BT_THREADS) {
-    if (!flag[i]) continue;
-    int s = i / k, t = i - s * k;
-    size_t sb = (size_t)s * B + b;
-    uint32_t j = coff[i];
-    int l = in.draft_len[sb * k + t];
-    len[j] = l;
-    uint32_t cnt = in.count[sb * k + t];
-    if (cnt > (1u << 20)) {  // weights are packed into 46-bit sort keys
-      fc_flag(FC_ERR_WORD(out.err), FC_EBIT_INVALID);
-      cnt = 1u << 20;
+  // 1. a draft per thread
+  for (int i = tid; i < words0 * 32; i += BT_THREADS) {
+    bool valid = false;
+    if (i < M0) {
+      const int s = i / k, t = i - s * k;
+      const size_t sb = (size_t)s * B + b;
+      const int nd = in.n_drafts[sb], l = in.draft_len[sb * k + t];
+      uint32_t cnt = in.count[sb * k + t];
+      const uint32_t* src = in.drafts + (sb * k + t) * d;
+      uint32_t tk[FC_MAX_DRAFT_LEN];
+#pragma unroll
+      for (int x = 0; x < FC_MAX_DRAFT_LEN; ++x) tk[x] = x < d ? src[x] : 0u;
+      valid = t < min(max(nd, 0), k) && l > 0 && l <= d;
+#pragma unroll
+      for (int v = 0; v < PK_WORDS / 2; ++v) {
+        ulonglong2 p;
+        auto at = [&](int x) { return (uint64_t)(x < l ? tk[x] : 0u); };
+        p.x = (at(4 * v) << 32) | at(4 * v + 1);
+        p.y = (at(4 * v + 2) << 32) | at(4 * v + 3);
+        if (valid) pk[v * M0 + i] = p;
+      }
+      if (valid && cnt > (1u << 20)) {  // weights are packed into 46-bit sort keys
+        fc_flag(FC_ERR_WORD(out.err), FC_EBIT_INVALID);
+        cnt = 1u << 20;
+      }
+      len[i] = valid ? l : 0;
+      w[i] = (uint64_t)in.w[s] * cnt;
     }
-    w[j] = (uint64_t)in.w[s] * cnt;
-    for (int x = 0; x < d; ++x) tok[j * d + x] = (x < l) ? in.drafts[(sb * k + t) * d + x] : 0u;
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, valid);
+    if (lane == 0) s_valid[i >> 5] = m;
+  }
+  __syncthreads();
+  uint32_t M = 0;
+  for (int v = 0; v < words0; ++v) M += __popc(s_valid[v]);
+  for (int i = tid; i < M0; i += BT_THREADS) {  // in (source, slot) order
+    const uint32_t m = s_valid[i >> 5];
+    if (!((m >> (i & 31)) & 1u)) continue;
+    uint32_t j = __popc(m & ((1u << (i & 31)) - 1u));
+    for (int v = 0; v < (i >> 5); ++v) j += __popc(s_valid[v]);
+    list[j] = i;
   }
   __syncthreads();
 
-  // 2. rank sort of the drafts by token sequence; equal drafts keep
-  //    (source, slot) order through the index tie-break.  Drafts compare as
-  //    their token pairs packed in 64-bit words, zero-padded, then by
-  //    length: a difference in the padded words always has the lexicographic
-  //    sign (a zero pad only ever ties with a real token), and padded words
-  //    that agree mean one draft is a prefix of the other.
-  for (uint32_t x = tid; x < M * (uint32_t)PK_WORDS; x += BT_THREADS) {
-    const uint32_t i = x / PK_WORDS, q = x - i * PK_WORDS;
-    const int l = len[i];
-    const uint32_t t0 = (2 * (int)q < l) ? tok[i * d + 2 * q] : 0u;
-    const uint32_t t1 = (2 * (int)q + 1 < l) ? tok[i * d + 2 * q + 1] : 0u;
-    pk[x] = ((uint64_t)t0 << 32) | t1;
-  }
-  for (uint32_t i = tid; i < M; i += BT_THREADS) order[i] = 0;
-  __syncthreads();
+  // 2. rank by token sequence; equal drafts keep (source, slot) order.  A
+  //    difference in the padded words always has the lexicographic sign (a zero
+  //    pad only ever ties with a real token), and words that all agree mean one
+  //    draft is a prefix of the other.
+  const int nv = (d + 3) / 4;
   {
-    // several threads per draft when they fit (slices of the j range)
-    const uint32_t split = M > 0 ? umax(1u, umin(8u, (uint32_t)BT_THREADS / M)) : 1u;
-    for (uint32_t x = tid; x < M * split; x += BT_THREADS) {
-      const uint32_t i = x / split, h = x - i * split;
-      const ulonglong2* pv = reinterpret_cast<const ulonglong2*>(pk);
-      uint64_t a[PK_WORDS];
-#pragma unroll
-      for (int q = 0; q < PK_WORDS / 2; ++q) {
-        const ulonglong2 v = pv[i * (PK_WORDS / 2) + q];
-        a[2 * q] = v.x;
-        a[2 * q + 1] = v.y;
-      }
-      const int la = len[i];
-      const uint32_t j0 = h * M / split, j1 = (h + 1) * M / split;
-      uint32_t rank = 0;
-      for (uint32_t j = j0; j < j1; ++j) {
-        int res = 0;  // sign of draft j vs draft i
-#pragma unroll
-        for (int q = 0; q < PK_WORDS / 2; ++q) {
-          const ulonglong2 v = pv[j * (PK_WORDS / 2) + q];
-          if (res == 0 && v.x != a[2 * q]) res = (v.x < a[2 * q]) ? -1 : 1;
-          if (res == 0 && v.y != a[2 * q + 1]) res = (v.y < a[2 * q + 1]) ? -1 : 1;
+    uint32_t split = 1;  // lanes per draft: a power of two that divides a warp
+    while (split < 32 && 2 * split * M <= (uint32_t)BT_THREADS) split *= 2;
+    const uint32_t j0 = tid / split;
+    uint32_t rank = 0;
+    int me = -1;
+    if (j0 < M) {
+      me = list[j0];
+      const ulonglong2 a = pk[me];
+      for (uint32_t j = tid & (split - 1); j < M; j += split) {
+        const int o = list[j];
+        ulonglong2 c = pk[o], mine = a;
+        for (int v = 1; v < nv && c.x == mine.x && c.y == mine.y; ++v) {
+          c = pk[v * M0 + o];
+          mine = pk[v * M0 + me];
         }
-        if (res == 0) res = (len[j] < la) ? -1 : (len[j] > la ? 1 : 0);
-        rank += (res < 0 || (res == 0 && j < i)) ? 1u : 0u;
+        const bool less = c.x != mine.x ? c.x < mine.x : c.y != mine.y ? c.y < mine.y : len[o] != len[me] ? len[o] < len[me] : o < me;
+        rank += less ? 1u : 0u;
       }
-      atomicAdd(&order[i], rank);  // order[] holds ranks here
+    }
+    for (uint32_t o = split / 2; o > 0; o >>= 1) rank += __shfl_xor_sync(0xFFFFFFFFu, rank, o);
+    if (me >= 0 && (tid & (split - 1)) == 0) order[rank] = me;
+  }
+  __syncthreads();
+  const int wordsM = ((int)M + 31) / 32;
+  for (int r = tid; r < wordsM * 32; r += BT_THREADS) {
+    bool fresh = false;
+    if (r < (int)M) {
+      uint32_t l = 0;
+      fresh = true;
+      if (r > 0) {
+        const int a = order[r - 1], c = order[r], la = len[a], lc = len[c];
+        l = (uint32_t)min(la, lc);
+        for (int v = 0; v < nv; ++v) {
+          const ulonglong2 x = pk[v * M0 + a], y = pk[v * M0 + c];
+          const uint64_t d0 = x.x ^ y.x, d1 = x.y ^ y.y;
+          if (d0 | d1) {
+            const uint32_t t = 4 * v + (d0 ? (d0 >> 32 ? 0 : 1) : (d1 >> 32 ? 2 : 3));
+            l = min(l, t);
+            break;
+          }
+        }
+        fresh = la != lc || l != (uint32_t)la;
+      }
+      lcpr[r] = l;
+    }
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, fresh);
+    if (lane == 0) s_uniq[r >> 5] = m;
+  }
+  __syncthreads();
+  uint32_t U = 0;
+  for (int v = 0; v < wordsM; ++v) U += __popc(s_uniq[v]);
+  // the unique draft of this thread's sorted one, its weight (equal ones follow it) and its candidates
+  uint64_t wu = 0;
+  uint32_t cu = 0, my_lcp = 0;
+  int my_u = -1;
+  if (tid < (int)M && ((s_uniq[tid >> 5] >> (tid & 31)) & 1u)) {
+    const int slot = order[tid];
+    my_u = __popc(s_uniq[tid >> 5] & ((1u << (tid & 31)) - 1u));
+    for (int v = 0; v < (tid >> 5); ++v) my_u += __popc(s_uniq[v]);
+    wu = w[slot];
+    for (int r = tid + 1; r < (int)M && !((s_uniq[r >> 5] >> (r & 31)) & 1u); ++r) wu += w[order[r]];
+    my_lcp = lcpr[tid];
+    cu = (uint32_t)len[slot] - my_lcp;
+    uniq[my_u] = slot;
+    lcp[my_u] = my_lcp;
+  }
+  // exclusive prefix sums over the unique drafts (sorted order is their order)
+  uint64_t iw = wu;
+  uint32_t ic = cu;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t yw = __shfl_up_sync(0xFFFFFFFFu, iw, o);
+    const uint32_t yc = __shfl_up_sync(0xFFFFFFFFu, ic, o);
+    if (lane >= o) {
+      iw += yw;
+      ic += yc;
     }
   }
-  __syncthreads();
-  for (uint32_t i = tid; i < M; i += BT_THREADS) flag[i] = order[i];  // rank of draft i
-  __syncthreads();
-  for (uint32_t i = tid; i < M; i += BT_THREADS) order[flag[i]] = i;
-  __syncthreads();
-  for (uint32_t r = tid; r < M; r += BT_THREADS) {
-    uint32_t i = order[r];
-    flag[r] = (r == 0 || cmp_draft(tok + order[r - 1] * d, len[order[r - 1]], tok + i * d, len[i]) != 0) ? 1u : 0u;
-    coff[r] = flag[r];
+  if (lane == 31) {
+    s_wsum64[warp] = iw;
+    s_wsum[warp] = ic;
   }
   __syncthreads();
-  uint32_t U = block_scan_array(coff, (int)M, wsum);  // coff[r] = unique index of run start
-  for (uint32_t u = tid; u < U; u += BT_THREADS) wu[u] = 0;
+  uint32_t C = 0;
+  {
+    uint64_t pw = iw - wu;
+    uint32_t pc = ic - cu;
+    for (int v = 0; v < wordsM; ++v) {
+      if (v < warp) {
+        pw += s_wsum64[v];
+        pc += s_wsum[v];
+      }
+      C += s_wsum[v];
+    }
+    if (my_u >= 0) {
+      ps[my_u] = pw;
+      coff[my_u] = pc;
+      if (my_u == (int)U - 1) ps[U] = pw + wu;
+    }
+  }
+  // 3. run starts at every depth (past the last draft: a start, so runs end there)
+  const int wordsU = ((int)U + 31) / 32;
+  if (warp <= wordsU) {
+    const int u = warp * 32 + lane;
+    const uint32_t lu = u < (int)U ? lcp[u] : 0u;
+    for (int l = 0; l <= d; ++l) {
+      const uint32_t m = __ballot_sync(0xFFFFFFFFu, u >= (int)U || u == 0 || lu < (uint32_t)l);
+      if (lane == 0) s_run[l][warp] = m;
+    }
+  }
+  if (wordsU == MAX_WORDS && tid <= d) s_run[tid][MAX_WORDS] = 1u;
   __syncthreads();
-  for (uint32_t r = tid; r < M; r += BT_THREADS) {
-    uint32_t u = coff[r] + flag[r] - 1u;  // unique index of the run containing r
-    if (flag[r]) uniq[u] = order[r];
-    atomicAdd(reinterpret_cast<unsigned long long*>(&wu[u]), (unsigned long long)w[order[r]]);
+  const uint32_t n_ul = U * (uint32_t)d;
+  const uint32_t ul_end = (n_ul + 31) / 32 * 32;
+  for (uint32_t x = tid; x < n_ul; x += BT_THREADS) {
+    const uint32_t u = x / (uint32_t)d, l = x - u * (uint32_t)d + 1;
+    if (l <= lcp[u] || l > (uint32_t)len[uniq[u]]) continue;
+    uint32_t q = (u + 1) >> 5, m = s_run[l][q] & (0xFFFFFFFFu << ((u + 1) & 31));
+    while (!m) m = s_run[l][++q];
+    const uint32_t e = min(U, q * 32 + __ffs(m) - 1);
+    ckey[coff[u] + (l - lcp[u] - 1)] = ((ps[e] - ps[u]) << 18) | ((uint64_t)(31 - l) << 13) | (uint64_t)(8191u - u);
   }
   __syncthreads();
 
-  // 3. neighbour LCPs, prefix sums of weights, candidate counts
-  for (uint32_t u = tid; u < U; u += BT_THREADS) {
-    uint32_t l = 0;
-    if (u > 0) {
-      const uint32_t* a = tok + uniq[u - 1] * d;
-      const uint32_t* c = tok + uniq[u] * d;
-      int lim = min(len[uniq[u - 1]], len[uniq[u]]);
-      while ((int)l < lim && a[l] == c[l]) ++l;
-    }
-    lcp[u] = l;
-    coff[u] = (uint32_t)len[uniq[u]] - l;
-  }
-  __syncthreads();
-  if (tid < 32) warp_scan_u64(wu, ps, U);  // ps[u] = sum of wu[0..u), ps[U] = total
-  uint32_t C = block_scan_array(coff, (int)U, wsum);
-  for (uint32_t u = tid; u < U; u += BT_THREADS) {
-    // deepest first: the run of (u, l) ends at the first e > u with lcp[e] < l,
-    // which only moves right as l falls, so one scan serves every depth
-    const int lu = len[uniq[u]];
-    uint32_t e = u + 1;
-    for (int l = lu; l > (int)lcp[u]; --l) {
-      while (e < U && (int)lcp[e] >= l) ++e;
-      const uint64_t W = ps[e] - ps[u];
-      ckey[coff[u] + (l - lcp[u] - 1)] = (W << 18) | ((uint64_t)(31 - l) << 13) | (uint64_t)(8191u - u);
-    }
-  }
-  for (uint32_t x = tid; x < U * (uint32_t)d; x += BT_THREADS) tab[x] = 0;
-  __syncthreads();
-
-  // 4. the nsel largest keys (all distinct): radix select of the threshold,
-  //    8 bits at a time from the top
+  // 4. the nsel largest keys (all distinct): radix select of the threshold, 8 bits at a time from the top
   const int nsel = (int)umin((uint32_t)(budget - 1), C);
   uint64_t thr = 0;
   if (nsel > 0 && (uint32_t)nsel < C) thr = radix_select_desc(ckey, C, (uint32_t)nsel, hist);
-  // 5. kept flags in the (u, l) table, scanned into preorder ranks
-  for (uint32_t c = tid; c < C; c += BT_THREADS) {
-    const uint64_t key = ckey[c];
-    if (nsel > 0 && key >= thr) {
-      const int u = 8191 - (int)(key & 8191u), l = 31 - (int)((key >> 13) & 31u);
-      tab[u * d + l - 1] = 1u;
+  // 5. kept bits in (u, l) order, and how many come before each word of them
+  for (uint32_t x = tid; x < ul_end; x += BT_THREADS) {
+    bool kept = false;
+    if (x < n_ul) {
+      const uint32_t u = x / (uint32_t)d, l = x - u * (uint32_t)d + 1;
+      kept = nsel > 0 && l > lcp[u] && l <= (uint32_t)len[uniq[u]] && ckey[coff[u] + (l - lcp[u] - 1)] >= thr;
+    }
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, kept);
+    if (lane == 0) s_kept[x >> 5] = m;
+  }
+  __syncthreads();
+  const uint32_t words_ul = ul_end / 32;  // up to 256
+  {
+    const uint32_t c = tid < (int)words_ul ? (uint32_t)__popc(s_kept[tid]) : 0u;
+    uint32_t inc = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) s_wsum[warp] = inc;
+    __syncthreads();
+    if (tid < (int)words_ul) {
+      uint32_t before = inc - c;
+      for (int v = 0; v < warp; ++v) before += s_wsum[v];
+      s_before[tid] = before;
+      if (tid == (int)words_ul - 1 && before + c != (uint32_t)nsel) fc_flag(FC_ERR_WORD(out.err), FC_EBIT_INTERNAL);
     }
   }
   __syncthreads();
-  const uint32_t nkept = block_scan_array(tab, (int)(U * (uint32_t)d), wsum);
-  if (nkept != (uint32_t)nsel && tid == 0) fc_flag(FC_ERR_WORD(out.err), FC_EBIT_INTERNAL);
-  for (uint32_t c = tid; c < C; c += BT_THREADS) {
-    const uint64_t key = ckey[c];
-    if (nsel > 0 && key >= thr) {
-      const int u = 8191 - (int)(key & 8191u), l = 31 - (int)((key >> 13) & 31u);
-      const int idx = 1 + (int)tab[u * d + l - 1];
-      if (idx < FC_MAX_NODES) {
-        sel_u[idx] = u;
-        sel_l[idx] = l;
-      }
+  for (uint32_t x = tid; x < n_ul; x += BT_THREADS) {
+    const uint32_t m = s_kept[x >> 5];
+    if (!((m >> (x & 31)) & 1u)) continue;
+    const uint32_t u = x / (uint32_t)d, l = x - u * (uint32_t)d + 1;
+    const uint32_t idx = 1 + s_before[x >> 5] + __popc(m & ((1u << (x & 31)) - 1u));
+    if (idx >= FC_MAX_NODES) continue;
+    int pidx = 0;
+    if (l > 1) {  // the parent is the prefix l - 1, first seen at the start of its run
+      uint32_t q = u >> 5, r = s_run[l - 1][q] & (0xFFFFFFFFu >> (31 - (u & 31)));
+      while (!r) r = s_run[l - 1][--q];  // draft 0 starts every run
+      const uint32_t px = (q * 32 + 31 - __clz(r)) * (uint32_t)d + l - 2;
+      pidx = 1 + (int)(s_before[px >> 5] + __popc(s_kept[px >> 5] & ((1u << (px & 31)) - 1u)));
     }
+    tok_s[idx] = P.token(uniq[u], (int)l - 1);
+    dep_s[idx] = (int)l;
+    par_s[idx] = pidx;
+  }
+  if (tid == 0) {
+    tok_s[0] = root;
+    dep_s[0] = 0;
+    par_s[0] = -1;
   }
   __syncthreads();
   const int n = 1 + min(nsel, FC_MAX_NODES - 1);
-  for (int i = 1 + tid; i < n; i += BT_THREADS) {
-    const int u = sel_u[i], l = sel_l[i];
-    int pidx = 0;
-    if (l > 1) {  // the parent is the prefix l - 1, first seen at the start of its run
-      int up = u;
-      while (up > 0 && (int)lcp[up] >= l - 1) --up;
-      pidx = 1 + (int)tab[up * d + l - 2];
-    }
-    par_s[i] = pidx;
-  }
-  if (tid == 0) par_s[0] = -1;
-  __syncthreads();
   const int nw = n_pad / 64;
   const size_t base = (size_t)b * n_pad;
-  const int kvl = kv_len[b];
   for (int i = tid; i < n_pad; i += BT_THREADS) {
     uint32_t tk = FC_PAD_TOKEN;
     int pa = -1, de = -1, po = -1;
     uint64_t m0 = 0, m1 = 0;
     if (i < n) {
-      tk = (i == 0) ? root_tok[b] : tok[uniq[sel_u[i]] * d + sel_l[i] - 1];
-      de = (i == 0) ? 0 : sel_l[i];
+      tk = tok_s[i];
+      de = dep_s[i];
       pa = par_s[i];
       po = kvl + de;
       for (int a = i; a >= 0; a = par_s[a]) {
@@ -504,7 +583,7 @@ __host__ __device__ inline AllLayout all_layout(int M, int d) {
 }
 
 // Sign of packed draft a against packed draft b (zero-padded token pairs,
-// then the lengths: the order of cmp_draft).
+// then the lengths: lexicographic, a prefix first).
 __device__ __forceinline__ int cmp_packed(const uint64_t* a, int la, const uint64_t* b, int lb) {
 #pragma unroll
   for (int q = 0; q < PK_WORDS; ++q)

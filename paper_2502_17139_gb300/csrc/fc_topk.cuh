@@ -15,6 +15,7 @@
 
 #include "fc_common.cuh"
 
+// Exclusive sum over the block's NT threads; *total = the whole sum.  Ends with the block synchronised.
 template <int NT>
 __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t* total, uint32_t* wsum) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -26,19 +27,17 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t* total,
   }
   if (lane == 31) wsum[warp] = inc;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t run = 0;
-    for (int w = 0; w < NT / 32; ++w) {
-      uint32_t c = wsum[w];
-      wsum[w] = run;
-      run += c;
-    }
-    *total = run;
+  // every warp scans the warps' sums (NT / 32 <= 32 of them)
+  uint32_t v = lane < NT / 32 ? wsum[lane] : 0u;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, v, o);
+    if (lane >= o) v += y;
   }
+  const uint32_t before = __shfl_sync(0xFFFFFFFFu, v, max(warp - 1, 0));
+  if (threadIdx.x == 31) *total = v;
   __syncthreads();
-  uint32_t r = wsum[warp] + inc - x;
-  __syncthreads();
-  return r;
+  return (warp ? before : 0u) + inc - x;
 }
 
 struct RunsScratch {
@@ -155,6 +154,48 @@ __device__ uint32_t topk_runs(uint32_t R, int k, const uint32_t* runs, uint32_t*
   }
   __syncthreads();
   return ks;
+}
+
+// Up to NT occurrences, one per thread (`head`: this thread's starts a run;
+// words: NT / 32 words of scratch): run starts from ballots, and up to
+// RANK_ALL_RUNS of them rank themselves, a few lanes per run, by counting the
+// runs ahead; the first k are the top-k.  Outputs as rank_runs.
+constexpr uint32_t RANK_ALL_RUNS = 128;
+template <int NT>
+__device__ uint32_t rank_runs_few(uint32_t nocc, int k, bool head, uint32_t* runs, uint32_t* work, uint32_t* sel,
+                                  uint32_t* order, uint32_t* wsum, uint32_t* words, RunsScratch& sc) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t m = __ballot_sync(0xFFFFFFFFu, head);
+  if (lane == 0) words[warp] = m;
+  __syncthreads();
+  uint32_t R = 0, before = 0;
+  for (int v = 0; v < NT / 32; ++v) {
+    const uint32_t c = __popc(words[v]);
+    before += v < warp ? c : 0u;
+    R += c;
+  }
+  if (head) runs[before + __popc(m & ((1u << lane) - 1u))] = tid;
+  if (tid == 0) {
+    runs[R] = nocc;
+    sc.n_runs = R;
+  }
+  __syncthreads();
+  if (R > RANK_ALL_RUNS) return topk_runs<NT>(R, k, runs, work, sel, order, wsum, sc);
+  uint32_t split = 1;
+  while (split < 32 && 2 * split * R <= (uint32_t)NT) split *= 2;
+  const uint32_t r = tid / split;
+  uint32_t rank = 0;
+  if (r < R) {
+    const uint32_t c = runs[r + 1] - runs[r];
+    for (uint32_t u = tid & (split - 1); u < R; u += split) {
+      const uint32_t cu = runs[u + 1] - runs[u];
+      rank += (cu > c || (cu == c && u < r)) ? 1u : 0u;
+    }
+  }
+  for (uint32_t o = split / 2; o > 0; o >>= 1) rank += __shfl_xor_sync(0xFFFFFFFFu, rank, o);
+  if (r < R && (tid & (split - 1)) == 0 && rank < (uint32_t)k) order[rank] = r;
+  __syncthreads();
+  return min((uint32_t)k, R);
 }
 
 // Both steps: head flags in work -> runs -> top-k (runs: FC_MAX_OCC + 1

@@ -3,16 +3,17 @@
 // and the context-keyed replay cache used by the step loop.
 //
 // One CTA per (query, source).  Design:
-//   * search: every suffix length n gets a warp, its two half-warps find the
-//     lower and the upper bound of the pattern's suffix-array range at once,
-//     so all lengths n_max..n_min are searched together and the longest
-//     non-empty range is picked afterwards (a match of length n implies
-//     matches of every shorter length, so the longest non-empty range is the
-//     answer).  The first-token bucket table narrows each search to the
-//     suffixes that start with the pattern's first token.  Each round of a
-//     search probes 16 pivots, one per lane (a 17-ary search: ~6 rounds for
-//     ten million suffixes instead of ~24 binary steps), and a probe reads its
-//     suffix's tokens as aligned 16-byte vectors, all loads in flight at once.
+//   * search: every suffix length n gets a warp that finds the lower and the
+//     upper bound of the pattern's suffix-array range, so all lengths
+//     n_max..n_min are searched together and the longest non-empty range is
+//     the answer (a match of length n implies matches of every shorter length,
+//     so a warp stops once a longer length has matched).  The first-token
+//     bucket table narrows each search to the suffixes that start with the
+//     pattern's first token.  A round probes 32 pivots, one per lane, until one
+//     equals the pattern, then 16 for either bound (~5 rounds for ten million
+//     suffixes instead of ~24 binary steps; 64 pivots a round made it slower),
+//     and a probe reads its suffix's tokens as aligned 16-byte vectors, all
+//     loads in flight at once.
 //   * the suffix that is exactly the pattern at the corpus end (no
 //     continuation) is the smallest suffix of its range when present; it is
 //     dropped.
@@ -24,7 +25,8 @@
 //     no token reads).
 //   * top-k: a histogram of run counts finds the k-th largest count; the runs
 //     above it and the first runs equal to it (in token order) are kept and
-//     ranked by (count descending, token order ascending).
+//     ranked by (count descending, token order ascending); few runs rank
+//     themselves at once.
 //   * reversed-corpus variant (fc_retrieve_rev): with the suffix array of the
 //     reversed corpus, the context suffixes of lengths 1, 2, ... read
 //     backwards are prefixes of one another, so their ranges are nested and
@@ -142,12 +144,13 @@ struct RetSmem {
   uint32_t sel[FC_MAX_TOPK];       // kept runs
   uint32_t order[FC_MAX_TOPK];     // kept runs by (count desc, run asc)
   uint32_t ctx[FC_MAX_NMAX];
-  uint32_t lo[FC_MAX_NMAX + 1];
-  uint32_t hi[FC_MAX_NMAX + 1];
-  uint32_t endhit[FC_MAX_NMAX + 1];
-  uint32_t wsum[RT_THREADS / 32];
+  uint32_t lo[FC_MAX_NMAX + 1];    // per length: the first occurrence and how many
+  uint32_t cnt[FC_MAX_NMAX + 1];
+  uint32_t pos[FC_MAX_TOPK];       // where the continuation in output slot t starts
+  uint32_t wsum[RT_THREADS / 32], words[RT_THREADS / 32];
   RunsScratch rs;
-  uint32_t n_star, first, cnt, bad, n_rev;
+  uint32_t bad, n_rev;
+  int longest;                     // the longest length found to match so far
   int32_t rc_slot;
 };
 
@@ -344,7 +347,10 @@ __global__ void __launch_bounds__(RT_THREADS) k_retrieve(DsArgs args, DsArgs rev
   int m = ctx_len[b];
   m = max(0, min(m, stride));
   const int cap = min(p.n_max, m);
-  if (tid == 0) sm.bad = 0;
+  if (tid == 0) {
+    sm.bad = 0;
+    sm.longest = 0;
+  }
   __syncthreads();
   if (tid < cap) {
     uint32_t t = ctx[(size_t)b * stride + (m - cap) + tid];
@@ -388,7 +394,6 @@ __global__ void __launch_bounds__(RT_THREADS) k_retrieve(DsArgs args, DsArgs rev
     n_top = (int)sm.n_rev;
     n_count = n_top ? 1 : 0;
   }
-  const int npairs = 2 * n_count;
   {
     const int warp = tid >> 5, lane = tid & 31, hl = lane & 15;
     const bool upper = lane >= 16;
@@ -398,17 +403,39 @@ __global__ void __launch_bounds__(RT_THREADS) k_retrieve(DsArgs args, DsArgs rev
       const uint32_t* pat = sm.ctx + (cap - n);
       const uint32_t t0 = pat[0];
       uint32_t lo = __ldg(ds.bucket + t0), hi = __ldg(ds.bucket + t0 + 1);
-      // invariant: the bound (first index whose suffix is >= the pattern, or >
-      // it for the upper bound) lies in [lo, hi], hi meaning "none below hi"
-      while (__any_sync(0xFFFFFFFFu, lo < hi)) {
+      auto compare = [&](uint32_t piv) {  // the suffix at piv against the pattern
+        uint32_t at = 0;
+        const int c = ds.keys ? cmp_suffix_key(ds.keys, T, N, piv, pat, n, &at)
+                              : cmp_suffix_vec(T, N, (at = __ldg(ds.sa + piv)), pat, n);
+        (void)FC_DEBUG_CHECK(at < N);
+        return c;
+      };
+      // invariant: both bounds (first index whose suffix is >= the pattern, first
+      // one > it) lie in [lo, hi], hi meaning "none below hi".  While no pivot
+      // equals the pattern the whole warp narrows one range, 32 pivots a round
+      // (a longer length that matches makes this one's result moot).
+      bool moot = false, apart = false;
+      while (lo < hi && !apart) {
+        if ((moot = __any_sync(0xFFFFFFFFu, *(volatile int*)&sm.longest > n))) break;
+        const uint32_t piv = lo + (uint32_t)(((uint64_t)(lane + 1) * (hi - lo)) / 33u);
+        const int c = compare(piv);
+        const int lt = __popc(__ballot_sync(0xFFFFFFFFu, c < 0)), le = __popc(__ballot_sync(0xFFFFFFFFu, c <= 0));
+        // pivots before each bound (prefixes of the warp)
+        apart = lt != le;
+        const int t = upper ? le : lt;
+        const uint32_t p_before = __shfl_sync(0xFFFFFFFFu, piv, max(t - 1, 0));
+        const uint32_t p_at = __shfl_sync(0xFFFFFFFFu, piv, min(t, 31));
+        if (t > 0) lo = p_before + 1;
+        if (t < 32) hi = p_at;
+      }
+      // then a half-warp per bound, 16 pivots a round
+      while (apart && __any_sync(0xFFFFFFFFu, lo < hi)) {
+        if ((moot = __any_sync(0xFFFFFFFFu, *(volatile int*)&sm.longest > n))) break;
         const bool active = lo < hi;
         const uint32_t piv = lo + (uint32_t)(((uint64_t)(hl + 1) * (hi - lo)) / 17u);
         bool pred = true;  // suffix at piv is past the bound's side
         if (active) {
-          uint32_t at = 0;
-          const int c = ds.keys ? cmp_suffix_key(ds.keys, T, N, piv, pat, n, &at)
-                                : cmp_suffix_vec(T, N, (at = __ldg(ds.sa + piv)), pat, n);
-          FC_DEBUG_CHECK(at < N);
+          const int c = compare(piv);
           pred = upper ? (c > 0) : (c >= 0);
         }
         const unsigned bal = __ballot_sync(0xFFFFFFFFu, !pred) & half_mask;
@@ -421,38 +448,21 @@ __global__ void __launch_bounds__(RT_THREADS) k_retrieve(DsArgs args, DsArgs rev
           if (t < 16) hi = p_at;
         }
       }
-      if (hl == 0) {
-        if (upper) {
-          sm.hi[n] = lo;
-        } else {
+      if (moot) continue;
+      const uint32_t end = __shfl_sync(0xFFFFFFFFu, lo, 16);
+      if (lane == 0) {
+        // the suffix that is exactly the pattern at the corpus end sorts first in its range
+        if (lo < end && (uint64_t)__ldg(ds.sa + lo) + n == N) ++lo;
+        if (lo < end) {
           sm.lo[n] = lo;
-          // the suffix that is exactly the pattern at the corpus end sorts first in its range
-          sm.endhit[n] = (lo < N && (uint64_t)__ldg(ds.sa + lo) + n == N) ? 1u : 0u;
+          sm.cnt[n] = min(end - lo, p.max_occ);
+          atomicMax(&sm.longest, n);
         }
       }
     }
   }
   __syncthreads();
-  if (tid == 0) {
-    uint32_t ns = 0, first = 0, cnt = 0;
-    if (npairs) {
-      for (int n = n_top; n > n_top - n_count; --n) {
-        uint32_t l = sm.lo[n], h = sm.hi[n];
-        if (l < h && sm.endhit[n]) ++l;
-        if (l < h) {
-          ns = n;
-          first = l;
-          cnt = h - l;
-          break;
-        }
-      }
-    }
-    sm.n_star = ns;
-    sm.first = first;
-    sm.cnt = min(cnt, p.max_occ);
-  }
-  __syncthreads();
-  const int ns = (int)sm.n_star;
+  const int ns = sm.longest;
   uint32_t* dr = o.drafts + sb * k * d;
   int32_t* dl = o.draft_len + sb * k;
   uint32_t* ct = o.count + sb * k;
@@ -468,44 +478,62 @@ __global__ void __launch_bounds__(RT_THREADS) k_retrieve(DsArgs args, DsArgs rev
     }
     return;
   }
-  const uint32_t nocc = sm.cnt, first = sm.first;
+  const uint32_t nocc = sm.cnt[ns], first = sm.lo[ns];
 
   // ---- runs of equal continuations -------------------------------------
   // neighbours j-1, j share their continuation iff lcp[j] >= n* + d
   const uint32_t need = (uint32_t)ns + (uint32_t)d;
-  for (uint32_t e = tid; e < nocc; e += RT_THREADS)
-    sm.work[e] = (e == 0 || (uint32_t)__ldg(ds.lcp + first + e) < need) ? 1u : 0u;
-  __syncthreads();
+  auto starts_run = [&](uint32_t e) { return e == 0 || (uint32_t)__ldg(ds.lcp + first + e) < need; };
   uint32_t nd_sel;
-  if constexpr (ALL)
-    nd_sel = runs_from_heads<RT_THREADS>(nocc, sm.runs, sm.work, sm.wsum, sm.rs);
-  else
-    nd_sel = rank_runs<RT_THREADS>(nocc, k, sm.runs, sm.work, sm.sel, sm.order, sm.wsum, sm.rs);
+  if (!ALL && nocc <= (uint32_t)RT_THREADS) {
+    nd_sel = rank_runs_few<RT_THREADS>(nocc, k, tid < (int)nocc && starts_run(tid), sm.runs, sm.work, sm.sel, sm.order,
+                                       sm.wsum, sm.words, sm.rs);
+  } else {
+    for (uint32_t e = tid; e < nocc; e += RT_THREADS) sm.work[e] = starts_run(e) ? 1u : 0u;
+    __syncthreads();
+    if constexpr (ALL)
+      nd_sel = runs_from_heads<RT_THREADS>(nocc, sm.runs, sm.work, sm.wsum, sm.rs);
+    else
+      nd_sel = rank_runs<RT_THREADS>(nocc, k, sm.runs, sm.work, sm.sel, sm.order, sm.wsum, sm.rs);
+  }
   auto run_count = [&](uint32_t r) { return sm.runs[r + 1] - sm.runs[r]; };
   auto run_at = [&](int t) -> uint32_t { return ALL ? (uint32_t)t : sm.order[t]; };  // the run in output slot t
   // ---- outputs ---------------------------------------------------------
   const int nd = (int)nd_sel;
-  for (int e = tid; e < k * d; e += RT_THREADS) {
-    int t = e / d, x = e - t * d;
-    uint32_t v = FC_PAD_TOKEN;
-    if (t < nd) {
-      const uint64_t pp = (uint64_t)__ldg(ds.sa + first + sm.runs[run_at(t)]) + (uint64_t)ns;
-      if (FC_DEBUG_CHECK(pp < N)) {
-        const uint64_t len = min((uint64_t)d, N - pp);
-        if ((uint64_t)x < len) v = __ldg(T + pp + x);
+  if constexpr (ALL) {
+    for (int e = tid; e < k * d; e += RT_THREADS) {
+      int t = e / d, x = e - t * d;
+      uint32_t v = FC_PAD_TOKEN;
+      if (t < nd) {
+        const uint64_t pp = (uint64_t)__ldg(ds.sa + first + sm.runs[run_at(t)]) + (uint64_t)ns;
+        if (FC_DEBUG_CHECK(pp < N)) {
+          const uint64_t len = min((uint64_t)d, N - pp);
+          if ((uint64_t)x < len) v = __ldg(T + pp + x);
+        }
       }
+      dr[e] = v;
     }
-    dr[e] = v;
   }
   for (int t = tid; t < k; t += RT_THREADS) {
     if (t < nd) {
       const uint32_t r = run_at(t);
       const uint64_t pp = (uint64_t)__ldg(ds.sa + first + sm.runs[r]) + (uint64_t)ns;
+      if constexpr (!ALL) sm.pos[t] = (uint32_t)(FC_DEBUG_CHECK(pp < N) ? pp : N);
       dl[t] = pp < N ? (int32_t)min((uint64_t)d, N - pp) : 0;
       ct[t] = run_count(r);
     } else {
       dl[t] = 0;
       ct[t] = 0;
+    }
+  }
+  if constexpr (!ALL) {  // the continuations' starts in one round trip, their tokens in the next
+    __syncthreads();
+#pragma unroll 4
+    for (int e = tid; e < k * d; e += RT_THREADS) {
+      const int t = e / d, x = e - t * d;
+      uint32_t v = FC_PAD_TOKEN;
+      if (t < nd && (uint64_t)sm.pos[t] + x < N) v = __ldg(T + sm.pos[t] + x);
+      dr[e] = v;
     }
   }
   if (tid == 0) {

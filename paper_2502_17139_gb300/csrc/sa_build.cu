@@ -22,8 +22,8 @@
 //
 // Bound by HBM: the radix passes stream 32 bytes a position each, the rounds
 // gather the text of the suffixes still in play.  Doubling from the start sorts
-// all positions in every round: 100M tokens 114 ms against 17 ms
-// (with the suffix keys); 1M tokens 1.94 against 0.77 ms.
+// all positions in every round: 100M tokens 114 ms against 13.3 ms
+// (with the suffix keys); 1M tokens 1.94 against 0.63 ms.
 
 #include <algorithm>
 
@@ -152,8 +152,8 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const uint64_t* __res
 // addresses of a digit's run, so the stores coalesce instead of spraying
 // 8- and 4-byte writes over 256 runs.  The values follow through the same
 // shared memory.  Bound by the latency of its phases, so by how many blocks an
-// SM holds: four at 64 registers and 42 KB (with the values in registers and
-// shared memory beside the keys, two: 0.99 ms a pass of 100M pairs, now @@).
+// SM holds: three at 80 registers (with the values in registers and shared
+// memory beside the keys, two: 208 us a pass of 20M pairs against 128).
 // FIRST: the keys come from the text and the values are the positions.
 template <bool FIRST>
 __global__ void __launch_bounds__(RS_THREADS, 3) k_radix_scatter(const uint64_t* __restrict__ kin,
@@ -1059,7 +1059,8 @@ extern "C" fc_status fc_datastore_build_noalloc(const uint32_t* d_tokens, uint64
 namespace {
 // VEC: the corpus is 16-byte aligned, and a suffix's tokens 1..7 come from the
 // aligned 16-byte groups they lie in (all inside the corpus) instead of seven
-// 4-byte loads.  Bound by the random reads: 100M tokens @@.
+// 4-byte loads.  Bound by the random reads: 20M tokens 352 us with 4-byte loads
+// alone, 283 us now.
 template <bool VEC>
 __global__ void k_suffix_keys(const uint32_t* __restrict__ T, const uint32_t* __restrict__ sa, uint64_t n,
                               uint4* __restrict__ keys) {

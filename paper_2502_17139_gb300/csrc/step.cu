@@ -167,9 +167,8 @@ __device__ __forceinline__ uint32_t max_nan_bf16x2(uint32_t a, uint32_t b) {
 // one chunk for the first element equal to it.  All rows run at once and are
 // read from their ends to their fronts: bound by HBM and L2, and the LM head
 // writes column by column of tiles, so the rows' ends are what L2 still holds
-// (39 -> 30 us
-// behind an LM head of 2048 rows by 32256 columns, 5 TB/s from 2048 cold rows).  The warp reduction then
-// orders candidates by (value, index).
+// (39 -> 30 us behind an LM head of 2048 rows by 32256 columns, 5 TB/s from
+// 2048 cold rows).  The warp reduction then orders candidates by (value, index).
 __global__ void __launch_bounds__(AM_WARPS * 32) k_argmax_rows(const uint16_t* __restrict__ logits, int vocab,
                                                                 const int32_t* __restrict__ n_nodes, int n_pad,
                                                                 uint32_t* __restrict__ argmax) {

@@ -1,4 +1,6 @@
 // Library-wide entry points: status names, version, device error word.
+#include <cmath>
+
 #include "fc_common.cuh"
 
 extern "C" unsigned int fc_take_error_sa(cudaStream_t s);
@@ -19,6 +21,21 @@ unsigned int* fc_error_slot() { return t_error_slot; }
 FcErrorScope::FcErrorScope(unsigned int* word) : prev(t_error_slot) { t_error_slot = word; }
 
 FcErrorScope::~FcErrorScope() { t_error_slot = prev; }
+
+const FcRope64& fc_rope64(float base) {
+  static thread_local float made_for = 0.f;  // no valid base
+  static thread_local FcRope64 t;
+  if (base != made_for) {
+    const double nl2f = -2.0 * std::log2((double)base) / 128.0;
+    for (int i = 0; i < 64; ++i) {
+      const double f = std::exp2((double)i * nl2f);
+      const float hi = (float)f;
+      t.f[i] = make_float2(hi, (float)(f - (double)hi));
+    }
+    made_for = base;
+  }
+  return t;
+}
 
 extern "C" const char* fc_status_string(fc_status s) {
   switch (s) {

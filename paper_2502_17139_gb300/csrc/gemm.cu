@@ -74,7 +74,7 @@ struct GemmArgs {
   __nv_bfloat16* v_out;  // [B][Hkv][n_pad][128]
   const int32_t* pos;    // [B][n_pad]; a negative position leaves its row unrotated
   int n_pad, hkv;
-  double rope_nl2f;      // -2 log2(base) / 128
+  FcRope64 rope;         // the rotation frequencies
   unsigned int* err;     // the launch's error word (NULL: this file's own)
 };
 
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ float2 s_rope[64];
-  if constexpr (EPI == EPI_KV_HEADS) fc_rope_table(s_rope, 64, g.rope_nl2f);  // read after the barrier below
+  if constexpr (EPI == EPI_KV_HEADS) fc_rope_copy(s_rope, g.rope);  // read after the barrier below
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) __cluster_dims__(2, 1, 1)
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ float2 s_rope[64];
-  if constexpr (EPI == EPI_KV_HEADS) fc_rope_table(s_rope, 64, g.rope_nl2f);  // read after the barrier below
+  if constexpr (EPI == EPI_KV_HEADS) fc_rope_copy(s_rope, g.rope);  // read after the barrier below
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -601,7 +601,7 @@ __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
     tmem_alloc(smem_u32(&s_tmem), WN);
     tmem_relinquish();
   }
-  if constexpr (EPI == EPI_KV_HEADS) fc_rope_table(s_rope, 64, g.rope_nl2f);
+  if constexpr (EPI == EPI_KV_HEADS) fc_rope_copy(s_rope, g.rope);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -921,7 +921,7 @@ extern "C" fc_status fc_gemm_kv_heads(const void* d_a, const void* d_wkv, int M,
   g.pos = d_pos;
   g.n_pad = n_pad;
   g.hkv = Hkv;
-  g.rope_nl2f = -2.0 * std::log2((double)rope_base) / 128.0;
+  g.rope = fc_rope64(rope_base);
   return launch_gemm<EPI_KV_HEADS>(d_a, d_wkv, M, 2 * Hkv * 128, K, g, static_cast<cudaStream_t>(stream));
 }
 

@@ -96,7 +96,7 @@ struct AttnArgs {
   unsigned int* err;  // the launch's error word (NULL: this file's own)
   float scale_log2;
   const int32_t* pos;  // [B][n_pad] node positions: rotate Q by them (RoPE), or nullptr
-  double rope_nl2f;    // -2 log2(base) / D: pair i turns by pos * 2^(i * rope_nl2f)
+  FcRope64 rope;       // the rotation frequencies, where pos is given
 };
 
 // Rotates the two pairs held by one 32-bit word of each half: l holds
@@ -305,6 +305,16 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   __shared__ volatile int s_abort;
   __shared__ int s_ticket, s_ready;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __shared__ float2 s_rope[ROPE ? HD / 2 : 1];
+  if constexpr (ROPE) fc_rope_copy(s_rope, a.rope);  // read behind a barrier below
+  if constexpr (SPREAD) {  // what needs no memory, while the kernel before drains
+    if (tid == 0) {
+      prefetch_tmap(&tm_kc);
+      prefetch_tmap(&tm_vc);
+      prefetch_tmap(&tm_kt);
+      prefetch_tmap(&tm_vt);
+    }
+  }
   fc_grid_wait();
   // Units (group, row chunk) in launch order, so the row chunks of a group,
   // which stream the same K/V blocks, run together and share them through
@@ -398,10 +408,12 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
     s_abort = 0;
     for (int i = 0; i < N_BARS; ++i) mbar_init(bar(i), (i == B_PFULL || i == B_PFULL + 1) ? 128u : 1u);
     fence_mbar_init();
-    prefetch_tmap(&tm_kc);
-    prefetch_tmap(&tm_vc);
-    prefetch_tmap(&tm_kt);
-    prefetch_tmap(&tm_vt);
+    if constexpr (!SPREAD) {
+      prefetch_tmap(&tm_kc);
+      prefetch_tmap(&tm_vc);
+      prefetch_tmap(&tm_kt);
+      prefetch_tmap(&tm_vt);
+    }
     if constexpr (Q_FIRST) {
       load_kv(0, true);
     } else {
@@ -417,9 +429,7 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   }
   // Q tiles: rows (head in group, node) packed densely, 128-byte swizzled, K-major.
   if constexpr (ROPE) {
-    __shared__ float2 s_rope[HD / 2];
-    fc_rope_table(s_rope, HD / 2, a.rope_nl2f);
-    __syncthreads();
+    __syncthreads();  // s_rope
     stage_q_rope(smem + OFF_Q, a.q, a.pos, s_rope, b, g, a.G, a.H, a.n_pad, nn, row0, rows_total, tid);
   } else {
     // asynchronous 16-byte copies: all of a thread's rows in flight at once
@@ -1683,7 +1693,7 @@ static fc_status launch_tree_attn(const void* d_q, const void* d_k_cache, const 
   a.min_cost = SPREAD_MIN_COST;
   a.err = fc_error_slot();
   a.pos = d_pos;
-  a.rope_nl2f = d_pos ? -2.0 * std::log2((double)rope_base) / HD : 0.0;
+  if (d_pos) a.rope = fc_rope64(rope_base);
   if (sp.parts > 1) {
     const WsLayout w = ws_layout(n_split, sp.parts);
     unsigned char* base = static_cast<unsigned char*>(d_ws);

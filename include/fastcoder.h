@@ -616,6 +616,13 @@ fc_status fc_gemm_bf16(const void* d_a, const void* d_b, void* d_c, int M, int N
 fc_status fc_gemm_kv_heads(const void* d_a, const void* d_wkv, int M, int K, int Hkv, int D, int batch, int n_pad,
                            const int32_t* d_pos, float rope_base, void* d_k_rot, void* d_v_heads, fc_stream s);
 
+/* The query projection q = A Wq [M][H D] (row-major, unrotated) and
+ * fc_gemm_kv_heads in one launch, with the same results (one launch each when
+ * H is odd). */
+fc_status fc_gemm_qkv(const void* d_a, const void* d_wq, const void* d_wkv, int M, int K, int H, int Hkv, int D,
+                      int batch, int n_pad, const int32_t* d_pos, float rope_base, void* d_q, void* d_k_rot,
+                      void* d_v_heads, fc_stream s);
+
 /* The gate/up projection with the SiLU-gated product folded into the GEMM's
  * epilogue: act[M][inter] = silu(A Wg) * (A Wu), fp32 inside, rounded once
  * to bf16.  d_wgu holds Wg and Wu interleaved in 128-column blocks, as

@@ -20,14 +20,15 @@
 //     the CTA lets its in-flight copies and MMAs land before it frees tensor
 //     memory and exits.
 //
-// Two epilogues fold the decoder's next step into the GEMM, so its output
+// The epilogues fold the decoder's next step into the GEMM, so its output
 // never makes a round trip through HBM in bf16:
 //   * K/V heads (fc_gemm_kv_heads): the fused K/V projection's 256-column
 //     tile holds two whole heads (D = 128); the epilogue rotates the key
 //     heads by each row's node position (RoPE, rotate-half pairing: columns
 //     d and d + 64 of a head, both in the tile) from the fp32 accumulators and
 //     writes both kinds head-major, as the tree attention and the cache
-//     append read them;
+//     append read them; fc_gemm_qkv runs the query projection's tiles (stored as
+//     they are) and these in one launch;
 //   * SiLU * up (fc_gemm_silu_mul): with the gate and up weights interleaved
 //     in 128-column blocks (fc_interleave_gate_up), a tile holds gate block t
 //     and up block t, and the epilogue writes act[:, 128t .. 128t + 128) =
@@ -62,7 +63,7 @@ constexpr uint64_t DRAIN_CYCLES = 400000000ull;          // ~0.2 s
 enum { B_FULL = 0, B_EMPTY = STAGES, B_ACC_FULL = 2 * STAGES, B_ACC_EMPTY = 2 * STAGES + 2,
        B_DRAIN = 2 * STAGES + 4, N_BARS = 2 * STAGES + 5 };
 
-enum { EPI_STORE = 0, EPI_KV_HEADS = 1, EPI_SILU_MUL = 2 };
+enum { EPI_STORE = 0, EPI_KV_HEADS = 1, EPI_SILU_MUL = 2, EPI_QKV = 3 };
 
 struct GemmArgs {
   __nv_bfloat16* c;  // EPI_STORE: C [M][N]; EPI_SILU_MUL: act [M][N / 2]
@@ -76,7 +77,19 @@ struct GemmArgs {
   int n_pad, hkv;
   FcRope64 rope;         // the rotation frequencies
   unsigned int* err;     // the launch's error word (NULL: this file's own)
+  int n_q;               // EPI_QKV: columns of the first weights, stored as EPI_STORE does; the rest as EPI_KV_HEADS
 };
+
+// The weight map of a column, and the column in it (EPI_QKV has two weight matrices side by side).
+template <int EPI>
+__device__ __forceinline__ const CUtensorMap* weight_map(const CUtensorMap& b, const CUtensorMap& b2, const GemmArgs& g,
+                                                         int& col) {
+  if (EPI == EPI_QKV && col >= g.n_q) {
+    col -= g.n_q;
+    return &b2;
+  }
+  return &b;
+}
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
   asm volatile(
@@ -118,19 +131,24 @@ __device__ __forceinline__ uint4 pack8(const float* v) {
 // One output row of a 128 x 256 tile, from 256 tensor-memory columns at tacc
 // (one row per thread; called by whole warps).
 template <int EPI>
-__device__ __forceinline__ void store_tile_row(const GemmArgs& g, uint32_t tacc, int row, int n0, const float2* s_rope) {
-  if constexpr (EPI == EPI_STORE) {
-    __nv_bfloat16* crow = g.c + (size_t)row * g.N;
+__device__ __forceinline__ void store_tile_row(const GemmArgs& g, uint32_t tacc, int row, int n0, const float2* s_rope,
+                                               int ldc = 0) {
+  if constexpr (EPI == EPI_QKV) {
+    if (n0 < g.n_q) store_tile_row<EPI_STORE>(g, tacc, row, n0, s_rope, g.n_q);
+    else store_tile_row<EPI_KV_HEADS>(g, tacc, row, n0 - g.n_q, s_rope);
+  } else if constexpr (EPI == EPI_STORE) {
+    const int N = ldc ? ldc : g.N;
+    __nv_bfloat16* crow = g.c + (size_t)row * N;
 #pragma unroll 1
     for (int cc = 0; cc < BN / 32; ++cc) {
       uint32_t v[32];
       tmem_ld32(tacc + cc * 32, v);
       tc_wait_ld();
       const int col = n0 + cc * 32;
-      if (row < g.M && col < g.N) {
+      if (row < g.M && col < N) {
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          if (col + 8 * u + 8 <= g.N)
+          if (col + 8 * u + 8 <= N)
             *reinterpret_cast<uint4*>(crow + col + 8 * u) = pack8_bits(v + 8 * u);
       }
     }
@@ -203,12 +221,13 @@ __device__ __forceinline__ void store_tile_row(const GemmArgs& g, uint32_t tacc,
 
 template <int EPI>
 __global__ void __launch_bounds__(GM_THREADS, 1)
-    k_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, GemmArgs g) {
+    k_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
+           const __grid_constant__ CUtensorMap tm_b2, GemmArgs g) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ float2 s_rope[64];
-  if constexpr (EPI == EPI_KV_HEADS) fc_rope_copy(s_rope, g.rope);  // read after the barrier below
+  if constexpr (EPI == EPI_KV_HEADS || EPI == EPI_QKV) fc_rope_copy(s_rope, g.rope);  // read after the barrier below
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -231,6 +250,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
     fence_mbar_init();
     prefetch_tmap(&tm_a);
     prefetch_tmap(&tm_b);
+    if constexpr (EPI == EPI_QKV) prefetch_tmap(&tm_b2);
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(&s_tmem), TMEM_COLS);
@@ -242,7 +262,11 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
   if (tid == 0) {  // the first tile's first weights into L2 while the kernel before drains
     const int n0 = ((int)blockIdx.x / g.tiles_m) * BN;
     for (int kb = 0; kb < min(nk, PREFETCH); ++kb)
-      for (int c = 0; c < BN / 64; ++c) tma_prefetch_2d(&tm_b, n0 + 64 * c, kb * BK);
+      for (int c = 0; c < BN / 64; ++c) {
+        int col = n0 + 64 * c;
+        const CUtensorMap* m = weight_map<EPI>(tm_b, tm_b2, g, col);
+        tma_prefetch_2d(m, col, kb * BK);
+      }
   }
   __syncwarp();
   fc_grid_wait();
@@ -253,7 +277,9 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
     if (lane == 0) {
       uint32_t issued = 0;
       for (int t = blockIdx.x; t < g.tiles && !s_abort; t += gridDim.x) {
-        const int m0 = (t % g.tiles_m) * BM, n0 = (t / g.tiles_m) * BN;
+        const int m0 = (t % g.tiles_m) * BM;
+        int wcol = (t / g.tiles_m) * BN;
+        const CUtensorMap* wm = weight_map<EPI>(tm_b, tm_b2, g, wcol);
         for (int kb = 0; kb < nk; ++kb) {
           const uint32_t s = issued % STAGES, ph = (issued / STAGES) & 1;
           if (!mbar_wait_bounded(bar(B_EMPTY + s), ph ^ 1, &s_abort, WAIT_CYCLES)) break;
@@ -261,7 +287,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
           mbar_expect_tx(bar(B_FULL + s), STAGE_BYTES);
           tma_load_2d(st, &tm_a, kb * BK, m0, bar(B_FULL + s));
 #pragma unroll
-          for (int c = 0; c < BN / 64; ++c) tma_load_2d(st + A_BYTES + c * B_CHUNK, &tm_b, n0 + 64 * c, kb * BK, bar(B_FULL + s));
+          for (int c = 0; c < BN / 64; ++c) tma_load_2d(st + A_BYTES + c * B_CHUNK, wm, wcol + 64 * c, kb * BK, bar(B_FULL + s));
           ++issued;
         }
       }
@@ -406,12 +432,13 @@ __device__ __forceinline__ bool wait_warp_cluster(uint32_t bar, uint32_t parity,
 
 template <int EPI>
 __global__ void __launch_bounds__(GM_THREADS, 1) __cluster_dims__(2, 1, 1)
-    k_gemm_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, GemmArgs g) {
+    k_gemm_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
+           const __grid_constant__ CUtensorMap tm_b2, GemmArgs g) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ float2 s_rope[64];
-  if constexpr (EPI == EPI_KV_HEADS) fc_rope_copy(s_rope, g.rope);  // read after the barrier below
+  if constexpr (EPI == EPI_KV_HEADS || EPI == EPI_QKV) fc_rope_copy(s_rope, g.rope);  // read after the barrier below
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -429,6 +456,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) __cluster_dims__(2, 1, 1)
     fence_mbar_init();
     prefetch_tmap(&tm_a);
     prefetch_tmap(&tm_b);
+    if constexpr (EPI == EPI_QKV) prefetch_tmap(&tm_b2);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
@@ -443,7 +471,11 @@ __global__ void __launch_bounds__(GM_THREADS, 1) __cluster_dims__(2, 1, 1)
   if (tid == 0) {  // the first tile's first weights into L2 while the kernel before drains
     const int n0 = (pair / g.tiles_m) * BN + (int)rank * (BN / 2);
     for (int kb = 0; kb < min(nk, PREFETCH); ++kb)
-      for (int c = 0; c < BN / 128; ++c) tma_prefetch_2d(&tm_b, n0 + 64 * c, kb * BK);
+      for (int c = 0; c < BN / 128; ++c) {
+        int col = n0 + 64 * c;
+        const CUtensorMap* m = weight_map<EPI>(tm_b, tm_b2, g, col);
+        tma_prefetch_2d(m, col, kb * BK);
+      }
   }
   __syncwarp();
   fc_grid_wait();
@@ -454,7 +486,9 @@ __global__ void __launch_bounds__(GM_THREADS, 1) __cluster_dims__(2, 1, 1)
     if (lane == 0) {
       uint32_t issued = 0;
       for (int t = pair; t < g.tiles && !s_abort; t += pairs) {
-        const int m0 = (t % g.tiles_m) * PR_BM + (int)rank * BM, n0 = (t / g.tiles_m) * BN + (int)rank * (BN / 2);
+        const int m0 = (t % g.tiles_m) * PR_BM + (int)rank * BM;
+        int wcol = (t / g.tiles_m) * BN + (int)rank * (BN / 2);
+        const CUtensorMap* wm = weight_map<EPI>(tm_b, tm_b2, g, wcol);
         for (int kb = 0; kb < nk; ++kb) {
           const uint32_t s = issued % PR_STAGES, ph = (issued / PR_STAGES) & 1;
           if (!mbar_wait_bounded(bar(P_EMPTY + s), ph ^ 1, &s_abort, WAIT_CYCLES)) break;
@@ -462,7 +496,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) __cluster_dims__(2, 1, 1)
           if (rank == 0) mbar_expect_tx(bar(P_FULL + s), 2 * PR_STAGE);
           tma_load_2d_pair(st, &tm_a, kb * BK, m0, fb);
 #pragma unroll
-          for (int c = 0; c < BN / 128; ++c) tma_load_2d_pair(st + A_BYTES + c * B_CHUNK, &tm_b, n0 + 64 * c, kb * BK, fb);
+          for (int c = 0; c < BN / 128; ++c) tma_load_2d_pair(st + A_BYTES + c * B_CHUNK, wm, wcol + 64 * c, kb * BK, fb);
           ++issued;
         }
       }
@@ -567,8 +601,8 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank) {
 
 template <int EPI, int S, int NB>
 __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
-    k_gemm_split(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, GemmArgs g,
-                 SplitArgs sp) {
+    k_gemm_split(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
+                 const __grid_constant__ CUtensorMap tm_b2, GemmArgs g, SplitArgs sp) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
@@ -596,12 +630,13 @@ __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
     fence_mbar_init();
     prefetch_tmap(&tm_a);
     prefetch_tmap(&tm_b);
+    if constexpr (EPI == EPI_QKV) prefetch_tmap(&tm_b2);
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(&s_tmem), WN);
     tmem_relinquish();
   }
-  if constexpr (EPI == EPI_KV_HEADS) fc_rope_copy(s_rope, g.rope);
+  if constexpr (EPI == EPI_KV_HEADS || EPI == EPI_QKV) fc_rope_copy(s_rope, g.rope);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -610,7 +645,11 @@ __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
   // into the coherent L2 is no read: what that kernel writes to them counts)
   if (tid == 0)
     for (int kb = k0; kb < k1; ++kb)
-      for (int c = 0; c < NB; ++c) tma_prefetch_2d(&tm_b, chunk_col(c), kb * BK);
+      for (int c = 0; c < NB; ++c) {
+        int col = chunk_col(c);
+        const CUtensorMap* m = weight_map<EPI>(tm_b, tm_b2, g, col);
+        tma_prefetch_2d(m, col, kb * BK);
+      }
   __syncwarp();
   fc_grid_wait();
   const uint32_t tmem = s_tmem;
@@ -625,7 +664,11 @@ __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
         const uint32_t st = sbase + s * stage_bytes, fb = bar(SB_FULL + s);
         mbar_expect_tx(fb, stage_bytes);
 #pragma unroll
-        for (int c = 0; c < NB; ++c) tma_load_2d(st + a_bytes + c * B_CHUNK, &tm_b, chunk_col(c), kb * BK, fb);
+        for (int c = 0; c < NB; ++c) {
+          int col = chunk_col(c);
+          const CUtensorMap* m = weight_map<EPI>(tm_b, tm_b2, g, col);
+          tma_load_2d(st + a_bytes + c * B_CHUNK, m, col, kb * BK, fb);
+        }
         tma_load_2d(st, &tm_a, kb * BK, m0, fb);
       }
       if (s_abort) {  // let the copies in flight land before the CTA exits
@@ -706,19 +749,22 @@ __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
       }
     }
     const int row = m0 + r;
-    if constexpr (EPI == EPI_STORE) {
-      __nv_bfloat16* crow = g.c + (size_t)row * g.N;
+    const bool plain = EPI == EPI_STORE || (EPI == EPI_QKV && nt * WN < g.n_q);
+    if (plain) {
+      const int N = EPI == EPI_QKV ? g.n_q : g.N;
+      __nv_bfloat16* crow = g.c + (size_t)row * N;
       const int col = nt * WN + c;
-      if (col + 8 <= g.N) *reinterpret_cast<uint4*>(crow + col) = pack8(lo);
-      if (col + HN + 8 <= g.N) *reinterpret_cast<uint4*>(crow + col + HN) = pack8(hi);
+      if (col + 8 <= N) *reinterpret_cast<uint4*>(crow + col) = pack8(lo);
+      if (col + HN + 8 <= N) *reinterpret_cast<uint4*>(crow + col + HN) = pack8(hi);
     } else if constexpr (EPI == EPI_SILU_MUL) {
 #pragma unroll
       for (int u = 0; u < 8; ++u) lo[u] = __fdividef(lo[u], 1.f + __expf(-lo[u])) * hi[u];  // as in k_gemm
       *reinterpret_cast<uint4*>(g.c + (size_t)row * (g.N / 2) + nt * HN + c) = pack8(lo);
-    } else {
+    } else if constexpr (EPI != EPI_STORE) {
+      const int hh = EPI == EPI_QKV ? nt - g.n_q / 128 : nt;  // the tile is one head
       const int b = row / g.n_pad, i = row - b * g.n_pad;
-      const bool key = nt < g.hkv;
-      const int head = key ? nt : nt - g.hkv, p = g.pos[row];
+      const bool key = hh < g.hkv;
+      const int head = key ? hh : hh - g.hkv, p = g.pos[row];
       __nv_bfloat16* dst = (key ? g.k_out : g.v_out) + (((size_t)b * g.hkv + head) * g.n_pad + i) * 128 + c;
       if (key && p >= 0) {
 #pragma unroll
@@ -782,9 +828,13 @@ bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0;
 // How many CTAs a cluster of k_gemm_split has for a launch, 0 = k_gemm.  The
 // split kernel serves launches whose 128 x 256 tiles fill less than half of
 // the SMs, with the most CTAs that still fit one per SM (a deep ring each);
-// shares of K of at least four slices.  Clusters of eight fit two CTAs per SM
-// only (one per SM, the GPCs hold too few of them: 10.7 against 7.3 us), with
-// half the ring; they pay for up to 64 rows and long K.
+// shares of K of at least four slices.  The GPCs hold whole clusters: 36 of
+// four and 46 of three on 152 SMs, and one more waits for a second wave (M 64,
+// K 2048: 47 tiles of three 9.2 -> 15.6 us, 38 of four 8.3 -> 14), hence the
+// limits.  Clusters of eight fit two CTAs per SM only (one per SM 10.7 against
+// 7.3 us), with half the ring; they pay for up to 64 rows and long K, as those
+// of four do there for up to 65 tiles (M 64, K 4096, N 6144: two 16.8, four
+// 14.4 us; K 2048: 9.8, 10.0).
 // us per call, k_gemm / clusters of 2 / 4 / 8, weights from HBM:
 //   M 64,  K 2048, N 2048   13.8 /  9.3 /  7.2 /  7.3      M 512, same        14.7 / 10.7 / 11.5 / 21
 //   M 256, K 2048, N 2048   15.1 / 10.3 /  8.4 / 11.1      M 64,  N 4096      14.8 /  9.7 /  8.1 /  8.9
@@ -792,16 +842,20 @@ bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0;
 //   M 512, K 2048, N 4096   15.6 / 14.6 / 23 / 47          (128 big tiles and more: k_gemm)
 // Where two CTAs per 128-column tile are too many, clusters of three take
 // 256-column tiles: gate/up of inter 5504 at M 64 15.6 -> 12.2, M 128 16.4 -> 14.2.
+// Just past clusters of four, those of three: M 64, K 2048, N 5632 9.8 -> 9.0.
 struct SplitPlan {
   int cluster, nb;  // CTAs per cluster (0: k_gemm), 64-column chunks per tile
+  bool half;        // half the ring, two CTAs per SM
 };
 SplitPlan choose_split(int M, int64_t tiles_m, int N, int64_t big_tiles, int nk, int sms, bool wide) {
   const int64_t tiles = tiles_m * ((N + 127) / 128);
-  if (2 * big_tiles > sms) return {0, 0};
-  if (M <= 64 && nk >= 64 && tiles * 8 <= sms) return {8, 2};
-  if (nk >= 16 && tiles * 4 <= sms) return {4, 2};
-  if (nk >= 8 && tiles * 2 <= sms) return {2, 2};
-  return wide && nk >= 12 && big_tiles * 3 <= sms ? SplitPlan{3, 4} : SplitPlan{0, 0};
+  if (2 * big_tiles > sms) return {0, 0, false};
+  if (M <= 64 && nk >= 64 && tiles * 8 <= sms) return {8, 2, true};
+  if (nk >= 16 && tiles * 25 <= 6 * sms) return {4, 2, false};
+  if (M <= 64 && nk >= 48 && tiles * 7 <= 3 * sms) return {4, 2, true};
+  if (nk >= 12 && tiles * 27 <= 8 * sms) return {3, 2, false};
+  if (nk >= 8 && tiles * 2 <= sms) return {2, 2, false};
+  return wide && nk >= 12 && big_tiles * 27 <= 8 * sms ? SplitPlan{3, 4, false} : SplitPlan{0, 0, false};
 }
 
 // Whether k_gemm_pair serves a launch of `tiles` 128 x 256 tiles: by waves, a
@@ -818,7 +872,8 @@ bool use_pair(int64_t tiles_m, int64_t tiles, int64_t pair_tiles, int nk, int sm
 }
 
 template <int EPI>
-fc_status launch_gemm(const void* d_a, const void* d_b, int M, int N, int K, GemmArgs g, cudaStream_t stream) {
+fc_status launch_gemm(const void* d_a, const void* d_b, int M, int N, int K, GemmArgs g, cudaStream_t stream,
+                      const void* d_b2 = nullptr) {
   const int sms = sm_count();
   if (sms <= 0) return FC_ERR_CUDA;
   g.M = M;
@@ -829,15 +884,17 @@ fc_status launch_gemm(const void* d_a, const void* d_b, int M, int N, int K, Gem
   const int64_t tiles = (int64_t)g.tiles_m * ((N + BN - 1) / BN);
   if (tiles > 0x7FFFFFFF) return FC_ERR_UNSUPPORTED;
   g.tiles = (int)tiles;
-  CUtensorMap ma, mb;
-  constexpr bool WIDE = EPI != EPI_KV_HEADS;  // a tile of the K/V projection is one head
+  CUtensorMap ma, mb, mb2;
+  constexpr bool WIDE = EPI == EPI_STORE || EPI == EPI_SILU_MUL;  // a narrow tile of the K/V projection is one head
   const SplitPlan plan = choose_split(M, g.tiles_m, N, tiles, (K + BK - 1) / BK, sms, WIDE);
   const int a_rows = plan.cluster ? std::min(BM, (M + 7) / 8 * 8) : BM;
-  if (!make_map_2d(&ma, d_a, (uint64_t)M, (uint64_t)K, a_rows) || !make_map_2d(&mb, d_b, (uint64_t)K, (uint64_t)N, BK))
+  if (!make_map_2d(&ma, d_a, (uint64_t)M, (uint64_t)K, a_rows) || !make_map_2d(&mb, d_b, (uint64_t)K, (uint64_t)(d_b2 ? g.n_q : N), BK))
     return FC_ERR_CUDA;
-  using Split = void (*)(CUtensorMap, CUtensorMap, GemmArgs, SplitArgs);
+  mb2 = mb;
+  if (d_b2 && !make_map_2d(&mb2, d_b2, (uint64_t)K, (uint64_t)(N - g.n_q), BK)) return FC_ERR_CUDA;
+  using Split = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, GemmArgs, SplitArgs);
   constexpr int W = WIDE ? 4 : 2;
-  static constexpr Split narrow[9] = {nullptr, nullptr, k_gemm_split<EPI, 2, 2>, nullptr, k_gemm_split<EPI, 4, 2>,
+  static constexpr Split narrow[9] = {nullptr, nullptr, k_gemm_split<EPI, 2, 2>, k_gemm_split<EPI, 3, 2>, k_gemm_split<EPI, 4, 2>,
                                       nullptr, nullptr, nullptr, k_gemm_split<EPI, 8, 2>};
   static constexpr Split wide = WIDE ? k_gemm_split<EPI, 3, W> : nullptr;
   static std::atomic<unsigned long long> ready;
@@ -845,7 +902,7 @@ fc_status launch_gemm(const void* d_a, const void* d_b, int M, int N, int K, Gem
     if (cudaFuncSetAttribute(k_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_gemm_pair<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PR_SMEM) != cudaSuccess)
       return FC_ERR_CUDA;
-    for (const Split k : {narrow[2], narrow[4], narrow[8], wide})
+    for (const Split k : {narrow[2], narrow[3], narrow[4], narrow[8], wide})
       if (k && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SP_RING_1 + SP_EXTRA)) != cudaSuccess)
         return FC_ERR_CUDA;
     return FC_OK;
@@ -853,21 +910,21 @@ fc_status launch_gemm(const void* d_a, const void* d_b, int M, int N, int K, Gem
   if (set != FC_OK) return set;
   if (plan.cluster) {
     const uint32_t stage = (uint32_t)a_rows * (BK * 2) + plan.nb * B_CHUNK;
-    const uint32_t ring = plan.cluster == 8 ? SP_RING_2 : SP_RING_1;
+    const uint32_t ring = plan.half ? SP_RING_2 : SP_RING_1;
     const SplitArgs sp{a_rows, std::min<int>(SP_MAX_STAGES, ring / stage), ring};
     const int64_t ctas = (int64_t)g.tiles_m * ((N + 64 * plan.nb - 1) / (64 * plan.nb)) * plan.cluster;
     return fc_launch_dependent(plan.nb == 4 ? wide : narrow[plan.cluster], dim3((unsigned)ctas), SP_THREADS,
-                               ring + SP_EXTRA, stream, (unsigned)plan.cluster, ma, mb, g, sp);
+                               ring + SP_EXTRA, stream, (unsigned)plan.cluster, ma, mb, mb2, g, sp);
   }
   const int64_t pair_tiles = (int64_t)((M + PR_BM - 1) / PR_BM) * ((N + BN - 1) / BN);
   if (use_pair(g.tiles_m, tiles, pair_tiles, (K + BK - 1) / BK, sms)) {
     g.tiles_m = (M + PR_BM - 1) / PR_BM;
     g.tiles = (int)pair_tiles;
     return fc_launch_dependent(k_gemm_pair<EPI>, dim3((unsigned)(2 * std::min(g.tiles, sms / 2))), GM_THREADS, PR_SMEM,
-                               stream, 0, ma, mb, g);
+                               stream, 0, ma, mb, mb2, g);
   }
   const int grid = (int)std::min<int64_t>(tiles, sms);
-  return fc_launch_dependent(k_gemm<EPI>, dim3((unsigned)grid), GM_THREADS, SMEM_BYTES, stream, 0, ma, mb, g);
+  return fc_launch_dependent(k_gemm<EPI>, dim3((unsigned)grid), GM_THREADS, SMEM_BYTES, stream, 0, ma, mb, mb2, g);
 }
 
 // gate/up weights [K][2 * inter] (gate columns, then up columns) -> 128-column
@@ -923,6 +980,34 @@ extern "C" fc_status fc_gemm_kv_heads(const void* d_a, const void* d_wkv, int M,
   g.hkv = Hkv;
   g.rope = fc_rope64(rope_base);
   return launch_gemm<EPI_KV_HEADS>(d_a, d_wkv, M, 2 * Hkv * 128, K, g, static_cast<cudaStream_t>(stream));
+}
+
+extern "C" fc_status fc_gemm_qkv(const void* d_a, const void* d_wq, const void* d_wkv, int M, int K, int H, int Hkv, int D,
+                                 int batch, int n_pad, const int32_t* d_pos, float rope_base, void* d_q, void* d_k_rot,
+                                 void* d_v_heads, fc_stream stream) {
+  FC_NVTX_RANGE();
+  if (M < 0 || K < 1 || H < 1 || Hkv < 1 || batch < 0 || n_pad < 1 || M != batch * n_pad) return FC_ERR_INVALID_ARG;
+  if (D != 128 || K % 8) return FC_ERR_UNSUPPORTED;
+  if (!(rope_base > 0.f) || !std::isfinite(rope_base)) return FC_ERR_INVALID_ARG;
+  if (M == 0) return FC_OK;
+  if (!d_a || !d_wq || !d_wkv || !d_pos || !d_q || !d_k_rot || !d_v_heads) return FC_ERR_INVALID_ARG;
+  if (!aligned16(d_a) || !aligned16(d_wq) || !aligned16(d_wkv) || !aligned16(d_q) || !aligned16(d_k_rot) ||
+      !aligned16(d_v_heads))
+    return FC_ERR_INVALID_ARG;
+  if (H % 2) {  // a 256-column tile would hold columns of both
+    const fc_status st = fc_gemm_bf16(d_a, d_wq, d_q, M, H * D, K, nullptr, 0, stream);
+    return st != FC_OK ? st : fc_gemm_kv_heads(d_a, d_wkv, M, K, Hkv, D, batch, n_pad, d_pos, rope_base, d_k_rot, d_v_heads, stream);
+  }
+  GemmArgs g{};
+  g.c = static_cast<__nv_bfloat16*>(d_q);
+  g.n_q = H * D;
+  g.k_out = static_cast<__nv_bfloat16*>(d_k_rot);
+  g.v_out = static_cast<__nv_bfloat16*>(d_v_heads);
+  g.pos = d_pos;
+  g.n_pad = n_pad;
+  g.hkv = Hkv;
+  g.rope = fc_rope64(rope_base);
+  return launch_gemm<EPI_QKV>(d_a, d_wq, M, (H + 2 * Hkv) * D, K, g, static_cast<cudaStream_t>(stream), d_wkv);
 }
 
 extern "C" fc_status fc_gemm_silu_mul(const void* d_a, const void* d_wgu, int M, int K, int inter, void* d_act,

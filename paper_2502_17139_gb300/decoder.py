@@ -4,8 +4,8 @@ tree ancestors at position kv_len + depth), for a LLaMA-family decoder like
 the paper's models, composed from the C-ABI calls (argument marshalling
 only; every step runs in the library's kernels).
 
-Per layer: add + RMSNorm -> Q projection -> the K/V projection, whose GEMM
-epilogue rotates the key heads and writes both head-major (fc_gemm_kv_heads)
+Per layer: add + RMSNorm -> the Q and K/V projections, whose GEMM epilogue
+rotates the key heads and writes keys and values head-major (fc_gemm_qkv)
 -> tree attention with the queries rotated inside the kernel
 (fc_tree_attn_rope) over the layer's rotated cache -> output projection ->
 add + RMSNorm -> the gate/up projection, whose GEMM epilogue applies SiLU *
@@ -78,8 +78,8 @@ class TreeDecoder:
         r = None
         for l, Lw in enumerate(W["layers"]):
             fc.fc_add_rmsnorm(self.x, r, Lw["attn_norm"], self.h, s.eps)
-            fc.fc_gemm_bf16(self.h, Lw["wq"], out=self.q)
-            fc.fc_gemm_kv_heads(self.h, Lw["wkv"], B, n_pad, s.Hkv, pos, s.rope_base, self.k_rot[l], self.v_heads[l])
+            fc.fc_gemm_qkv(self.h, Lw["wq"], Lw["wkv"], B, n_pad, s.Hkv, pos, s.rope_base, self.q, self.k_rot[l],
+                           self.v_heads[l])
             ev = None
             if events is not None and "attn" in events:
                 ev = (torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))

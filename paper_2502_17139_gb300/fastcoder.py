@@ -77,7 +77,7 @@ EXPORTS = ["fc_status_string", "fc_version", "fc_get_error", "fc_datastore_build
            "fc_datastore_build_noalloc", "fc_datastore_keys", "fc_datastore_save", "fc_datastore_file_info", "fc_datastore_load",
            "fc_retrieve", "fc_retrieve_all", "fc_retrieve_rev", "fc_reverse_tokens", "fc_rcache_bytes", "fc_rcache_init", "fc_rcache_lookup", "fc_rcache_insert", "fc_retrieve_cached",
            "fc_cache_init", "fc_cache_search", "fc_cache_update", "fc_missing_bytes", "fc_missing_init",
-           "fc_missing_insert", "fc_build_tree", "fc_build_tree_all_workspace", "fc_build_tree_all", "fc_tree_mask", "fc_tree_attn", "fc_tree_attn_workspace", "fc_tree_attn_parts", "fc_tree_attn_streamed", "fc_rope", "fc_tree_attn_rope", "fc_gemm_workspace", "fc_gemm_bf16", "fc_gemm_kv_heads", "fc_gemm_silu_mul", "fc_interleave_gate_up", "fc_embed",
+           "fc_missing_insert", "fc_build_tree", "fc_build_tree_all_workspace", "fc_build_tree_all", "fc_tree_mask", "fc_tree_attn", "fc_tree_attn_workspace", "fc_tree_attn_parts", "fc_tree_attn_streamed", "fc_rope", "fc_tree_attn_rope", "fc_gemm_workspace", "fc_gemm_bf16", "fc_gemm_kv_heads", "fc_gemm_qkv", "fc_gemm_silu_mul", "fc_interleave_gate_up", "fc_embed",
            "fc_add_rmsnorm", "fc_silu_mul", "fc_rope_heads", "fc_selftest_wait", "fc_accept", "fc_argmax_accept", "fc_kv_append", "fc_synth_argmax",
            "fc_pipeline_create", "fc_pipeline_step", "fc_pipeline_step_part", "fc_pipeline_join_part", "fc_pipeline_stream", "fc_pipeline_error", "fc_pipeline_join",
            "fc_pipeline_capture_part", "fc_pipeline_graph_launch", "fc_pipeline_graph_kernels", "fc_pipeline_graph_destroy",
@@ -138,6 +138,7 @@ def _load():
         "fc_selftest_wait": (C.c_int, [i32, C.c_ulonglong, vp]),
         "fc_gemm_bf16": (C.c_int, [vp, vp, vp, i32, i32, i32, vp, sz, vp]),
         "fc_gemm_kv_heads": (C.c_int, [vp, vp, i32, i32, i32, i32, i32, i32, vp, C.c_float, vp, vp, vp]),
+        "fc_gemm_qkv": (C.c_int, [vp, vp, vp, i32, i32, i32, i32, i32, i32, i32, vp, C.c_float, vp, vp, vp, vp]),
         "fc_gemm_silu_mul": (C.c_int, [vp, vp, i32, i32, i32, vp, vp]),
         "fc_interleave_gate_up": (C.c_int, [vp, vp, i32, i32, vp]),
         "fc_embed": (C.c_int, [vp, i32, vp, i32, i32, vp, vp]),
@@ -742,6 +743,24 @@ def fc_gemm_kv_heads(a, wkv, batch, n_pad, Hkv, pos, rope_base, k_rot, v_heads):
         _need(t, torch.bfloat16, name, (batch, Hkv, n_pad, D))
     _check("fc_gemm_kv_heads", LIB.fc_gemm_kv_heads(_ptr(a), _ptr(wkv), M, K, Hkv, D, batch, n_pad, _ptr(pos),
                                                     C.c_float(rope_base), _ptr(k_rot), _ptr(v_heads), _stream()))
+
+
+def fc_gemm_qkv(a, wq, wkv, batch, n_pad, Hkv, pos, rope_base, q, k_rot, v_heads):
+    """q [batch * n_pad, H * 128] = a @ wq, and fc_gemm_kv_heads, in one launch."""
+    _need(a, torch.bfloat16, "a")
+    _need(wq, torch.bfloat16, "wq")
+    _need(wkv, torch.bfloat16, "wkv")
+    _need(pos, torch.int32, "pos", (batch, n_pad))
+    M, K = a.shape
+    D = 128
+    H = wq.shape[1] // D
+    if tuple(wq.shape) != (K, H * D) or tuple(wkv.shape) != (K, 2 * Hkv * D):
+        raise ValueError("wq must be [K, H * 128] and wkv [K, 2 * Hkv * 128]")
+    _need(q, torch.bfloat16, "q", (M, H * D))
+    for t, name in ((k_rot, "k_rot"), (v_heads, "v_heads")):
+        _need(t, torch.bfloat16, name, (batch, Hkv, n_pad, D))
+    _check("fc_gemm_qkv", LIB.fc_gemm_qkv(_ptr(a), _ptr(wq), _ptr(wkv), M, K, H, Hkv, D, batch, n_pad, _ptr(pos),
+                                          C.c_float(rope_base), _ptr(q), _ptr(k_rot), _ptr(v_heads), _stream()))
 
 
 def fc_interleave_gate_up(wgu, out=None):

@@ -174,8 +174,10 @@ def test_gemm_silu_mul(fc, M, K, inter):
 @pytest.mark.parametrize("M,N,K", [
     (1, 8, 512), (64, 136, 1032), (64, 2048, 5504), (64, 2432, 4104),        # clusters of 2, 4 and 8; ragged N and K
     (65, 2048, 2048), (128, 4096, 1024), (200, 1000, 1016), (300, 2048, 520),  # two and three row tiles
-    (64, 4864, 1024), (64, 4872, 1024),                                       # the last tile count of clusters of 4, the first of 2
+    (64, 4864, 1024), (64, 4872, 1024), (64, 4608, 1024), (64, 4616, 1024),   # about the last tile count of clusters of 4
+    (64, 5760, 776), (65, 5768, 776), (64, 8320, 3080), (64, 8328, 3080),     # of 3, and of 4 with two CTAs per SM
     (64, 9728, 520), (64, 9736, 1000), (70, 12800, 776), (3, 12808, 1024),    # clusters of 3 on wide tiles, and past them
+    (70, 11520, 776), (70, 11528, 776),
 ])
 def test_gemm_split_shapes(fc, M, N, K):
     """Few tiles: K cut over the CTAs of a cluster, partial tiles summed in CTA
@@ -222,3 +224,26 @@ def test_gemm_pair_silu_mul(fc, M, K, inter):
 @pytest.mark.parametrize("batch,n_pad,Hkv,K", [(5, 128, 33, 200), (9, 64, 5, 3080)])
 def test_gemm_pair_kv_heads(fc, orc, batch, n_pad, Hkv, K):
     test_gemm_kv_heads(fc, orc, batch, n_pad, Hkv, K)
+
+
+@pytest.mark.parametrize("batch,n_pad,H,Hkv,K", [
+    (1, 64, 2, 1, 4104), (1, 64, 4, 2, 1032), (1, 64, 16, 16, 2048), (3, 40, 2, 3, 520),  # clusters of 8, 4, 3 and 2
+    (5, 64, 2, 3, 256), (2, 128, 32, 8, 4096), (5, 128, 34, 33, 200),                     # whole tiles, single and paired
+    (1, 64, 3, 1, 520),                                                                   # an odd H: two launches
+])
+def test_gemm_qkv(fc, orc, batch, n_pad, H, Hkv, K):
+    """The query projection beside the K/V projection: both within the bounds
+    of the separate calls."""
+    class OneLaunch:
+        fc_get_error = staticmethod(fc.fc_get_error)
+
+        @staticmethod
+        def fc_gemm_kv_heads(a, w, batch, n_pad, Hkv, pos, base, k_rot, v_heads):
+            wq = operands(1, H * 128, K, K + H)[1]
+            q = torch.full((a.shape[0] + 1, H * 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+            fc.fc_gemm_qkv(a, wq, w, batch, n_pad, Hkv, pos, base, q[:-1], k_rot, v_heads)
+            torch.cuda.synchronize()
+            bound_check(a, wq, q[:-1])
+            assert torch.isnan(q[-1]).all()
+
+    test_gemm_kv_heads(OneLaunch, orc, batch, n_pad, Hkv, K)

@@ -22,8 +22,8 @@
 //
 // Bound by HBM: the radix passes stream 32 bytes a position each, the rounds
 // gather the text of the suffixes still in play.  Doubling from the start sorts
-// all positions in every round: 100M tokens 114 ms against 13.3 ms
-// (with the suffix keys); 1M tokens 1.94 against 0.63 ms.
+// all positions in every round: 100M tokens 114 ms against 11.4 ms
+// (with the suffix keys); 1M tokens 1.94 against 0.47 ms.
 
 #include <algorithm>
 
@@ -123,21 +123,33 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const uint64_t* __res
   key = fc_after_wait(key);
   h[threadIdx.x] = 0;
   __syncthreads();
-  uint64_t base = blockIdx.x * (uint64_t)RS_TILE;
+  const uint64_t base = blockIdx.x * (uint64_t)RS_TILE + threadIdx.x;
   bool bad = false;
-#pragma unroll 4
-  for (int k = 0; k < RS_ITEMS; ++k) {
-    uint64_t idx = base + (uint64_t)k * RS_THREADS + threadIdx.x;
-    if (idx < n) {
-      uint64_t x;
+  if (FIRST && tx.y.bits < 8) {  // the digit holds several symbols
+    for (int k = 0; k < RS_ITEMS; ++k) {
+      const uint64_t idx = base + (uint64_t)k * RS_THREADS;
+      if (idx >= n) break;
+      bad |= __ldg(tx.T + idx) >= vocab;
+      atomicAdd(&h[(uint32_t)(pack_key(tx.T, n, idx, tx.y.bits, tx.y.count) >> shift) & 255u], 1u);
+    }
+  } else {  // every load in flight at once (100M keys 196 us a pass in groups of four loads)
+    uint32_t d[RS_ITEMS];  // the digit (FIRST: of the key's last symbol), 256 past the end
+#pragma unroll
+    for (int k = 0; k < RS_ITEMS; ++k) {
+      const uint64_t idx = base + (uint64_t)k * RS_THREADS;
+      d[k] = 256u;
+      if (idx >= n) continue;
       if constexpr (FIRST) {
-        x = pack_key(tx.T, n, idx, tx.y.bits, tx.y.count);
+        const uint64_t last = idx + (uint64_t)tx.y.count - 1;
+        d[k] = last < n ? (__ldg(tx.T + last) + 1u) & 255u : 0u;
         bad |= __ldg(tx.T + idx) >= vocab;
       } else {
-        x = key[idx];
+        d[k] = (uint32_t)(key[idx] >> shift) & 255u;
       }
-      atomicAdd(&h[(uint32_t)(x >> shift) & 255u], 1u);
     }
+#pragma unroll
+    for (int k = 0; k < RS_ITEMS; ++k)
+      if (d[k] < 256u) atomicAdd(&h[d[k]], 1u);
   }
   if (FIRST && bad) atomicOr(ctl, 1u);
   __syncthreads();
@@ -182,17 +194,22 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_radix_scatter(const uint64_t*
   uint64_t key[RS_ITEMS];
   if constexpr (FIRST) {  // the tile's symbols (0 past the end) and the seven after it, staged
     const int bits = tx.y.bits;
-    const bool pairs = tx.y.count == 4 && bits <= 16;  // staged as pairs of neighbours: two make a key
-    for (int i = tid; i < RS_TILE + 8; i += RS_THREADS) {
-      const uint32_t a = b0 + i < n ? __ldg(tx.T + b0 + i) + 1u : 0u;
-      const uint32_t b = pairs && b0 + i + 1 < n ? __ldg(tx.T + b0 + i + 1) + 1u : 0u;
-      sval[i] = pairs ? (a << bits) | b : a;
+    uint32_t sym[RS_ITEMS + 1];  // every load in flight at once (100M tokens: 1.24 ms one after the other, 0.79 now)
+#pragma unroll
+    for (int q = 0; q < RS_ITEMS + 1; ++q) {
+      const int i = tid + q * RS_THREADS;
+      sym[q] = i < RS_TILE + 8 && b0 + i < n ? __ldg(tx.T + b0 + i) + 1u : 0u;
     }
+#pragma unroll
+    for (int q = 0; q < RS_ITEMS + 1; ++q)
+      if (tid + q * RS_THREADS < RS_TILE + 8) sval[tid + q * RS_THREADS] = sym[q];
     __syncthreads();
     const uint32_t* sy = sval + warp * RS_WARP_CHUNK + lane;
-    if (pairs) {
+    if (tx.y.count == 4 && bits <= 16) {
 #pragma unroll
-      for (int it = 0; it < RS_ITEMS; ++it) key[it] = ((uint64_t)sy[32 * it] << (2 * bits)) | sy[32 * it + 2];
+      for (int it = 0; it < RS_ITEMS; ++it)
+        key[it] = ((uint64_t)((sy[32 * it] << bits) | sy[32 * it + 1]) << (2 * bits)) |
+                  ((sy[32 * it + 2] << bits) | sy[32 * it + 3]);
     } else {
 #pragma unroll
       for (int it = 0; it < RS_ITEMS; ++it) {
@@ -277,6 +294,95 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_radix_scatter(const uint64_t*
   for (int k = 0; k < RS_ITEMS; ++k) {
     const uint32_t j = tid + k * RS_THREADS;
     if (j < count) vout[pos[k]] = sval[j];
+  }
+}
+
+// All passes over up to RO_MAX pairs in one CTA, the pairs in registers and put
+// in order through shared memory: the digits [shift, bits) in steps of eight.
+// A pass over a few tiles is three launches that wait for each other (10 us for
+// 5000 pairs, six here: a build of 1M tokens 497 -> 468 us).
+constexpr int RO_THREADS = 512, RO_WARPS = RO_THREADS / 32, RO_MAX = RO_THREADS * RS_ITEMS;
+constexpr uint32_t RO_SMEM = RO_MAX * (8 + 4) + RO_WARPS * 256 * 4;
+__global__ void __launch_bounds__(RO_THREADS) k_radix_one(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout,
+                                                          int m, int shift, int bits) {
+  extern __shared__ __align__(16) unsigned char ro_smem[];
+  uint64_t* skey = reinterpret_cast<uint64_t*>(ro_smem);
+  uint32_t* sval = reinterpret_cast<uint32_t*>(ro_smem + RO_MAX * 8);
+  uint32_t* wbin = sval + RO_MAX;  // [warp][256]
+  __shared__ uint32_t wsum[8];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int first_item = warp * RS_WARP_CHUNK + lane, left = m - first_item;  // this lane's pairs: every 32
+  const uint32_t lt = (1u << lane) - 1u;
+  fc_grid_wait();
+  uint64_t key[RS_ITEMS];
+  uint32_t val[RS_ITEMS], at[RS_ITEMS / 2];
+#pragma unroll
+  for (int it = 0; it < RS_ITEMS; ++it) {
+    key[it] = 32 * it < left ? kin[first_item + 32 * it] : 0ull;
+    val[it] = 32 * it < left ? vin[first_item + 32 * it] : 0u;
+  }
+  for (; shift < bits; shift += 8) {
+    for (int d = tid; d < RO_WARPS * 256; d += RO_THREADS) wbin[d] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < RS_ITEMS; ++it) {
+      if (32 * it >= m - warp * RS_WARP_CHUNK) break;  // (the warp has no more)
+      const bool ok = 32 * it < left;
+      const uint32_t d = ok ? ((uint32_t)(key[it] >> shift) & 255u) : 256u;
+      const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+      uint32_t cnt = 0;
+      if (ok && (peers & lt) == 0) cnt = atomicAdd(&wbin[warp * 256 + d], (uint32_t)__popc(peers));
+      const uint32_t r = __shfl_sync(0xFFFFFFFFu, cnt, __ffs(peers) - 1) + __popc(peers & lt);
+      at[it / 2] = it & 1 ? at[it / 2] | (r << 16) : r;
+    }
+    __syncthreads();
+    uint32_t run = 0, inc = 0;  // threads 0 .. 255: a digit's pairs, and where each warp's start
+    if (tid < 256) {
+#pragma unroll
+      for (int w = 0; w < RO_WARPS; ++w) run += wbin[w * 256 + tid];
+      inc = run;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      if (lane == 31) wsum[warp] = inc;
+    }
+    __syncthreads();
+    if (tid < 256) {
+      uint32_t first = inc - run;
+      for (int w = 0; w < warp; ++w) first += wsum[w];
+#pragma unroll
+      for (int w = 0; w < RO_WARPS; ++w) {
+        const uint32_t c = wbin[w * 256 + tid];
+        wbin[w * 256 + tid] = first;
+        first += c;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < RS_ITEMS; ++it) {
+      if (32 * it < left) {
+        const uint32_t p = wbin[warp * 256 + ((uint32_t)(key[it] >> shift) & 255u)] + ((at[it / 2] >> (16 * (it & 1))) & 0xFFFFu);
+        skey[p] = key[it];
+        sval[p] = val[it];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < RS_ITEMS; ++it) {
+      if (32 * it < left) {
+        key[it] = skey[first_item + 32 * it];
+        val[it] = sval[first_item + 32 * it];
+      }
+    }
+  }
+#pragma unroll
+  for (int it = 0; it < RS_ITEMS; ++it) {
+    if (32 * it < left) {
+      kout[first_item + 32 * it] = key[it];
+      vout[first_item + 32 * it] = val[it];
+    }
   }
 }
 
@@ -584,8 +690,8 @@ __global__ void __launch_bounds__(SPL_THREADS) k_split(const uint64_t* __restric
 // sub-range's place), equal (they go on), and the largest smaller one (the LCP
 // at the new sub-range's start).  Several rounds run in the tile before what is
 // left goes back to a list: the next symbols lie beside the last ones, and a
-// launch and a list's way through memory are saved (1M tokens 628 -> 533 us a
-// build, 100M 13.3 -> 12.9 ms).  Where every tile has its own CTA there is
+// launch and a list's way through memory are saved (a build of 1M tokens
+// 628 -> 533 us, of 100M 13.3 -> 12.9 ms).  Where every tile has its own CTA there is
 // nothing to gain from packing: RFS_DEEP rounds.  Else `many`: one in the first
 // round, which leaves a quarter of its elements, then eight (an eighth goes
 // each round).
@@ -657,95 +763,139 @@ __global__ void __launch_bounds__(RFS_THREADS) k_refine_small(const uint32_t* __
   }
 }
 
-// One round over the ranges of 33 to 4096 suffixes: a CTA sorts a range's
-// (next symbols, position) pairs in shared memory (bitonic) and splits it.
-constexpr int RFM_THREADS = 512;
-constexpr uint32_t RFM_SMEM = MID_MAX * (8 + 4);
+// One round over the ranges of 33 to 4096 suffixes: a group of threads sorts a
+// range's (next symbols, position) pairs in shared memory (bitonic) and splits
+// it.  Bound by the latency of the sort's steps, so by how many ranges an SM has
+// in work: 64 threads take a range of up to 512, the whole CTA a longer one
+// (100M tokens: 1097 us a round with a CTA for each, 605 now).
+constexpr int RFM_THREADS = 512, RFM_GROUP = 64, RFM_GROUPS = RFM_THREADS / RFM_GROUP;
+constexpr uint32_t RFM_GROUP_MAX = MID_MAX / RFM_GROUPS, RFM_SMEM = MID_MAX * (8 + 4);
+struct MidShared {  // one range's: key and position arrays for its size, heads, and a few words
+  uint64_t* key;
+  uint32_t *pos, *head, *wsum, *base;
+};
+template <int NT>
+__device__ __forceinline__ void mid_sync(int bar) {
+  asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(NT) : "memory");
+}
+// One range by NT threads (tid: within them), whose barrier is `bar`.
+template <int NT>
+__device__ __forceinline__ void mid_range(const Range g, const MidShared sh, int tid, int bar, const uint32_t* __restrict__ T,
+                                          uint64_t n, Sym y, uint32_t* sa, uint8_t* __restrict__ lcp, Range* next, Elem* small,
+                                          Counts* ct, int out) {
+  const int lane = tid & 31, warp = tid >> 5;
+  uint32_t p2 = 64;
+  while (p2 < g.size) p2 *= 2;
+  for (uint32_t i = tid; i < p2; i += NT) {
+    uint32_t pos = 0xFFFFFFFFu;  // padding sorts behind every suffix
+    uint64_t k = ~0ull;
+    if (i < g.size) {
+      pos = sa[g.start + i];
+      k = pack_key(T, n, (uint64_t)pos + g.depth, y.bits, y.count);
+    }
+    sh.key[i] = k;
+    sh.pos[i] = pos;
+  }
+  mid_sync<NT>(bar);
+  for (uint32_t len = 2; len <= p2; len *= 2)
+    for (uint32_t st = len / 2; st > 0; st /= 2) {
+      for (uint32_t i = tid; i < p2 / 2; i += NT) {
+        const uint32_t a = 2 * i - (i & (st - 1)), b = a + st;
+        const uint64_t ka = sh.key[a], kb = sh.key[b];
+        const uint32_t pa = sh.pos[a], pb = sh.pos[b];
+        const bool up = (a & len) == 0, gt = ka > kb || (ka == kb && pa > pb);
+        if (gt == up) {
+          sh.key[a] = kb, sh.key[b] = ka;
+          sh.pos[a] = pb, sh.pos[b] = pa;
+        }
+      }
+      // a step of up to 32 stays in its warp's 64 elements
+      if (st >= 64 || (st == 1 && len >= 64)) mid_sync<NT>(bar);  // (the next step's is st / 2, or len)
+      else __syncwarp();
+    }
+  const uint32_t words = (g.size + 31) / 32 + 1;
+  for (uint32_t i = tid; i < words * 32; i += NT) {
+    const bool head = i >= g.size || i == 0 || sh.key[i] != sh.key[i - 1];
+    const uint32_t w = __ballot_sync(0xFFFFFFFFu, head);  // whole warps: words * 32 elements
+    if (lane == 0) sh.head[i >> 5] = w;
+  }
+  mid_sync<NT>(bar);
+  // a thread takes consecutive elements, so that its small ones stay in order
+  const uint32_t per = (g.size + NT - 1) / NT, i0 = min(g.size, tid * per), i1 = min(g.size, i0 + per);
+  auto range_of = [&](uint32_t i, uint32_t& hd, uint32_t& nx) {  // the bounds of i's sub-range
+    uint32_t w = i >> 5, v = sh.head[w] & (0xFFFFFFFFu >> (31 - (i & 31)));
+    while (!v) v = sh.head[--w];  // element 0 is a head
+    hd = w * 32 + 31 - __clz(v);
+    w = (i + 1) >> 5, v = sh.head[w] & (0xFFFFFFFFu << ((i + 1) & 31));
+    while (!v) v = sh.head[++w];  // the word past the last element is all heads
+    nx = min(g.size, w * 32 + __ffs(v) - 1);
+  };
+  uint32_t n_out = 0;
+  for (uint32_t i = i0; i < i1; ++i) {
+    sa[g.start + i] = sh.pos[i];
+    uint32_t hd, nx;
+    range_of(i, hd, nx);
+    const uint32_t size = nx - hd;
+    if (i == hd && i > 0) lcp[g.start + i] = cap_lcp(g.depth + common_syms(sh.key[i], sh.key[i - 1], y));
+    if (size > SMALL_MAX) {
+      if (i == hd) next[atomicAdd(&ct->mid[out], 1u)] = Range{g.start + hd, size, g.depth + (uint32_t)y.count};
+    } else if (size > 1) {
+      ++n_out;
+    }
+  }
+  uint32_t inc = n_out;  // the small ones before this thread's
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  if (lane == 31) sh.wsum[warp] = inc;
+  mid_sync<NT>(bar);
+  uint32_t at = inc - n_out, total = 0;
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) {
+    const uint32_t v = sh.wsum[w];
+    at += w < warp ? v : 0u;
+    total += v;
+  }
+  if (tid == 0 && total) *sh.base = atomicAdd(&ct->small[out], total);
+  mid_sync<NT>(bar);
+  at += *sh.base;
+  if (n_out)
+    for (uint32_t i = i0; i < i1; ++i) {
+      uint32_t hd, nx;
+      range_of(i, hd, nx);
+      if (nx - hd > 1 && nx - hd <= SMALL_MAX)
+        small[at++] = make_uint2(g.start + i, ((g.depth + (uint32_t)y.count) << 8) | (i - hd));
+    }
+  mid_sync<NT>(bar);
+}
 __global__ void __launch_bounds__(RFM_THREADS) k_refine_mid(const uint32_t* __restrict__ T, uint64_t n, Sym y, uint32_t* sa,
                                                             uint8_t* __restrict__ lcp, const Range* ranges, Range* next,
                                                             Elem* small, Counts* ct, int in, int out) {
   extern __shared__ __align__(16) unsigned char rfm_smem[];
-  uint64_t* s_key = reinterpret_cast<uint64_t*>(rfm_smem);
-  uint32_t* s_pos = reinterpret_cast<uint32_t*>(rfm_smem + MID_MAX * 8);
-  __shared__ uint32_t s_head[MID_MAX / 32 + 2], wsum[32], s_total, s_base;
-  const int tid = threadIdx.x, lane = tid & 31;
+  __shared__ uint32_t s_head[MID_MAX / 32 + 2 * RFM_GROUPS], s_wsum[RFM_THREADS / 32], s_base[RFM_GROUPS];
+  const int tid = threadIdx.x, lane = tid & 31, grp = tid / RFM_GROUP;
   fc_grid_wait();
   const uint32_t ng = *(volatile uint32_t*)&ct->mid[in];
   if (blockIdx.x == 0 && tid == 0) ct->small[3 - in - out] = ct->mid[3 - in - out] = 0u;  // the round after next's
-  for (uint32_t gi = blockIdx.x; gi < ng; gi += gridDim.x) {
+  uint64_t* key = reinterpret_cast<uint64_t*>(rfm_smem);
+  uint32_t* pos = reinterpret_cast<uint32_t*>(rfm_smem + MID_MAX * 8);
+  const MidShared part{key + grp * RFM_GROUP_MAX, pos + grp * RFM_GROUP_MAX, s_head + grp * (RFM_GROUP_MAX / 32 + 2),
+                       s_wsum + grp * (RFM_GROUP / 32), s_base + grp};
+  for (uint32_t gi = blockIdx.x * RFM_GROUPS + grp; gi < ng; gi += gridDim.x * RFM_GROUPS) {
     const Range g = ranges[gi];
-    uint32_t p2 = 64;
-    while (p2 < g.size) p2 *= 2;
-    for (uint32_t i = tid; i < p2; i += RFM_THREADS) {
-      uint32_t pos = 0xFFFFFFFFu;  // padding sorts behind every suffix
-      uint64_t k = ~0ull;
-      if (i < g.size) {
-        pos = sa[g.start + i];
-        k = pack_key(T, n, (uint64_t)pos + g.depth, y.bits, y.count);
-      }
-      s_key[i] = k;
-      s_pos[i] = pos;
-    }
-    __syncthreads();
-    for (uint32_t len = 2; len <= p2; len *= 2)
-      for (uint32_t st = len / 2; st > 0; st /= 2) {
-        for (uint32_t i = tid; i < p2 / 2; i += RFM_THREADS) {
-          const uint32_t a = 2 * i - (i & (st - 1)), b = a + st;
-          const uint64_t ka = s_key[a], kb = s_key[b];
-          const uint32_t pa = s_pos[a], pb = s_pos[b];
-          const bool up = (a & len) == 0, gt = ka > kb || (ka == kb && pa > pb);
-          if (gt == up) {
-            s_key[a] = kb, s_key[b] = ka;
-            s_pos[a] = pb, s_pos[b] = pa;
-          }
-        }
-        // a step of up to 32 stays in its warp's 64 elements
-        if (st >= 64 || (st == 1 && len >= 64)) __syncthreads();  // (the next step's is st / 2, or len)
-        else __syncwarp();
-      }
-    const uint32_t words = (g.size + 31) / 32 + 1;
-    for (uint32_t i = tid; i < words * 32; i += RFM_THREADS) {
-      const bool head = i >= g.size || i == 0 || s_key[i] != s_key[i - 1];
-      const uint32_t w = __ballot_sync(0xFFFFFFFFu, head);  // whole warps: words * 32 elements
-      if (lane == 0) s_head[i >> 5] = w;
-    }
-    __syncthreads();
-    // a thread takes consecutive elements, so that its small ones stay in order
-    const uint32_t per = (g.size + RFM_THREADS - 1) / RFM_THREADS, i0 = min(g.size, tid * per), i1 = min(g.size, i0 + per);
-    auto range_of = [&](uint32_t i, uint32_t& hd, uint32_t& nx) {  // the bounds of i's sub-range
-      uint32_t w = i >> 5, v = s_head[w] & (0xFFFFFFFFu >> (31 - (i & 31)));
-      while (!v) v = s_head[--w];  // element 0 is a head
-      hd = w * 32 + 31 - __clz(v);
-      w = (i + 1) >> 5, v = s_head[w] & (0xFFFFFFFFu << ((i + 1) & 31));
-      while (!v) v = s_head[++w];  // the word past the last element is all heads
-      nx = min(g.size, w * 32 + __ffs(v) - 1);
-    };
-    uint32_t n_out = 0;
-    for (uint32_t i = i0; i < i1; ++i) {
-      sa[g.start + i] = s_pos[i];
-      uint32_t hd, nx;
-      range_of(i, hd, nx);
-      const uint32_t size = nx - hd;
-      if (i == hd && i > 0)
-        lcp[g.start + i] = cap_lcp(g.depth + common_syms(s_key[i], s_key[i - 1], y));
-      if (size > SMALL_MAX) {
-        if (i == hd) next[atomicAdd(&ct->mid[out], 1u)] = Range{g.start + hd, size, g.depth + (uint32_t)y.count};
-      } else if (size > 1) {
-        ++n_out;
-      }
-    }
-    uint32_t at = block_sum_scan(n_out, wsum, &s_total);
-    if (tid == 0 && s_total) s_base = atomicAdd(&ct->small[out], s_total);
-    __syncthreads();
-    at += s_base;
-    if (n_out)
-      for (uint32_t i = i0; i < i1; ++i) {
-        uint32_t hd, nx;
-        range_of(i, hd, nx);
-        if (nx - hd > 1 && nx - hd <= SMALL_MAX)
-          small[at++] = make_uint2(g.start + i, ((g.depth + (uint32_t)y.count) << 8) | (i - hd));
-      }
-    __syncthreads();
+    if (g.size <= RFM_GROUP_MAX)
+      mid_range<RFM_GROUP>(g, part, tid % RFM_GROUP, 1 + grp, T, n, y, sa, lcp, next, small, ct, out);
+  }
+  __syncthreads();
+  const MidShared all{key, pos, s_head, s_wsum, s_base};
+  for (uint32_t g0 = blockIdx.x; g0 < ng; g0 += gridDim.x * 32) {  // 32 of this CTA's ranges at a time
+    const uint32_t mine = g0 + lane * gridDim.x;
+    uint32_t longer = __ballot_sync(0xFFFFFFFFu, mine < ng && ranges[mine].size > RFM_GROUP_MAX);
+    for (; longer; longer &= longer - 1)
+      mid_range<RFM_THREADS>(ranges[g0 + (__ffs(longer) - 1) * gridDim.x], all, tid, 1 + RFM_GROUPS, T, n, y, sa, lcp, next,
+                             small, ct, out);
   }
 }
 
@@ -870,6 +1020,11 @@ extern "C" fc_status fc_datastore_build(const uint32_t* d_tokens, uint64_t n, ui
   };
   // The passes from digit `d` on over the low `bits` bits, from one pair of buffers to the other.
   auto passes = [&](uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, uint64_t m, int d, int bits) {
+    if (m <= (uint64_t)RO_MAX && 8 * d < bits) {
+      const bool odd = ((bits - 8 * d + 7) / 8) % 2 != 0;
+      return fc_launch_dependent(k_radix_one, dim3(1), RO_THREADS, RO_SMEM, s, 0, k0, v0, odd ? k1 : k0, odd ? v1 : v0, (int)m,
+                                 8 * d, bits) == FC_OK;
+    }
     for (; 8 * d < bits; ++d) {
       if (!pass(k0, v0, k1, v1, m, 8 * d)) return false;
       std::swap(k0, k1);
@@ -878,7 +1033,8 @@ extern "C" fc_status fc_datastore_build(const uint32_t* d_tokens, uint64_t n, ui
     return true;
   };
 
-  if (cudaFuncSetAttribute(k_refine_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RFM_SMEM) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_refine_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RFM_SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(k_radix_one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RO_SMEM) != cudaSuccess)
     return FC_ERR_CUDA;
   if (cudaMemsetAsync(ctl, 0, 64, s) != cudaSuccess) return FC_ERR_CUDA;
 
@@ -963,7 +1119,7 @@ extern "C" fc_status fc_datastore_build(const uint32_t* d_tokens, uint64_t n, ui
     }
     const int o = (round + 1) % 3, li = round & 1;
     const int many = round == 0 ? 1 : 8;
-    const unsigned gs = (unsigned)std::min<uint64_t>(cdiv(n, RFS_HEADS), 8ull * sms), gm = 3u * sms;
+    const unsigned gs = (unsigned)std::min<uint64_t>(cdiv(n, RFS_HEADS), 8ull * sms), gm = 4u * sms;
     if (fc_launch_dependent(k_refine_small, dim3(gs), RFS_THREADS, 0, s, 0, d_tokens, n, y, d_sa, d_lcp, lists[li],
                             lists[li ^ 1], ct, in, o, many) != FC_OK ||
         fc_launch_dependent(k_refine_mid, dim3(gm), RFM_THREADS, RFM_SMEM, s, 0, d_tokens, n, y, d_sa, d_lcp, mids[li],

@@ -76,6 +76,11 @@ def _sa_corpus(kind):
     if kind == "tile_edges":  # runs of 31 to 33 and of 4095 to 4097 equal keys around the tiles of 2048
         runs = [31, 32, 33, 1, 2, 2016, 32, 33, 64, 4095, 4096, 4097, 31]
         return np.concatenate([np.concatenate([np.full(r, 5, np.uint32), [100 + i]]) for i, r in enumerate(runs)]).astype(np.uint32), 200
+    if kind == "group_edges":  # ranges of 63 to 65, 511 to 513 and 4096 suffixes
+        runs = [63, 64, 65, 511, 512, 513, 514, 515, 516, 4096, 4099]
+        return np.concatenate([np.concatenate([np.tile([7, 8, 9, 10, 11 + i], r), [100]]) for i, r in enumerate(runs)]).astype(np.uint32), 200
+    if kind.isdigit():  # about the most pairs that one CTA sorts
+        return z(int(kind), 3000), 3000
     if kind == "equal_pairs":  # many pairs, triples, ... of 40 equal tokens: several rounds, the LCP inside them
         grams = rng.integers(0, 30_000, (200, 40))
         return np.concatenate([np.concatenate([grams[i], rng.integers(0, 30_000, 3)]) for i in rng.integers(0, 200, 900)]).astype(np.uint32), 30_000
@@ -94,7 +99,7 @@ def _sa_corpus(kind):
 
 
 @pytest.mark.parametrize("kind", ["zipf", "sparse_vocab", "eight_bits", "tile_edges", "equal_pairs", "twice", "long_repeats",
-                                  "periodic", "one_token"])
+                                  "periodic", "one_token", "group_edges", "1", "33", "8191", "8192", "8193"])
 def test_sa_build_paths(fc, orc, kind):
     """Corpora whose ranges of equal keys take each path of the refinement."""
     T, vocab = _sa_corpus(kind)

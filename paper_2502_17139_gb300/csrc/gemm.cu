@@ -580,6 +580,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) __cluster_dims__(2, 1, 1)
 // ---------------------------------------------------------------------------
 constexpr int SP_THREADS = 192, SP_MAX_STAGES = 12;
 constexpr uint32_t SP_RING_1 = 208 * 1024, SP_RING_2 = 96 * 1024;  // one CTA per SM, or two; a partial tile is 32 NB KB
+static_assert(SP_RING_1 >= 4 * 32 * 1024 && SP_RING_2 >= 2 * 32 * 1024, "a partial tile lies in the ring");
 constexpr uint32_t SP_EXTRA = 256 + 1024;                       // barriers + alignment slack
 enum { SB_FULL = 0, SB_EMPTY = SP_MAX_STAGES, SB_ACC = 2 * SP_MAX_STAGES, SB_DRAIN, SB_COUNT };
 

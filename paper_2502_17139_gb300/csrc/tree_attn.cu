@@ -292,14 +292,55 @@ __device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a, int units) 
   return p;
 }
 
+// Launches of a few waves of units: the sequence at `place` when the batch is
+// ordered by the work of a row chunk, longest first, so that what runs last is
+// short (and what is split is shorter still).  Lengths live on the device:
+// a warp of each CTA ranks the batch, a sequence or two per lane.
+struct Seq {
+  int b, nn, kvl;  // the sequence, its n_nodes and kv_len as given
+};
+constexpr int ORDER_MAX = 64;  // sequences
+__device__ __forceinline__ Seq work_order(const AttnArgs& a, int place) {
+  const int lane = threadIdx.x & 31;
+  int nn[2], kvl[2], rank[2] = {0, 0};
+  uint32_t key[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int b = lane + 32 * h;
+    nn[h] = b < a.B ? a.n_nodes[b] : 0;
+    kvl[h] = b < a.B ? a.kv_len[b] : 0;
+    const bool none = nn[h] < 1 || nn[h] > a.n_pad || kvl[h] < 0 || kvl[h] > a.kv_cap;
+    const uint32_t cost = none ? 0u : (uint32_t)((kvl[h] + BN - 1) / BN + 1) * (a.G * nn[h] > BM ? 4u : 3u);
+    key[h] = (min(cost, (1u << 26) - 1) << 6) | (uint32_t)(ORDER_MAX - 1 - b);  // distinct
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (h && a.B <= 32) break;
+#pragma unroll
+    for (int l = 0; l < 32; ++l) {
+      const uint32_t k = __shfl_sync(0xFFFFFFFFu, key[h], l);
+      rank[0] += k > key[0];
+      rank[1] += k > key[1];
+    }
+  }
+  const unsigned lo = __ballot_sync(0xFFFFFFFFu, lane < a.B && rank[0] == place);
+  const unsigned hi = __ballot_sync(0xFFFFFFFFu, lane + 32 < a.B && rank[1] == place);
+  const int src = __ffs(lo ? lo : hi) - 1;
+  return {src + (lo ? 0 : 32), __shfl_sync(0xFFFFFFFFu, lo ? nn[0] : nn[1], src),
+          __shfl_sync(0xFFFFFFFFu, lo ? kvl[0] : kvl[1], src)};
+}
+
 // ROPE: the queries arrive unrotated and are rotated by a.pos while staged
 // (a separate instance, so the plain kernel's code is unchanged).
-// SPREAD: the CTA's unit and share of its keys come from spread_plan, and
+// MODE_SPREAD: the CTA's unit and share of its keys come from spread_plan, and
 // shared units' partial sums are merged by k_attn_merge, launched behind.
-template <bool ROPE, bool SPREAD>
+// MODE_ORDERED: the sequences run in work_order.
+enum { MODE_PLAIN = 0, MODE_SPREAD = 1, MODE_ORDERED = 2 };
+template <bool ROPE, int MODE>
 __global__ void __launch_bounds__(TA_THREADS, 1)
     k_tree_attn(const __grid_constant__ CUtensorMap tm_kc, const __grid_constant__ CUtensorMap tm_vc,
                 const __grid_constant__ CUtensorMap tm_kt, const __grid_constant__ CUtensorMap tm_vt, AttnArgs a) {
+  constexpr bool SPREAD = MODE == MODE_SPREAD;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
@@ -339,9 +380,26 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
     nparts = a.parts;
   }
   const int su = unit - a.u_split;  // index among the split units
-  const int bg = unit / a.ctas, c = unit - bg * a.ctas;
-  const int b = bg / a.Hkv, g = bg - b * a.Hkv;
-  const int nn_raw = a.n_nodes[b], kvl = a.kv_len[b];
+  int bg = unit / a.ctas;
+  const int c = unit - bg * a.ctas;
+  int b = bg / a.Hkv;
+  const int g = bg - b * a.Hkv;
+  int nn_raw, kvl;
+  if constexpr (MODE == MODE_ORDERED) {
+    __shared__ Seq s_seq;
+    if (warp == 0) {
+      const Seq seq = work_order(a, b);
+      if (lane == 0) s_seq = seq;
+    }
+    __syncthreads();
+    b = s_seq.b;
+    bg = b * a.Hkv + g;
+    nn_raw = s_seq.nn;
+    kvl = s_seq.kvl;
+  } else {
+    nn_raw = a.n_nodes[b];
+    kvl = a.kv_len[b];
+  }
   const bool bad = nn_raw < 1 || nn_raw > a.n_pad || kvl < 0 || kvl > a.kv_cap;
   const int nn = bad ? 0 : nn_raw;
   if (bad && c == 0 && part == 0 && tid == 0) fc_flag(FC_ERR_WORD(a.err), FC_EBIT_INVALID);
@@ -1558,6 +1616,21 @@ bool use_stream(uint64_t units, int G, int n_pad, int kv_cap, bool rope) {
   return waves * nb * (uint64_t)sms <= units * (nb + STREAM_OVERHEAD_BLOCKS);
 }
 
+// Whether a launch's sequences run longest first: from a little over one wave
+// of units to four (us per launch, in order / longest first, trees and caches
+// of mixed sizes: 256 units of two tiles and 16384 keys 362 / 316, 320 of 16384
+// 359 / 309, 512 of 16384 569 / 546, 512 of 9000 346 / 329; more waves even out
+// by themselves, 768 of 6000 349 / 351).  The ranking costs a CTA 0.6 to 1.4 us:
+// caches of 8192 keys and more (equal lengths: 256 units of 8192 keys 221 / 222,
+// 512 of 4096 240 / 245), and units of two tiles (one-tile units are bound by
+// the K/V stream: 149 / 155).
+constexpr uint64_t ORDER_MIN_BLOCKS = 64;
+bool use_order(int batch, uint64_t units, int rows, int kv_cap) {
+  const uint64_t sms = (uint64_t)sm_count();
+  const uint64_t nb = (uint64_t)(kv_cap + BN - 1) / BN + 1;
+  return rows > BM && batch > 1 && batch <= ORDER_MAX && nb >= ORDER_MIN_BLOCKS && 4 * units >= 5 * sms && units <= 4 * sms;
+}
+
 uint64_t attn_units(int batch, int n_pad, int H, int Hkv) {
   return (uint64_t)batch * Hkv * (((uint64_t)(H / Hkv) * n_pad + TILES * BM - 1) / (TILES * BM));
 }
@@ -1656,12 +1729,14 @@ static fc_status launch_tree_attn(const void* d_q, const void* d_k_cache, const 
     return FC_ERR_CUDA;
   // the streaming kernel keeps three K/V stages when a group's rows fit 64
   const bool three = streamed && G * n_pad <= 64;
-  static constexpr AttnKernel kernels[6] = {k_tree_attn<false, false>, k_tree_attn<true, false>, k_tree_attn<false, true>,
-                                            k_tree_attn<true, true>,   k_tree_attn_stream<2>,    k_tree_attn_stream<3>};
-  const int which = streamed ? 4 + three : 2 * (spread > 0) + (d_pos != nullptr);
+  static constexpr AttnKernel kernels[8] = {
+      k_tree_attn<false, MODE_PLAIN>,   k_tree_attn<true, MODE_PLAIN>,   k_tree_attn<false, MODE_SPREAD>, k_tree_attn<true, MODE_SPREAD>,
+      k_tree_attn<false, MODE_ORDERED>, k_tree_attn<true, MODE_ORDERED>, k_tree_attn_stream<2>,           k_tree_attn_stream<3>};
+  const bool ordered = !streamed && !spread && use_order(batch, units, G * n_pad, kv_cap);
+  const int which = streamed ? 6 + three : 2 * (spread ? MODE_SPREAD : ordered ? MODE_ORDERED : MODE_PLAIN) + (d_pos != nullptr);
   const AttnKernel kern = kernels[which];
   const uint32_t smem_bytes = streamed ? (three ? StreamLayout<3>::SMEM : StreamLayout<2>::SMEM) : SMEM_BYTES;
-  static std::atomic<unsigned long long> ready[6];  // per kernel: the devices it is set up on
+  static std::atomic<unsigned long long> ready[8];  // per kernel: the devices it is set up on
   const fc_status set = fc_once_per_device(ready[which], [&](int) -> fc_status {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) != cudaSuccess)
       return FC_ERR_CUDA;

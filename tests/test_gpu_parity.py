@@ -601,6 +601,40 @@ def test_attn_spread_limits(fc):
     assert parts(4, 769) > 1 and parts(4, 768) == 1 and parts(4, 4096, 0) == 1
 
 
+@pytest.mark.parametrize("B,n_pad,H,Hkv", [(13, 128, 32, 8), (32, 128, 16, 4), (33, 64, 32, 8), (64, 64, 32, 8), (3, 128, 64, 32)])
+@pytest.mark.parametrize("rope", [False, True])
+def test_attn_ordered(fc, orc, B, n_pad, H, Hkv, rope):
+    """Launches of one to four waves over long caches run the longest sequences
+    first (up to 64 of them): lengths that tie, empty caches and an invalid
+    sequence, whose rows are zero; every row as without a workspace, sampled
+    rows against the oracle."""
+    cap, rng = 8100, np.random.default_rng(B)
+    kvl = [[0, 1, 128, 700, 700, 1500][b % 6] if b % 5 else int(rng.integers(0, 1500)) for b in range(B)]
+    nn = [int(rng.integers(1, n_pad + 1)) if b % 4 else n_pad for b in range(B)]
+    if not rope:
+        _attn_case(fc, orc, 41, B, n_pad, H, Hkv, kvl, cap, nn=nn, full_rows=False, sample=300)
+    bad, D = B // 2, 128
+    q = synth.randn_bf16((B, n_pad, H, D), 71, "cuda")
+    kc, vc = (synth.randn_bf16((B, Hkv, cap, D), s, "cuda") for s in (72, 73))
+    kt, vt = (synth.randn_bf16((B, Hkv, n_pad, D), s, "cuda") for s in (74, 75))
+    mask = torch.ones((B, n_pad, n_pad // 64), dtype=torch.int64, device="cuda")
+    nn[bad] = n_pad + 1
+    pos = torch.arange(n_pad, dtype=torch.int32, device="cuda").expand(B, n_pad).contiguous()
+    run = lambda sel, n: (fc.fc_tree_attn_rope(*(t[sel].contiguous() for t in (q, kc, vc, dev(np.array(kvl, np.int32)), kt, vt, mask)),
+                                               dev(np.array(n, np.int32)), pos[sel].contiguous()) if rope else
+                          fc.fc_tree_attn(*(t[sel].contiguous() for t in (q, kc, vc, dev(np.array(kvl, np.int32)), kt, vt, mask)),
+                                          dev(np.array(n, np.int32))))
+    got = run(slice(None), nn)
+    torch.cuda.synchronize()
+    assert fc.fc_get_error() == "FC_ERR_INVALID_ARG"
+    assert (got[bad] == 0).all()
+    for b in [b for b in range(B) if b != bad][:: max(1, B // 8)]:  # one sequence at a time runs in no order
+        one = run(slice(b, b + 1), [nn[b]])
+        torch.cuda.synchronize()
+        check_no_error(fc)
+        assert (one.float() - got[b:b + 1].float()).abs().max().item() <= ATOL
+
+
 def test_attn_stream_c1_shape(fc, orc):
     """The c1 launch (1024 one-tile groups, 512-key caches) runs on the
     streaming kernel: several groups per CTA."""

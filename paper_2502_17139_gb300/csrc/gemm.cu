@@ -371,14 +371,6 @@ enum { P_FULL = 0, P_EMPTY = PR_STAGES, P_ACC_FULL = 2 * PR_STAGES, P_ACC_EMPTY 
        P_DRAIN = P_ACC_EMPTY + 2, P_COUNT };
 static_assert(P_COUNT * 8 <= 256, "barrier area");
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));

@@ -87,6 +87,9 @@ def _sa_corpus(kind):
     if kind == "twice":  # a corpus and its copy: prefix doubling over all positions
         t = z(20_000, 5000)
         return np.concatenate([t, t]), 5000
+    if kind == "twice_odd":  # a scan of flags that ends inside a thread's eight
+        t = z(20_001, 5000)
+        return np.concatenate([t, t, t[:1]]), 5000
     if kind == "long_repeats":  # repeats of 140 to 1000 tokens among others: doubling for a few
         t = z(60_000, 5000)
         for ln in (140, 300, 1000, 129, 133):
@@ -98,7 +101,7 @@ def _sa_corpus(kind):
     return np.zeros(9000, np.uint32), 1  # "one_token"
 
 
-@pytest.mark.parametrize("kind", ["zipf", "sparse_vocab", "eight_bits", "tile_edges", "equal_pairs", "twice", "long_repeats",
+@pytest.mark.parametrize("kind", ["zipf", "sparse_vocab", "eight_bits", "tile_edges", "equal_pairs", "twice", "twice_odd", "long_repeats",
                                   "periodic", "one_token", "group_edges", "1", "33", "8191", "8192", "8193"])
 def test_sa_build_paths(fc, orc, kind):
     """Corpora whose ranges of equal keys take each path of the refinement."""

@@ -34,6 +34,7 @@ struct fc_pipeline {
   std::vector<cudaEvent_t> ev_pre, ev_post, ev_done, ev_fork;
   cudaEvent_t ev_start = nullptr;
   int p_chain = 0, p_attn = 0;                    // the two streams' priorities
+  std::vector<char> unshared;                     // per sub-batch: its attention gets no workspace (see create)
   std::vector<cudaGraphNode_t>* capture_attn = nullptr;  // while capturing: the attention nodes
 };
 
@@ -125,6 +126,23 @@ extern "C" fc_status fc_pipeline_create(const fc_pipeline_desc* d, fc_pipeline**
   pl->p_chain = p_chain;
   pl->p_attn = p_attn;
   const int n = d->n_parts;
+  // A launch of few row chunks has the SMs share their keys, which pays while
+  // SMs would be idle.  The sub-batches' launches run side by side: where
+  // together they have more than 5/4 chunks an SM, a CTA per chunk is enough
+  // (8 steps of 64-node trees and 4000 keys: 4 x 8 sequences, 256 chunks, 1606
+  // us with shared keys, 1273 without; 4 x 7, 224 chunks, 1530 and 1258; 4 x 6,
+  // 192 chunks, 1393 and 1232; 2 x 9, 144 chunks, 1182 and 1225).  Without a
+  // workspace nothing is shared; launches of more than half as many chunks as
+  // SMs never are.
+  int dev = 0, sms = 0;
+  ok = ok && cudaGetDevice(&dev) == cudaSuccess &&
+       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+  auto chunks = [&](int h) {
+    return (int64_t)d->parts[h].batch * d->Hkv * (((int64_t)(d->H / d->Hkv) * d->n_pad + 255) / 256);
+  };
+  int64_t total = 0;
+  for (int h = 0; h < n; ++h) total += chunks(h);
+  for (int h = 0; h < n; ++h) pl->unshared.push_back(4 * total > 5 * (int64_t)sms && 2 * chunks(h) <= sms);
   pl->chain.assign(n, nullptr);
   pl->attn.assign(n, nullptr);
   pl->ev_pre.assign(n, nullptr);
@@ -249,13 +267,14 @@ fc_status enqueue_part(fc_pipeline* pl, int h, int c, bool attention, const void
     stage_event(stage_events, h, 2, 0, sa);
     std::vector<cudaGraphNode_t> before;  // capturing: what the attention launches follow
     if (pl->capture_attn) FC_TRY(capture_heads(sa, &before));
+    void* ws = pl->unshared[h] ? nullptr : P.attn_ws;
+    const size_t ws_bytes = ws ? P.attn_ws_bytes : 0;
     if (rope)
       FC_TRY(fc_tree_attn_rope(q, P.k_cache, P.v_cache, d.kv_cap, P.kv_len[c], kt, vt, P.mask, P.n_nodes, B, Np,
-                               d.H, d.Hkv, d.D, d.scale, P.pos, d.rope_base, P.attn_out, P.attn_ws,
-                               P.attn_ws_bytes, sa));
+                               d.H, d.Hkv, d.D, d.scale, P.pos, d.rope_base, P.attn_out, ws, ws_bytes, sa));
     else
       FC_TRY(fc_tree_attn(q, P.k_cache, P.v_cache, d.kv_cap, P.kv_len[c], kt, vt, P.mask, P.n_nodes, B, Np, d.H,
-                          d.Hkv, d.D, d.scale, P.attn_out, P.attn_ws, P.attn_ws_bytes, sa));
+                          d.Hkv, d.D, d.scale, P.attn_out, ws, ws_bytes, sa));
     stage_event(stage_events, h, 2, 1, sa);
     if (pl->capture_attn) FC_TRY(note_attn_nodes(sa, before, pl->capture_attn));
     if (cudaEventRecord(pl->ev_post[h], sa) != cudaSuccess ||

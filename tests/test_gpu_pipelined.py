@@ -172,6 +172,34 @@ def test_pipelined_kv_split_workspaces(fc):
     assert fc.fc_get_error() == "FC_OK"
 
 
+@pytest.mark.parametrize("B", [16, 24])
+def test_pipelined_shared_keys(fc, B):
+    """Four sub-batches of 4 sequences x 8 heads, whose attention launches share
+    their chunks' keys over the GPU, and of 6 x 8, which together have a chunk
+    for every SM and do not: both equal the single loop."""
+    from paper_2502_17139_gb300.step import PipelinedStepLoop, StepLoop
+    rng = synth.rng_for(79)
+    T, _ = synth.make_corpus(rng, 300_000, 1.2, synth.VOCAB, n_grams=500, len_range=(8, 64))
+    steps, n_pad, H, Hkv, D, kv0 = 3, 64, 8, 8, 128, 1100
+    ctx, cl, _ = synth.make_contexts(rng, B, 128, 16, [T, None], [0.75, 0.25], 1.1, ctx_stride=128 + 48)
+    hits = synth.cache_hit_pattern(rng, steps, B)
+    draws = [synth.argmax_draws(rng, B, n_pad) for _ in range(steps)]
+    cap = kv0 + steps * 12
+    args = ([fc.fc_datastore_build(dev(T), synth.VOCAB)], ctx, cl, fc.params(16, 2, 64, 10, 4096), n_pad, n_pad, [1], H, Hkv, D)
+    kw = dict(kv_cap=cap, kv_len0=kv0, vocab=synth.VOCAB)
+    kc0, vc0 = (synth.randn_bf16((B, Hkv, cap, D), s, "cuda") for s in (210, 211))
+    single = StepLoop(*args, **kw, k_cache=kc0.clone(), v_cache=vc0.clone())
+    piped = PipelinedStepLoop(4, *args, **kw, k_cache=kc0.clone(), v_cache=vc0.clone())
+    for s in range(steps):
+        ins = (synth.randn_bf16((B, n_pad, H, D), 310 + s, "cuda"), synth.randn_bf16((B, Hkv, n_pad, D), 340 + s, "cuda"),
+               synth.randn_bf16((B, Hkv, n_pad, D), 370 + s, "cuda"), dev(hits[s]), dev(draws[s][0]), dev(draws[s][1]))
+        single.step(*ins)
+        piped.step(*ins)
+        piped.join()
+        same(state(single), state(piped))
+    assert fc.fc_get_error() == "FC_OK"
+
+
 def test_pipelined_rope_matches_single_loop(fc, setup):
     """The executor's RoPE path (tree keys rotated by fc_rope, queries inside
     the attention kernel) against the single loop's."""

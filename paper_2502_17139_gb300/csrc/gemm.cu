@@ -287,7 +287,8 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
           mbar_expect_tx(bar(B_FULL + s), STAGE_BYTES);
           tma_load_2d(st, &tm_a, kb * BK, m0, bar(B_FULL + s));
 #pragma unroll
-          for (int c = 0; c < BN / 64; ++c) tma_load_2d(st + A_BYTES + c * B_CHUNK, wm, wcol + 64 * c, kb * BK, bar(B_FULL + s));
+          for (int c = 0; c < BN / 64; ++c)
+            tma_load_2d(st + A_BYTES + c * B_CHUNK, wm, wcol + 64 * c, kb * BK, bar(B_FULL + s));
           ++issued;
         }
       }
@@ -564,11 +565,14 @@ __global__ void __launch_bounds__(GM_THREADS, 1) __cluster_dims__(2, 1, 1)
 // ring), and after a cluster barrier CTA r sums every S-th group of eight
 // columns of both halves over the S partials, in CTA order, and applies the
 // epilogue (column c of either half is what the epilogues need together: gate
-// and up, or the rotation's partners).  fp32 throughout, no scratch memory.  Bound by the
-// latency of its steps (a copy, the MMAs, the exchange: 5 us for the smallest
-// shape) and then by the weights' stream: the ring is as deep as the SM allows.
-//   The ring's slices carry only as many rows of A as the matrix has (the MMA then reads 128 - a_rows rows of the slice's B as A
-// rows, into accumulator rows that nothing reads).
+// and up, or the rotation's partners).  fp32 throughout, no scratch memory.
+// Bound by the latency of its steps (a copy, the MMAs, the exchange: 5 us for
+// the smallest shape) and then by the weights' stream: the ring is as deep as
+// the SM allows (shallower ones, with which the next launch's CTAs would fit
+// beside this one's, measured no better).
+//   The ring's slices carry only as many rows of A as the matrix has (the MMA
+// then reads 128 - a_rows rows of the slice's B as A rows, into accumulator rows
+// that nothing reads).
 // ---------------------------------------------------------------------------
 constexpr int SP_THREADS = 192, SP_MAX_STAGES = 12;
 constexpr uint32_t SP_RING_1 = 208 * 1024, SP_RING_2 = 96 * 1024;  // one CTA per SM, or two; a partial tile is 32 NB KB
@@ -881,7 +885,8 @@ fc_status launch_gemm(const void* d_a, const void* d_b, int M, int N, int K, Gem
   constexpr bool WIDE = EPI == EPI_STORE || EPI == EPI_SILU_MUL;  // a narrow tile of the K/V projection is one head
   const SplitPlan plan = choose_split(M, g.tiles_m, N, tiles, (K + BK - 1) / BK, sms, WIDE);
   const int a_rows = plan.cluster ? std::min(BM, (M + 7) / 8 * 8) : BM;
-  if (!make_map_2d(&ma, d_a, (uint64_t)M, (uint64_t)K, a_rows) || !make_map_2d(&mb, d_b, (uint64_t)K, (uint64_t)(d_b2 ? g.n_q : N), BK))
+  if (!make_map_2d(&ma, d_a, (uint64_t)M, (uint64_t)K, a_rows) ||
+      !make_map_2d(&mb, d_b, (uint64_t)K, (uint64_t)(d_b2 ? g.n_q : N), BK))
     return FC_ERR_CUDA;
   mb2 = mb;
   if (d_b2 && !make_map_2d(&mb2, d_b2, (uint64_t)K, (uint64_t)(N - g.n_q), BK)) return FC_ERR_CUDA;
@@ -989,7 +994,9 @@ extern "C" fc_status fc_gemm_qkv(const void* d_a, const void* d_wq, const void* 
     return FC_ERR_INVALID_ARG;
   if (H % 2) {  // a 256-column tile would hold columns of both
     const fc_status st = fc_gemm_bf16(d_a, d_wq, d_q, M, H * D, K, nullptr, 0, stream);
-    return st != FC_OK ? st : fc_gemm_kv_heads(d_a, d_wkv, M, K, Hkv, D, batch, n_pad, d_pos, rope_base, d_k_rot, d_v_heads, stream);
+    return st != FC_OK ? st
+                       : fc_gemm_kv_heads(d_a, d_wkv, M, K, Hkv, D, batch, n_pad, d_pos, rope_base, d_k_rot, d_v_heads,
+                                          stream);
   }
   GemmArgs g{};
   g.c = static_cast<__nv_bfloat16*>(d_q);

@@ -1730,10 +1730,12 @@ static fc_status launch_tree_attn(const void* d_q, const void* d_k_cache, const 
   // the streaming kernel keeps three K/V stages when a group's rows fit 64
   const bool three = streamed && G * n_pad <= 64;
   static constexpr AttnKernel kernels[8] = {
-      k_tree_attn<false, MODE_PLAIN>,   k_tree_attn<true, MODE_PLAIN>,   k_tree_attn<false, MODE_SPREAD>, k_tree_attn<true, MODE_SPREAD>,
-      k_tree_attn<false, MODE_ORDERED>, k_tree_attn<true, MODE_ORDERED>, k_tree_attn_stream<2>,           k_tree_attn_stream<3>};
+      k_tree_attn<false, MODE_PLAIN>,   k_tree_attn<true, MODE_PLAIN>,   k_tree_attn<false, MODE_SPREAD>,
+      k_tree_attn<true, MODE_SPREAD>,   k_tree_attn<false, MODE_ORDERED>, k_tree_attn<true, MODE_ORDERED>,
+      k_tree_attn_stream<2>,            k_tree_attn_stream<3>};
   const bool ordered = !streamed && !spread && use_order(batch, units, G * n_pad, kv_cap);
-  const int which = streamed ? 6 + three : 2 * (spread ? MODE_SPREAD : ordered ? MODE_ORDERED : MODE_PLAIN) + (d_pos != nullptr);
+  const int mode = spread ? MODE_SPREAD : ordered ? MODE_ORDERED : MODE_PLAIN;
+  const int which = streamed ? 6 + three : 2 * mode + (d_pos != nullptr);
   const AttnKernel kern = kernels[which];
   const uint32_t smem_bytes = streamed ? (three ? StreamLayout<3>::SMEM : StreamLayout<2>::SMEM) : SMEM_BYTES;
   static std::atomic<unsigned long long> ready[8];  // per kernel: the devices it is set up on

@@ -175,7 +175,10 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+// A barrier of all threads of the cluster's CTAs.  The instructions are .aligned: all lanes of a warp
+// execute them together, and nothing but __syncwarp() brings lanes that took different branches back together.
 __device__ __forceinline__ void cluster_sync_all() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 

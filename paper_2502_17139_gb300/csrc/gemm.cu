@@ -777,7 +777,6 @@ __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
       *reinterpret_cast<uint4*>(dst + 64) = pack8(hi);
     }
   }
-  __syncwarp();
   cluster_sync_all();  // no CTA leaves while another may still read its partial tile
   if (tid == 0 && s_abort) fc_flag(FC_ERR_WORD(g.err), FC_EBIT_TIMEOUT);
   if (warp == 1) {

@@ -90,6 +90,10 @@ def _sa_corpus(kind):
     if kind == "twice_odd":  # a scan of flags that ends inside a thread's eight
         t = z(20_001, 5000)
         return np.concatenate([t, t, t[:1]]), 5000
+    if kind.startswith("flags"):  # that many flags to scan in doubling: its last warp has whole and ragged eights of them
+        n = int(kind[5:])
+        t = z((n + 1) // 2, 5000)
+        return np.concatenate([t, t])[:n], 5000
     if kind == "long_repeats":  # repeats of 140 to 1000 tokens among others: doubling for a few
         t = z(60_000, 5000)
         for ln in (140, 300, 1000, 129, 133):
@@ -102,7 +106,8 @@ def _sa_corpus(kind):
 
 
 @pytest.mark.parametrize("kind", ["zipf", "sparse_vocab", "eight_bits", "tile_edges", "equal_pairs", "twice", "twice_odd", "long_repeats",
-                                  "periodic", "one_token", "group_edges", "1", "33", "8191", "8192", "8193"])
+                                  "periodic", "one_token", "group_edges", "1", "33", "8191", "8192", "8193",
+                                  "flags4097", "flags4104", "flags65528", "flags65535"])
 def test_sa_build_paths(fc, orc, kind):
     """Corpora whose ranges of equal keys take each path of the refinement."""
     T, vocab = _sa_corpus(kind)

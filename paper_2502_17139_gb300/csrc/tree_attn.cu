@@ -979,8 +979,10 @@ __global__ void __launch_bounds__(TILES* BM) k_attn_merge(AttnArgs a) {
     float m_new = m;
 #pragma unroll
     for (int q = 0; q < MERGE_ROUND; ++q) m_new = fmaxf(m_new, v[q].x);
+    // parts whose keys all score -inf for this row have m = -inf, l = 0 and O = 0: a reference of 0 keeps their weights 0
+    const float m_use = m_new == -INFINITY ? 0.f : m_new;
     if (h0 > 0) {
-      const float w = exp2f(m - m_new);
+      const float w = exp2f(m - m_use);
       lstar *= w;
 #pragma unroll
       for (int u = 0; u < MERGE_COLS; ++u) acc[u] *= w;
@@ -989,7 +991,7 @@ __global__ void __launch_bounds__(TILES* BM) k_attn_merge(AttnArgs a) {
 #pragma unroll
     for (int q = 0; q < MERGE_ROUND; ++q) {
       if (h0 + q >= p.y) break;
-      const float w = exp2f(v[q].x - m);
+      const float w = exp2f(v[q].x - m_use);
       lstar += v[q].y * w;
 #pragma unroll
       for (int u = 0; u < MERGE_COLS / 4; ++u) {

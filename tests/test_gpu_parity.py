@@ -601,6 +601,39 @@ def test_attn_spread(fc, orc, B, n_pad, H, Hkv, cap, kv, nn):
     _attn_case(fc, orc, 32, B, n_pad, H, Hkv, kv, cap, nn=nn, full_rows=False, sample=500, workspace=few, want_parts=2)
 
 
+@pytest.mark.parametrize("B,n_pad,H,Hkv,cap,dead", [
+    (1, 64, 8, 8, 16384, 3000), (1, 64, 8, 8, 16384, 8000), (1, 64, 8, 8, 16384, 16384),  # 19 parts: 3, 9 and 18 of them dead
+    (2, 128, 32, 8, 9000, 6000),                                                          # two-tile units, four or five parts
+    (13, 128, 32, 8, 8100, 8000),                                                         # longest first, a split last wave
+])
+def test_attn_dead_keys(fc, B, n_pad, H, Hkv, cap, dead):
+    """Keys that a bias dimension of -inf switches off at the front of a long
+    cache: whole parts have no key that counts for a row, and the row is that
+    of the call without a workspace (and of the live keys alone)."""
+    D = 128
+    q = synth.randn_bf16((B, n_pad, H, D), 81, "cuda")
+    kc, vc = (synth.randn_bf16((B, Hkv, cap, D), s, "cuda") for s in (82, 83))
+    kt, vt = (synth.randn_bf16((B, Hkv, n_pad, D), s, "cuda") for s in (84, 85))
+    q[..., D - 1] = 1.0
+    kc[..., D - 1] = 0.0
+    kt[..., D - 1] = 0.0
+    kc[:, :, :dead, D - 1] = float("-inf")
+    kvl = dev(np.array([cap - 37 * b for b in range(B)], np.int32))
+    nn = dev(np.array([n_pad - b for b in range(B)], np.int32))
+    mask = torch.zeros((B, n_pad, n_pad // 64), dtype=torch.int64, device="cuda")
+    mask[..., 0] = 1  # every row sees node 0 of its tree, in either word of the mask no other
+    got, one = torch.full_like(q, float("nan")), torch.full_like(q, float("nan"))
+    assert fc.LIB.fc_tree_attn_parts(B, n_pad, H, Hkv, cap, 1 << 40) > 1
+    fc.fc_tree_attn(q, kc, vc, kvl, kt, vt, mask, nn, out=got)
+    fc.fc_tree_attn(q, kc, vc, kvl, kt, vt, mask, nn, out=one, workspace=None)
+    torch.cuda.synchronize()
+    check_no_error(fc)
+    assert torch.isfinite(one.float()).all() and torch.isfinite(got.float()).all()
+    assert (got.float() - one.float()).abs().max().item() <= ATOL
+    k, v = (torch.cat([c[0, 0, dead:], t[0, 0, :1]]).float() for c, t in ((kc, kt), (vc, vt)))
+    assert (torch.softmax(k @ q[0, 0, 0].float() * D ** -0.5, 0) @ v - got[0, 0, 0].float()).abs().max().item() <= ATOL
+
+
 def test_attn_spread_limits(fc):
     """One unit more than half the SMs, or caches too short, are not spread."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count

@@ -31,6 +31,7 @@
 #include <mutex>
 
 #include "fc_common.cuh"
+#include "fc_merge.cuh"
 
 FC_DEFINE_ERROR_WORD(attn)
 
@@ -788,8 +789,9 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
       }
     } else if constexpr (SPREAD) {
       // This CTA's share of the unit's sums goes to its slot, column-major (the
-      // warp's rows are adjacent, so its 16-byte stores fill whole lines).
-      if (fin && row_ok) a.ws_ml[(size_t)blockIdx.x * (TILES * BM) + x * BM + r] = make_float2(m_run, l_run);
+      // warp's rows are adjacent, so its 16-byte stores fill whole lines).  A
+      // wait that ran out leaves the mark of no result.
+      if (row_ok) a.ws_ml[(size_t)blockIdx.x * (TILES * BM) + x * BM + r] = fin ? make_float2(m_run, l_run) : FC_NO_PART;
       float4* od = reinterpret_cast<float4*>(a.ws_o) + (size_t)blockIdx.x * (TILES * BM * HD / 4) + x * BM + r;
       if (fin) {
 #pragma unroll
@@ -934,9 +936,8 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   }
 }
 
-// The merge of a spread launch: with m* = max m_t, l* = sum l_t 2^(m_t - m*) and
-// O = sum O_t 2^(m_t - m*) / l* over a unit's parts, in part order.  One CTA
-// takes MERGE_COLS columns of a unit's rows, one row per thread: a warp's
+// The merge of a spread launch: a unit's parts in part order.  One CTA takes
+// MERGE_COLS columns of a unit's rows, one row per thread: a warp's
 // 16-byte loads of a part are consecutive.  Launched as a programmatic
 // dependent of the attention (2 us less than a plain launch); units that one
 // CTA served are already written.  A dependent chain of L2 reads: 8 columns
@@ -959,11 +960,8 @@ __global__ void __launch_bounds__(TILES* BM) k_attn_merge(AttnArgs a) {
   const float2* ml = a.ws_ml + (size_t)p.x * (TILES * BM) + r;
   const float4* os = reinterpret_cast<const float4*>(a.ws_o) + (size_t)p.x * (TILES * BM * HD / 4) +
                      (size_t)(col / 4) * (TILES * BM) + r;
-  // parts in rounds of MERGE_ROUND, every load of a round in flight at once;
-  // the reference maximum moves from round to round
-  float m = -INFINITY, lstar = 0.f, acc[MERGE_COLS];
-#pragma unroll
-  for (int u = 0; u < MERGE_COLS; ++u) acc[u] = 0.f;
+  // parts in rounds of MERGE_ROUND, every load of a round in flight at once
+  FcRowMerge<MERGE_COLS> row;
   for (int h0 = 0; h0 < p.y; h0 += MERGE_ROUND) {
     float2 v[MERGE_ROUND];
     float4 o[MERGE_ROUND][MERGE_COLS / 4];
@@ -976,39 +974,16 @@ __global__ void __launch_bounds__(TILES* BM) k_attn_merge(AttnArgs a) {
       for (int u = 0; u < MERGE_COLS / 4; ++u)
         o[q][u] = __ldcg(os + (size_t)(h0 + q) * (TILES * BM * HD / 4) + u * (TILES * BM));
     }
-    float m_new = m;
-#pragma unroll
-    for (int q = 0; q < MERGE_ROUND; ++q) m_new = fmaxf(m_new, v[q].x);
-    // parts whose keys all score -inf for this row have m = -inf, l = 0 and O = 0: a reference of 0 keeps their weights 0
-    const float m_use = m_new == -INFINITY ? 0.f : m_new;
-    if (h0 > 0) {
-      const float w = exp2f(m - m_use);
-      lstar *= w;
-#pragma unroll
-      for (int u = 0; u < MERGE_COLS; ++u) acc[u] *= w;
-    }
-    m = m_new;
-#pragma unroll
-    for (int q = 0; q < MERGE_ROUND; ++q) {
-      if (h0 + q >= p.y) break;
-      const float w = exp2f(v[q].x - m_use);
-      lstar += v[q].y * w;
-#pragma unroll
-      for (int u = 0; u < MERGE_COLS / 4; ++u) {
-        acc[4 * u] += o[q][u].x * w;
-        acc[4 * u + 1] += o[q][u].y * w;
-        acc[4 * u + 2] += o[q][u].z * w;
-        acc[4 * u + 3] += o[q][u].w * w;
-      }
-    }
+    row.round(v, o, p.y - h0, h0 == 0);
   }
-  const float inv = 1.f / lstar;
+  if (!row.whole) return;  // a part gave up (the error word says so): the row stays as it was
+  const float inv = 1.f / row.l;
   const int hh = rg / nn, i = rg - hh * nn;
   uint2* dst = reinterpret_cast<uint2*>(a.out + (((size_t)b * a.n_pad + i) * a.H + g * a.G + hh) * HD + col);
 #pragma unroll
   for (int u = 0; u < MERGE_COLS / 4; ++u)
-    dst[u] = make_uint2(pack_bf16x2(acc[4 * u] * inv, acc[4 * u + 1] * inv),
-                        pack_bf16x2(acc[4 * u + 2] * inv, acc[4 * u + 3] * inv));
+    dst[u] = make_uint2(pack_bf16x2(row.acc[4 * u] * inv, row.acc[4 * u + 1] * inv),
+                        pack_bf16x2(row.acc[4 * u + 2] * inv, row.acc[4 * u + 3] * inv));
 }
 
 // ---------------------------------------------------------------------------

@@ -596,6 +596,14 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank) {
   return v;
 }
 
+// Raises the abort flag at this address in all S CTAs of the cluster (before a cluster barrier, so that behind it
+// they agree).
+template <int S>
+__device__ __forceinline__ void abort_cluster(uint32_t flag) {
+  for (uint32_t r = 0; r < S; ++r)
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(flag, r)), "r"(1u) : "memory");
+}
+
 template <int EPI, int S, int NB>
 __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
     k_gemm_split(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
@@ -672,6 +680,7 @@ __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
         volatile int dummy = 0;
         for (int i = max(0, issued - sp.stages); i < issued; ++i)
           mbar_wait_bounded(bar(SB_FULL + i % sp.stages), (i / sp.stages) & 1, &dummy, DRAIN_CYCLES);
+        abort_cluster<S>(smem_u32((const void*)&s_abort));
       }
     }
     __syncwarp();
@@ -694,11 +703,14 @@ __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
       tc_commit(bar(SB_DRAIN));
       volatile int dummy = 0;
       mbar_wait_bounded(bar(SB_DRAIN), 0, &dummy, DRAIN_CYCLES);
+      abort_cluster<S>(smem_u32((const void*)&s_abort));
     }
   } else {  // ---------------- warps 2-5: the partial tile to shared memory ----------------
     const int q4 = warp & 3;
     // every MMA has read the ring and every copy has landed: the ring is free
-    if (wait_warp(bar(SB_ACC), 0, &s_abort) && q4 * 32 < rows) {
+    if (!wait_warp(bar(SB_ACC), 0, &s_abort)) {
+      abort_cluster<S>(smem_u32((const void*)&s_abort));
+    } else if (q4 * 32 < rows) {
       tc_fence_after();
       float4* red = reinterpret_cast<float4*>(smem) + q4 * 32 + lane;  // [column / 4][row]
 #pragma unroll
@@ -718,7 +730,8 @@ __global__ void __launch_bounds__(SP_THREADS, NB == 2 ? 2 : 1)
 
   // ---------------- this CTA's columns of the tile, eight of each half per item ----------------
   constexpr int QUAD = S < 4 ? S : 4;  // partials whose loads are in flight together
-  const int groups = (HN / 8 - (int)rank + S - 1) / S;  // groups rank, rank + S, ... of the half's eights
+  // groups rank, rank + S, ... of the half's eights; none where a CTA of the cluster gave up: the tile stays as it was
+  const int groups = s_abort ? 0 : (HN / 8 - (int)rank + S - 1) / S;
   for (int e = tid; e < rows * groups; e += SP_THREADS) {
     const int cg = e / rows, r = e - cg * rows, c = ((int)rank + cg * S) * 8;
     float lo[8], hi[8];

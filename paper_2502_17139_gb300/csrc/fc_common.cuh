@@ -132,8 +132,9 @@ fc_status fc_launch_dependent(void (*kern)(P...), dim3 grid, unsigned threads, s
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = cluster ? 2 : 1;
-  if (cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...) != cudaSuccess) return FC_ERR_CUDA;
-  return FC_CHECK_LAUNCH();
+  const cudaError_t launched = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+  const fc_status left = FC_CHECK_LAUNCH();  // also takes the error off the runtime: the next call is not to report it
+  return launched == cudaSuccess ? left : FC_ERR_CUDA;
 }
 __device__ __forceinline__ void fc_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // A pointer argument as read after the wait: loads through a const __restrict__

@@ -230,7 +230,9 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_radix_scatter(const uint64_t*
     const bool ok = 32 * it < left;
     const uint32_t d = ok ? ((uint32_t)(key[it] >> shift) & 255u) : 256u;
     const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
-    // the equal digits' first lane adds them all: a warp's atomics apply in order, and the iterations overlap
+    // the equal digits' first lane adds them all, behind the iterations before it: other lanes' atomics on a
+    // counter are ordered by the warp's barrier alone, and the pass has to be stable
+    __syncwarp();
     uint32_t cnt = 0;
     if (ok && (peers & lt) == 0) cnt = atomicAdd(&wbin[warp][d], (uint32_t)__popc(peers));
     const uint32_t r = __shfl_sync(0xFFFFFFFFu, cnt, __ffs(peers) - 1) + __popc(peers & lt);
@@ -330,6 +332,7 @@ __global__ void __launch_bounds__(RO_THREADS) k_radix_one(const uint64_t* kin, c
       const bool ok = 32 * it < left;
       const uint32_t d = ok ? ((uint32_t)(key[it] >> shift) & 255u) : 256u;
       const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+      __syncwarp();  // orders the iterations' atomics, as in k_radix_scatter
       uint32_t cnt = 0;
       if (ok && (peers & lt) == 0) cnt = atomicAdd(&wbin[warp * 256 + d], (uint32_t)__popc(peers));
       const uint32_t r = __shfl_sync(0xFFFFFFFFu, cnt, __ffs(peers) - 1) + __popc(peers & lt);

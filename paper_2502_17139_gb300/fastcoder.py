@@ -615,23 +615,56 @@ def fc_tree_mask(parent, n_nodes, kv_len):
 
 # --------------------------------------------------------------- attention
 _ATTN_WS = {}        # (device, bytes) -> a workspace of launches that split at most their last wave
-_ATTN_WS_BYTES = {}  # (device, shape) -> (bytes, whether the launch is spread over the GPU)
+_ATTN_WS_BYTES = {}  # (device, shape) -> (bytes, few row chunks, the shortest caches whose launch is then spread over the GPU)
 
 
-def attn_workspace(B, Np, H, Hkv, device):
+def _shortest_spread(B, Np, H, Hkv, n):
+    """The smallest kv_cap for which a launch with n bytes of workspace shares its keys."""
+    spread = lambda cap: LIB.fc_tree_attn_parts(B, Np, H, Hkv, cap, n) > 1  # noqa: E731
+    lo, hi = 1, 1 << 24
+    if not spread(hi):
+        return None
+    while lo < hi:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if spread(mid) else (mid + 1, hi)
+    return lo
+
+
+def _kept_for_replay(t):
+    """Whether t, allocated while the current stream is captured, lies in a pool of its own graph (torch's captures).
+    In any other capture the allocator hands its memory on while the graph still writes there."""
+    at = t.data_ptr()
+    try:
+        seg = next(s for s in torch.cuda.memory_snapshot() if s["address"] <= at < s["address"] + s["total_size"])
+    except (StopIteration, RuntimeError):  # not an allocation of the caching allocator
+        return False
+    return tuple(seg["segment_pool_id"]) != (0, 0)
+
+
+def attn_workspace(B, Np, H, Hkv, device, kv_cap=None):
     """A device workspace of fc_tree_attn_workspace() bytes for this shape.
-    Launches of at most half as many row chunks as SMs use theirs on every
-    call, so each gets one of its own from the caching allocator (any stream,
-    thread or capture); the others share a cached one per size."""
+    Launches of at most half as many row chunks as SMs write to theirs on every
+    call if their caches are long enough to share (kv_cap; None: any), so each
+    gets one of its own from the caching allocator, for any stream or thread.
+    They get None, with which the call shares no keys, where the caches are
+    short, where there is no memory, and in a capture that is not torch's.
+    Larger launches share a cached workspace per size."""
     key = (device, B, Np, H, Hkv)
     got = _ATTN_WS_BYTES.get(key)
     if got is None:
         chunks = B * Hkv * -(-(H // Hkv) * Np // 256) if Hkv and H % Hkv == 0 else 0
         sms = torch.cuda.get_device_properties(device).multi_processor_count
-        got = _ATTN_WS_BYTES[key] = (max(int(LIB.fc_tree_attn_workspace(B, Np, H, Hkv)), 16), 2 * chunks <= sms)
-    n, own = got
+        n = max(int(LIB.fc_tree_attn_workspace(B, Np, H, Hkv)), 16)
+        got = _ATTN_WS_BYTES[key] = (n, 2 * chunks <= sms, _shortest_spread(B, Np, H, Hkv, n) if 2 * chunks <= sms else None)
+    n, own, shortest = got
     if own:
-        return torch.empty(n, dtype=torch.uint8, device=device)
+        if kv_cap is not None and (shortest is None or kv_cap < shortest):
+            return None
+        try:
+            ws = torch.empty(n, dtype=torch.uint8, device=device)
+        except torch.cuda.OutOfMemoryError:
+            return None
+        return ws if not torch.cuda.is_current_stream_capturing() or _kept_for_replay(ws) else None
     key = (str(device), n)
     if key not in _ATTN_WS:
         _ATTN_WS[key] = torch.empty(n, dtype=torch.uint8, device=device)
@@ -642,7 +675,7 @@ def fc_tree_attn(q, k_cache, v_cache, kv_len, k_tree, v_tree, mask, n_nodes, sca
     """q [B, Np, H, D]; caches [B, Hkv, cap, D]; tree K/V [B, Hkv, Np, D] (bf16).
 
     ``workspace``: "auto" (attn_workspace: one of the full size, shared by every
-    call with that size unless the batch is small: calls that may overlap on
+    call with that size unless there are few row chunks: calls that may overlap on
     different streams must each pass their own), None (no key split) or a uint8
     device tensor."""
     _need(q, torch.bfloat16, "q")
@@ -658,7 +691,7 @@ def fc_tree_attn(q, k_cache, v_cache, kv_len, k_tree, v_tree, mask, n_nodes, sca
     o = out if out is not None else torch.empty_like(q)
     sc = float(scale) if scale is not None else D ** -0.5
     if isinstance(workspace, str):
-        workspace = attn_workspace(B, Np, H, Hkv, q.device)
+        workspace = attn_workspace(B, Np, H, Hkv, q.device, cap)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     _check("fc_tree_attn", LIB.fc_tree_attn(_ptr(q), _ptr(k_cache), _ptr(v_cache), cap, _ptr(kv_len), _ptr(k_tree),
                                             _ptr(v_tree), _ptr(mask), _ptr(n_nodes), B, Np, H, Hkv, D, sc, _ptr(o),
@@ -701,7 +734,7 @@ def fc_tree_attn_rope(q, k_cache, v_cache, kv_len, k_tree_rot, v_tree, mask, n_n
     o = out if out is not None else torch.empty_like(q)
     sc = float(scale) if scale is not None else D ** -0.5
     if isinstance(workspace, str):
-        workspace = attn_workspace(B, Np, H, Hkv, q.device)
+        workspace = attn_workspace(B, Np, H, Hkv, q.device, cap)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     _check("fc_tree_attn_rope", LIB.fc_tree_attn_rope(
         _ptr(q), _ptr(k_cache), _ptr(v_cache), cap, _ptr(kv_len), _ptr(k_tree_rot), _ptr(v_tree), _ptr(mask),

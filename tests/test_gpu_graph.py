@@ -2,6 +2,8 @@
 and replayed with inputs updated in place give the same trajectory as eager
 steps (integer outputs bit-exact, attention within the step's max-abs 2e-2),
 for the replay-cache loop and for the loop with Algorithm 1's CACHE."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -83,3 +85,65 @@ def test_graph_replay_matches_eager(fc, seq_cache):
         for name in ("ctx", "cl", "kv", "acc", "nn", "kc"):
             assert torch.equal(w[name], gt[name]), name
         assert (w["attn"] - gt["attn"]).abs().max().item() <= 2e-2
+
+
+def _small_attn(cap):
+    B, n_pad, H, Hkv, D = 1, 64, 8, 8, 128
+    t = [synth.randn_bf16(sh, 91 + i, "cuda") for i, sh in enumerate([(B, n_pad, H, D)] + 2 * [(B, Hkv, cap, D)] + 2 * [(B, Hkv, n_pad, D)])]
+    mask = torch.ones((B, n_pad, 1), dtype=torch.int64, device="cuda")
+    return t[0], t[1], t[2], dev(np.array([cap], np.int32)), t[3], t[4], mask, dev(np.array([n_pad], np.int32))
+
+
+@pytest.mark.parametrize("by", ["torch", "runtime"])
+def test_small_attention_in_a_capture(fc, by):
+    """A launch that shares its keys over the GPU, in a graph that torch
+    captures and in one captured through the CUDA runtime: replayed, it gives
+    the call's result and writes to no memory that others have since been
+    given."""
+    args = _small_attn(4096)
+    want = fc.fc_tree_attn(*args)
+    out, stream = torch.zeros_like(want), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    n = fc.LIB.fc_tree_attn_workspace(1, 64, 8, 8)
+    if by == "torch":
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            fc.fc_tree_attn(*args, out=out)
+        replay = g.replay
+    else:
+        rt = C.CDLL(next(line.split()[-1] for line in open("/proc/self/maps") if "libcudart" in line))
+        h, graph, ex = C.c_void_p(stream.cuda_stream), C.c_void_p(), C.c_void_p()
+        with torch.cuda.stream(stream):
+            fc.fc_tree_attn(*args)
+            assert rt.cudaStreamBeginCapture(h, 2) == 0
+            fc.fc_tree_attn(*args, out=out)
+            assert rt.cudaStreamEndCapture(h, C.byref(graph)) == 0
+        assert rt.cudaGraphInstantiate(C.byref(ex), graph, C.c_ulonglong(0)) == 0
+        replay = lambda: rt.cudaGraphLaunch(ex, h)  # noqa: E731
+    with torch.cuda.stream(stream):
+        others = [torch.full((n,), 7, dtype=torch.uint8, device="cuda") for _ in range(4)]
+    torch.cuda.synchronize()
+    replay()
+    torch.cuda.synchronize()
+    assert fc.fc_get_error() == "FC_OK"
+    assert (out.float() - want.float()).abs().max().item() <= 2e-2
+    assert by == "runtime" or torch.equal(out, want)  # torch's capture shares the keys as the call does
+    assert all((t == 7).all() for t in others)
+
+
+def test_small_attention_without_workspace(fc, monkeypatch):
+    """Caches too short to share ask for no workspace, and where there is no
+    memory for one the call does without."""
+    assert fc.attn_workspace(1, 64, 8, 8, "cuda", 768) is None
+    assert fc.attn_workspace(1, 64, 8, 8, "cuda", 769).numel() == fc.LIB.fc_tree_attn_workspace(1, 64, 8, 8)
+    args = _small_attn(2000)
+    want, out = fc.fc_tree_attn(*args, workspace=None), torch.zeros_like(args[0])
+
+    def no_memory(*a, **k):
+        raise torch.cuda.OutOfMemoryError("none left")
+
+    monkeypatch.setattr(torch, "empty", no_memory)
+    fc.fc_tree_attn(*args, out=out)
+    monkeypatch.undo()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want) and fc.fc_get_error() == "FC_OK"

@@ -204,11 +204,13 @@ fc_status note_attn_nodes(cudaStream_t s, const std::vector<cudaGraphNode_t>& be
         std::find(out->begin(), out->end(), v) != out->end())
       continue;
     out->push_back(v);
-    cudaGraphNode_t d[16];  // a stream's node follows the nodes its stream and its event waits ended on
-    cudaGraphEdgeData e[16];
-    size_t n = 16;
-    if (cudaGraphNodeGetDependencies(v, d, e, &n) != cudaSuccess || n > 16) return FC_ERR_CUDA;
-    todo.insert(todo.end(), d, d + n);
+    size_t n = 0;  // a stream's node follows the nodes its stream and its event waits ended on: first how many
+    if (cudaGraphNodeGetDependencies(v, nullptr, nullptr, &n) != cudaSuccess) return FC_ERR_CUDA;
+    if (n == 0) continue;
+    std::vector<cudaGraphEdgeData> edges(n);  // (programmatic edges are refused to a caller that does not take them)
+    const size_t at = todo.size();
+    todo.resize(at + n);
+    if (cudaGraphNodeGetDependencies(v, todo.data() + at, edges.data(), &n) != cudaSuccess) return FC_ERR_CUDA;
   }
   return FC_OK;
 }

@@ -104,7 +104,11 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, i
                "r"(x), "r"(y)
                : "memory");
 }
-constexpr int PREFETCH = 8;  // weight slices of a CTA's first tile that k_gemm prefetches
+// Weight slices of a CTA's first tile that k_gemm and k_gemm_pair prefetch while the kernel before drains.  The thread
+// that copies issues them, so with nothing to wait for they delay its first copies: us a call, weights from HBM, none /
+// 2 / 8: M 4096, K 1024, N 1024 10.5 / 10.6 / 11.4; M 64, K 4096, N 32256 43.7 / 44.2 / 45.8.  Behind a norm they pay,
+// two as much as eight (both launches): M 64, K 2048, N 32256 27.7 / 27.1 / 27.4; M 448 51.6 / 50.8 / 50.4.
+constexpr int PREFETCH = 2;
 
 __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort) {
   return __all_sync(0xFFFFFFFFu, mbar_wait_bounded(bar, parity, abort, WAIT_CYCLES));

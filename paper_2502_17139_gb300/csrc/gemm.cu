@@ -871,17 +871,23 @@ SplitPlan choose_split(int M, int64_t tiles_m, int N, int64_t big_tiles, int nk,
   return wide && nk >= 12 && big_tiles * 27 <= 8 * sms ? SplitPlan{3, 4, false} : SplitPlan{0, 0, false};
 }
 
-// Whether k_gemm_pair serves a launch of `tiles` 128 x 256 tiles: by waves, a
-// pair's being the shorter (16.4 thousand cycles of MMAs per 2048 of K either
-// way; k_gemm reaches 69% of that).  One row of tiles would waste half of each
-// pair, and in a single wave of short K the pair's set-up (a cluster barrier,
-// 0.6 us) is not earned back.  us per call, k_gemm / pairs:
+// Whether k_gemm_pair serves a launch of `tiles` 128 x 256 tiles: by waves.
+// A pair's wave is 3 to 20% shorter at K of 1024 and more, and not below (the
+// epilogues are the longer part then), so it may have one wave in eight more,
+// which an odd number of row tiles costs it.  One row of tiles would waste
+// half of each pair, and in a single wave of short K the pair's set-up (a
+// cluster barrier, 0.6 us) is not earned back.  us per call, k_gemm / pairs:
 //   M 2048, K 2048, N 32256  178.3 / 145.4    M 2048, K 2048, gate/up 11008  60.2 / 51.2
 //   M 2048, K 5504, N 2048    31.6 /  30.1    M 512,  K 2048, N 32256        59.1 / 47.9
 //   M 1000, K 2048, N 4096    16.6 /  17.7    M 2048, K 2048, N 2048         15.2 / 15.8
+// and with weights from HBM, waves of either in brackets:
+//   M 320, K 1024, N 32256 (3, 4)  28.2 / 32.5    M 320, K 4096, N 32256 (3, 4)  84.1 / 84.0
+//   M 640, K 4096, gate/up 22016 (3, 4)  78.1 / 81.6
+//   M 4096, K 256, N 2048 (2, 2)  9.8 / 11.6      M 3000, K 768, N 8192 (6, 6)  37.6 / 38.4
+//   M 4096, K 1024, N 2048 (2, 2)  18.9 / 18.1
 bool use_pair(int64_t tiles_m, int64_t tiles, int64_t pair_tiles, int nk, int sms) {
   const int64_t waves = (tiles + sms - 1) / sms, pair_waves = (pair_tiles + sms / 2 - 1) / (sms / 2);
-  return tiles_m > 1 && 20 * pair_waves < 29 * waves && (waves > 1 || nk >= 48);
+  return tiles_m > 1 && 8 * pair_waves <= 9 * waves && nk >= (waves > 1 ? 16 : 48);
 }
 
 template <int EPI>

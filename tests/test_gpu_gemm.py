@@ -203,10 +203,12 @@ def test_gemm_split_kv_heads(fc, orc, batch, n_pad, Hkv, K):
     test_gemm_kv_heads(fc, orc, batch, n_pad, Hkv, K)
 
 
-@pytest.mark.parametrize("M,N,K", [(257, 20000, 136), (300, 39000, 72), (2500, 4104, 200), (1281, 2056, 3080), (129, 19464, 3072)])
+@pytest.mark.parametrize("M,N,K", [(257, 20000, 136), (300, 39000, 72), (2500, 4104, 200), (1281, 2056, 3080), (129, 19464, 3072),
+                                   (390, 39000, 1032), (1410, 9736, 1000), (400, 20008, 960),    # pairs from K 961 on
+                                   (270, 39000, 1032)])                                         # and not with a quarter more waves
 def test_gemm_pair_shapes(fc, M, N, K):
-    """Many tiles: 256 x 256 tiles on pairs of CTAs, over several waves, with
-    ragged rows (a whole half tile past M among them), columns and K."""
+    """Many tiles: 256 x 256 tiles on pairs of CTAs (short K: 128 x 256 on one),
+    over several waves, with ragged rows (a whole half tile past M among them), columns and K."""
     a, b = operands(M, N, K, M + N + K)
     c = torch.full((M + 1, N), float("nan"), dtype=torch.bfloat16, device="cuda")
     fc.fc_gemm_bf16(a, b, out=c[:M])
@@ -216,19 +218,19 @@ def test_gemm_pair_shapes(fc, M, N, K):
     assert torch.isnan(c[M]).all()
 
 
-@pytest.mark.parametrize("M,K,inter", [(390, 200, 11008), (1100, 3080, 384)])
+@pytest.mark.parametrize("M,K,inter", [(390, 200, 11008), (1100, 3080, 384), (390, 1032, 11008)])
 def test_gemm_pair_silu_mul(fc, M, K, inter):
     test_gemm_silu_mul(fc, M, K, inter)
 
 
-@pytest.mark.parametrize("batch,n_pad,Hkv,K", [(5, 128, 33, 200), (9, 64, 5, 3080)])
+@pytest.mark.parametrize("batch,n_pad,Hkv,K", [(5, 128, 33, 200), (9, 64, 5, 3080), (5, 128, 33, 1032)])
 def test_gemm_pair_kv_heads(fc, orc, batch, n_pad, Hkv, K):
     test_gemm_kv_heads(fc, orc, batch, n_pad, Hkv, K)
 
 
 @pytest.mark.parametrize("batch,n_pad,H,Hkv,K", [
     (1, 64, 2, 1, 4104), (1, 64, 4, 2, 1032), (1, 64, 16, 16, 2048), (3, 40, 2, 3, 520),  # clusters of 8, 4, 3 and 2
-    (5, 64, 2, 3, 256), (2, 128, 32, 8, 4096), (5, 128, 34, 33, 200),                     # whole tiles, single and paired
+    (5, 64, 2, 3, 256), (2, 128, 32, 8, 4096), (5, 128, 34, 33, 200), (5, 128, 34, 33, 1032),  # whole tiles, single and paired
     (1, 64, 3, 1, 520),                                                                   # an odd H: two launches
 ])
 def test_gemm_qkv(fc, orc, batch, n_pad, H, Hkv, K):

@@ -93,7 +93,7 @@ struct AttnArgs {
   float* ws_o;     // [split units][parts][256 rows][128]: unnormalised O of a partial, by part
   // spread launches (fewer row chunks than SMs; ws_ml and ws_o then have one slot per CTA):
   int2* ws_plan;   // [units]: the unit's first CTA and how many CTAs share its keys
-  int min_cost;    // the least work of one CTA, in quarter blocks of a two-tile chunk
+  int min_cost;    // the least work of one CTA, in eighths of a block of a two-tile chunk
   unsigned int* err;  // the launch's error word (NULL: this file's own)
   float scale_log2;
   const int32_t* pos;  // [B][n_pad] node positions: rotate Q by them (RoPE), or nullptr
@@ -222,71 +222,96 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // Spread launches: with U units on P SMs and U well below P, one CTA per
 // unit leaves most of the GPU idle, so the launch has P CTAs and every unit's
 // KV blocks are shared by as many of them as its work asks for.  The lengths
-// live on the device, so each warp works the same plan out for itself: the
+// live on the device, so a warp of each CTA works the same plan out: the
 // smallest work per CTA, T, for which the units' shares max(1, ceil(cost / T))
-// fit the P CTAs; CTAs are then dealt to the units in order.  A two-tile block
-// costs 4, a one-tile block 3 (1.6 against 1.2 us, measured).  With `sum` the
+// fit the P CTAs; CTAs are then dealt to the units in order.  The Hkv units of
+// a row chunk are alike, so the plan is made of row chunks.  A two-tile block
+// costs 8, a one-tile block 5 (1.54 against 0.94 us, measured).  With `sum` the
 // units' whole cost, T >= sum / P, and T = sum / (P - U) always fits: the 32
 // lanes try 32 values between the two at once (a bisection by the whole warp
 // took 1.5 us longer, on every launch's critical path).
-constexpr int SPREAD_LANE_UNITS = 3;  // units per lane: launches of up to 96 units
-constexpr int SPREAD_MAX_UNITS = 32 * SPREAD_LANE_UNITS;
+// Sharing has to save more than the merge takes (SPREAD_MERGE_COST and the
+// partial sums on their way through L2, a tile's rows of a part
+// 1 / SPREAD_MERGE_TILES); else every unit has a CTA of its own, and the launch
+// costs 1.5 to 2 us more than one that is not spread: the lengths are not known
+// when it is made.  us, a CTA each / spread, 64 one-tile units: 64 keys 7.8 /
+// 9.5, 1200 keys 15.9 / 16.0, 3200 31.2 / 26.3 (with all shared that could be
+// and a merge of 1024 CTAs: 13.0, 20.2, 30.4); 32 two-tile units: 400 keys 16.7 /
+// 17.4, 1200 25.8 / 19.3, 16000 205 / 67.
+constexpr int SPREAD_LANE_CHUNKS = 3;  // row chunks per lane
+constexpr int SPREAD_MAX_UNITS = 32 * SPREAD_LANE_CHUNKS;
+constexpr float SPREAD_MERGE_COST = 10.f, SPREAD_MERGE_TILES = 14.f;
 struct SpreadPlan {
   int unit, part, nparts;  // unit = -1: nothing left for this CTA
+  bool shared;             // some unit of the launch has more than one CTA
 };
-__device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a, int units) {
-  const int lane = threadIdx.x & 31, P = (int)gridDim.x;
-  float cost[SPREAD_LANE_UNITS], sum = 0.f, top = 0.f;
+__device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a) {
+  const int lane = threadIdx.x & 31, P = (int)gridDim.x, me = (int)blockIdx.x, chunks = a.B * a.ctas;
+  float cost[SPREAD_LANE_CHUNKS];  // negative: of a two-tile chunk
+  uint32_t sum = 0, top = 0;
 #pragma unroll
-  for (int k = 0; k < SPREAD_LANE_UNITS; ++k) {
-    const int u = k * 32 + lane;
-    cost[k] = 0.f;  // no work: one CTA writes the zero rows
-    if (u < units) {
-      const int bg = u / a.ctas, b = bg / a.Hkv;
-      const int nn = a.n_nodes[b], kvl = a.kv_len[b];
-      const int rows = a.G * nn - (u - bg * a.ctas) * (TILES * BM);  // this unit's rows and the later ones'
-      if (nn >= 1 && nn <= a.n_pad && kvl >= 0 && kvl <= a.kv_cap && rows > 0)
-        cost[k] = (float)(((kvl + BN - 1) / BN + 1) * (rows > BM ? 4 : 3));
+  for (int k = 0; k < SPREAD_LANE_CHUNKS; ++k) {
+    const int j = k * 32 + lane;
+    uint32_t c = 0;  // no work: one CTA writes the zero rows
+    bool two = false;
+    if (j < chunks) {
+      const int b = j / a.ctas, nn = a.n_nodes[b], kvl = a.kv_len[b];
+      const int rows = a.G * nn - (j - b * a.ctas) * (TILES * BM);  // this chunk's rows and the later ones'
+      if (nn >= 1 && nn <= a.n_pad && kvl >= 0 && kvl <= a.kv_cap && rows > 0) {
+        c = min((uint32_t)((kvl + BN - 1) / BN + 1), 1u << 21) * (rows > BM ? 8u : 5u);  // (96 of them fit 32 bits)
+        two = rows > BM;
+      }
     }
-    sum += cost[k];
-    top = fmaxf(top, cost[k]);
+    cost[k] = two ? -(float)c : (float)c;
+    sum += c;
+    top = max(top, c);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-    top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
-  }
-  const float lo = fmaxf((float)a.min_cost, sum / (float)P), hi = fmaxf(lo, sum / (float)(P - units));
+  sum = __reduce_add_sync(0xFFFFFFFFu, sum) * (uint32_t)a.Hkv;
+  top = __reduce_max_sync(0xFFFFFFFFu, top);
+  const float lo = fmaxf((float)a.min_cost, (float)sum / (float)P);
+  // a share never exceeds the unit's blocks: a block costs at most 8 <= min_cost <= T
+  auto share = [](float c, float inv) { return fmaxf(1.f, ceilf(fabsf(c) * inv - 1e-3f)); };
+  const int units = chunks * a.Hkv;
+  SpreadPlan p{me < units ? me : -1, 0, 1, false};  // a CTA per unit
+  if ((float)top <= lo + SPREAD_MERGE_COST) return p;
+  const float hi = fmaxf(lo, (float)sum / (float)(P - units));
   const float mine = lo + (hi - lo) * ((float)lane * (1.f / 31.f));
-  // a share never exceeds the unit's blocks: a block costs at most 4 <= min_cost <= T
-  auto share = [](float c, float inv) { return fmaxf(1.f, ceilf(c * inv - 1e-3f)); };
-  float inv = 1.f / mine, used = 0.f;
+  float inv = 1.f / mine, used = 0.f, partials = 0.f;  // CTAs; tiles whose rows the merge reads
 #pragma unroll
-  for (int k = 0; k < SPREAD_LANE_UNITS; ++k) {
-    const int here = min(32, units - 32 * k);
-    for (int u = 0; u < here; ++u) used += share(__shfl_sync(0xFFFFFFFFu, cost[k], u), inv);
+  for (int k = 0; k < SPREAD_LANE_CHUNKS; ++k) {
+    const int here = min(32, chunks - 32 * k);
+    for (int j = 0; j < here; ++j) {
+      const float c = __shfl_sync(0xFFFFFFFFu, cost[k], j), n = share(c, inv);
+      used += n;
+      partials += n > 1.f ? (c < 0.f ? 2.f * n : n) : 0.f;
+    }
   }
-  const unsigned fits = __ballot_sync(0xFFFFFFFFu, used <= (float)P);
-  inv = fits ? __shfl_sync(0xFFFFFFFFu, inv, __ffs(fits) - 1) : 1.f / fmaxf(top, 1.f);  // (none: one CTA per unit)
-  SpreadPlan p{-1, 0, 1};
-  int first = 0;  // CTAs of the units before this row of 32
+  const bool pays = (float)top > mine + SPREAD_MERGE_COST + partials * ((float)a.Hkv / SPREAD_MERGE_TILES);
+  const unsigned fits = __ballot_sync(0xFFFFFFFFu, used * (float)a.Hkv <= (float)P);
+  const unsigned worth = __ballot_sync(0xFFFFFFFFu, pays);
+  const int least = max(__ffs(fits) - 1, 0);
+  if (!fits || !(worth >> least & 1u)) return p;  // (the last value fits but for rounding)
+  inv = __shfl_sync(0xFFFFFFFFu, inv, least);
+  p = SpreadPlan{-1, 0, 1, true};
+  int first = 0;  // CTAs of the chunks before this row of 32
 #pragma unroll
-  for (int k = 0; k < SPREAD_LANE_UNITS; ++k) {
-    if (k * 32 >= units) break;
-    const int n = k * 32 + lane < units ? (int)share(cost[k], inv) : 0;
-    int inc = n;
+  for (int k = 0; k < SPREAD_LANE_CHUNKS; ++k) {
+    if (k * 32 >= chunks) break;
+    const int n = k * 32 + lane < chunks ? (int)share(cost[k], inv) : 0;
+    int inc = n * a.Hkv;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
       if (lane >= o) inc += y;
     }
-    const int at = first + inc - n, me = (int)blockIdx.x;  // at: this unit's first CTA
-    const unsigned hit = __ballot_sync(0xFFFFFFFFu, me >= at && me < at + n);
+    const int at = me - (first + inc - n * a.Hkv);  // this CTA among the chunk's
+    const unsigned hit = __ballot_sync(0xFFFFFFFFu, at >= 0 && at < n * a.Hkv);
     if (hit) {
-      const int src = __ffs(hit) - 1;
-      p.unit = k * 32 + src;
+      const int src = __ffs(hit) - 1, j = k * 32 + src, b = j / a.ctas;
       p.nparts = __shfl_sync(0xFFFFFFFFu, n, src);
-      p.part = me - __shfl_sync(0xFFFFFFFFu, at, src);
+      const int g = __shfl_sync(0xFFFFFFFFu, at, src) / p.nparts;
+      p.part = __shfl_sync(0xFFFFFFFFu, at, src) - g * p.nparts;
+      p.unit = (b * a.Hkv + g) * a.ctas + (j - b * a.ctas);
     }
     first += __shfl_sync(0xFFFFFFFFu, inc, 31);
   }
@@ -346,6 +371,7 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ int s_ticket, s_ready;
+  __shared__ SpreadPlan s_plan;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   __shared__ float2 s_rope[ROPE ? HD / 2 : 1];
   if constexpr (ROPE) fc_rope_copy(s_rope, a.rope);  // read behind a barrier below
@@ -364,11 +390,16 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   // (launched last: whole units first, the short split CTAs fill the tail).
   int unit, part, nparts;
   if constexpr (SPREAD) {
-    const SpreadPlan sp = spread_plan(a, a.B * a.Hkv * a.ctas);
-    if (sp.unit < 0) return;
-    unit = sp.unit;
-    part = sp.part;
-    nparts = sp.nparts;
+    if (warp == 0) {
+      const SpreadPlan p = spread_plan(a);
+      if (lane == 0) s_plan = p;
+    }
+    __syncthreads();
+    if (!s_plan.shared) fc_grid_release();  // the merge has nothing to do: its CTAs may come and wait
+    unit = s_plan.unit;
+    part = s_plan.part;
+    nparts = s_plan.nparts;
+    if (unit < 0) return;
     if (part == 0 && tid == 0) a.ws_plan[unit] = make_int2(blockIdx.x, nparts);
   } else if ((int)blockIdx.x < a.u_split) {
     unit = blockIdx.x;
@@ -440,8 +471,8 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   // empty when a unit has fewer blocks than parts.
   const int kb = part * nblk_all / nparts;
   const int nblk = (part + 1) * nblk_all / nparts - kb;
-  int n_contrib = 0;
-  for (int h = 0; h < nparts; ++h) n_contrib += ((h + 1) * nblk_all / nparts > h * nblk_all / nparts);
+  int n_contrib = SPREAD ? nparts : 0;  // (a plan's parts all have blocks)
+  for (int h = SPREAD ? nparts : 0; h < nparts; ++h) n_contrib += ((h + 1) * nblk_all / nparts > h * nblk_all / nparts);
   if (nblk == 0) {
     zero_pad(0, TA_THREADS);
     return;
@@ -937,19 +968,22 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
 }
 
 // The merge of a spread launch: a unit's parts in part order.  One CTA takes
-// MERGE_COLS columns of a unit's rows, one row per thread: a warp's
-// 16-byte loads of a part are consecutive.  Launched as a programmatic
-// dependent of the attention (2 us less than a plain launch); units that one
-// CTA served are already written.  A dependent chain of L2 reads: 8 columns
-// and eight parts a round measured best of {4, 8, 16} x {4, 8}.
+// COLS columns of a unit's rows, one row per thread: a warp's 16-byte loads
+// of a part are consecutive.  Launched as a programmatic dependent of the
+// attention (2 us less than a plain launch); units that one CTA served are
+// already written.  A dependent chain of L2 reads: for few units 8 columns and
+// eight parts a round (best of {4, 8, 16} x {4, 8}); the more units, the fewer
+// parts each has and the more columns a CTA takes, since a launch that finds
+// nothing shared still starts and ends them all (64 one-tile units, 8 / 32
+// columns: 64 keys 11.6 / 9.9 us, 1200 keys 20.4 / 17.8).
 //
 // Spread launches against one CTA per unit (back-to-back calls, three input
 // sets in turn): 8 units of 16384 keys 184 -> 28 us, 32 units of 10-16k keys
 // and 256 rows 178 -> 55 us, 32 one-tile units of 1400-2300 keys 24 -> 18 us,
 // 16 such units 21 -> 14 us.
-constexpr int MERGE_COLS = 8, MERGE_ROUND = 8;
+template <int COLS, int ROUND>
 __global__ void __launch_bounds__(TILES* BM) k_attn_merge(AttnArgs a) {
-  const int unit = blockIdx.y, r = threadIdx.x, col = blockIdx.x * MERGE_COLS;
+  const int unit = blockIdx.y, r = threadIdx.x, col = blockIdx.x * COLS;
   const int bg = unit / a.ctas, c = unit - bg * a.ctas;
   const int b = bg / a.Hkv, g = bg - b * a.Hkv;
   fc_grid_release();
@@ -960,18 +994,18 @@ __global__ void __launch_bounds__(TILES* BM) k_attn_merge(AttnArgs a) {
   const float2* ml = a.ws_ml + (size_t)p.x * (TILES * BM) + r;
   const float4* os = reinterpret_cast<const float4*>(a.ws_o) + (size_t)p.x * (TILES * BM * HD / 4) +
                      (size_t)(col / 4) * (TILES * BM) + r;
-  // parts in rounds of MERGE_ROUND, every load of a round in flight at once
-  FcRowMerge<MERGE_COLS> row;
-  for (int h0 = 0; h0 < p.y; h0 += MERGE_ROUND) {
-    float2 v[MERGE_ROUND];
-    float4 o[MERGE_ROUND][MERGE_COLS / 4];
+  // parts in rounds, every load of a round in flight at once
+  FcRowMerge<COLS> row;
+  for (int h0 = 0; h0 < p.y; h0 += ROUND) {
+    float2 v[ROUND];
+    float4 o[ROUND][COLS / 4];
 #pragma unroll
-    for (int q = 0; q < MERGE_ROUND; ++q) {
+    for (int q = 0; q < ROUND; ++q) {
       v[q] = make_float2(-INFINITY, 0.f);
       if (h0 + q >= p.y) continue;
       v[q] = __ldcg(ml + (h0 + q) * (TILES * BM));
 #pragma unroll
-      for (int u = 0; u < MERGE_COLS / 4; ++u)
+      for (int u = 0; u < COLS / 4; ++u)
         o[q][u] = __ldcg(os + (size_t)(h0 + q) * (TILES * BM * HD / 4) + u * (TILES * BM));
     }
     row.round(v, o, p.y - h0, h0 == 0);
@@ -981,7 +1015,7 @@ __global__ void __launch_bounds__(TILES* BM) k_attn_merge(AttnArgs a) {
   const int hh = rg / nn, i = rg - hh * nn;
   uint2* dst = reinterpret_cast<uint2*>(a.out + (((size_t)b * a.n_pad + i) * a.H + g * a.G + hh) * HD + col);
 #pragma unroll
-  for (int u = 0; u < MERGE_COLS / 4; ++u)
+  for (int u = 0; u < COLS / 4; ++u)
     dst[u] = make_uint2(pack_bf16x2(row.acc[4 * u] * inv, row.acc[4 * u + 1] * inv),
                         pack_bf16x2(row.acc[4 * u + 2] * inv, row.acc[4 * u + 3] * inv));
 }
@@ -1549,12 +1583,12 @@ SplitPlan choose_split(uint64_t units, int kv_cap, size_t ws_bytes) {
   return sp;
 }
 
-// Spread launches (k_tree_attn<., true> and k_attn_merge): at most half as
-// many units as SMs, and caches long enough (SPREAD_MIN_BLOCKS blocks with the
+// Spread launches (k_tree_attn<., MODE_SPREAD> and k_attn_merge): at most half
+// as many units as SMs, and caches that may be long enough (SPREAD_MIN_BLOCKS blocks with the
 // tree's) that sharing a unit's keys pays for the merge launch.  The grid is
 // the CTAs that the SMs and the workspace's slots allow; 0 = not spread.
 constexpr int SPREAD_MIN_BLOCKS = 8;
-constexpr int SPREAD_MIN_COST = 8;  // a CTA's share: two blocks of a two-tile unit
+constexpr int SPREAD_MIN_COST = 16;  // a CTA's share: two blocks of a two-tile unit
 struct SpreadLayout {
   size_t plan, ml, o, total;
 };
@@ -1767,8 +1801,9 @@ static fc_status launch_tree_attn(const void* d_q, const void* d_k_cache, const 
   const fc_status st = fc_launch_dependent(kern, dim3((unsigned)grid), TA_THREADS, smem_bytes,
                                            static_cast<cudaStream_t>(stream), 0, mkc, mvc, mkt, mvt, a);
   if (st != FC_OK || !spread) return st;
-  return fc_launch_dependent(k_attn_merge, dim3(HD / MERGE_COLS, (unsigned)units), TILES * BM, 0,
-                             static_cast<cudaStream_t>(stream), 0, a);
+  const int cols = units <= 18 ? 8 : units <= 38 ? 16 : 32;  // 8, 4 or 2 CTAs and more for a unit
+  return fc_launch_dependent(cols == 8 ? k_attn_merge<8, 8> : cols == 16 ? k_attn_merge<16, 4> : k_attn_merge<32, 2>,
+                             dim3((unsigned)(HD / cols), (unsigned)units), TILES * BM, 0, static_cast<cudaStream_t>(stream), 0, a);
 }
 
 extern "C" fc_status fc_tree_attn(const void* d_q, const void* d_k_cache, const void* d_v_cache, int kv_cap,

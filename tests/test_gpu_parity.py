@@ -587,6 +587,9 @@ def test_attn_kv_split_deterministic(fc):
     (3, 128, 32, 8, 2048, [2048, 1, 128], [128, 40, 1]),                       # second row chunks partly empty
     (4, 128, 16, 1, 900, [900, 899, 640, 641], [128, 64, 17, 16]),             # 16 heads a group: eight chunks
     (76, 64, 1, 1, 1000, [(37 * b) % 1001 for b in range(76)], [1 + (5 * b) % 64 for b in range(76)]),  # the most units
+    (2, 64, 32, 32, 4096, [300, 64], [64, 40]),                                # short in long buffers: nothing is shared
+    (6, 64, 32, 8, 9000, [60, 128, 9000, 700, 0, 2500], [64, 30, 64, 64, 1, 64]),  # two long ones among short ones
+    (2, 128, 32, 4, 3000, [3000, 17], [128, 33]),                              # row chunks shared, alone and without rows
 ])
 def test_attn_spread(fc, orc, B, n_pad, H, Hkv, cap, kv, nn):
     """Launches of at most half as many units as SMs share every unit's keys

@@ -615,7 +615,7 @@ def fc_tree_mask(parent, n_nodes, kv_len):
 
 # --------------------------------------------------------------- attention
 _ATTN_WS = {}        # (device, bytes) -> a workspace of launches that split at most their last wave
-_ATTN_WS_BYTES = {}  # (device, shape) -> (bytes, few row chunks, the shortest caches whose launch is then spread over the GPU)
+_ATTN_WS_SHAPE = {}  # (device, shape) -> (bytes, few row chunks: a template of theirs, the shortest caches whose launch is spread over the GPU)
 
 
 def _shortest_spread(B, Np, H, Hkv, n):
@@ -650,21 +650,23 @@ def attn_workspace(B, Np, H, Hkv, device, kv_cap=None):
     short, where there is no memory, and in a capture that is not torch's.
     Larger launches share a cached workspace per size."""
     key = (device, B, Np, H, Hkv)
-    got = _ATTN_WS_BYTES.get(key)
+    got = _ATTN_WS_SHAPE.get(key)
     if got is None:
         chunks = B * Hkv * -(-(H // Hkv) * Np // 256) if Hkv and H % Hkv == 0 else 0
         sms = torch.cuda.get_device_properties(device).multi_processor_count
         n = max(int(LIB.fc_tree_attn_workspace(B, Np, H, Hkv)), 16)
-        got = _ATTN_WS_BYTES[key] = (n, 2 * chunks <= sms, _shortest_spread(B, Np, H, Hkv, n) if 2 * chunks <= sms else None)
-    n, own, shortest = got
-    if own:
+        few = 2 * chunks <= sms
+        got = _ATTN_WS_SHAPE[key] = (n, torch.empty(1, dtype=torch.uint8, device=device).expand(n) if few else None,
+                                     _shortest_spread(B, Np, H, Hkv, n) if few else None)
+    n, few, shortest = got
+    if few is not None:
         if kv_cap is not None and (shortest is None or kv_cap < shortest):
             return None
         try:
-            ws = torch.empty(n, dtype=torch.uint8, device=device)
+            ws = torch.empty_like(few)  # (1.0 us; torch.empty reads its options for 1.4)
         except torch.cuda.OutOfMemoryError:
             return None
-        return ws if not torch.cuda.is_current_stream_capturing() or _kept_for_replay(ws) else None
+        return None if torch._C._cuda_isCurrentStreamCapturing() and not _kept_for_replay(ws) else ws
     key = (str(device), n)
     if key not in _ATTN_WS:
         _ATTN_WS[key] = torch.empty(n, dtype=torch.uint8, device=device)

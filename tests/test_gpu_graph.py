@@ -135,14 +135,15 @@ def test_small_attention_without_workspace(fc, monkeypatch):
     """Caches too short to share ask for no workspace, and where there is no
     memory for one the call does without."""
     assert fc.attn_workspace(1, 64, 8, 8, "cuda", 768) is None
-    assert fc.attn_workspace(1, 64, 8, 8, "cuda", 769).numel() == fc.LIB.fc_tree_attn_workspace(1, 64, 8, 8)
+    ws = fc.attn_workspace(1, 64, 8, 8, "cuda", 769)
+    assert ws.is_contiguous() and ws.numel() == ws.untyped_storage().nbytes() == fc.LIB.fc_tree_attn_workspace(1, 64, 8, 8)
     args = _small_attn(2000)
     want, out = fc.fc_tree_attn(*args, workspace=None), torch.zeros_like(args[0])
 
     def no_memory(*a, **k):
         raise torch.cuda.OutOfMemoryError("none left")
 
-    monkeypatch.setattr(torch, "empty", no_memory)
+    monkeypatch.setattr(torch, "empty_like", no_memory)
     fc.fc_tree_attn(*args, out=out)
     monkeypatch.undo()
     torch.cuda.synchronize()

@@ -321,14 +321,16 @@ __device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a) {
 // Launches of a few waves of units: the sequence at `place` when the batch is
 // ordered by the work of a row chunk, longest first, so that what runs last is
 // short (and what is split is shorter still).  Lengths live on the device:
-// a warp of each CTA ranks the batch, a sequence or two per lane.
+// every warp of the CTA has the batch in its lanes, a sequence or two each, and
+// ranks its share of it (by one warp 0.6 us more a wave: 512 units of 300 equal
+// keys 82.8 us, now 80.8); the warp that has the sequence writes it.
 struct Seq {
   int b, nn, kvl;  // the sequence, its n_nodes and kv_len as given
 };
 constexpr int ORDER_MAX = 64;  // sequences
-__device__ __forceinline__ Seq work_order(const AttnArgs& a, int place) {
-  const int lane = threadIdx.x & 31;
-  int nn[2], kvl[2], rank[2] = {0, 0};
+__device__ __forceinline__ void work_order(const AttnArgs& a, int place, Seq* out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int nn[2], kvl[2];
   uint32_t key[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -337,23 +339,13 @@ __device__ __forceinline__ Seq work_order(const AttnArgs& a, int place) {
     kvl[h] = b < a.B ? a.kv_len[b] : 0;
     const bool none = nn[h] < 1 || nn[h] > a.n_pad || kvl[h] < 0 || kvl[h] > a.kv_cap;
     const uint32_t cost = none ? 0u : (uint32_t)((kvl[h] + BN - 1) / BN + 1) * (a.G * nn[h] > BM ? 4u : 3u);
-    key[h] = (min(cost, (1u << 26) - 1) << 6) | (uint32_t)(ORDER_MAX - 1 - b);  // distinct
+    key[h] = (min(cost, (1u << 26) - 1) << 6) | (uint32_t)(ORDER_MAX - 1 - b);  // distinct, and past the batch the last
   }
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    if (h && a.B <= 32) break;
-#pragma unroll
-    for (int l = 0; l < 32; ++l) {
-      const uint32_t k = __shfl_sync(0xFFFFFFFFu, key[h], l);
-      rank[0] += k > key[0];
-      rank[1] += k > key[1];
-    }
+  for (int b = warp; b < a.B; b += TA_THREADS / 32) {
+    const uint32_t k = __shfl_sync(0xFFFFFFFFu, b < 32 ? key[0] : key[1], b & 31);
+    const int ahead = __popc(__ballot_sync(0xFFFFFFFFu, key[0] > k)) + __popc(__ballot_sync(0xFFFFFFFFu, key[1] > k));
+    if (ahead == place && lane == (b & 31)) *out = b < 32 ? Seq{b, nn[0], kvl[0]} : Seq{b, nn[1], kvl[1]};
   }
-  const unsigned lo = __ballot_sync(0xFFFFFFFFu, lane < a.B && rank[0] == place);
-  const unsigned hi = __ballot_sync(0xFFFFFFFFu, lane + 32 < a.B && rank[1] == place);
-  const int src = __ffs(lo ? lo : hi) - 1;
-  return {src + (lo ? 0 : 32), __shfl_sync(0xFFFFFFFFu, lo ? nn[0] : nn[1], src),
-          __shfl_sync(0xFFFFFFFFu, lo ? kvl[0] : kvl[1], src)};
 }
 
 // ROPE: the queries arrive unrotated and are rotated by a.pos while staged
@@ -419,10 +411,7 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   int nn_raw, kvl;
   if constexpr (MODE == MODE_ORDERED) {
     __shared__ Seq s_seq;
-    if (warp == 0) {
-      const Seq seq = work_order(a, b);
-      if (lane == 0) s_seq = seq;
-    }
+    work_order(a, b, &s_seq);
     __syncthreads();
     b = s_seq.b;
     bg = b * a.Hkv + g;
@@ -1629,12 +1618,15 @@ bool use_stream(uint64_t units, int G, int n_pad, int kv_cap, bool rope) {
 
 // Whether a launch's sequences run longest first: from a little over one wave
 // of units to four (us per launch, in order / longest first, trees and caches
-// of mixed sizes: 256 units of two tiles and 16384 keys 362 / 316, 320 of 16384
-// 359 / 309, 512 of 16384 569 / 546, 512 of 9000 346 / 329; more waves even out
-// by themselves, 768 of 6000 349 / 351).  The ranking costs a CTA 0.6 to 1.4 us:
-// caches of 8192 keys and more (equal lengths: 256 units of 8192 keys 221 / 222,
-// 512 of 4096 240 / 245), and units of two tiles (one-tile units are bound by
-// the K/V stream: 149 / 155).
+// of mixed sizes: 256 units of two tiles and 16384 keys 404 / 345, 384 of 16384
+// 521 / 462, 512 of 16384 649 / 623; more waves even out by themselves, 768 of
+// 6000 349 / 351).  Over 134 mixed launches of 192 to 512 units and buffers of
+// 8192 to 16384 keys, half of them filled to a tenth, 4% less time; the worst
+// took 7% more (512 units of 400 to 1000 keys, 86 / 92: an order that happened
+// to be good).  With nothing to gain the ranking costs 0.8 us a wave: caches of
+// 8192 keys and more (equal lengths: 512 units of 300 keys 78.2 / 80.8, of 1000
+// 104.0 / 106.4, of 4000 237 / 239), and units of two tiles (one-tile units are
+// bound by the K/V stream: 149 / 155).
 constexpr uint64_t ORDER_MIN_BLOCKS = 64;
 bool use_order(int batch, uint64_t units, int rows, int kv_cap) {
   const uint64_t sms = (uint64_t)sm_count();

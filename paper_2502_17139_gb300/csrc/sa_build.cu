@@ -595,6 +595,7 @@ struct Counts {  // device counters
   uint32_t flag, groups;     // bad token; doubling's number of ranks
   uint32_t small[3], mid[3];  // list elements and ranges: a round reads one, fills the next, clears the third
   uint32_t huge[2], total;
+  unsigned long long mid_work;  // suffixes sorted by k_refine_mid so far
 };
 
 // Exclusive sum over the block; *total = the whole sum (warps of 32, up to 32 of them).
@@ -841,6 +842,7 @@ __device__ __forceinline__ void mid_range(const Range g, const MidShared sh, int
                                           uint64_t n, Sym y, uint32_t* sa, uint8_t* __restrict__ lcp, Range* next, Elem* small,
                                           Counts* ct, int out) {
   const int lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) atomicAdd(&ct->mid_work, (unsigned long long)g.size);
   uint32_t p2 = 64;
   while (p2 < g.size) p2 *= 2;
   for (uint32_t i = tid; i < p2; i += NT) {
@@ -1162,13 +1164,19 @@ extern "C" fc_status fc_datastore_build(const uint32_t* d_tokens, uint64_t n, ui
   // Rounds of y.count more tokens over the rest.
   const int sms = std::max(1, sm_count());
   int round = 0, check = 0;
+  unsigned long long mid_before = 0;  // mid_work after the first two rounds
   while (!doubling) {
     const int in = round % 3;
     if (round == check) {
       if (round && !read_counts()) return FC_ERR_CUDA;
       if (hc.small[in] == 0 && hc.mid[in] == 0) break;
-      // most suffixes still together after six rounds, or repeats of more than about 130 tokens
-      if (round >= 32 || (round >= 6 && hc.small[in] > n / 4)) {
+      if (round == 2) mid_before = hc.mid_work;
+      // Most suffixes still together after six rounds, or 34 rounds; or mid ranges that stay (a text of hundreds of
+      // tokens in many copies): sorting n / 2 suffixes of theirs takes as long as a round of doubling.  5M tokens, ms,
+      // doubling from the start / without this line / n suffixes / n / 2 / n / 4: 3000 copies of 200 tokens 5.2 / 5.7 /
+      // 4.3 / 4.3 / 3.8, of 100 4.6 / 3.2 / 3.2 / 3.3 / 3.1, 100 of 3000 8.0 / 8.6 / 8.4 / 6.9 / 6.6; 50M tokens, 3000
+      // of 400 73 / 32 / 32 / 31 / 35.
+      if (round >= 32 || (round >= 6 && (hc.small[in] > n / 4 || (hc.mid[in] && hc.mid_work - mid_before > n / 2)))) {
         doubling = true;
         break;
       }

@@ -94,6 +94,11 @@ def _sa_corpus(kind):
         n = int(kind[5:])
         t = z((n + 1) // 2, 5000)
         return np.concatenate([t, t])[:n], 5000
+    if kind == "copies":  # 60 copies of 400 tokens: ranges of 33 to 4096 suffixes that stay, then doubling
+        t, text = z(60_000, 5000), rng.integers(0, 5000, 400)
+        for at in range(60):
+            t[1000 * at:1000 * at + 400] = text
+        return t, 5000
     if kind == "long_repeats":  # repeats of 140 to 1000 tokens among others: doubling for a few
         t = z(60_000, 5000)
         for ln in (140, 300, 1000, 129, 133):
@@ -107,7 +112,7 @@ def _sa_corpus(kind):
 
 @pytest.mark.parametrize("kind", ["zipf", "sparse_vocab", "eight_bits", "tile_edges", "equal_pairs", "twice", "twice_odd", "long_repeats",
                                   "periodic", "one_token", "group_edges", "1", "33", "8191", "8192", "8193",
-                                  "flags4097", "flags4104", "flags65528", "flags65535"])
+                                  "flags4097", "flags4104", "flags65528", "flags65535", "copies"])
 def test_sa_build_paths(fc, orc, kind):
     """Corpora whose ranges of equal keys take each path of the refinement."""
     T, vocab = _sa_corpus(kind)

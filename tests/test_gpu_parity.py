@@ -99,7 +99,11 @@ def _sa_corpus(kind):
         for at in range(60):
             t[1000 * at:1000 * at + 400] = text
         return t, 5000
-    if kind == "long_repeats":  # repeats of 140 to 1000 tokens among others: doubling for a few
+    if kind == "longest_repeat":  # more than 34 rounds of 32 times 4 tokens for a few suffixes: then doubling, from their list
+        t = z(60_000, 5000)
+        t[40_000:46_000] = t[10_000:16_000]
+        return t, 5000
+    if kind == "long_repeats":  # repeats of 140 to 1000 tokens among others: many rounds of small ranges
         t = z(60_000, 5000)
         for ln in (140, 300, 1000, 129, 133):
             a, b = rng.integers(0, 29_000), rng.integers(30_000, 59_000 - ln)
@@ -112,7 +116,7 @@ def _sa_corpus(kind):
 
 @pytest.mark.parametrize("kind", ["zipf", "sparse_vocab", "eight_bits", "tile_edges", "equal_pairs", "twice", "twice_odd", "long_repeats",
                                   "periodic", "one_token", "group_edges", "1", "33", "8191", "8192", "8193",
-                                  "flags4097", "flags4104", "flags65528", "flags65535", "copies"])
+                                  "flags4097", "flags4104", "flags65528", "flags65535", "copies", "longest_repeat"])
 def test_sa_build_paths(fc, orc, kind):
     """Corpora whose ranges of equal keys take each path of the refinement."""
     T, vocab = _sa_corpus(kind)

@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_retrieve(DsArgs args, DsArgs rev
   }
   if (sm.bad && tid == 0) fc_flag(FC_ERR_WORD(o.err), FC_EBIT_INVALID);
 
-  // ---- search: one warp per n, one half-warp per bound, 16 pivots a round
+  // ---- search: one warp per n, 32 pivots a round until one matches, then a half-warp per bound
   // (lengths n_top down to n_top - n_count + 1; with the reversed corpus only n*)
   int n_top = cap, n_count = (cap >= p.n_min && !sm.bad) ? cap - p.n_min + 1 : 0;
   if constexpr (REV) {

@@ -15,10 +15,23 @@
 //   * longer: the ranges' suffixes are gathered and go through the radix sort
 //     again, (range, next tokens) as the key.
 // Where a range splits, its two neighbours' first different token is their
-// common prefix, so the LCP array comes out of the same comparisons.  Corpora
-// with repeats of more than about 130 tokens end with prefix doubling: after a
-// round at h every position carries the dense rank of its first h tokens, and
-// sorting by (rank[i], rank[i + h] + 1) gives the ranks of the first 2h.
+// common prefix, so the LCP array comes out of the same comparisons.
+//
+// What the rounds do not resolve ends with prefix doubling over all positions:
+// after a round at h every position carries the dense rank of its first h
+// tokens (of h or more: ranges that were refined further keep their places),
+// and sorting by (rank[i], rank[i + h] + 1) gives the ranks of the first 2h.
+// With k tokens a key, that is where
+//   * the ranges of more than 4096 suffixes do not halve from one round to the
+//     next: a text of more than k or 2k tokens in more than 4096 copies, from
+//     h = k on (5M tokens, 5000 copies of 16: 2.6 ms where doubling from the
+//     start takes 3.2 and a corpus without them 0.94; 20M, 100000 of 40: 11.6,
+//     15.2);
+//   * after six rounds a quarter of the suffixes is still in small ranges, or
+//     mid ranges have taken n / 2 suffixes through their sort (33 to 4096
+//     copies of long texts);
+//   * 34 rounds have gone: k tokens each in mid ranges, 8 k to 32 k in small ones
+//     (2 to 32 copies of more than about 1000 to 4300 tokens at k = 4).
 //
 // Bound by HBM: the radix passes stream 32 bytes a position each, the rounds
 // gather the text of the suffixes still in play.  Doubling from the start sorts
@@ -454,9 +467,11 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(uint32_t* __restric
   }
 }
 
-// Up to SC_MAX numbers by one cluster of eight CTAs, each with a stretch of them:
-// one launch instead of three (a build of 1M tokens, with eight such scans of
-// 63k: 463 -> 450 us).
+// Up to SC_MAX numbers by one cluster of eight CTAs (the most that is portable),
+// each with a stretch of them: one launch instead of three (a build of 1M
+// tokens, with eight such scans of 63k: 463 -> 450 us).  Eight numbers a thread
+// are two 16-byte loads in flight; the digit counts of 1M tokens just fit, and
+// those of more take three launches, each over the whole GPU.
 constexpr int SC_CTAS = 8, SC_ITEMS = 8, SC_MAX = SC_CTAS * SCAN_THREADS * SC_ITEMS;
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_cluster(uint32_t* data, uint32_t n) {
   __shared__ uint32_t s_tot;
@@ -1135,7 +1150,7 @@ extern "C" fc_status fc_datastore_build(const uint32_t* d_tokens, uint64_t n, ui
   int hin = 0;
   uint64_t before = ~0ull;
   bool doubling = false;
-  uint64_t h = (uint64_t)y.count;  // tokens that every range is known to share
+  uint64_t h = (uint64_t)y.count;  // tokens that every range is known to share (some share more)
   for (;;) {
     k_huge_base<<<1, SCAN_THREADS, 0, s>>>(huges[hin], ct, hin);
     if (!read_counts()) return FC_ERR_CUDA;

@@ -517,8 +517,8 @@ fc_status fc_tree_mask(const int32_t* d_parent, const int32_t* d_n_nodes, const 
  *             fc_tree_attn_workspace() bytes the call may split each row
  *             chunk's keys over up to 4 CTAs (so that the grid fills the GPU
  *             in whole waves), or, when there are few row chunks, over as many
- *             as fill the GPU, and merge their partial softmax sums; with less
- *             it uses fewer parts.  Owned by the caller, no initial contents
+ *             as fill the GPU (where the lengths make that pay), and merge
+ *             their partial softmax sums; with less it uses fewer parts.  Owned by the caller, no initial contents
  *             needed (the call clears its counters on the stream first).
  *             Concurrent calls on different streams need separate workspaces.
  * Supported: D = 128, n_pad in {64, 128}, H % Hkv == 0, H / Hkv <= 16,
@@ -549,7 +549,8 @@ int fc_tree_attn_streamed(int batch, int n_pad, int H, int Hkv, int kv_cap);
 /* How many parts fc_tree_attn splits each row chunk's keys into for this
  * shape and workspace size on the current device (1 = no split; 0 for an
  * unsupported shape; with few row chunks the device deals its CTAs out by the
- * lengths, and this is their mean per chunk, rounded up).  Host-only, launches nothing. */
+ * lengths, and this is their mean per chunk, rounded up; over short caches it
+ * leaves each chunk one CTA).  Host-only, launches nothing. */
 int fc_tree_attn_parts(int batch, int n_pad, int H, int Hkv, int kv_cap, size_t ws_bytes);
 
 /* ------------------------------------------------------------------------

@@ -243,7 +243,6 @@ constexpr int SPREAD_MAX_UNITS = 32 * SPREAD_LANE_CHUNKS;
 constexpr float SPREAD_MERGE_COST = 10.f, SPREAD_MERGE_TILES = 14.f;
 struct SpreadPlan {
   int unit, part, nparts;  // unit = -1: nothing left for this CTA
-  bool shared;             // some unit of the launch has more than one CTA
 };
 __device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a) {
   const int lane = threadIdx.x & 31, P = (int)gridDim.x, me = (int)blockIdx.x, chunks = a.B * a.ctas;
@@ -272,7 +271,7 @@ __device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a) {
   // a share never exceeds the unit's blocks: a block costs at most 8 <= min_cost <= T
   auto share = [](float c, float inv) { return fmaxf(1.f, ceilf(fabsf(c) * inv - 1e-3f)); };
   const int units = chunks * a.Hkv;
-  SpreadPlan p{me < units ? me : -1, 0, 1, false};  // a CTA per unit
+  SpreadPlan p{me < units ? me : -1, 0, 1};  // a CTA per unit
   if ((float)top <= lo + SPREAD_MERGE_COST) return p;
   const float hi = fmaxf(lo, (float)sum / (float)(P - units));
   const float mine = lo + (hi - lo) * ((float)lane * (1.f / 31.f));
@@ -292,7 +291,7 @@ __device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a) {
   const int least = max(__ffs(fits) - 1, 0);
   if (!fits || !(worth >> least & 1u)) return p;  // (the last value fits but for rounding)
   inv = __shfl_sync(0xFFFFFFFFu, inv, least);
-  p = SpreadPlan{-1, 0, 1, true};
+  p.unit = -1;
   int first = 0;  // CTAs of the chunks before this row of 32
 #pragma unroll
   for (int k = 0; k < SPREAD_LANE_CHUNKS; ++k) {
@@ -387,7 +386,6 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
       if (lane == 0) s_plan = p;
     }
     __syncthreads();
-    if (!s_plan.shared) fc_grid_release();  // the merge has nothing to do: its CTAs may come and wait
     unit = s_plan.unit;
     part = s_plan.part;
     nparts = s_plan.nparts;

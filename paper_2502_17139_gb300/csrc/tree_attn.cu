@@ -222,14 +222,15 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // Spread launches: with U units on P SMs and U well below P, one CTA per
 // unit leaves most of the GPU idle, so the launch has P CTAs and every unit's
 // KV blocks are shared by as many of them as its work asks for.  The lengths
-// live on the device, so a warp of each CTA works the same plan out: the
+// live on the device, so each warp works the same plan out for itself: the
 // smallest work per CTA, T, for which the units' shares max(1, ceil(cost / T))
 // fit the P CTAs; CTAs are then dealt to the units in order.  The Hkv units of
 // a row chunk are alike, so the plan is made of row chunks.  A two-tile block
 // costs 8, a one-tile block 5 (1.54 against 0.94 us, measured).  With `sum` the
 // units' whole cost, T >= sum / P, and T = sum / (P - U) always fits: the 32
 // lanes try 32 values between the two at once (a bisection by the whole warp
-// took 1.5 us longer, on every launch's critical path).
+// took 1.5 us longer, on every launch's critical path; one warp planning for
+// the CTA 0.3 us, and 1.3 in the decoder behind its projections).
 // Sharing has to save more than the merge takes (SPREAD_MERGE_COST and the
 // partial sums on their way through L2, a tile's rows of a part
 // 1 / SPREAD_MERGE_TILES); else every unit has a CTA of its own, and the launch
@@ -362,7 +363,6 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ int s_ticket, s_ready;
-  __shared__ SpreadPlan s_plan;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   __shared__ float2 s_rope[ROPE ? HD / 2 : 1];
   if constexpr (ROPE) fc_rope_copy(s_rope, a.rope);  // read behind a barrier below
@@ -381,14 +381,10 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
   // (launched last: whole units first, the short split CTAs fill the tail).
   int unit, part, nparts;
   if constexpr (SPREAD) {
-    if (warp == 0) {
-      const SpreadPlan p = spread_plan(a);
-      if (lane == 0) s_plan = p;
-    }
-    __syncthreads();
-    unit = s_plan.unit;
-    part = s_plan.part;
-    nparts = s_plan.nparts;
+    const SpreadPlan sp = spread_plan(a);
+    unit = sp.unit;
+    part = sp.part;
+    nparts = sp.nparts;
     if (unit < 0) return;
     if (part == 0 && tid == 0) a.ws_plan[unit] = make_int2(blockIdx.x, nparts);
   } else if ((int)blockIdx.x < a.u_split) {

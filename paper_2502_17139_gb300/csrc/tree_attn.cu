@@ -226,14 +226,15 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // smallest work per CTA, T, for which the units' shares max(1, ceil(cost / T))
 // fit the P CTAs; CTAs are then dealt to the units in order.  The Hkv units of
 // a row chunk are alike, so the plan is made of row chunks.  A two-tile block
-// costs 8, a one-tile block 5 (1.54 against 0.94 us, measured).  With `sum` the
+// costs 8, a one-tile block 6.  With `sum` the
 // units' whole cost, T >= sum / P, and T = sum / (P - U) always fits: the 32
 // lanes try 32 values between the two at once (a bisection by the whole warp
 // took 1.5 us longer, on every launch's critical path; one warp planning for
 // the CTA 0.3 us, and 1.3 in the decoder behind its projections).
-// Sharing has to save more than the merge takes (SPREAD_MERGE_COST and the
+// Sharing has to save more time than the merge takes (SPREAD_MERGE_COST and the
 // partial sums on their way through L2, a tile's rows of a part
-// 1 / SPREAD_MERGE_TILES); else every unit has a CTA of its own, and the launch
+// 1 / SPREAD_MERGE_TILES; in eighths of a two-tile block's 1.54 us, a one-tile
+// block's 0.94 being 5 of them); else every unit has a CTA of its own, and the launch
 // costs 1.5 to 2 us more than one that is not spread: the lengths are not known
 // when it is made.  us, a CTA each / spread, 64 one-tile units: 64 keys 7.8 /
 // 9.5, 1200 keys 15.9 / 16.0, 3200 31.2 / 26.3 (with all shared that could be
@@ -249,6 +250,7 @@ __device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a) {
   const int lane = threadIdx.x & 31, P = (int)gridDim.x, me = (int)blockIdx.x, chunks = a.B * a.ctas;
   float cost[SPREAD_LANE_CHUNKS];  // negative: of a two-tile chunk
   uint32_t sum = 0, top = 0;
+  bool two_tiles = false;
 #pragma unroll
   for (int k = 0; k < SPREAD_LANE_CHUNKS; ++k) {
     const int j = k * 32 + lane;
@@ -258,11 +260,12 @@ __device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a) {
       const int b = j / a.ctas, nn = a.n_nodes[b], kvl = a.kv_len[b];
       const int rows = a.G * nn - (j - b * a.ctas) * (TILES * BM);  // this chunk's rows and the later ones'
       if (nn >= 1 && nn <= a.n_pad && kvl >= 0 && kvl <= a.kv_cap && rows > 0) {
-        c = min((uint32_t)((kvl + BN - 1) / BN + 1), 1u << 21) * (rows > BM ? 8u : 5u);  // (96 of them fit 32 bits)
+        c = min((uint32_t)((kvl + BN - 1) / BN + 1), 1u << 21) * (rows > BM ? 8u : 6u);  // (96 of them fit 32 bits)
         two = rows > BM;
       }
     }
     cost[k] = two ? -(float)c : (float)c;
+    two_tiles = two_tiles || two;
     sum += c;
     top = max(top, c);
   }
@@ -273,7 +276,9 @@ __device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a) {
   auto share = [](float c, float inv) { return fmaxf(1.f, ceilf(fabsf(c) * inv - 1e-3f)); };
   const int units = chunks * a.Hkv;
   SpreadPlan p{me < units ? me : -1, 0, 1};  // a CTA per unit
-  if ((float)top <= lo + SPREAD_MERGE_COST) return p;
+  // the time of a unit of cost: the longest chunk's, which two tiles decide where any chunk has them
+  const float unit_time = __any_sync(0xFFFFFFFFu, two_tiles) ? 1.f : 5.f / 6.f;
+  if (((float)top - lo) * unit_time <= SPREAD_MERGE_COST) return p;
   const float hi = fmaxf(lo, (float)sum / (float)(P - units));
   const float mine = lo + (hi - lo) * ((float)lane * (1.f / 31.f));
   float inv = 1.f / mine, used = 0.f, partials = 0.f;  // CTAs; tiles whose rows the merge reads
@@ -286,7 +291,7 @@ __device__ __forceinline__ SpreadPlan spread_plan(const AttnArgs& a) {
       partials += n > 1.f ? (c < 0.f ? 2.f * n : n) : 0.f;
     }
   }
-  const bool pays = (float)top > mine + SPREAD_MERGE_COST + partials * ((float)a.Hkv / SPREAD_MERGE_TILES);
+  const bool pays = ((float)top - mine) * unit_time > SPREAD_MERGE_COST + partials * ((float)a.Hkv / SPREAD_MERGE_TILES);
   const unsigned fits = __ballot_sync(0xFFFFFFFFu, used * (float)a.Hkv <= (float)P);
   const unsigned worth = __ballot_sync(0xFFFFFFFFu, pays);
   const int least = max(__ffs(fits) - 1, 0);

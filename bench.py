@@ -56,9 +56,9 @@ UNIT = "steps/s"
 # ratio x the algorithmic bytes per launch of its own launches.  The ratio is valid
 # only for the kernel sources it was taken on (their SHA-256 below); otherwise the
 # bench reports traffic as null until it is measured again.
-ATTN_TRAFFIC = {"ratio": 1.0662,
+ATTN_TRAFFIC = {"ratio": 1.0665,
                 "sources": ["paper_2502_17139_gb300/csrc/tree_attn.cu", "paper_2502_17139_gb300/csrc/fc_common.cuh"],
-                "sha256": "b9c61e2a9b5b793d523c8d7ee67b6dce7748f874a90dc27f1a30d7d29bca3eb1"}
+                "sha256": "9b943c02c73fd894284c1eec364e8403e233c2a3879e79d0a6a3591d73d6e6c8"}
 
 WORKLOAD = ("full step loop: two-source datastore 100M (Zipf 1.1) + 5M (Zipf 1.3, 20k planted repeats) tokens, "
             "vocab 32256, batch 32, ctx 128, n 16->2, top-64 x 10 tokens per source, tree <=128 nodes, "
